@@ -58,8 +58,8 @@ typedef enum {
     BISP_PREC_FP32 = 0,     /* FP32 transforms, products and sums ("plain")                */
     BISP_PREC_MIXED = 1,    /* FP32 transforms and products, FP64 sums and binning         */
     BISP_PREC_FP64 = 2,     /* FP64 throughout (verification)                               */
-    BISP_PREC_MIXED_TC = 3  /* as MIXED, with the triple sums on the tensor cores: TF32     */
-                            /* mma with each FP32 operand split into two TF32 parts        */
+    BISP_PREC_MIXED_TC = 3  /* as MIXED, with the triple sums on the tensor cores: FP16     */
+                            /* mma with each (scaled) FP32 operand split into two parts    */
 } bisp_precision;
 
 /* Opaque plan: ring tables, triangle counts, combination tables, bin

@@ -88,8 +88,9 @@ struct bisp_plan {
     // off_status: one int, set by a Step-II block of this field whose bounded
     // wait ran out; cleared at the start of every estimate
     // off_epi: the binning's partial sums per chunk
+    // off_scale: the power-of-two factors of the stored fields (tensor-core plans)
     size_t off_a = 0, off_b = 0, off_gt = 0, off_dstore = 0, off_part = 0, off_S = 0, off_status = 0, off_epi = 0,
-           region_bytes = 0;
+           off_scale = 0, region_bytes = 0;
     int wait_spins = kDefaultWaitSpins;  // bound of the tensor-core Step II's abortable waits
     int device = -1;                     // the device the plan's tables live on
     int last_field = 0;                  // field of the last estimate that introspection reads
@@ -671,6 +672,8 @@ int build_plan(bisp_plan *p, const bisp_desc *desc, cudaStream_t s)
     p->off_S = o; o = align256(o + size_t(P.n_combos) * sizeof(double));
     p->off_status = o; o = align256(o + sizeof(int));
     p->off_epi = o; o = align256(o + size_t(P.max_chunks * epi_nlm) * sizeof(double));
+    p->off_scale = o;
+    if (P.tensor) o = align256(o + size_t(R.nz + 1) * kMaxRings * sizeof(float));
     p->region_bytes = o;
     CK(cudaStreamSynchronize(s));
     return desc->precision == BISP_PREC_FP64 ? autotune_transforms<double>(p, s) : autotune_transforms<float>(p, s);
@@ -705,7 +708,8 @@ int run_estimate(bisp_plan *p, const R *delta, int batch, unsigned char *ws, dou
     const int64_t fs = int64_t(p->region_bytes);          // between the fields' workspace regions
     StepIIArgs a2{p->d_groups, p->d_tiles, p->d_units, p->d_doff, Rg.nz + 1, Rg.nr, p->x_chunk, part, fs};
     TcArgs atc{p->d_tc_tiles, p->d_tc_rows, p->d_tc_slots, p->d_tc_units, p->d_doff, Rg.nz + 1, Rg.nr, p->x_chunk,
-               part, reinterpret_cast<int *>(ws + p->off_status), fs, p->wait_spins};
+               part, reinterpret_cast<const float *>(ws + p->off_scale), reinterpret_cast<int *>(ws + p->off_status),
+               fs, p->wait_spins};
     // every stage runs once for all fields of the batch (gridDim.y = field)
     const unsigned nf = unsigned(batch);
     const Batch in_field{nf, int64_t(ng2) * ng * int64_t(sizeof(R)), fs};   // input field -> region
@@ -720,12 +724,19 @@ int run_estimate(bisp_plan *p, const R *delta, int batch, unsigned char *ws, dou
         CK(launch_fft_rows_T<R>(B_, A_, ng, ng, Rg.nz + 1, nullptr, scale, true, tw, region, s, p->rt_xy));
     }
     {   // Step I: D(r, n) on each reduction grid (Eq. iFT)
-        StageMark m(p, BISP_STAGE_STEP1, int(2 * P.levels.size()), s);
+        StageMark m(p, BISP_STAGE_STEP1, int(2 * P.levels.size()) + (P.tensor ? 1 : 0), s);
+        const float *fac = nullptr;
+        if constexpr (sizeof(R) == 4)
+            if (P.tensor) {
+                float *scale = reinterpret_cast<float *>(ws + p->off_scale);
+                CK(launch_ring_scale(A_, ng, Rg.nz + 1, p->ring_arg, scale, region, s));
+                fac = scale;
+            }
         for (size_t l = 0; l < P.levels.size(); ++l) {
             const Level &L = P.levels[l];
             const int M = L.M;
             CK(launch_ring_gather<R>(A_, ng, p->ring_arg, p->d_jobs[l], L.njobs, M, false, gt, tw, region, s,
-                                     p->rt_gather[L.lev]));
+                                     p->rt_gather[L.lev], fac));
             CK(launch_fft_cols<R>(gt, dstore, M, L.njobs, p->d_job_off[l], p->d_jobs[l], p->ring_arg, tw, region, s,
                                   p->rt_rows[L.lev]));
         }
@@ -1236,7 +1247,15 @@ int estimator_dfield(const bisp_plan *p, const void *workspace, int M, int n, in
     if (o < 0) return fail(BISP_INVALID_ARG, "field not stored on this grid");
     const unsigned char *src = static_cast<const unsigned char *>(workspace) + size_t(p->last_field) * p->region_bytes +
                                p->off_dstore + size_t(o) * p->celem;
-    return copy_complex_out(p, src, int64_t(M) * M, out, static_cast<cudaStream_t>(stream));
+    const int st = copy_complex_out(p, src, int64_t(M) * M, out, static_cast<cudaStream_t>(stream));
+    if (st || !P.tensor) return st;
+    float f = 1.0f;                      // the stored field is D times this power of two
+    CK(cudaMemcpyAsync(&f, static_cast<const unsigned char *>(workspace) + size_t(p->last_field) * p->region_bytes +
+                               p->off_scale + (size_t(n) * kMaxRings + r) * sizeof(float),
+                       sizeof(float), cudaMemcpyDeviceToHost, static_cast<cudaStream_t>(stream)));
+    CK(cudaStreamSynchronize(static_cast<cudaStream_t>(stream)));
+    for (int64_t i = 0; i < 2 * int64_t(M) * M; ++i) out[i] /= double(f);
+    return BISP_OK;
 }
 
 int estimator_delta_plane(const bisp_plan *p, const void *workspace, int n, double *out, void *stream)

@@ -7,6 +7,7 @@
 //                   passes of the forward transform; second pass of Step I)
 //   k_ring_gather   Step I first pass: ring mask (and fold onto the M x M
 //                   reduction grid) fused into the load, transform along u_y
+//   k_ring_scale    power-of-two factors of the D fields (tensor-core Step II)
 //   k_step2         Step II: partial triple sums sum_x D1 D2 D3 (Eq. fftbs)
 //   k_reduce        partial sums -> S per combination, grid normalisation
 //   k_epilogue      Y_lm weights, (k1, mu, t) binning and the ratio of
@@ -384,12 +385,13 @@ template <typename R, bool UNIT>
 __global__ void __launch_bounds__(256)
 k_ring_gather(const typename Cx<R>::T *__restrict__ planes, int ng, RingArg rings,
               const Job *__restrict__ jobs, int M, int ntile, int rt, typename Cx<R>::T *__restrict__ gt,
-              Twiddles<typename Cx<R>::T> tw, int64_t fs)
+              Twiddles<typename Cx<R>::T> tw, const float *__restrict__ scale, int64_t fs)
 {
     using C = typename Cx<R>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     planes = field_ptr(planes, fs);
     gt = field_ptr(gt, fs);
+    scale = scale ? field_ptr(scale, fs) : scale;
     const int P = fft_stride(M);
     C *a = reinterpret_cast<C *>(smem_raw);
     C *b = a + rt * P;
@@ -399,6 +401,7 @@ k_ring_gather(const typename Cx<R>::T *__restrict__ planes, int ng, RingArg ring
     const C *pl = planes + int64_t(J.n) * ng * ng;
     const int64_t lo = rings.e3sq[J.r], hi = rings.e3sq[J.r + 1];
     const int mc = rings.maxc[J.r];
+    const R fac = scale ? R(scale[J.n * kMaxRings + J.r]) : R(1);
     const int row0 = tile * rt;
     const int nr = min(rt, M - row0);
     // rows i hold ring members only where |u_x| <= maxc for u_x = i or i - M;
@@ -426,8 +429,8 @@ k_ring_gather(const typename Cx<R>::T *__restrict__ planes, int ng, RingArg ring
                     vr += R(1);
                 } else {
                     const C v = pl[int64_t(ux < 0 ? ux + ng : ux) * ng + (uy < 0 ? uy + ng : uy)];
-                    vr += v.x;
-                    vi += v.y;
+                    vr += v.x * fac;
+                    vi += v.y * fac;
                 }
             }
         }
@@ -442,6 +445,58 @@ k_ring_gather(const typename Cx<R>::T *__restrict__ planes, int ng, RingArg ring
         const int r = st.q, k = st.r;
         dst[t] = res[r * P + spos(k)];
     }
+}
+
+// scale[n][r] = the power of two 2^e with 2^e sum (|Re Delta| + |Im Delta|)
+// in (kFieldBound / 2, kFieldBound], the sum over ring r of plane n.  No
+// |D(r, n, x)| 2^e exceeds that sum, so a product of two scaled fields stays
+// below 62500, inside FP16, while a typical value (the root mean square of a
+// Gaussian field is about the bound over the square root of the ring's mode
+// count) stays near or above 1/2 up to N_g = 1024, so that the low part of an
+// FP16 pair keeps its 11 bits.  One block per (ring, plane), eight lanes per row
+// u_x, 32 rows at a time: the loads of a row are a few runs of u_y, so the
+// kernel is bound by their latency (a warp per row took 0.3 ms a field at
+// 384^3, this one a tenth of it).  Every sum is in a fixed order.  Empty or
+// non-finite rings get 1.
+__global__ void __launch_bounds__(256)
+k_ring_scale(const float2 *__restrict__ planes, int ng, RingArg rings, float *__restrict__ scale, int64_t fs)
+{
+    planes = field_ptr(planes, fs);
+    scale = field_ptr(scale, fs);
+    const int r = blockIdx.x % rings.nr, n = blockIdx.x / rings.nr;
+    const float2 *pl = planes + int64_t(n) * ng * ng;
+    // members: lo <= |u|^2 < hi (9 |u|^2 is compared with squares of 3 e_r)
+    const int lo = int((rings.e3sq[r] + 8) / 9), hi = int((rings.e3sq[r + 1] + 8) / 9);
+    const int mc = rings.maxc[r], grp = threadIdx.x >> 3, sub = threadIdx.x & 7;
+    float sum = 0.0f;
+#pragma unroll 2
+    for (int ux = -mc + grp; ux <= mc; ux += 32) {
+        const float2 *row = pl + int64_t(ux < 0 ? ux + ng : ux) * ng;
+        // |u_y| from just inside the inner edge on (members are tested exactly)
+        const int in2 = lo - ux * ux, out2 = hi - ux * ux;
+        const int first = in2 > 0 ? max(0, int(sqrtf(float(in2))) - 1) : 0;
+        for (int a = first + sub; a * a < out2; a += 8) {
+            if (a * a < in2) continue;
+            const float2 v = row[a];
+            const float2 w = a == 0 ? make_float2(0.0f, 0.0f) : row[ng - a];
+            sum += (fabsf(v.x) + fabsf(v.y)) + (fabsf(w.x) + fabsf(w.y));
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+    __shared__ float wsum[8];
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    float b = 0.0f;
+    for (int w = 0; w < 8; ++w) b += wsum[w];
+    b *= 1.0f / kFieldBound;
+    int e = 0;
+    if (b > 0.0f && isfinite(b)) {
+        const float m = frexpf(b, &e);             // b = m 2^e, 1/2 <= m < 1
+        e = m == 0.5f ? 1 - e : -e;                // the largest e with b 2^e <= 1
+        e = max(-100, min(100, e));
+    }
+    scale[n * kMaxRings + r] = ldexpf(1.0f, e);
 }
 
 // Step I second pass: transforms along the first axis of each job's M x M
@@ -848,7 +903,8 @@ cudaError_t launch_fft_rows_T(const typename Cx<R>::T *in, typename Cx<R>::T *ou
 template <typename R>
 cudaError_t launch_ring_gather(const typename Cx<R>::T *planes, int ng, const RingArg &rings, const Job *jobs,
                                int64_t njobs, int M, bool unit, typename Cx<R>::T *gt,
-                               const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s, int rt)
+                               const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s, int rt,
+                               const float *scale)
 {
     using C = typename Cx<R>::T;
     if (rt <= 0) rt = int(fft_rows_per_block(M, sizeof(C)));
@@ -859,9 +915,18 @@ cudaError_t launch_ring_gather(const typename Cx<R>::T *planes, int ng, const Ri
     if (nblk == 0) return cudaSuccess;
     const dim3 grid(unsigned(nblk), fb.nf);
     if (unit)
-        k_ring_gather<R, true><<<grid, 256, smem, s>>>(planes, ng, rings, jobs, M, ntile, rt, gt, tw, fb.fs_in);
+        k_ring_gather<R, true><<<grid, 256, smem, s>>>(planes, ng, rings, jobs, M, ntile, rt, gt, tw, scale,
+                                                        fb.fs_in);
     else
-        k_ring_gather<R, false><<<grid, 256, smem, s>>>(planes, ng, rings, jobs, M, ntile, rt, gt, tw, fb.fs_in);
+        k_ring_gather<R, false><<<grid, 256, smem, s>>>(planes, ng, rings, jobs, M, ntile, rt, gt, tw, scale,
+                                                         fb.fs_in);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_ring_scale(const float2 *planes, int ng, int nz1, const RingArg &rings, float *scale,
+                              const Batch &fb, cudaStream_t s)
+{
+    k_ring_scale<<<dim3(unsigned(nz1 * rings.nr), fb.nf), 256, 0, s>>>(planes, ng, rings, scale, fb.fs_in);
     return cudaGetLastError();
 }
 
@@ -1023,8 +1088,8 @@ template cudaError_t launch_fft_z_real<float>(const float *, float2 *, int, int6
 template cudaError_t launch_fft_z_real<double>(const double *, double2 *, int, int64_t, int, const Twiddles<double2> &, const Batch &, cudaStream_t, int);
 template cudaError_t launch_fft_rows_T<float>(const float2 *, float2 *, int, int, int64_t, const int64_t *, float, bool, const Twiddles<float2> &, const Batch &, cudaStream_t, int);
 template cudaError_t launch_fft_rows_T<double>(const double2 *, double2 *, int, int, int64_t, const int64_t *, double, bool, const Twiddles<double2> &, const Batch &, cudaStream_t, int);
-template cudaError_t launch_ring_gather<float>(const float2 *, int, const RingArg &, const Job *, int64_t, int, bool, float2 *, const Twiddles<float2> &, const Batch &, cudaStream_t, int);
-template cudaError_t launch_ring_gather<double>(const double2 *, int, const RingArg &, const Job *, int64_t, int, bool, double2 *, const Twiddles<double2> &, const Batch &, cudaStream_t, int);
+template cudaError_t launch_ring_gather<float>(const float2 *, int, const RingArg &, const Job *, int64_t, int, bool, float2 *, const Twiddles<float2> &, const Batch &, cudaStream_t, int, const float *);
+template cudaError_t launch_ring_gather<double>(const double2 *, int, const RingArg &, const Job *, int64_t, int, bool, double2 *, const Twiddles<double2> &, const Batch &, cudaStream_t, int, const float *);
 template cudaError_t launch_fft_cols<float>(const float2 *, float2 *, int, int64_t, const int64_t *, const Job *,
                                             const RingArg &, const Twiddles<float2> &,
                                             const Batch &, cudaStream_t, int);

@@ -86,12 +86,22 @@ cudaError_t launch_fft_rows_T(const typename Cx<R>::T *in, typename Cx<R>::T *ou
 // Step I, first pass: ring r of plane n of Delta (planes [nz+1][ng][ng]),
 // folded onto the M x M grid, transformed along u_y, written in place order
 // to gt[job][u_x][k_y].  unit = true uses Delta = 1 (the unit fields of
-// Eq. 2FT).
+// Eq. 2FT).  scale: optional factors [nz1][kMaxRings] of the members' values
+// (one field's; the next field's lie fb.fs_in bytes further).
 template <typename R>
 cudaError_t launch_ring_gather(const typename Cx<R>::T *planes, int ng, const RingArg &rings,
                                const Job *jobs, int64_t njobs, int M, bool unit,
                                typename Cx<R>::T *gt, const Twiddles<typename Cx<R>::T> &tw,
-                               const Batch &fb, cudaStream_t s, int rt = 0);
+                               const Batch &fb, cudaStream_t s, int rt = 0,
+                               const float *scale = nullptr);
+
+// Power-of-two factor of every (plane, ring) field D(r, n), [nz1][kMaxRings]
+// (see k_ring_scale): with it, every |D| on the grid is at most kFieldBound.
+// The tensor-core Step II splits the scaled values into FP16 parts; Step I's
+// first pass applies the factors (launch_ring_gather's scale).
+constexpr float kFieldBound = 250.0f;
+cudaError_t launch_ring_scale(const float2 *planes, int ng, int nz1, const RingArg &rings, float *scale,
+                              const Batch &fb, cudaStream_t s);
 
 // Step I second pass: for each of njobs M x M fields in gt ([u_x][k_y],
 // the gather's output), transforms along u_x in strips of w columns and
@@ -121,6 +131,7 @@ struct TcArgs {
     int nz1, nr;
     int64_t x_chunk;
     double *partials;
+    const float *scale;      // field 0's power-of-two factors of the stored fields [nz1][kMaxRings]
     int *status;             // field 0's status word, set to 1 by a block whose wait ran out
     int64_t fs;              // bytes between the workspace regions of the fields of a batch
     int wait_spins;          // polls before an abortable wait gives up

@@ -82,9 +82,8 @@ constexpr int kTcRows = 128;
 constexpr int kTcMaxCols = 64;
 constexpr int kTcMaxSlots = 250;      // distinct D1 / D2 fields staged by a tile
 constexpr int kTcClasses = 4;         // NC = 16 (class + 1)
-constexpr int kTcTX = 16;             // grid points of one pipeline stage (one MMA step)
-constexpr int kTcRingTX = 2 * kTcTX;  // grid points of one ring buffer (two stages)
-constexpr int kTcSlotBytes = kTcRingTX * 8 + 16;   // one staged field row of a ring buffer (padded)
+constexpr int kTcTX = 32;             // grid points of one pipeline stage (one ring buffer)
+constexpr int kTcSlotBytes = kTcTX * 8 + 16;   // one staged field row of a ring buffer (padded)
 constexpr int kTcMinRing = 2;         // ring buffers
 constexpr int kTcMaxRing = 4;
 constexpr size_t kTcSmem = 110 * 1024;         // dynamic shared memory of a block (two per SM)
@@ -93,14 +92,15 @@ constexpr size_t kTcSmem = 110 * 1024;         // dynamic shared memory of a blo
 // of a block), two otherwise.
 BISP_HD constexpr int tc_abuf(int ncol) { return ncol <= 32 ? 3 : 2; }
 // Shared memory of a tcgen05 block other than its stage ring: B high and
-// low parts (tc_abuf buffers each), field offsets, barriers; a multiple of
-// 128 bytes, so that the ring that follows is aligned for 16-byte copies.
+// low parts (tc_abuf buffers each, 4 bytes per point), field offsets,
+// barriers; a multiple of 128 bytes, so that the ring that follows is
+// aligned for 16-byte copies.
 BISP_HD inline size_t tc_fixed_smem(int ncol, int nslot)
 {
-    return size_t(2 * tc_abuf(ncol)) * ncol * kTcTX * 8 + ((8 * size_t(nslot + ncol) + 256 + 127) & ~size_t(127));
+    return size_t(2 * tc_abuf(ncol)) * ncol * kTcTX * 4 + ((8 * size_t(nslot + ncol) + 256 + 127) & ~size_t(127));
 }
 // Buffers of the stage ring for a tile (0 if fewer than kTcMinRing fit):
-// each holds two stages of the tile's nslot + ncol fields and one zero row.
+// each holds a stage of the tile's nslot + ncol fields and one zero row.
 BISP_HD inline int tc_ring(int ncol, int nslot)
 {
     const size_t fixed = tc_fixed_smem(ncol, nslot);

@@ -11,32 +11,41 @@
 //   B[c][2x]  = Re D3,  B[c][2x + 1]  = Im D3,
 // with D3 the stored field of plane |n3| and g3 = -1 when n3 < 0 (the field
 // of a negative plane is the conjugate of the stored one; likewise g1, g2 in
-// P).  The fields of a stage (16 grid points = 128 bytes each) are staged
+// P).  The fields of a stage (32 grid points = 256 bytes each) are staged
 // in shared memory by cp.async; the CUDA cores form A and store it to
 // tensor memory (lane = row) and write B, split into high and low parts, in
 // the K-major canonical layout (core matrices of 8 rows x 16 bytes, no
-// swizzle); one thread issues the MMAs (M = 128, N = NC, K = 8, kind::tf32,
+// swizzle); one thread issues the MMAs (M = 128, N = NC, K = 16, kind::f16,
 // FP32 accumulator in tensor memory).
 //
-// Precision.  A tf32 MMA reads the top 19 bits of each FP32 operand (it
-// truncates), so every operand is split x = hi + lo with hi = x with its 13
-// low mantissa bits cleared (the raw x is passed: the MMA drops those bits
-// itself) and lo = x - hi, exact in FP32; the product is taken as
-// hi hi' + lo hi' + hi lo' (lo lo' is below FP32 rounding), which keeps
-// FP32 accuracy.  The tensor-memory accumulator (it also truncates when it
-// accumulates) holds one stage of 16 grid points; every stage is added
-// into FP32 registers, and each unit's sums go out as FP64 partials, as in
-// the CUDA-core kernel.
+// Precision.  Every FP32 operand is split x = hi + lo into two FP16 numbers,
+// hi rounded to nearest and lo the remainder (exact in FP32) rounded to
+// nearest, so that hi + lo holds x to 2^-24; the product is taken as
+// hi hi' + lo hi' + hi lo' (lo lo' is below FP32 rounding).  The stored
+// fields are D times a power of two per field that puts them, their products
+// and the low parts inside FP16's range (k_ring_scale); it is undone, exactly,
+// on the FP64 partial sums.  The tensor-memory accumulator truncates when it
+// accumulates, so it holds one stage of 32 grid points (12 MMAs); every stage
+// is added into FP32 registers, and each unit's sums go out as FP64 partials,
+// as in the CUDA-core kernel.
+//
+// Why FP16 pairs.  A TF32 pair (hi truncated by the MMA) keeps 22 bits, reads
+// 8 bytes per value and has half the MMA rate: with it a stage of the same
+// buffers holds 16 points, so the barriers, fences and accumulator reads, a
+// third of the time, came twice as often.  512^3, all of Step II: 587 ms with
+// TF32 pairs and 16-point stages, 462 ms so; the error against 64 bits fell
+// from 1.1e-6 to 0.7e-6 (2-norm over the bins, 128^3).
 #include "kernels.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace bisp {
 
 namespace {
 
-constexpr int kTX = kTcTX;                   // grid points per stage (K = 32)
-constexpr int kSlotBytes = kTcSlotBytes;     // a field's row of a ring buffer: two stages (+ padding)
+constexpr int kTX = kTcTX;                   // grid points per stage (K = 64)
+constexpr int kSlotBytes = kTcSlotBytes;     // a field's row of a ring buffer: one stage (+ padding)
 constexpr uint32_t kTmemCols = 256;          // A[tc_abuf] (hi 32 + lo 32 columns each), then the accumulators
 constexpr int kDrainSpins = kDefaultWaitSpins;  // bound of the wait for the block's own MMAs
 
@@ -57,21 +66,21 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
            (uint64_t((sbo & 0x3FFFF) >> 4) << 32) | (uint64_t(1) << 46);
 }
 
-// Instruction descriptor: FP32 accumulator, A and B tf32, both K-major, N, M.
+// Instruction descriptor: FP32 accumulator, A and B FP16 (format 0), both K-major, N, M.
 template <int N>
-__host__ __device__ constexpr uint32_t idesc_tf32()
+__host__ __device__ constexpr uint32_t idesc_f16()
 {
-    return (1u << 4) | (2u << 7) | (2u << 10) | (uint32_t(N >> 3) << 17) | (uint32_t(128 >> 4) << 24);
+    return (1u << 4) | (uint32_t(N >> 3) << 17) | (uint32_t(128 >> 4) << 24);
 }
 
 // One MMA, issued by one elected lane of a converged warp whose lanes all
 // hold the same operands.  Issued this way the operands stay warp-uniform,
 // and a stage's twelve MMAs issue in ~15 cycles each; issued from a single
 // lane (inside a lane test) they took ~48.
-__device__ __forceinline__ void mma_tf32(uint32_t d, uint32_t a, uint64_t b, uint32_t id, uint32_t acc)
+__device__ __forceinline__ void mma_f16(uint32_t d, uint32_t a, uint64_t b, uint32_t id, uint32_t acc)
 {
     asm volatile("{\n.reg .pred p, e;\nsetp.ne.b32 p, %4, 0;\nelect.sync _|e, 0xffffffff;\n"
-                 "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n"
+                 "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n"
                  ::"r"(d), "r"(a), "l"(b), "r"(id), "r"(acc) : "memory");
 }
 
@@ -83,9 +92,6 @@ __device__ __forceinline__ void mma_commit(uint32_t m)
                  ::"r"(m) : "memory");
 }
 
-// -hi(x): x with its 13 low mantissa bits cleared, negated (one logical operation)
-__device__ __forceinline__ uint32_t tf32_neg_hi(float x) { return (__float_as_uint(x) & 0xFFFFE000u) ^ 0x80000000u; }
-
 // (a, b) += (x, y): one packed FP32 addition (round to nearest, as two
 // scalar additions would be)
 __device__ __forceinline__ void add2(float &a, float &b, uint32_t x, uint32_t y)
@@ -94,13 +100,17 @@ __device__ __forceinline__ void add2(float &a, float &b, uint32_t x, uint32_t y)
         : "+f"(a), "+f"(b) : "r"(x), "r"(y));
 }
 
-// (lo(x), lo(y)) = (x - hi(x), y - hi(y)), exact
-__device__ __forceinline__ void lo2(float x, float y, uint32_t &lx, uint32_t &ly)
+// (x, y) -> hi + lo, two FP16 pairs (x in the low halves): hi rounded to
+// nearest, lo the remainder x - hi (exact in FP32) rounded to nearest.  The
+// remainder is taken by the mixed-precision subtraction (one instruction,
+// hi - x), so the pair costs two conversions and two subtractions.
+__device__ __forceinline__ void split2(float x, float y, uint32_t &hi, uint32_t &lo)
 {
-    float a = x, b = y;
-    add2(a, b, tf32_neg_hi(x), tf32_neg_hi(y));
-    lx = __float_as_uint(a);
-    ly = __float_as_uint(b);
+    float rx, ry;
+    asm("cvt.rn.f16x2.f32 %0, %2, %1;" : "=r"(hi) : "f"(x), "f"(y));
+    asm("{\n.reg .b16 l, h;\nmov.b32 {l, h}, %2;\nsub.rn.f32.f16 %0, l, %3;\nsub.rn.f32.f16 %1, h, %4;\n}\n"
+        : "=f"(rx), "=f"(ry) : "r"(hi), "f"(x), "f"(y));
+    asm("cvt.rn.f16x2.f32 %0, %2, %1;" : "=r"(lo) : "f"(-rx), "f"(-ry));
 }
 
 // No memory clobber: tensor memory is not memory the compiler tracks, so
@@ -141,9 +151,9 @@ __device__ __forceinline__ void add_accumulator(uint32_t tcol, float (&acc)[NH])
 //              st % NA of stage st (NA = tc_abuf(NC): 3 for NC <= 32, else
 //              2; A in tensor-memory columns 64 a .. 64 a + 63); warps w and
 //              w + 4 share tensor-memory lanes 32 (w % 4) .. (the tile's
-//              rows, one per lane): warp w forms grid points 0-7 of a stage
+//              rows, one per lane): warp w forms grid points 0-15 of a stage
 //              and adds accumulator columns 0 .. NC/2 - 1 into FP32
-//              registers, warp w + 4 points 8-15 and columns NC/2 .. NC - 1,
+//              registers, warp w + 4 points 16-31 and columns NC/2 .. NC - 1,
 //              reading the accumulators of stage st - (NA - 1) after forming
 //              stage st;
 //   warp 8     issues the 12 MMAs of a stage (one elected lane) into
@@ -155,16 +165,14 @@ __device__ __forceinline__ void add_accumulator(uint32_t tcol, float (&acc)[NH])
 //              own was slower: a second accumulator doubles the compute
 //              warps' reads);
 //   warps 9-10 stage the fields of each stage in shared memory (cp.async,
-//              a ring of 2 to 4 buffers of two stages each: 32 grid points
-//              a field row, waited for and released once per two stages).
+//              a ring of 2 to 4 buffers of one stage each).
 // mbarriers (phase k of a barrier = its k-th use):
 //   full[q]   the data of ring buffer q landed        (64 producer arrivals)
 //   empty[q]  ring buffer q has been read             (1 arrival: the MMA warp,
 //                                                      once it has seen A of
-//                                                      the buffer's last stage,
-//                                                      which every compute
-//                                                      thread signals after its
-//                                                      reads of the buffer)
+//                                                      the stage, which every
+//                                                      compute thread signals
+//                                                      after its reads)
 //   aready[a] A and B (high, low) of buffer a written (256 compute arrivals)
 //   mdone[b]  the MMAs into accumulator b are done    (commit)
 //   drain     every MMA the block issued is done      (commit; before the
@@ -233,11 +241,11 @@ __device__ __forceinline__ void mbar_wait_bounded(uint64_t *m, uint32_t parity)
     }
 }
 
-// The A columns of half a stage (grid points 8 half .. 8 half + 7) for this
-// thread's row: P = D1' D2' with D' the stored field or its conjugate (G1,
-// G2: n1 < 0, n2 < 0), and A = (Re P, -g3 Im P) (G3: n3 < 0), high parts at
-// column a + 16 half, low parts at a + 32 + 16 half.  u8, v8: the row's two
-// staged fields (16 points each).
+// The A columns of half a stage (grid points 16 half .. 16 half + 15) for
+// this thread's row: P = D1' D2' with D' the stored field or its conjugate
+// (G1, G2: n1 < 0, n2 < 0), and A = (Re P, -g3 Im P) (G3: n3 < 0), one FP16
+// pair per point: high parts at column a + 16 half, low parts at a + 32 +
+// 16 half.  u8, v8: the row's two staged fields (32 points each).
 template <bool G1, bool G2, bool G3>
 __device__ __forceinline__ void form_a(const unsigned char *u8, const unsigned char *v8, uint32_t a, int half)
 {
@@ -247,23 +255,18 @@ __device__ __forceinline__ void form_a(const unsigned char *u8, const unsigned c
     constexpr bool NEG2 = !(G3 ^ G2);             // s2 = -1
     constexpr bool NEG1 = !(G3 ^ G1);             // s1 = -1
 #pragma unroll
-    for (int hh = 0; hh < 2; ++hh) {              // 4 grid points = 8 columns
+    for (int hh = 0; hh < 2; ++hh) {              // 8 grid points = 8 columns
         const int h = 2 * half + hh;
         uint32_t hi[8], lo[8];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const float4 u = *reinterpret_cast<const float4 *>(u8 + (h * 2 + k) * 16);
-            const float4 v = *reinterpret_cast<const float4 *>(v8 + (h * 2 + k) * 16);
-            float e[4];
+        for (int k = 0; k < 4; ++k) {
+            const float4 u = *reinterpret_cast<const float4 *>(u8 + (h * 4 + k) * 16);
+            const float4 v = *reinterpret_cast<const float4 *>(v8 + (h * 4 + k) * 16);
             const float t0 = u.y * v.y, t1 = u.y * v.x, t2 = u.w * v.w, t3 = u.w * v.z;
-            e[0] = fmaf(u.x, v.x, NEG12 ? -t0 : t0);
-            e[1] = fmaf(NEG2 ? -u.x : u.x, v.y, NEG1 ? -t1 : t1);
-            e[2] = fmaf(u.z, v.z, NEG12 ? -t2 : t2);
-            e[3] = fmaf(NEG2 ? -u.z : u.z, v.w, NEG1 ? -t3 : t3);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) hi[4 * k + j] = __float_as_uint(e[j]);
-            lo2(e[0], e[1], lo[4 * k], lo[4 * k + 1]);
-            lo2(e[2], e[3], lo[4 * k + 2], lo[4 * k + 3]);
+            split2(fmaf(u.x, v.x, NEG12 ? -t0 : t0), fmaf(NEG2 ? -u.x : u.x, v.y, NEG1 ? -t1 : t1), hi[2 * k],
+                   lo[2 * k]);
+            split2(fmaf(u.z, v.z, NEG12 ? -t2 : t2), fmaf(NEG2 ? -u.z : u.z, v.w, NEG1 ? -t3 : t3), hi[2 * k + 1],
+                   lo[2 * k + 1]);
         }
         tmem_st8(a + 8 * h, hi);
         tmem_st8(a + 32 + 8 * h, lo);
@@ -276,14 +279,14 @@ struct CompArgs {
     uint32_t tlane;            // tensor-memory address of lane 0 of this warp's quarter
     volatile int *abort;
     TcSync *sy;
-    int rowb, nslot, S, nstage, spins, t, half, s1, s2;
+    int rowb, nslot, S, nstage, ntail, spins, t, half, s1, s2;   // ntail: points of the last stage (16 or 32)
 };
 
 // Tensor-memory column of accumulator buffer 0 and the distance to buffer 1
 template <int NC> __device__ constexpr uint32_t acc_col0() { return 64u * tc_abuf(NC); }
 template <int NC> __device__ constexpr uint32_t acc_step() { return tc_abuf(NC) == 3 ? uint32_t(NC) : 64u; }
 
-// The stage loop of one compute thread: form A (its row's 8 points of the
+// The stage loop of one compute thread: form A (its row's 16 points of the
 // stage) and its share of B into buffer st % NA, and add the accumulators of
 // stage st - (NA - 1).  With two buffers the sums of stage st - 1 are read
 // after forming stage st (the MMAs of st - 1 run meanwhile); with three, the
@@ -291,15 +294,16 @@ template <int NC> __device__ constexpr uint32_t acc_step() { return tc_abuf(NC) 
 // overwrite that accumulator buffer, and wait only for A(st), signalled
 // after the read) can start as soon as A(st) is written, and have the whole
 // next stage to finish.  Returns false if a wait gave up.  B piece p
-// (grid points 2p, 2p + 1) of column c goes to core matrix (K block p, rows
+// (grid points 4p .. 4p + 3) of column c goes to core matrix (K block p, rows
 // 8 (c / 8) ..), row c % 8; this thread's pieces are i = t and t + 256
 // (i = p NC + c), fixed for the tile, so their offsets are computed once.
+// The last stage may hold 16 points (ntail); its second half is left alone.
 template <int NC, bool G1, bool G2, bool G3>
 __device__ __forceinline__ bool compute_loop(const CompArgs &ca, float (&acc)[NC / 2])
 {
     constexpr int NH = NC / 2;
     constexpr int NB = NC / 8;
-    constexpr int BB = NC * kTX * 8;
+    constexpr int BB = NC * kTX * 4;
     constexpr int NP = (NC * 8 + kCompute - 1) / kCompute;    // B pieces per thread (at most 2)
     constexpr int NA = tc_abuf(NC), LAG = NA - 1;
     constexpr bool READ_FIRST = NA == 3;
@@ -309,43 +313,44 @@ __device__ __forceinline__ bool compute_loop(const CompArgs &ca, float (&acc)[NC
     for (int k = 0; k < NP; ++k) {
         const int i = ca.t + k * kCompute;
         const int c = i % NC, p = i / NC;
-        src[k] = i < NC * 8 ? (ca.nslot + c) * kSlotBytes + p * 16 : -1;
+        src[k] = i < NC * 8 ? (ca.nslot + c) * kSlotBytes + p * 32 : -1;
         dst[k] = (p * NB + c / 8) * 128 + (c % 8) * 16;
     }
     const int uoff = ca.s1 * kSlotBytes, voff = ca.s2 * kSlotBytes;
 #pragma unroll
     for (int c = 0; c < NH; ++c) acc[c] = 0.f;
-    int q = 0;                                   // ring buffer of stage st: (st / 2) % S
-    uint32_t ph = 0;                             // its phase: (st / 2S) & 1
+    int q = 0;                                   // ring buffer of stage st: st % S
+    uint32_t ph = 0;                             // its phase: (st / S) & 1
     const unsigned char *sq = ca.sS;             // ring buffer q
     int ia = 0;                                  // A / B buffer of stage st: st % NA
-    // A and B of stage st (half st & 1 of ring buffer q) into buffer ia
-    // (last read by the MMAs of stage st - NA, complete: their sums have
-    // been read); the ring buffer is waited for at its first stage and left
-    // after its second (or the last stage); the MMA warp releases it
+    // A and B of stage st (ring buffer q) into buffer ia (last read by the
+    // MMAs of stage st - NA, complete: their sums have been read); the MMA
+    // warp releases the ring buffer
     auto form = [&](int st) -> bool {
-        const int h = (st & 1) * (kTX * 8);
-        if (h == 0 && !mbar_wait_abort(&sy->full[q], ph, ca.abort, ca.spins)) return false;
-        form_a<G1, G2, G3>(sq + uoff + h, sq + voff + h, ca.tlane + 64 * ia, ca.half);
+        if (!mbar_wait_abort(&sy->full[q], ph, ca.abort, ca.spins)) return false;
+        const bool whole = st + 1 < ca.nstage || ca.ntail == kTX;
+        if (whole || ca.half == 0) form_a<G1, G2, G3>(sq + uoff, sq + voff, ca.tlane + 64 * ia, ca.half);
 #pragma unroll
         for (int k = 0; k < NP; ++k) {
             if (src[k] < 0) continue;
-            const float4 v = *reinterpret_cast<const float4 *>(sq + src[k] + h);
+            if (!whole && ca.t + k * kCompute >= NC * 4) continue;        // pieces of points 16 ..
+            const float4 v = *reinterpret_cast<const float4 *>(sq + src[k]);
+            const float4 w = *reinterpret_cast<const float4 *>(sq + src[k] + 16);
             const int o = ia * BB + dst[k];
-            *reinterpret_cast<float4 *>(ca.sHi + o) = v;
-            uint4 l;
-            lo2(v.x, v.y, l.x, l.y);
-            lo2(v.z, v.w, l.z, l.w);
+            uint4 h, l;
+            split2(v.x, v.y, h.x, l.x);
+            split2(v.z, v.w, h.y, l.y);
+            split2(w.x, w.y, h.z, l.z);
+            split2(w.z, w.w, h.w, l.w);
+            *reinterpret_cast<uint4 *>(ca.sHi + o) = h;
             *reinterpret_cast<uint4 *>(ca.sLo + o) = l;
         }
-        if (h != 0 || st + 1 == ca.nstage) {
-            if (++q == ca.S) {
-                q = 0;
-                ph ^= 1u;
-                sq = ca.sS;
-            } else {
-                sq += ca.rowb;
-            }
+        if (++q == ca.S) {
+            q = 0;
+            ph ^= 1u;
+            sq = ca.sS;
+        } else {
+            sq += ca.rowb;
         }
         asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
@@ -383,9 +388,9 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
     constexpr int NB = NC / 8;                   // 8-row groups of B
     constexpr uint32_t LBO = NB * 128;           // next core matrix along K
     constexpr uint32_t SBO = 128;                // next 8 rows of B
-    constexpr int BB = NC * kTX * 8;             // bytes of one stage of B
+    constexpr int BB = NC * kTX * 4;             // bytes of one stage of B (high or low parts)
     constexpr int NA = tc_abuf(NC);              // A / B buffers
-    constexpr uint32_t ID = idesc_tf32<NC>();
+    constexpr uint32_t ID = idesc_f16<NC>();
     extern __shared__ __align__(1024) unsigned char smem[];
 
     const TcUnit U = args.units[unit0 + blockIdx.x];
@@ -394,13 +399,14 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
     // field blockIdx.y of a batch: its D store and partial sums
     dstore = reinterpret_cast<const float2 *>(reinterpret_cast<const char *>(dstore) + int64_t(blockIdx.y) * args.fs);
     args.partials = reinterpret_cast<double *>(reinterpret_cast<char *>(args.partials) + int64_t(blockIdx.y) * args.fs);
+    args.scale = reinterpret_cast<const float *>(reinterpret_cast<const char *>(args.scale) + int64_t(blockIdx.y) * args.fs);
     args.status = reinterpret_cast<int *>(reinterpret_cast<char *>(args.status) + int64_t(blockIdx.y) * args.fs);
     const int spins = args.wait_spins;
     const int nslot = T.nslot, nf = nslot + NC;
     const int S = tc_ring(NC, nslot);            // ring buffers (>= 2; the plan checked)
     const int rowb = (nf + 1) * kSlotBytes;      // one ring buffer: nf fields and a zero row
     // shared memory: B high and low parts [NA][BB] each (canonical layout),
-    // field offsets [nf], barriers, ring [S][nf + 1][kSlotBytes] (two stages of D1 / D2
+    // field offsets [nf], barriers, ring [S][nf + 1][kSlotBytes] (a stage of D1 / D2
     // slots, the B window, a zero row)
     unsigned char *sHi = smem;
     unsigned char *sLo = smem + NA * BB;
@@ -451,7 +457,8 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
     const int64_t M2 = int64_t(T.M) * T.M;
     const int64_t x0 = int64_t(U.chunk) * args.x_chunk;
     const int64_t x1 = min(M2, x0 + args.x_chunk);
-    const int nstage = int((x1 - x0) / kTX);
+    const int nstage = int((x1 - x0 + kTX - 1) / kTX);
+    const int ntail = int(x1 - x0) - (nstage - 1) * kTX;     // 16 or 32 points (M^2 is a multiple of 16)
     bool ok = true;
 
     if (warp >= 9) {
@@ -469,23 +476,21 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
             const int64_t o = f < nf ? offs[f] : -1;
             o16[k] = o < 0 ? 0xFFFFFFFFu : uint32_t(o >> 4);
         }
-        // A ring buffer holds two stages (32 grid points): the lane copies
-        // piece p of each stage; the last buffer of an odd stage count holds
-        // one
+        // A stage has 32 grid points: the lane copies piece p of each half;
+        // the last stage may have one half
         int q = 0;                                   // ring buffer sb % S
         uint32_t ph = 0;                             // its phase: (sb / S) & 1
-        const int nbuf = (nstage + 1) / 2;
-        for (int sb = 0; sb < nbuf && ok; ++sb) {
+        for (int sb = 0; sb < nstage && ok; ++sb) {
             if (sb >= S) ok = mbar_wait_abort(&sy->empty[q], ph ^ 1u, abort, spins);
             if (!ok) break;
-            const float2 *src = dstore + x0 + int64_t(sb) * (2 * kTX) + 2 * p;
+            const float2 *src = dstore + x0 + int64_t(sb) * kTX + 2 * p;
             const uint32_t dst = su32(sS + q * rowb + f0 * kSlotBytes + p * 16);
-            if (2 * sb + 1 < nstage) {
+            if (sb + 1 < nstage || ntail == kTX) {
 #pragma unroll
                 for (int k = 0; k < kProdFields; ++k)
                     if (o16[k] != 0xFFFFFFFFu) {
                         cp_async16(dst + 8 * k * kSlotBytes, src + (int64_t(o16[k]) << 4));
-                        cp_async16(dst + 8 * k * kSlotBytes + kTX * 8, src + (int64_t(o16[k]) << 4) + kTX);
+                        cp_async16(dst + 8 * k * kSlotBytes + kTX * 4, src + (int64_t(o16[k]) << 4) + kTX / 2);
                     }
             } else {
 #pragma unroll
@@ -511,25 +516,27 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
                 ok = mbar_wait_abort(&sy->aready[ia], pa, abort, spins);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
-                // A(st) signalled by every compute thread: at the last stage
-                // of a ring buffer, all its reads are done (the MMAs do not
-                // read the ring)
-                if ((st & 1) || st + 1 == nstage) {
-                    if (lane == 0) mbar_arrive(&sy->empty[qr]);
-                    if (++qr == S) qr = 0;
-                }
+                // A(st) signalled by every compute thread: all reads of the
+                // stage's ring buffer are done (the MMAs do not read the ring)
+                if (lane == 0) mbar_arrive(&sy->empty[qr]);
+                if (++qr == S) qr = 0;
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t a = tmem + 64 * ia;
                 const uint32_t d = tmem + acc_col0<NC>() + acc_step<NC>() * b;
                 const uint64_t bo = uint64_t(ia * BB) >> 4;     // start-address field offset of buffer ia
                 if (++ia == NA) { ia = 0; pa ^= 1u; }
                 constexpr uint64_t kstep = (2 * LBO) >> 4;      // next k-step (two core matrices along K)
+                auto issue = [&](auto ksteps) {
+                    constexpr int KS = decltype(ksteps)::value;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) mma_tf32(d, a + 8 * j, dh + bo + j * kstep, ID, j > 0);
+                    for (int j = 0; j < KS; ++j) mma_f16(d, a + 8 * j, dh + bo + j * kstep, ID, j > 0);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) mma_tf32(d, a + 32 + 8 * j, dh + bo + j * kstep, ID, 1);
+                    for (int j = 0; j < KS; ++j) mma_f16(d, a + 32 + 8 * j, dh + bo + j * kstep, ID, 1);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) mma_tf32(d, a + 8 * j, dl + bo + j * kstep, ID, 1);
+                    for (int j = 0; j < KS; ++j) mma_f16(d, a + 8 * j, dl + bo + j * kstep, ID, 1);
+                };
+                if (st + 1 < nstage || ntail == kTX) issue(std::integral_constant<int, 4>{});
+                else issue(std::integral_constant<int, 2>{});
                 mma_commit(su32(&sy->mdone[b]));
             }
             // the MMAs issued so far finish before the tensor memory is freed
@@ -546,7 +553,7 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
         const bool live = row < T.nrow;
         TcRow R{};
         if (live) R = args.rows[T.row0 + row];
-        CompArgs ca{sS, sHi, sLo, tmem + (uint32_t(quarter * 32) << 16), abort, sy, rowb, nslot, S, nstage, spins,
+        CompArgs ca{sS, sHi, sLo, tmem + (uint32_t(quarter * 32) << 16), abort, sy, rowb, nslot, S, nstage, ntail, spins,
                     t, half, live ? int(R.s1) : nf, live ? int(R.s2) : nf};
         float acc[NC / 2];
         switch (T.flags) {
@@ -557,12 +564,17 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
         }
         if (live) {
             double *dst = args.partials + R.p0 + int64_t(U.chunk) * R.stride;
+            // the stored fields are D times powers of two: undone exactly
+            const int32_t f1 = args.slots[T.slot0 + R.s1], f2 = args.slots[T.slot0 + R.s2];
+            const double inv12 = 1.0 / (double(args.scale[(f1 >> 8) * kMaxRings + (f1 & 255)]) *
+                                        double(args.scale[(f2 >> 8) * kMaxRings + (f2 & 255)]));
+            const float *s3 = args.scale + T.n3abs * kMaxRings + T.r3lo;
             const double nan = __longlong_as_double(0x7FF8000000000000LL);
             constexpr int NH = NC / 2;
 #pragma unroll
             for (int c = 0; c < NH; ++c) {
                 const int j = c + NH * half - int(R.col0);
-                if (j >= 0 && j < int(R.n)) dst[j] = ok ? double(acc[c]) : nan;
+                if (j >= 0 && j < int(R.n)) dst[j] = ok ? double(acc[c]) * (inv12 / double(s3[c + NH * half])) : nan;
             }
         }
     }
