@@ -70,6 +70,7 @@ struct bisp_plan {
     TcTile *d_tc_tiles = nullptr;        // tcgen05 Step II (MIXED_TC)
     TcRow *d_tc_rows = nullptr;
     int32_t *d_tc_slots = nullptr;
+    TcLane *d_tc_lanes = nullptr;
     TcUnit *d_tc_units = nullptr;
     int64_t *d_doff = nullptr;
     Record *d_rec = nullptr;
@@ -601,6 +602,7 @@ int build_plan(bisp_plan *p, const bisp_desc *desc, cudaStream_t s)
     if (!st) st = upload(p, &p->d_tc_tiles, P.tc_tiles, s);
     if (!st) st = upload(p, &p->d_tc_rows, P.tc_rows, s);
     if (!st) st = upload(p, &p->d_tc_slots, P.tc_slots, s);
+    if (!st) st = upload(p, &p->d_tc_lanes, P.tc_lanes, s);
     if (!st) st = upload(p, &p->d_tc_units, P.tc_units, s);
     if (!st) st = upload(p, &p->d_doff, P.doff, s);
     if (!st) st = upload(p, &p->d_rec, P.records, s);
@@ -707,7 +709,7 @@ int run_estimate(bisp_plan *p, const R *delta, int batch, unsigned char *ws, dou
     const R scale = R(P.volume / (double(ng2) * ng));
     const int64_t fs = int64_t(p->region_bytes);          // between the fields' workspace regions
     StepIIArgs a2{p->d_groups, p->d_tiles, p->d_units, p->d_doff, Rg.nz + 1, Rg.nr, p->x_chunk, part, fs};
-    TcArgs atc{p->d_tc_tiles, p->d_tc_rows, p->d_tc_slots, p->d_tc_units, p->d_doff, Rg.nz + 1, Rg.nr, p->x_chunk,
+    TcArgs atc{p->d_tc_tiles, p->d_tc_rows, p->d_tc_slots, p->d_tc_lanes, p->d_tc_units, p->d_doff, Rg.nz + 1, Rg.nr, p->x_chunk,
                part, reinterpret_cast<const float *>(ws + p->off_scale), reinterpret_cast<int *>(ws + p->off_status),
                fs, p->wait_spins};
     // every stage runs once for all fields of the batch (gridDim.y = field)

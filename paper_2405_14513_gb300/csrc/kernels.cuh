@@ -126,6 +126,7 @@ struct TcArgs {
     const TcTile *tiles;
     const TcRow *rows;
     const int32_t *slots;
+    const TcLane *lanes;
     const TcUnit *units;
     const int64_t *doff;     // [kMaxLevels][nz+1][kMaxRings]
     int nz1, nr;

@@ -206,6 +206,105 @@ void enumerate_pair(const HostPlan &P, int n1, int n2, PairOut &out)
     }
 }
 
+// Lanes of a tcgen05 tile.  A lane (= row) reads its two fields with 16-byte
+// shared-memory loads.  Such a load of a warp is served in four passes of
+// eight lanes, but in two of sixteen when every lane l reads the same address
+// as lane l ^ 1, or every lane the same as lane l ^ 2 (measured: 2.09 and 4.00
+// cycles a load).  So rows are put side by side that share a field: four rows
+// (two D1 fields times two D2 fields) on lanes 4q .. 4q + 3 as (a, x), (a, y),
+// (b, x), (b, y) halve both loads, two rows of one D1 field on lanes 2q, 2q + 1
+// halve the first, two of one D2 field the second.  The condition is on whole
+// warps, so the lanes are filled in the order: quads, D1 pairs, rows alone,
+// D2 pairs, and where the tile has lanes to spare, each kind starts a warp.
+// key1, key2: the rows' fields.  Returns lane -> row (-1: no row) and the
+// row whose fields a lane without a row repeats (so that it breaks no pair).
+struct LaneOrder {
+    int row[kTcRows], like[kTcRows];
+    bool pair1[kTcRows / 32], pair2[kTcRows / 32];    // per warp: the D1 / D2 loads take two passes
+};
+LaneOrder arrange_lanes(const std::vector<int32_t> &key1, const std::vector<int32_t> &key2)
+{
+    const int n = int(key1.size());
+    std::vector<int> by1(n);
+    for (int i = 0; i < n; ++i) by1[i] = i;
+    std::sort(by1.begin(), by1.end(), [&](int a, int b) {
+        return key1[a] != key1[b] ? key1[a] < key1[b] : key2[a] < key2[b];
+    });
+    std::vector<std::vector<int>> run;                // rows of each D1 field, by D2 field
+    for (int i : by1) {
+        if (run.empty() || key1[run.back()[0]] != key1[i]) run.emplace_back();
+        run.back().push_back(i);
+    }
+    std::vector<int> kind[4];                         // quads, D1 pairs, alone, D2 pairs
+    for (size_t a = 0; a < run.size(); ++a)
+        for (size_t b = a + 1; b < std::min(run.size(), a + 4) && run[a].size() >= 2; ++b) {
+            std::vector<std::pair<int, int>> both;    // rows of a and b with the same D2 field
+            for (int i : run[a])
+                for (int j : run[b])
+                    if (key2[i] == key2[j]) both.emplace_back(i, j);
+            for (size_t k = 0; k + 1 < both.size(); k += 2) {
+                const int q[4] = {both[k].first, both[k + 1].first, both[k].second, both[k + 1].second};
+                kind[0].insert(kind[0].end(), q, q + 4);
+                for (int h = 0; h < 4; ++h) {
+                    std::vector<int> &r = h < 2 ? run[a] : run[b];
+                    r.erase(std::find(r.begin(), r.end(), q[h]));
+                }
+            }
+        }
+    std::vector<int> left;
+    for (auto &r : run)
+        for (size_t k = 0; k < r.size(); ++k) {
+            if (k + 1 < r.size()) {
+                kind[1].insert(kind[1].end(), {r[k], r[k + 1]});
+                ++k;
+            } else {
+                left.push_back(r[k]);
+            }
+        }
+    std::stable_sort(left.begin(), left.end(), [&](int a, int b) { return key2[a] < key2[b]; });
+    for (size_t k = 0; k < left.size(); ++k) {
+        if (k + 1 < left.size() && key2[left[k]] == key2[left[k + 1]]) {
+            kind[3].insert(kind[3].end(), {left[k], left[k + 1]});
+            ++k;
+        } else {
+            kind[2].push_back(left[k]);
+        }
+    }
+    std::stable_sort(kind[2].begin(), kind[2].end(), [&](int a, int b) {
+        return key1[a] != key1[b] ? key1[a] < key1[b] : key2[a] < key2[b];
+    });
+    LaneOrder L;
+    int at = 0, spare = kTcRows - n;
+    for (int i = 0; i < kTcRows; ++i) L.row[i] = -1;
+    for (int k = 0; k < 4; ++k) {
+        const int pad = (32 - at % 32) % 32;
+        if (!kind[k].empty() && pad <= spare) {
+            at += pad;
+            spare -= pad;
+        }
+        for (int r : kind[k]) L.row[at++] = r;
+    }
+    // a lane without a row repeats the lane that its pairing mirrors, else the nearest row before it
+    for (int i = 0; i < kTcRows; ++i) {
+        L.like[i] = L.row[i];
+        if (L.row[i] >= 0) continue;
+        const int q = i & ~3;
+        L.like[i] = i == 0 ? 0 : L.like[i - 1];
+        if (i >= 4 && (i & 3)) L.like[i] = L.like[i - 1];
+        if (i != q && L.row[q] < 0) L.like[i] = L.like[q];
+    }
+    for (int w = 0; w < kTcRows / 32; ++w) {
+        auto merged = [&](const std::vector<int32_t> &key, int x) {
+            for (int l = 0; l < 32; ++l)
+                if (key[L.like[32 * w + l]] != key[L.like[32 * w + (l ^ x)]]) return false;
+            return true;
+        };
+        L.pair1[w] = merged(key1, 1) || merged(key1, 2);
+        L.pair2[w] = merged(key2, 1) || merged(key2, 2);
+    }
+    return L;
+}
+
 // tcgen05 tiles (see TcTile): the groups of each (grid, |n3|, signs of n1,
 // n2, n3) in order of n1, their rows by the centre of their r3 run, cut
 // greedily into tiles of at most 128 rows and a window of at most 64 r3
@@ -220,6 +319,7 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
     P.tc_tiles.clear();
     P.tc_rows.clear();
     P.tc_slots.clear();
+    P.tc_lanes.clear();
     P.tc_units.clear();
     P.tc_mma_products = 0;
     auto gflags = [](const Group &G) { return (G.n1 < 0 ? 1 : 0) | (G.n2 < 0 ? 2 : 0) | (G.n3 < 0 ? 4 : 0); };
@@ -257,10 +357,8 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
         if (cur_flags & 1) return "tcgen05 tiles need n1 >= 0";
         if (T.ncol > kTcMaxCols || T.nslot > kTcMaxSlots || T.nrow > kTcRows || tc_ring(T.ncol, T.nslot) == 0)
             return "tcgen05 tile limits";
-        // rows (tensor-memory lanes) in order of their D1 field, then D2
-        // field, and the staged fields numbered in that order: lanes of one
-        // shared-memory load phase then read the same D1 row (a broadcast) or
-        // consecutive slots (different banks)
+        // rows in order of their D1 field, then D2 field, and the staged
+        // fields in that order (arrange_lanes puts them on lanes)
         auto keys = [&](const std::pair<int32_t, int32_t> &gr) {
             const Group &G = P.groups[gr.first];
             const Row &rw = P.rows[gr.second];
@@ -276,31 +374,37 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
             if (slot_of(cur.slots, k.second) < 0) cur.slots.push_back(k.second);
         }
         if (int(cur.slots.size()) != T.nslot) return "tcgen05 tile slots";
+        std::vector<int32_t> key1, key2;
+        for (auto &gr : cur.rows) {
+            key1.push_back(keys(gr).first);
+            key2.push_back(keys(gr).second);
+        }
+        const LaneOrder lanes = arrange_lanes(key1, key2);
         // Bank groups: a 16-byte load of slot s falls in bank group s % 8
-        // (slot stride 144 bytes), and the 8 lanes of a load phase that read
-        // different slots of one group are served one after another.  Colour
-        // the fields greedily (first appearance order) so that the distinct
-        // D1 fields of each 8-row phase, and its distinct D2 fields, take
-        // distinct colours where they can, and number them colour + 8 k;
-        // numbers left free are padding slots that hold a field nothing
-        // stores (they read as zero).  Kept only if the tile still fits.
+        // (slot stride 272 bytes), and the lanes of a pass (8, or 16 that pair
+        // up) that read different slots of one group are served one after
+        // another.  Colour the fields greedily (first appearance order) so
+        // that the distinct D1 fields of each pass, and its distinct D2
+        // fields, take distinct colours where they can, and number them
+        // colour + 8 k; numbers left free are padding slots that hold a field
+        // nothing stores (they read as zero).  Kept only if the tile still fits.
         const int ns = T.nslot;
         std::vector<int> num(ns);
         {
             std::vector<std::vector<int>> adj(ns);
-            for (size_t g0 = 0; g0 < cur.rows.size(); g0 += 8) {
-                std::vector<int> U, V;
-                for (size_t r = g0; r < std::min(cur.rows.size(), g0 + 8); ++r) {
-                    const auto k = keys(cur.rows[r]);
-                    const int f1 = slot_of(cur.slots, k.first), f2 = slot_of(cur.slots, k.second);
-                    if (std::find(U.begin(), U.end(), f1) == U.end()) U.push_back(f1);
-                    if (std::find(V.begin(), V.end(), f2) == V.end()) V.push_back(f2);
-                }
-                for (const auto *grp : {&U, &V})
-                    for (int a : *grp)
-                        for (int b : *grp)
+            for (int side = 0; side < 2; ++side)
+                for (int g0 = 0; g0 < kTcRows;) {
+                    const int np = (side ? lanes.pair2 : lanes.pair1)[g0 / 32] ? 16 : 8;
+                    std::vector<int> grp;
+                    for (int l = g0; l < g0 + np; ++l) {
+                        const int f = slot_of(cur.slots, (side ? key2 : key1)[lanes.like[l]]);
+                        if (std::find(grp.begin(), grp.end(), f) == grp.end()) grp.push_back(f);
+                    }
+                    for (int a : grp)
+                        for (int b : grp)
                             if (a != b) adj[a].push_back(b);
-            }
+                    g0 += np;
+                }
             std::vector<int> col(ns, -1), cnt(8, 0), next(8, 0);
             int top = 0;
             for (int f = 0; f < ns; ++f) {
@@ -342,6 +446,10 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
             U_(cur_lev, a2, rw.r2) = 1;
             for (int j = 0; j < rw.n; ++j) U_(cur_lev, cur_n3, rw.r3a + j) = 1;
         }
+        for (int l = 0; l < kTcRows; ++l)
+            P.tc_lanes.push_back(TcLane{uint8_t(slot_of(cur.slots, key1[lanes.like[l]])),
+                                        uint8_t(slot_of(cur.slots, key2[lanes.like[l]])),
+                                        uint8_t(lanes.row[l] < 0 ? kTcNoRow : lanes.row[l]), 0});
         P.tc_slots.insert(P.tc_slots.end(), cur.slots.begin(), cur.slots.end());
         P.tc_mma_products += double(kTcRows) * T.ncol * double(M2);
         P.tc_tiles.push_back(T);

@@ -100,12 +100,12 @@ BISP_HD inline size_t tc_fixed_smem(int ncol, int nslot)
     return size_t(2 * tc_abuf(ncol)) * ncol * kTcTX * 4 + ((8 * size_t(nslot + ncol) + 256 + 127) & ~size_t(127));
 }
 // Buffers of the stage ring for a tile (0 if fewer than kTcMinRing fit):
-// each holds a stage of the tile's nslot + ncol fields and one zero row.
+// each holds a stage of the tile's nslot + ncol fields.
 BISP_HD inline int tc_ring(int ncol, int nslot)
 {
     const size_t fixed = tc_fixed_smem(ncol, nslot);
     if (fixed >= kTcSmem) return 0;
-    const size_t per = size_t(nslot + ncol + 1) * kTcSlotBytes;
+    const size_t per = size_t(nslot + ncol) * kTcSlotBytes;
     const int n = int((kTcSmem - fixed) / per);
     return n < kTcMinRing ? 0 : (n > kTcMaxRing ? kTcMaxRing : n);
 }
@@ -126,6 +126,12 @@ struct TcTile {
     int32_t ncol, nchunk;      // NC; x chunks of the M^2 grid
     int32_t flags;             // the rows' flags (all rows of a tile share them)
     int32_t pad;
+};
+// What tensor-memory lane `lane` of a tile does: its row of the tile (kTcNoRow:
+// none) and the two staged slots it multiplies (see arrange_lanes).
+constexpr int kTcNoRow = 255;
+struct TcLane {
+    uint8_t s1, s2, row, pad;
 };
 struct TcUnit {
     int32_t tile, chunk;
@@ -208,6 +214,7 @@ struct HostPlan {
     std::vector<TcTile> tc_tiles;
     std::vector<TcRow> tc_rows;
     std::vector<int32_t> tc_slots;
+    std::vector<TcLane> tc_lanes;       // kTcRows per tile
     std::vector<TcUnit> tc_units;       // by class (NC), then grid, x chunk, tile
     int64_t tc_class_begin[kTcClasses + 1] = {};
     double tc_mma_products = 0;         // sum over tiles of 128 NC M^2 (lane-column-points)

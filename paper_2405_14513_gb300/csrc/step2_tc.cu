@@ -66,7 +66,9 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
            (uint64_t((sbo & 0x3FFFF) >> 4) << 32) | (uint64_t(1) << 46);
 }
 
-// Instruction descriptor: FP32 accumulator, A and B FP16 (format 0), both K-major, N, M.
+// Instruction descriptor: FP32 accumulator, A and B FP16 (format 0), both
+// K-major, N, M; kNegA, kNegB: the operand is read negated.
+constexpr uint32_t kNegA = 1u << 13, kNegB = 1u << 14;
 template <int N>
 __host__ __device__ constexpr uint32_t idesc_f16()
 {
@@ -100,17 +102,17 @@ __device__ __forceinline__ void add2(float &a, float &b, uint32_t x, uint32_t y)
         : "+f"(a), "+f"(b) : "r"(x), "r"(y));
 }
 
-// (x, y) -> hi + lo, two FP16 pairs (x in the low halves): hi rounded to
-// nearest, lo the remainder x - hi (exact in FP32) rounded to nearest.  The
-// remainder is taken by the mixed-precision subtraction (one instruction,
-// hi - x), so the pair costs two conversions and two subtractions.
-__device__ __forceinline__ void split2(float x, float y, uint32_t &hi, uint32_t &lo)
+// (x, y) -> hi - nlo, two FP16 pairs (x in the low halves): hi rounded to
+// nearest, nlo the remainder hi - x (exact in FP32) rounded to nearest.  The
+// remainder is taken by the mixed-precision subtraction, one instruction; it
+// only gives hi - x, and the MMAs that read a low part negate it.
+__device__ __forceinline__ void split2(float x, float y, uint32_t &hi, uint32_t &nlo)
 {
     float rx, ry;
     asm("cvt.rn.f16x2.f32 %0, %2, %1;" : "=r"(hi) : "f"(x), "f"(y));
     asm("{\n.reg .b16 l, h;\nmov.b32 {l, h}, %2;\nsub.rn.f32.f16 %0, l, %3;\nsub.rn.f32.f16 %1, h, %4;\n}\n"
         : "=f"(rx), "=f"(ry) : "r"(hi), "f"(x), "f"(y));
-    asm("cvt.rn.f16x2.f32 %0, %2, %1;" : "=r"(lo) : "f"(-rx), "f"(-ry));
+    asm("cvt.rn.f16x2.f32 %0, %2, %1;" : "=r"(nlo) : "f"(rx), "f"(ry));
 }
 
 // No memory clobber: tensor memory is not memory the compiler tracks, so
@@ -183,7 +185,8 @@ __device__ __forceinline__ void add_accumulator(uint32_t tcol, float (&acc)[NH])
 // st + 2 wait for A(st + 2), signalled after that read.
 constexpr int kThreads = 352;
 constexpr int kCompute = 256;
-constexpr int kProdFields = (kTcMaxSlots + kTcMaxCols + 7) / 8;   // fields per producer lane
+constexpr int kProd0 = 288;                  // first producer thread
+constexpr int kProdFields = (kTcMaxSlots + kTcMaxCols + 7) / 8;   // most fields per producer lane
 
 struct TcSync {
     uint64_t full[kTcMaxRing], empty[kTcMaxRing], aready[3], mdone[2], drain;
@@ -377,6 +380,59 @@ __device__ __forceinline__ bool compute_loop(const CompArgs &ca, float (&acc)[NC
     return true;
 }
 
+// What a producer lane needs (see k_step2_tc).
+struct ProdArgs {
+    unsigned char *sS;
+    const int64_t *offs;
+    const float2 *src;         // the unit's first grid point
+    volatile int *abort;
+    TcSync *sy;
+    int nf, rowb, S, nstage, ntail, spins, pl;
+};
+
+// The producers' loop: lane pl of the 64 copies piece p = pl % 8 (grid points
+// 2p, 2p + 1) of each half of fields pl / 8, pl / 8 + 8, ... (at most NFL of
+// them); their offsets (in 16-element units: every stored field starts at a
+// multiple of 16) are held in registers.  The last stage may have one half.
+// Returns false if a wait gave up.
+template <int NFL>
+__device__ __forceinline__ bool produce(const ProdArgs &pa)
+{
+    const int p = pa.pl & 7, f0 = pa.pl >> 3;
+    uint32_t o16[NFL];
+#pragma unroll
+    for (int k = 0; k < NFL; ++k) {
+        const int f = f0 + 8 * k;
+        const int64_t o = f < pa.nf ? pa.offs[f] : -1;
+        o16[k] = o < 0 ? 0xFFFFFFFFu : uint32_t(o >> 4);
+    }
+    int q = 0;                                   // ring buffer st % S
+    uint32_t ph = 0;                             // its phase: (st / S) & 1
+    for (int st = 0; st < pa.nstage; ++st) {
+        if (st >= pa.S && !mbar_wait_abort(&pa.sy->empty[q], ph ^ 1u, pa.abort, pa.spins)) return false;
+        const float2 *src = pa.src + int64_t(st) * kTX + 2 * p;
+        const uint32_t dst = su32(pa.sS + q * pa.rowb + f0 * kSlotBytes + p * 16);
+        if (st + 1 < pa.nstage || pa.ntail == kTX) {
+#pragma unroll
+            for (int k = 0; k < NFL; ++k)
+                if (o16[k] != 0xFFFFFFFFu) {
+                    cp_async16(dst + 8 * k * kSlotBytes, src + (int64_t(o16[k]) << 4));
+                    cp_async16(dst + 8 * k * kSlotBytes + kTX * 4, src + (int64_t(o16[k]) << 4) + kTX / 2);
+                }
+        } else {
+#pragma unroll
+            for (int k = 0; k < NFL; ++k)
+                if (o16[k] != 0xFFFFFFFFu) cp_async16(dst + 8 * k * kSlotBytes, src + (int64_t(o16[k]) << 4));
+        }
+        asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(su32(&pa.sy->full[q])) : "memory");
+        if (++q == pa.S) {
+            q = 0;
+            ph ^= 1u;
+        }
+    }
+    return true;
+}
+
 // Two blocks per SM (sharing its 227 KB of shared memory and 512
 // tensor-memory columns) hold 22 warps, 6 on some of the SM's four
 // schedulers, whose register files are 16384 each: at most 80 registers a
@@ -404,10 +460,10 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
     const int spins = args.wait_spins;
     const int nslot = T.nslot, nf = nslot + NC;
     const int S = tc_ring(NC, nslot);            // ring buffers (>= 2; the plan checked)
-    const int rowb = (nf + 1) * kSlotBytes;      // one ring buffer: nf fields and a zero row
+    const int rowb = nf * kSlotBytes;            // one ring buffer: nf fields
     // shared memory: B high and low parts [NA][BB] each (canonical layout),
-    // field offsets [nf], barriers, ring [S][nf + 1][kSlotBytes] (a stage of D1 / D2
-    // slots, the B window, a zero row)
+    // field offsets [nf], barriers, ring [S][nf][kSlotBytes] (a stage of D1 / D2
+    // slots and the B window)
     unsigned char *sHi = smem;
     unsigned char *sLo = smem + NA * BB;
     int64_t *offs = reinterpret_cast<int64_t *>(smem + 2 * NA * BB);
@@ -442,10 +498,10 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
     __syncthreads();
-    // fields that are not stored (past the last ring), and the zero row, read as zero
-    for (int i = t; i < S * (nf + 1) * 16; i += kThreads) {
-        const int q = i / ((nf + 1) * 16), rem = i - q * (nf + 1) * 16, f = rem >> 4, p = rem & 15;
-        if (f < nf && offs[f] >= 0) continue;
+    // fields that are not stored (past the last ring, padding slots) read as zero
+    for (int i = t; i < S * nf * 16; i += kThreads) {
+        const int q = i / (nf * 16), rem = i - q * nf * 16, f = rem >> 4, p = rem & 15;
+        if (offs[f] >= 0) continue;
         *reinterpret_cast<float4 *>(sS + q * rowb + f * kSlotBytes + p * 16) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -462,44 +518,15 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
     bool ok = true;
 
     if (warp >= 9) {
-        // producers: lane l of the 64 copies piece p = l % 8 (grid points
-        // 2p, 2p + 1) of fields l / 8, l / 8 + 8, ...; their offsets (in
-        // 16-element units: every stored field starts at a multiple of 16)
-        // are held in registers
-        const int pl = t - 288, p = pl & 7, f0 = pl >> 3;
-        // (all kProdFields copies are issued under a predicate: a loop
-        // bound by the fields that exist was 6% slower)
-        uint32_t o16[kProdFields];
-#pragma unroll
-        for (int k = 0; k < kProdFields; ++k) {
-            const int f = f0 + 8 * k;
-            const int64_t o = f < nf ? offs[f] : -1;
-            o16[k] = o < 0 ? 0xFFFFFFFFu : uint32_t(o >> 4);
-        }
-        // A stage has 32 grid points: the lane copies piece p of each half;
-        // the last stage may have one half
-        int q = 0;                                   // ring buffer sb % S
-        uint32_t ph = 0;                             // its phase: (sb / S) & 1
-        for (int sb = 0; sb < nstage && ok; ++sb) {
-            if (sb >= S) ok = mbar_wait_abort(&sy->empty[q], ph ^ 1u, abort, spins);
-            if (!ok) break;
-            const float2 *src = dstore + x0 + int64_t(sb) * kTX + 2 * p;
-            const uint32_t dst = su32(sS + q * rowb + f0 * kSlotBytes + p * 16);
-            if (sb + 1 < nstage || ntail == kTX) {
-#pragma unroll
-                for (int k = 0; k < kProdFields; ++k)
-                    if (o16[k] != 0xFFFFFFFFu) {
-                        cp_async16(dst + 8 * k * kSlotBytes, src + (int64_t(o16[k]) << 4));
-                        cp_async16(dst + 8 * k * kSlotBytes + kTX * 4, src + (int64_t(o16[k]) << 4) + kTX / 2);
-                    }
-            } else {
-#pragma unroll
-                for (int k = 0; k < kProdFields; ++k)
-                    if (o16[k] != 0xFFFFFFFFu) cp_async16(dst + 8 * k * kSlotBytes, src + (int64_t(o16[k]) << 4));
-            }
-            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(su32(&sy->full[q])) : "memory");
-            if (++q == S) { q = 0; ph ^= 1u; }
-        }
+        // producers, with as many field copies unrolled as the tile needs (a
+        // copy that a lane does not need still issues its predicated
+        // instructions: at 512^3 tiles have 60 to 130 fields, 8 to 17 per lane,
+        // of the 40 that the largest could have)
+        const ProdArgs pa{sS, offs, dstore + x0, abort, sy, nf, rowb, S, nstage, ntail, spins, t - kProd0};
+        if (nf <= 8 * 10) ok = produce<10>(pa);
+        else if (nf <= 8 * 14) ok = produce<14>(pa);
+        else if (nf <= 8 * 20) ok = produce<20>(pa);
+        else ok = produce<kProdFields>(pa);
         asm volatile("cp.async.wait_all;\n" ::: "memory");
     } else if (warp == 8) {
         // MMA issue: high A x high B, low A x high B and high A x low B over
@@ -531,9 +558,9 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
 #pragma unroll
                     for (int j = 0; j < KS; ++j) mma_f16(d, a + 8 * j, dh + bo + j * kstep, ID, j > 0);
 #pragma unroll
-                    for (int j = 0; j < KS; ++j) mma_f16(d, a + 32 + 8 * j, dh + bo + j * kstep, ID, 1);
+                    for (int j = 0; j < KS; ++j) mma_f16(d, a + 32 + 8 * j, dh + bo + j * kstep, ID | kNegA, 1);
 #pragma unroll
-                    for (int j = 0; j < KS; ++j) mma_f16(d, a + 8 * j, dl + bo + j * kstep, ID, 1);
+                    for (int j = 0; j < KS; ++j) mma_f16(d, a + 8 * j, dl + bo + j * kstep, ID | kNegB, 1);
                 };
                 if (st + 1 < nstage || ntail == kTX) issue(std::integral_constant<int, 4>{});
                 else issue(std::integral_constant<int, 2>{});
@@ -545,16 +572,17 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
         }
         __syncwarp();
     } else {
-        // compute warps: the thread owns tensor-memory lane (row) 32 (warp % 4)
-        // + lane; rows past the tile's end read the zero row.  The loop is
-        // instantiated per sign pattern (uniform over the tile; n1 >= 0)
+        // compute warps: the thread owns tensor-memory lane 32 (warp % 4) +
+        // lane; a lane without a row repeats a neighbour's fields, and its sums
+        // go nowhere.  The loop is instantiated per sign pattern (uniform over
+        // the tile; n1 >= 0)
         const int quarter = warp & 3, half = warp >> 2;
-        const int row = quarter * 32 + lane;
-        const bool live = row < T.nrow;
+        const TcLane ln = args.lanes[size_t(U.tile) * kTcRows + quarter * 32 + lane];
+        const bool live = ln.row != kTcNoRow;
         TcRow R{};
-        if (live) R = args.rows[T.row0 + row];
+        if (live) R = args.rows[T.row0 + ln.row];
         CompArgs ca{sS, sHi, sLo, tmem + (uint32_t(quarter * 32) << 16), abort, sy, rowb, nslot, S, nstage, ntail, spins,
-                    t, half, live ? int(R.s1) : nf, live ? int(R.s2) : nf};
+                    t, half, int(ln.s1), int(ln.s2)};
         float acc[NC / 2];
         switch (T.flags) {
         case 0: ok = compute_loop<NC, false, false, false>(ca, acc); break;
