@@ -73,7 +73,8 @@ struct bisp_plan {
     TcLane *d_tc_lanes = nullptr;
     TcUnit *d_tc_units = nullptr;
     int64_t *d_doff = nullptr;
-    Record *d_rec = nullptr;
+    Record *d_rec = nullptr;             // binning records: FP64 plans keep these,
+    RecordF *d_recf = nullptr;           // the others their FP32 form
     int64_t *d_bin_start = nullptr;
     int64_t *d_chunk_lo = nullptr, *d_chunk_hi = nullptr, *d_bin_chunk = nullptr;   // binning chunks
     double *d_den = nullptr;
@@ -605,7 +606,9 @@ int build_plan(bisp_plan *p, const bisp_desc *desc, cudaStream_t s)
     if (!st) st = upload(p, &p->d_tc_lanes, P.tc_lanes, s);
     if (!st) st = upload(p, &p->d_tc_units, P.tc_units, s);
     if (!st) st = upload(p, &p->d_doff, P.doff, s);
-    if (!st) st = upload(p, &p->d_rec, P.records, s);
+    const bool fp64 = desc->precision == BISP_PREC_FP64;
+    if (!st && fp64) st = upload(p, &p->d_rec, P.records, s);
+    if (!st && !fp64) st = dev_alloc(p, &p->d_recf, P.records.size());
     if (!st) st = upload(p, &p->d_bin_start, P.bin_start, s);
     if (!st) st = upload(p, &p->d_chunk_lo, P.chunk_lo, s);
     if (!st) st = upload(p, &p->d_chunk_hi, P.chunk_hi, s);
@@ -616,20 +619,29 @@ int build_plan(bisp_plan *p, const bisp_desc *desc, cudaStream_t s)
     // plan-time denominators of Eq. bs_lm2_1 (FP64)
     {
         double *d_nt = nullptr, *d_epi = nullptr;
-        void *q = nullptr, *q2 = nullptr;
+        Record *d_rec = p->d_rec;
+        void *q = nullptr, *q2 = nullptr, *q3 = nullptr;
         if (cudaMalloc(&q, std::max<size_t>(P.rec_ntri.size() * sizeof(double), 16)) != cudaSuccess ||
-            cudaMalloc(&q2, std::max<size_t>(size_t(P.max_chunks * epi_nlm) * sizeof(double), 16)) != cudaSuccess) {
+            cudaMalloc(&q2, std::max<size_t>(size_t(P.max_chunks * epi_nlm) * sizeof(double), 16)) != cudaSuccess ||
+            (!fp64 && cudaMalloc(&q3, std::max<size_t>(P.records.size() * sizeof(Record), 16)) != cudaSuccess)) {
             cudaGetLastError();
             if (q) cudaFree(q);
+            if (q2) cudaFree(q2);
             return fail(BISP_OUT_OF_MEMORY, "device memory for the denominators");
         }
         d_nt = static_cast<double *>(q);
         d_epi = static_cast<double *>(q2);
         cudaError_t e = cudaMemcpyAsync(d_nt, P.rec_ntri.data(), P.rec_ntri.size() * sizeof(double),
                                         cudaMemcpyHostToDevice, s);
+        if (!fp64) {
+            d_rec = static_cast<Record *>(q3);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(d_rec, P.records.data(), P.records.size() * sizeof(Record), cudaMemcpyHostToDevice, s);
+            if (e == cudaSuccess) e = launch_records_f(d_rec, p->d_recf, int64_t(P.records.size()), s);
+        }
         for (const View &v : P.views)
             if (e == cudaSuccess) {
-                const EpiArgs ea{p->d_rec, p->d_chunk_lo + v.chunk_off, p->d_chunk_hi + v.chunk_off, v.n_chunks,
+                const EpiArgs ea{d_rec, nullptr, p->d_chunk_lo + v.chunk_off, p->d_chunk_hi + v.chunk_off, v.n_chunks,
                                  p->d_bin_chunk + v.bc_off, v.n_bins, d_epi, 0};
                 e = launch_epilogue<double>(1, ea, d_nt, v.l_lo, v.l_hi, nullptr, 1.0, p->d_den + v.out_off,
                                             Batch{}, s);
@@ -640,6 +652,7 @@ int build_plan(bisp_plan *p, const bisp_desc *desc, cudaStream_t s)
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         cudaFree(d_nt);
         cudaFree(d_epi);
+        if (q3) cudaFree(q3);
         if (e != cudaSuccess) return fail(BISP_CUDA_ERROR, std::string("denominators: ") + cudaGetErrorString(e));
         std::vector<double>().swap(P.rec_ntri);
     }
@@ -775,7 +788,7 @@ int run_estimate(bisp_plan *p, const R *delta, int batch, unsigned char *ws, dou
     {   // binning and the ratio of Eq. bs_lm2_1
         StageMark m(p, BISP_STAGE_BIN, int(2 * P.views.size()), s);
         for (const View &v : P.views) {
-            const EpiArgs ea{p->d_rec, p->d_chunk_lo + v.chunk_off, p->d_chunk_hi + v.chunk_off, v.n_chunks,
+            const EpiArgs ea{p->d_rec, p->d_recf, p->d_chunk_lo + v.chunk_off, p->d_chunk_hi + v.chunk_off, v.n_chunks,
                              p->d_bin_chunk + v.bc_off, v.n_bins, reinterpret_cast<double *>(ws + p->off_epi), fs};
             CK(launch_epilogue<W>(0, ea, Ssum, v.l_lo, v.l_hi, p->d_den + v.out_off, 1.0 / (P.volume * double(ng2)),
                                   B + v.out_off, to_out, s, p->precision != BISP_PREC_FP64));

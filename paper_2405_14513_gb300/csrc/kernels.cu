@@ -713,18 +713,62 @@ __constant__ double c_nlm[9][9];
 __constant__ double c_pref[9];
 // Legendre recurrence ratios (2l+1)/(l+1-m) and (l+m)/(l+1-m), l, m <= 8
 __constant__ double c_rec[2][9][9];
+// the same in FP32, so that the FP32 weights take them as operands
+__constant__ float c_nlm_f[9][9];
+__constant__ float c_rec_f[2][9][9];
+template <typename Y> __device__ __forceinline__ Y nlm_of(int l, int m)
+{
+    if constexpr (sizeof(Y) == 4) return c_nlm_f[l][m]; else return Y(c_nlm[l][m]);
+}
+template <typename Y> __device__ __forceinline__ Y rec_of(int k, int l, int m)
+{
+    if constexpr (sizeof(Y) == 4) return c_rec_f[k][l][m]; else return Y(c_rec[k][l][m]);
+}
+
+__global__ void __launch_bounds__(256)
+k_records_f(const Record *__restrict__ rec, RecordF *__restrict__ recf, int64_t n)
+{
+    for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < n; k += int64_t(gridDim.x) * blockDim.x) {
+        const Record r = rec[k];
+        recf[k] = RecordF{r.s_index, r.flags, float(r.pz), float(r.cphi)};
+    }
+}
+
+// w 2^-896, exactly, for a normal (or zero) w: the float's sign, exponent
+// field and mantissa moved to a double's, three integer operations.
+__device__ __forceinline__ double widen_scaled(float w)
+{
+    const int u = __float_as_int(w);
+    return __hiloint2double((u >> 3) & int(0x8FFFFFFFu), u << 29);
+}
 
 // W: type of the sums over records; Y: type the Y_lm of each record are
 // computed in (FP32 for the FP32-transform paths, whose tolerance is 1e-4;
 // FP64 for the FP64 path and the plan-time denominators).  The moments
 // written are lm_lo .. (LMAX/2 + 1)^2 - 1 (even l from l_lo = 2 sqrt(lm_lo)),
 // nlm_out = that count per bin, for out and den alike.
+//
+// One warp per chunk.  With FP32 weights and FP64 sums the slow FP64 pipe (two
+// lanes a clock and SM) bounds it, so a record costs it one FMA per moment and
+// two products: the weight is widened in the integer pipe (as w 2^-896; 2^448 goes
+// to the value and 2^448 to the sum, so neither can overflow below 1e173) where
+// a conversion instruction took as long as the FMA, and the orientation is read
+// as FP32 and the recurrences' constants are FP32 operands in constant memory.
+// The next record's value and the one after's record are loaded ahead.  With
+// conversions of all of these, and one thread per bin in k_epi_fin: 512^3 (1.1e8
+// records) 7.5 -> 3.2 ms, 256^3 1.21 -> 0.52 ms; 64^3, mostly for its shorter chunks
+// (bin_chunk_len), 184 -> 26 us.
 template <typename W, typename Y, int LMAX>
 __global__ void __launch_bounds__(256)
-k_epi_part(int mode, const Record *__restrict__ rec, const int64_t *__restrict__ chunk_lo,
-           const int64_t *__restrict__ chunk_hi, int64_t nchunks, const double *__restrict__ value,
-           double *__restrict__ partial, int64_t fs_in, int64_t fs_part)
+k_epi_part(int mode, const Record *__restrict__ rec, const RecordF *__restrict__ recf,
+           const int64_t *__restrict__ chunk_lo, const int64_t *__restrict__ chunk_hi, int64_t nchunks,
+           const double *__restrict__ value, double *__restrict__ partial, int64_t fs_in, int64_t fs_part)
 {
+    constexpr bool F32 = sizeof(Y) == 4;                  // FP32 weights (mode 0 only)
+    constexpr bool WIDEN = F32 && sizeof(W) == 8;
+    using Rec = typename std::conditional<F32, RecordF, Record>::type;
+    const Rec *recs;
+    if constexpr (F32) recs = recf; else recs = rec;
     value = field_ptr(value, fs_in);
     partial = field_ptr(partial, fs_part);
     constexpr int NLM = (LMAX / 2 + 1) * (LMAX / 2 + 1);
@@ -734,12 +778,24 @@ k_epi_part(int mode, const Record *__restrict__ rec, const int64_t *__restrict__
     W acc[NLM];
 #pragma unroll
     for (int i = 0; i < NLM; ++i) acc[i] = W(0);
-    const int64_t k0 = chunk_lo[ch], k1 = chunk_hi[ch];
-    for (int64_t k = k0 + lane; k < k1; k += 32) {
-        const Record R = rec[k];
+    const int64_t k1 = chunk_hi[ch];
+    int64_t k = chunk_lo[ch] + lane;
+    auto load_value = [&](const Rec &r, int64_t at) { return mode == 0 ? value[r.s_index] : value[at]; };
+    Rec R{}, Rn{};
+    double val = 0.0;
+    if (k < k1) {
+        R = recs[k];
+        if (k + 32 < k1) Rn = recs[k + 32];
+        val = load_value(R, k);
+    }
+    for (; k < k1; k += 32) {
+        double val_n = 0.0;
+        Rec Rnn{};
+        if (k + 64 < k1) Rnn = recs[k + 64];
+        if (k + 32 < k1) val_n = load_value(Rn, k + 32);
         const Y x = Y(R.pz), c = Y(R.cphi);
         const W mult = (R.flags & 1) ? W(1) : W(2);
-        const W v = W(mode == 0 ? value[R.s_index] : value[k]) * mult;
+        const W v = W(val) * (WIDEN ? W(0x1p448) * mult : mult);
         const bool deg = (R.flags & 2) != 0;
         const Y s = sqrt(max(Y(0), Y(1) - x * x));
         Y pmm = Y(1), tm1 = Y(1), tm2 = Y(1);   // P_m^m; cos(m phi), cos((m-1) phi)
@@ -754,35 +810,60 @@ k_epi_part(int mode, const Record *__restrict__ rec, const int64_t *__restrict__
 #pragma unroll
             for (int l = m; l <= LMAX; ++l) {
                 if ((l & 1) == 0) {
-                    const Y y = Y(c_nlm[l][m]) * pl;
+                    const Y y = nlm_of<Y>(l, m) * pl;
                     const int idx = (l >> 1) * (l >> 1) + m;
-                    if (mode == 0) {
+                    if (F32 || mode == 0) {
                         const Y w = deg ? (m == 0 ? y : Y(0)) : y * tm;
-                        acc[idx] += W(w) * v;
+                        if constexpr (WIDEN) acc[idx] = fma(widen_scaled(w), v, acc[idx]);
+                        else acc[idx] += W(w) * v;
                     } else {
                         acc[idx] += W(y) * W(y) * v;
                     }
                 }
                 // P_{l+1}^m = ((2l+1) x P_l^m - (l+m) P_{l-1}^m) / (l+1-m), with
                 // the two ratios from constant memory (no division per record)
-                const Y pn = Y(c_rec[0][l][m]) * x * pl - Y(c_rec[1][l][m]) * plm1;
+                const Y pn = rec_of<Y>(0, l, m) * x * pl - rec_of<Y>(1, l, m) * plm1;
                 plm1 = pl;
                 pl = pn;
             }
             tm2 = tm1;
             tm1 = tm;
         }
+        R = Rn;
+        Rn = Rnn;
+        val = val_n;
     }
+    // Sums across the warp: while more than one sum is left, the step of
+    // distance o gives half of them away (the lanes with bit o keep the upper
+    // half), so NLM sums cost about NLM exchanges and not 5 NLM; then plain
+    // halving steps.  At the end lane l holds sum (l's bits from the top).
+    constexpr int P2 = NLM <= 1 ? 1 : (NLM <= 4 ? 4 : (NLM <= 16 ? 16 : 32));
+    W red[P2];
 #pragma unroll
-    for (int i = 0; i < NLM; ++i) {
-        W v = acc[i];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) partial[ch * NLM + i] = double(v);
+    for (int i = 0; i < P2; ++i) red[i] = i < NLM ? acc[i] : W(0);
+    int idx = 0;
+#pragma unroll
+    for (int o = 16, n = P2; o >= 1; o >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int k = 0; k < P2 / 2; ++k) {
+                if (k >= n) break;
+                const W keep = up ? red[k + n] : red[k];
+                const W give = up ? red[k] : red[k + n];
+                red[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+            if (up) idx += n;
+        } else {
+            red[0] += __shfl_xor_sync(0xffffffffu, red[0], o);
+        }
     }
+    if ((lane & (32 / P2 - 1)) == 0 && idx < NLM) partial[ch * NLM + idx] = double(red[0]) * (WIDEN ? 0x1p448 : 1.0);
 }
 
-// One thread per bin: its chunks' partial sums in chunk order, then (mode
-// 0) the ratio of Eq. bs_lm2_1 or (mode 1) the sum itself.
+// One thread per bin and moment: the bin's chunks' partial sums in chunk
+// order, then (mode 0) the ratio of Eq. bs_lm2_1 or (mode 1) the sum itself.
 template <int LMAX>
 __global__ void __launch_bounds__(256)
 k_epi_fin(int mode, const int64_t *__restrict__ bin_chunk, int64_t nbins, const double *__restrict__ partial,
@@ -792,21 +873,21 @@ k_epi_fin(int mode, const int64_t *__restrict__ bin_chunk, int64_t nbins, const 
     partial = field_ptr(partial, fs_part);
     out = field_ptr(out, fs_out);
     constexpr int NLM = (LMAX / 2 + 1) * (LMAX / 2 + 1);
-    const int64_t b = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (b >= nbins) return;
+    const int64_t o = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (o >= nbins * nlm_out) return;
+    const int64_t b = o / nlm_out;
+    const int i = int(o - b * nlm_out) + lm_lo;
     const int64_t c0 = bin_chunk[b], c1 = bin_chunk[b + 1];
-    for (int i = lm_lo; i < NLM; ++i) {
-        double v = 0.0;
-        for (int64_t ch = c0; ch < c1; ++ch) v += partial[ch * NLM + i];
-        const int64_t o = b * nlm_out + (i - lm_lo);
-        if (mode == 0) {
-            int l = 0;
-            while ((l / 2 + 1) * (l / 2 + 1) <= i) l += 2;
-            const double d = den[o];
-            out[o] = d > 0.0 ? c_pref[l] * v * norm / d : __longlong_as_double(0x7ff8000000000000LL);
-        } else {
-            out[o] = v;
-        }
+    double v = 0.0;
+#pragma unroll 8
+    for (int64_t ch = c0; ch < c1; ++ch) v += partial[ch * NLM + i];
+    if (mode == 0) {
+        int l = 0;
+        while ((l / 2 + 1) * (l / 2 + 1) <= i) l += 2;
+        const double d = den[o];
+        out[o] = d > 0.0 ? c_pref[l] * v * norm / d : __longlong_as_double(0x7ff8000000000000LL);
+    } else {
+        out[o] = v;
     }
 }
 
@@ -990,9 +1071,9 @@ template <typename W, typename Y, int LMAX>
 cudaError_t epilogue_l(int mode, const EpiArgs &e, const double *value, const double *den, double norm, double *out,
                        const Batch &fb, int lo, int n, cudaStream_t s)
 {
-    const dim3 g1(unsigned((e.nchunks * 32 + 255) / 256), fb.nf), g2(unsigned((e.nbins + 255) / 256), fb.nf);
+    const dim3 g1(unsigned((e.nchunks * 32 + 255) / 256), fb.nf), g2(unsigned((e.nbins * n + 255) / 256), fb.nf);
     if (e.nchunks > 0)
-        k_epi_part<W, Y, LMAX><<<g1, 256, 0, s>>>(mode, e.rec, e.chunk_lo, e.chunk_hi, e.nchunks, value, e.partial,
+        k_epi_part<W, Y, LMAX><<<g1, 256, 0, s>>>(mode, e.rec, e.recf, e.chunk_lo, e.chunk_hi, e.nchunks, value, e.partial,
                                                   fb.fs_in, e.fs_part);
     k_epi_fin<LMAX><<<g2, 256, 0, s>>>(mode, e.bin_chunk, e.nbins, e.partial, den, norm, out, e.fs_part, fb.fs_out,
                                        lo, n);
@@ -1020,8 +1101,16 @@ cudaError_t launch_epilogue(int mode, const EpiArgs &e, const double *value, int
 {
     if (e.nbins == 0) return cudaSuccess;
     if (l_lo < 0 || l_lo > l_hi || (l_lo & 1)) return cudaErrorInvalidValue;
+    if (fp32_weights && mode != 0) return cudaErrorInvalidValue;
     if (fp32_weights) return epilogue_lmax<W, float>(mode, e, value, l_lo, l_hi, den, norm, out, fb, s);
     return epilogue_lmax<W, W>(mode, e, value, l_lo, l_hi, den, norm, out, fb, s);
+}
+
+cudaError_t launch_records_f(const Record *rec, RecordF *recf, int64_t n, cudaStream_t s)
+{
+    if (n == 0) return cudaSuccess;
+    k_records_f<<<unsigned(std::min<int64_t>((n + 255) / 256, 152 * 16)), 256, 0, s>>>(rec, recf, n);
+    return cudaGetLastError();
 }
 
 // Every kernel that takes more than 48 KB of dynamic shared memory is
@@ -1079,6 +1168,14 @@ cudaError_t set_ylm_constants(const double nlm[9][9], const double pref[9], cuda
     cudaError_t e = cudaMemcpyToSymbolAsync(c_nlm, nlm, sizeof(double) * 81, 0, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(c_pref, pref, sizeof(double) * 9, 0, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(c_rec, rec, sizeof(rec), 0, cudaMemcpyHostToDevice, s);
+    float nlm_f[9][9], rec_f[2][9][9];
+    for (int l = 0; l < 9; ++l)
+        for (int m = 0; m < 9; ++m) {
+            nlm_f[l][m] = float(nlm[l][m]);
+            for (int k = 0; k < 2; ++k) rec_f[k][l][m] = float(rec[k][l][m]);
+        }
+    if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(c_nlm_f, nlm_f, sizeof(nlm_f), 0, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaMemcpyToSymbolAsync(c_rec_f, rec_f, sizeof(rec_f), 0, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // the tables above live on this stack
     return e;
 }

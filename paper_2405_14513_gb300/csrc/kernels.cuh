@@ -170,7 +170,8 @@ cudaError_t launch_reduce_partials(const Group *groups, int64_t ngroups, const d
 // partial sums per moment in `partial` [nchunks][moments of l <= l_hi]),
 // then each bin adds its chunks in order (one thread per bin).
 struct EpiArgs {
-    const Record *rec;
+    const Record *rec;                    // fp32_weights: not read (recf is)
+    const RecordF *recf;
     const int64_t *chunk_lo, *chunk_hi;   // record range of each chunk
     int64_t nchunks;
     const int64_t *bin_chunk;             // [nbins + 1]: first chunk of each bin
@@ -181,6 +182,9 @@ struct EpiArgs {
 template <typename W>
 cudaError_t launch_epilogue(int mode, const EpiArgs &e, const double *value, int l_lo, int l_hi, const double *den,
                             double norm, double *out, const Batch &fb, cudaStream_t s, bool fp32_weights = false);
+
+// The records' FP32 form.
+cudaError_t launch_records_f(const Record *rec, RecordF *recf, int64_t n, cudaStream_t s);
 
 // Y_lm normalisations nlm[l][m] and the prefactors sqrt((2l+1)/(4 pi)).
 cudaError_t set_ylm_constants(const double nlm[9][9], const double pref[9], cudaStream_t s);

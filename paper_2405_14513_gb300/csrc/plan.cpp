@@ -920,8 +920,9 @@ void sort_records(HostPlan &P)
     }
     std::vector<Record>().swap(P.records_s);
     std::vector<double>().swap(P.ntri_s);
-    // binning chunks: each bin's records in runs of at most kBinChunk, so no
-    // warp of the binning walks a whole large bin alone
+    // binning chunks: each bin's records in runs of at most bin_chunk_len, so
+    // no warp of the binning walks a whole large bin alone
+    const int64_t chunk = bin_chunk_len(int64_t(n));
     P.chunk_lo.clear();
     P.chunk_hi.clear();
     P.bin_chunk.assign(total_bs, 0);
@@ -933,9 +934,9 @@ void sort_records(HostPlan &P)
         v.bc_off = bc;
         for (int64_t b = 0; b < v.n_bins; ++b) {
             P.bin_chunk[bc + b] = int64_t(P.chunk_lo.size()) - v.chunk_off;
-            for (int64_t k = bs[b]; k < bs[b + 1]; k += kBinChunk) {
+            for (int64_t k = bs[b]; k < bs[b + 1]; k += chunk) {
                 P.chunk_lo.push_back(k);
-                P.chunk_hi.push_back(std::min(k + kBinChunk, bs[b + 1]));
+                P.chunk_hi.push_back(std::min(k + chunk, bs[b + 1]));
             }
         }
         v.n_chunks = int64_t(P.chunk_lo.size()) - v.chunk_off;

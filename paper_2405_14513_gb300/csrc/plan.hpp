@@ -168,6 +168,13 @@ struct Record {
     double cphi;               // cos(phi) of p
 };
 
+// The same for the paths that weigh records in FP32: one 16-byte load, and no
+// conversion per record.
+struct RecordF {
+    int32_t s_index, flags;
+    float pz, cphi;
+};
+
 // A binning of the combinations (Eq. bs_lm2_1): the moments of even l
 // l_lo .. l_hi on an n_mu x n_t grid of (mu, t) bins; one field's output
 // block [n_k1][n_mu][n_t][n_lm] starts at out_off doubles, its records in
@@ -175,7 +182,7 @@ struct Record {
 // bin_start at bs_off of the plan's bin_start array (absolute record
 // indices).  One view (every l on the caller's n_mu x n_t) unless per-l
 // bins are asked for; then consecutive l with the same grid share a view.
-// The binning runs over chunks of at most kBinChunk records of one bin (a
+// The binning runs over chunks of at most bin_chunk_len records of one bin (a
 // bin's records cut in order), chunk_off .. chunk_off + n_chunks - 1 of the
 // plan's chunk arrays, and bin b's chunks are bin_chunk[bc_off + b] ..
 // bin_chunk[bc_off + b + 1] - 1.
@@ -185,7 +192,15 @@ struct View {
     int64_t n_bins = 0, out_off = 0, rec_off = 0, bs_off = 0;
     int64_t chunk_off = 0, n_chunks = 0, bc_off = 0;
 };
-constexpr int64_t kBinChunk = 2048;
+// Records of a binning chunk (one warp each): 2048 where a view has millions of
+// records, fewer where that would leave the SMs idle (4096 chunks are 27 warps
+// per SM), at least two per lane (the sum across the warp costs as much FP64
+// work as one record per lane).
+inline int64_t bin_chunk_len(int64_t nrec)
+{
+    const int64_t len = (nrec / 4096 + 31) / 32 * 32;
+    return len < 64 ? 64 : (len > 2048 ? 2048 : len);
+}
 
 struct Level {
     int lev = 0;               // index into Rings::grid
