@@ -529,8 +529,9 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
         else ok = produce<kProdFields>(pa);
         asm volatile("cp.async.wait_all;\n" ::: "memory");
     } else if (warp == 8) {
-        // MMA issue: high A x high B, low A x high B and high A x low B over
-        // the four k-steps of the stage.  The whole warp runs the loop (all
+        // MMA issue: low A x high B, high A x low B and high A x high B over
+        // the four k-steps of the stage: the small products first, so that the
+        // accumulator truncates at its full size only four times.  The whole warp runs the loop (all
         // lanes wait, one elected lane issues), so that its operands are
         // warp-uniform; a lane's wait that gives up stops the warp.
         {
@@ -556,11 +557,11 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
                 auto issue = [&](auto ksteps) {
                     constexpr int KS = decltype(ksteps)::value;
 #pragma unroll
-                    for (int j = 0; j < KS; ++j) mma_f16(d, a + 8 * j, dh + bo + j * kstep, ID, j > 0);
-#pragma unroll
-                    for (int j = 0; j < KS; ++j) mma_f16(d, a + 32 + 8 * j, dh + bo + j * kstep, ID | kNegA, 1);
+                    for (int j = 0; j < KS; ++j) mma_f16(d, a + 32 + 8 * j, dh + bo + j * kstep, ID | kNegA, j > 0);
 #pragma unroll
                     for (int j = 0; j < KS; ++j) mma_f16(d, a + 8 * j, dl + bo + j * kstep, ID | kNegB, 1);
+#pragma unroll
+                    for (int j = 0; j < KS; ++j) mma_f16(d, a + 8 * j, dh + bo + j * kstep, ID, 1);
                 };
                 if (st + 1 < nstage || ntail == kTX) issue(std::integral_constant<int, 4>{});
                 else issue(std::integral_constant<int, 2>{});
