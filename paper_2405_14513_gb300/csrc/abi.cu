@@ -38,6 +38,7 @@ int fail(int code, const std::string &msg)
 
 constexpr double kTwoPi = 6.283185307179586476925286766559;
 constexpr int64_t kXChunk = 16384;        // grid points of one Step-II unit
+constexpr size_t kStepShare = size_t(64) << 20;   // bytes of fields up to which Step-I grids share launches
 
 size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
 
@@ -51,6 +52,20 @@ int ilog2i(int v)
 }  // namespace
 
 namespace bisp {
+void make_twiddles(double2 *t)
+{
+    for (int F : {1, 3, 5, 7})
+        for (int s = 0, Ns = F; Ns <= 512; s += 3, Ns *= 8) {
+            double2 *o = t + Twiddles<double2>::offset(F) + Twiddles<double2>::stage(F, s);
+            for (int R : {8, 4, 2})
+                for (int r = 1; r < R; ++r)
+                    for (int k = 0; k < Ns; ++k) {
+                        const double a = -kTwoPi * double(r * k) / double(R * Ns);
+                        *o++ = make_double2(std::cos(a), std::sin(a));
+                    }
+        }
+}
+
 // Record a failure message for estimator_last_error() from another
 // translation unit of the library.
 int record_error(int code, const char *msg) { return fail(code, msg); }
@@ -83,22 +98,21 @@ struct bisp_plan {
     Twiddles<double2> tw_d{};
     GridArg grid_arg{};                  // reduction grid sides by level index
     RingArg ring_arg{};
-    std::vector<Job *> d_jobs;           // per level in use
-    std::vector<int64_t *> d_job_off;    // per level: output offsets of the jobs
+    std::vector<StepGrids> step1;        // the Step-I launches: one grid each, or several small ones (rt: first pass)
+    std::vector<StepGrids> step1_cols;   // the same grids (rt: columns of the second pass)
     // one field's workspace region (offsets within it); field f of a batch
     // uses bytes [f region_bytes, (f + 1) region_bytes) of the workspace
     // off_status: one int, set by a Step-II block of this field whose bounded
     // wait ran out; cleared at the start of every estimate
     // off_epi: the binning's partial sums per chunk
     // off_scale: the power-of-two factors of the stored fields (tensor-core plans)
-    size_t off_a = 0, off_b = 0, off_gt = 0, off_dstore = 0, off_part = 0, off_S = 0, off_status = 0, off_epi = 0,
+    size_t off_a = 0, off_b = 0, off_dstore = 0, off_part = 0, off_S = 0, off_status = 0, off_epi = 0,
            off_scale = 0, region_bytes = 0;
     int wait_spins = kDefaultWaitSpins;  // bound of the tensor-core Step II's abortable waits
     int device = -1;                     // the device the plan's tables live on
     int last_field = 0;                  // field of the last estimate that introspection reads
     // transform rows per block picked by the plan's autotuner (0 = default rule)
     int rt_z = 0, rt_xy = 0;
-    int rt_gather[kMaxLevels] = {}, rt_rows[kMaxLevels] = {};
     size_t resident = 0;
     // buffers of estimator_estimate_host
     void *own_ws = nullptr, *own_in = nullptr;
@@ -271,7 +285,7 @@ int compute_ntri(bisp_plan *p, cudaStream_t s)
                 need[lv * kMaxRings + a] = need[lv * kMaxRings + b] = need[lv * kMaxRings + c] = 1;
             }
     std::vector<int64_t> ioff(size_t(kMaxLevels) * kMaxRings, -1);
-    int64_t cur = 0, gtmax = 0;
+    int64_t cur = 0;
     std::vector<std::vector<Job>> jobs(kMaxLevels);
     for (int lv = 0; lv < R.ngrid; ++lv) {
         const int64_t M2 = int64_t(R.grid[lv]) * R.grid[lv];
@@ -281,7 +295,6 @@ int compute_ntri(bisp_plan *p, cudaStream_t s)
                 jobs[lv].push_back(Job{0, r, cur});
                 cur += M2;
             }
-        gtmax = std::max<int64_t>(gtmax, int64_t(jobs[lv].size()) * M2);
     }
 
     std::vector<void *> tmp;
@@ -293,13 +306,11 @@ int compute_ntri(bisp_plan *p, cudaStream_t s)
     };
     auto cleanup = [&]() { for (void *q : tmp) cudaFree(q); };
     double2 *I = (double2 *)talloc(size_t(cur) * sizeof(double2));
-    double2 *gt = (double2 *)talloc(size_t(gtmax) * sizeof(double2));
     int64_t *d_ioff = (int64_t *)talloc(ioff.size() * sizeof(int64_t));
     int32_t *d_tri = (int32_t *)talloc(tri.size() * sizeof(int32_t));
     double *d_raw = (double *)talloc(tri.size() / 4 * sizeof(double));
     Job *d_jobs = (Job *)talloc(size_t(nr) * sizeof(Job));
-    int64_t *d_joff = (int64_t *)talloc(size_t(nr) * sizeof(int64_t));
-    if (!I || !gt || !d_ioff || !d_tri || !d_raw || !d_jobs || !d_joff) {
+    if (!I || !d_ioff || !d_tri || !d_raw || !d_jobs) {
         cleanup();
         return fail(BISP_OUT_OF_MEMORY, "device memory for the triangle counts");
     }
@@ -308,15 +319,12 @@ int compute_ntri(bisp_plan *p, cudaStream_t s)
         CK(cudaMemcpyAsync(d_tri, tri.data(), tri.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
         for (int lv = 0; lv < R.ngrid; ++lv) {
             if (jobs[lv].empty()) continue;
-            const int M = R.grid[lv];
-            std::vector<int64_t> joff;
-            for (auto &j : jobs[lv]) joff.push_back(j.out_off);
             CK(cudaMemcpyAsync(d_jobs, jobs[lv].data(), jobs[lv].size() * sizeof(Job), cudaMemcpyHostToDevice, s));
-            CK(cudaMemcpyAsync(d_joff, joff.data(), joff.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-            CK(launch_ring_gather<double>(I, R.ng, p->ring_arg, d_jobs, int64_t(jobs[lv].size()), M, true, gt,
-                                          p->tw_d, Batch{}, s));
-            CK(launch_fft_cols<double>(gt, I, M, int64_t(jobs[lv].size()), d_joff, d_jobs, p->ring_arg, p->tw_d, Batch{},
-                                        s));
+            StepGrids gs;
+            gs.n = 1;
+            gs.g[0] = StepGrid{R.grid[lv], 0, d_jobs, int64_t(jobs[lv].size()), 0, 0, 0};
+            CK(launch_ring_gather<double>(I, R.ng, p->ring_arg, gs, true, I, p->tw_d, Batch{}, s));
+            CK(launch_fft_cols<double>(I, gs, p->ring_arg, p->tw_d, Batch{}, s));
             CK(cudaStreamSynchronize(s));   // the job tables are reused by the next grid
         }
         CK(launch_ntri(I, d_ioff, d_tri, int64_t(tri.size() / 4), p->grid_arg, d_raw, s));
@@ -392,7 +400,7 @@ int autotune_transforms(bisp_plan *p, cudaStream_t s)
         for (int n = 0; n <= Rg.nz; ++n)
             for (int r = 0; r < Rg.nr; ++r)
                 if (P.doff[(size_t(L.lev) * (Rg.nz + 1) + n) * kMaxRings + r] >= 0 && k++ % stride == 0)
-                    sample[l].push_back(Job{n, r, 0});
+                    sample[l].push_back(Job{n, r, int64_t(sample[l].size()) * L.M * L.M});
         jmax = std::max(jmax, int64_t(sample[l].size()) * L.M * L.M);
         nsamp += int64_t(sample[l].size());
     }
@@ -414,21 +422,16 @@ int autotune_transforms(bisp_plan *p, cudaStream_t s)
     C *planes = static_cast<C *>(talloc(bplanes));
     C *b0 = static_cast<C *>(talloc(bout));
     C *b1 = static_cast<C *>(talloc(brows));
-    // the sampled jobs and their output offsets (job j of a grid at j M^2)
-    int64_t *d_offs = static_cast<int64_t *>(talloc(sizeof(int64_t) * size_t(nsamp)));
+    // the sampled jobs (job j of a grid at j M^2 of the scratch)
     Job *d_samp = static_cast<Job *>(talloc(sizeof(Job) * size_t(nsamp)));
-    std::vector<int64_t> h_offs;
     std::vector<Job> h_samp;
     std::vector<int64_t> samp0;
     for (size_t l = 0; l < P.levels.size(); ++l) {
         samp0.push_back(int64_t(h_samp.size()));
-        for (size_t j = 0; j < sample[l].size(); ++j) {
-            h_offs.push_back(int64_t(j) * P.levels[l].M * P.levels[l].M);
-            h_samp.push_back(sample[l][j]);
-        }
+        h_samp.insert(h_samp.end(), sample[l].begin(), sample[l].end());
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (!zin || !planes || !b0 || !b1 || !d_offs || !d_samp || cudaEventCreate(&e0) != cudaSuccess ||
+    if (!zin || !planes || !b0 || !b1 || !d_samp || cudaEventCreate(&e0) != cudaSuccess ||
         cudaEventCreate(&e1) != cudaSuccess) {
         cudaGetLastError();
         cleanup();
@@ -439,14 +442,14 @@ int autotune_transforms(bisp_plan *p, cudaStream_t s)
     cudaMemsetAsync(planes, 0, bplanes, s);
     cudaMemsetAsync(b0, 0, bout, s);
     cudaMemsetAsync(b1, 0, brows, s);
-    cudaMemcpyAsync(d_offs, h_offs.data(), h_offs.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s);
     cudaMemcpyAsync(d_samp, h_samp.data(), h_samp.size() * sizeof(Job), cudaMemcpyHostToDevice, s);
     const size_t cand[] = {4096, 8192, 16384, 32768, 65536};
     // the fastest of the candidate rows per block for one launch
-    auto pick = [&](int M, int cap, auto &&launch) -> int {
+    auto pick = [&](int M, int cap, size_t most, auto &&launch) -> int {
         int best = 0, last = -1;
         float best_ms = 1e30f;
         for (size_t bytes : cand) {
+            if (bytes > most) continue;
             const int rt = std::min(int(fft_rows_per_block(M, sizeof(C), bytes)), cap);
             if (rt == last) continue;
             last = rt;
@@ -462,11 +465,12 @@ int autotune_transforms(bisp_plan *p, cudaStream_t s)
         return best;
     };
     // the fastest strip width (columns per block) of a grid's second pass
-    auto pick_w = [&](int M, auto &&launch) -> int {
+    auto pick_w = [&](int M, size_t most, auto &&launch) -> int {
         int best = 0;
         float best_ms = 1e30f;
         for (int w : {2, 4, 8, 16, 32}) {
             if (w > M || size_t(2) * w * fft_stride(M) * sizeof(C) > 227 * 1024) continue;
+            if (w > 4 && size_t(w) * M * sizeof(C) > most) continue;
             if (launch(w) != cudaSuccess) return -1;
             cudaEventRecord(e0, s);
             for (int r = 0; r < 3; ++r) launch(w);
@@ -480,27 +484,42 @@ int autotune_transforms(bisp_plan *p, cudaStream_t s)
     };
     const Batch one{};
     int st = BISP_OK;
-    p->rt_z = pick(ng, 256, [&](int rt) {
+    p->rt_z = pick(ng, 256, cand[4], [&](int rt) {
         return launch_fft_z_real<R>(zin, b0, ng, zrows, nz1, tw, one, s, rt);
     });
-    p->rt_xy = pick(ng, ng, [&](int rt) {
-        return launch_fft_rows_T<R>(b1, b0, ng, ng, npl, nullptr, R(1), false, tw, one, s, rt);
+    p->rt_xy = pick(ng, ng, cand[4], [&](int rt) {
+        return launch_fft_rows_T<R>(b1, b0, ng, ng, npl, R(1), false, tw, one, s, rt);
     });
     if (p->rt_z < 0 || p->rt_xy < 0) st = fail(BISP_CUDA_ERROR, "transform autotuner");
     for (size_t l = 0; l < P.levels.size() && !st; ++l) {
         const Level &L = P.levels[l];
         const int64_t nj = int64_t(sample[l].size());
-        const int64_t *d_off = d_offs + samp0[l];
         const Job *d_j = d_samp + samp0[l];
-        const int g = pick(L.M, L.M, [&](int rt) {
-            return launch_ring_gather<R>(planes, ng, p->ring_arg, d_j, nj, L.M, false, b0, tw, one, s, rt);
+        // a grid that shares its launches with others keeps to tiles that
+        // leave several blocks an SM
+        bool shared = false;
+        for (const StepGrids &gs : p->step1)
+            for (int i = 0; i < gs.n; ++i) shared |= gs.n > 1 && gs.g[i].M == L.M;
+        const size_t most = shared ? 16384 : 65536;
+        auto one_grid = [&](int rt) {
+            StepGrids gs;
+            gs.n = 1;
+            gs.g[0] = StepGrid{L.M, rt, d_j, nj, 0, 0, 0};
+            return gs;
+        };
+        const int g = pick(L.M, L.M, most, [&](int rt) {
+            return launch_ring_gather<R>(planes, ng, p->ring_arg, one_grid(rt), false, b0, tw, one, s);
         });
-        const int r = pick_w(L.M, [&](int w) {
-            return launch_fft_cols<R>(b0, b1, L.M, nj, d_off, d_j, p->ring_arg, tw, one, s, w);
+        const int r = pick_w(L.M, most, [&](int w) {
+            return launch_fft_cols<R>(b0, one_grid(w), p->ring_arg, tw, one, s);
         });
         if (g < 0 || r < 0) st = fail(BISP_CUDA_ERROR, "transform autotuner");
-        p->rt_gather[L.lev] = std::max(g, 0);
-        p->rt_rows[L.lev] = std::max(r, 0);
+        for (StepGrids &gs : p->step1)
+            for (int i = 0; i < gs.n; ++i)
+                if (gs.g[i].M == L.M) gs.g[i].rt = std::max(g, 0);
+        for (StepGrids &gs : p->step1_cols)
+            for (int i = 0; i < gs.n; ++i)
+                if (gs.g[i].M == L.M) gs.g[i].rt = std::max(r, 0);
     }
     cudaStreamSynchronize(s);
     cudaEventDestroy(e0);
@@ -538,39 +557,19 @@ int build_plan(bisp_plan *p, const bisp_desc *desc, cudaStream_t s)
     for (int r = 0; r < R.nr; ++r) p->ring_arg.maxc[r] = R.maxc[r];
 
     for (int l = 0; l < R.ngrid; ++l) p->grid_arg.M[l] = R.grid[l];
-    // twiddles in double: exp(-2 pi i k / (F x 2^lgF)), k < 7/8 of F x 2^lgF
-    // (radix-8 stages reach seven eighths of the circle), for the lengths
-    // F x 2^q <= N_g of the transforms, F = 1, 3, 5, 7
     {
-        const int ng = desc->n_g;
-        int lg2 = 0, lg3 = 0, lg5 = 0, lg7 = 0;
-        while ((2 << lg2) <= ng) ++lg2;
-        while (3 * (2 << lg3) <= ng) ++lg3;
-        while (5 * (2 << lg5) <= ng) ++lg5;
-        while (7 * (2 << lg7) <= ng) ++lg7;
-        if (lg3 < 1) lg3 = 1;
-        if (lg5 < 2) lg5 = 2;
-        if (lg7 < 2) lg7 = 2;
-        auto table = [&](int base, int count, float2 **df, double2 **dd) -> int {
-            std::vector<double2> twd(count);
-            std::vector<float2> twf(count);
-            for (int k = 0; k < count; ++k) {
-                const double a = -kTwoPi * double(k) / double(base);
-                twd[k] = make_double2(std::cos(a), std::sin(a));
-                twf[k] = make_float2(float(twd[k].x), float(twd[k].y));
-            }
-            int st = upload(p, dd, twd, s);
-            return st ? st : upload(p, df, twf, s);
-        };
-        float2 *f2 = nullptr, *f3 = nullptr, *f5 = nullptr, *f7 = nullptr;
-        double2 *d2 = nullptr, *d3 = nullptr, *d5 = nullptr, *d7 = nullptr;
-        int st = table(1 << lg2, (7 * (1 << lg2) + 7) / 8, &f2, &d2);
-        if (!st) st = table(3 << lg3, (7 * (3 << lg3) + 7) / 8, &f3, &d3);
-        if (!st) st = table(5 << lg5, (7 * (5 << lg5) + 7) / 8, &f5, &d5);
-        if (!st) st = table(7 << lg7, (7 * (7 << lg7) + 7) / 8, &f7, &d7);
+        std::vector<double2> twd(kTwiddles);
+        std::vector<float2> twf(kTwiddles);
+        make_twiddles(twd.data());
+        for (int k = 0; k < kTwiddles; ++k) twf[k] = make_float2(float(twd[k].x), float(twd[k].y));
+        double2 *dd = nullptr;
+        float2 *df = nullptr;
+        int st = upload(p, &dd, twd, s);
+        if (!st) st = upload(p, &df, twf, s);
         if (st) return st;
-        p->tw_f = Twiddles<float2>{f2, f3, lg2, lg3, f5, lg5, f7, lg7};
-        p->tw_d = Twiddles<double2>{d2, d3, lg2, lg3, d5, lg5, d7, lg7};
+        CK(cudaStreamSynchronize(s));              // the tables above are this block's
+        p->tw_d = Twiddles<double2>{dd};
+        p->tw_f = Twiddles<float2>{df};
     }
     // Y_lm normalisations
     {
@@ -656,32 +655,37 @@ int build_plan(bisp_plan *p, const bisp_desc *desc, cudaStream_t s)
         if (e != cudaSuccess) return fail(BISP_CUDA_ERROR, std::string("denominators: ") + cudaGetErrorString(e));
         std::vector<double>().swap(P.rec_ntri);
     }
-    // Step-I jobs per grid
+    // Step-I jobs per grid, and the launches: consecutive small grids share one
+    // while their fields together take at most kStepShare bytes; their kernels
+    // last a few us each, so a plan of small grids was bound by the launches
+    // (64^3, 11 grids: 22 launches, 151 us; in two, see DESIGN), while a large grid
+    // fills the GPU by itself and keeps the shared memory that suits it
+    size_t share = 0;
     for (const Level &L : P.levels) {
         std::vector<Job> jobs;
-        std::vector<int64_t> off;
         for (int n = 0; n <= R.nz; ++n)
             for (int r = 0; r < R.nr; ++r) {
                 int64_t o = P.doff[(size_t(L.lev) * (R.nz + 1) + n) * kMaxRings + r];
-                if (o >= 0) {
-                    jobs.push_back(Job{n, r, o});
-                    off.push_back(o);
-                }
+                if (o >= 0) jobs.push_back(Job{n, r, o});
             }
         Job *dj = nullptr;
-        int64_t *dof = nullptr;
         st = upload(p, &dj, jobs, s);
-        if (!st) st = upload(p, &dof, off, s);
         if (st) return st;
-        p->d_jobs.push_back(dj);
-        p->d_job_off.push_back(dof);
+        const size_t bytes = size_t(L.njobs) * L.M * L.M * p->celem;
+        share += bytes;
+        if (p->step1.empty() || share > kStepShare) {
+            p->step1.emplace_back();
+            share = bytes;
+        }
+        StepGrids &gs = p->step1.back();
+        gs.g[gs.n++] = StepGrid{L.M, 0, dj, L.njobs, 0, 0, 0};
     }
+    p->step1_cols = p->step1;
     // workspace layout
     const int64_t planes = int64_t(R.nz + 1) * desc->n_g * desc->n_g;
     size_t o = 0;
     p->off_a = o; o = align256(o + size_t(planes) * p->celem);
     p->off_b = o; o = align256(o + size_t(planes) * p->celem);
-    p->off_gt = o; o = align256(o + size_t(P.gt_elems) * p->celem);
     p->off_dstore = o; o = align256(o + size_t(P.dstore_elems) * p->celem);
     p->off_part = o; o = align256(o + size_t(P.n_partials) * sizeof(double));
     p->off_S = o; o = align256(o + size_t(P.n_combos) * sizeof(double));
@@ -714,7 +718,6 @@ int run_estimate(bisp_plan *p, const R *delta, int batch, unsigned char *ws, dou
     if constexpr (sizeof(R) == 8) tw = p->tw_d; else tw = p->tw_f;
     C *A_ = reinterpret_cast<C *>(ws + p->off_a);
     C *B_ = reinterpret_cast<C *>(ws + p->off_b);
-    C *gt = reinterpret_cast<C *>(ws + p->off_gt);
     C *dstore = reinterpret_cast<C *>(ws + p->off_dstore);
     double *part = reinterpret_cast<double *>(ws + p->off_part);
     double *Ssum = reinterpret_cast<double *>(ws + p->off_S);
@@ -735,11 +738,11 @@ int run_estimate(bisp_plan *p, const R *delta, int batch, unsigned char *ws, dou
     {   // forward transform: z (real, planes 0..N_g/3 kept) -> y -> x, scaled by V/N_g^3, Delta(0) = 0
         StageMark m(p, BISP_STAGE_FORWARD, 3, s);
         CK(launch_fft_z_real<R>(delta, A_, ng, ng2, Rg.nz + 1, tw, in_field, s, p->rt_z));
-        CK(launch_fft_rows_T<R>(A_, B_, ng, ng, Rg.nz + 1, nullptr, R(1), false, tw, region, s, p->rt_xy));
-        CK(launch_fft_rows_T<R>(B_, A_, ng, ng, Rg.nz + 1, nullptr, scale, true, tw, region, s, p->rt_xy));
+        CK(launch_fft_rows_T<R>(A_, B_, ng, ng, Rg.nz + 1, R(1), false, tw, region, s, p->rt_xy));
+        CK(launch_fft_rows_T<R>(B_, A_, ng, ng, Rg.nz + 1, scale, true, tw, region, s, p->rt_xy));
     }
     {   // Step I: D(r, n) on each reduction grid (Eq. iFT)
-        StageMark m(p, BISP_STAGE_STEP1, int(2 * P.levels.size()) + (P.tensor ? 1 : 0), s);
+        StageMark m(p, BISP_STAGE_STEP1, int(2 * p->step1.size()) + (P.tensor ? 1 : 0), s);
         const float *fac = nullptr;
         if constexpr (sizeof(R) == 4)
             if (P.tensor) {
@@ -747,13 +750,9 @@ int run_estimate(bisp_plan *p, const R *delta, int batch, unsigned char *ws, dou
                 CK(launch_ring_scale(A_, ng, Rg.nz + 1, p->ring_arg, scale, region, s));
                 fac = scale;
             }
-        for (size_t l = 0; l < P.levels.size(); ++l) {
-            const Level &L = P.levels[l];
-            const int M = L.M;
-            CK(launch_ring_gather<R>(A_, ng, p->ring_arg, p->d_jobs[l], L.njobs, M, false, gt, tw, region, s,
-                                     p->rt_gather[L.lev], fac));
-            CK(launch_fft_cols<R>(gt, dstore, M, L.njobs, p->d_job_off[l], p->d_jobs[l], p->ring_arg, tw, region, s,
-                                  p->rt_rows[L.lev]));
+        for (size_t l = 0; l < p->step1.size(); ++l) {
+            CK(launch_ring_gather<R>(A_, ng, p->ring_arg, p->step1[l], false, dstore, tw, region, s, fac));
+            CK(launch_fft_cols<R>(dstore, p->step1_cols[l], p->ring_arg, tw, region, s));
         }
     }
     {   // Step II: triple sums (Eq. fftbs), all units or one share of them

@@ -4,9 +4,10 @@
 //   k_fft_z_real    forward transform along the line of sight (real rows),
 //                   keeping planes 0..N_g/3, written plane-major
 //   k_fft_rows_T    batched row transforms written transposed (the y and x
-//                   passes of the forward transform; second pass of Step I)
+//                   passes of the forward transform)
 //   k_ring_gather   Step I first pass: ring mask (and fold onto the M x M
 //                   reduction grid) fused into the load, transform along u_y
+//   k_fft_cols      Step I second pass: transform along u_x, in place
 //   k_ring_scale    power-of-two factors of the D fields (tensor-core Step II)
 //   k_step2         Step II: partial triple sums sum_x D1 D2 D3 (Eq. fftbs)
 //   k_reduce        partial sums -> S per combination, grid normalisation
@@ -16,8 +17,7 @@
 //
 // All transforms use exp(-i k.x), the sign of Eq. iFT.  Transform lengths
 // are 2^q, 3 x 2^q, 5 x 2^q or 7 x 2^q (N_g and the reduction grids of the
-// plan); the twiddle tables, computed on the host in double, are
-// twF[k] = exp(-2 pi i k / (F x 2^lgF)), F = 1 (tw2), 3, 5, 7.
+// plan); the twiddle tables (Twiddles) are computed on the host in double.
 #include "kernels.cuh"
 
 #include <algorithm>
@@ -82,238 +82,218 @@ struct DivIter {
 // fft_stride(M) elements (kernels.cuh).
 __device__ __forceinline__ int spos(int i) { return i + (i >> 3); }
 
-// Stockham transform of nrows rows of length M = F x 2^q (F = 1, 3, 5 or 7)
-// held in shared memory (row stride P), X_k = sum_j x_j exp(-2 pi i jk / M):
-// one radix-F stage first when F > 1, then radix-8 stages and, for what is
-// left of the power of two, one radix-4 or radix-2 stage.  Every thread of
-// the block takes part; the caller synchronises before the call.  The result
-// is in the returned buffer (a or b).  Every index split below is a shift, or
-// a shift and a division by the constant F.
-template <typename C, int F>
-__device__ C *fft_smem_f(C *a, C *b, int M, int P, int nrows, const Twiddles<C> &tw)
+// DFT of R values in registers, X_m = sum_r v_r exp(-2 pi i r m / R), in place.
+template <int R, typename C> __device__ __forceinline__ void dft(C (&v)[R])
 {
-    using Rr = decltype(a[0].x);
-    const int p = __ffs(M) - 1;                 // M = F 2^p
-    auto divF = [](int x) { return F == 1 ? x : int(unsigned(x) / unsigned(F)); };
-    int Ns = 1;
-    if (F == 3) {
-        const int third = M / 3;
-        const int total = nrows * third;
+    using Rr = decltype(v[0].x);
+    if constexpr (R == 2) {
+        const C t = csub(v[0], v[1]);
+        v[0] = cadd(v[0], v[1]);
+        v[1] = t;
+    } else if constexpr (R == 3) {
         const Rr h = Rr(0.86602540378443864676);   // sqrt(3)/2
-        for (int t = threadIdx.x; t < total; t += blockDim.x) {
-            const int row = t >> p, j = t & (third - 1);
-            const C v0 = a[row * P + spos(j)], v1 = a[row * P + spos(j + third)], v2 = a[row * P + spos(j + 2 * third)];
-            const Rr sx = v1.x + v2.x, sy = v1.y + v2.y, dx = v1.x - v2.x, dy = v1.y - v2.y;
-            const Rr mx = v0.x - Rr(0.5) * sx, my = v0.y - Rr(0.5) * sy;
-            C y0, y1, y2;
-            y0.x = v0.x + sx; y0.y = v0.y + sy;
-            y1.x = mx + h * dy; y1.y = my - h * dx;
-            y2.x = mx - h * dy; y2.y = my + h * dx;
-            b[row * P + spos(3 * j)] = y0;
-            b[row * P + spos(3 * j + 1)] = y1;
-            b[row * P + spos(3 * j + 2)] = y2;
-        }
-        __syncthreads();
-        C *t2 = a;
-        a = b;
-        b = t2;
-        Ns = 3;
-    } else if (F == 5) {
-        // 5-point DFT of v_k = x[j + k M/5], w = exp(-2 pi i/5):
+        const Rr sx = v[1].x + v[2].x, sy = v[1].y + v[2].y, dx = v[1].x - v[2].x, dy = v[1].y - v[2].y;
+        const Rr mx = v[0].x - Rr(0.5) * sx, my = v[0].y - Rr(0.5) * sy;
+        v[0].x += sx; v[0].y += sy;
+        v[1].x = mx + h * dy; v[1].y = my - h * dx;
+        v[2].x = mx - h * dy; v[2].y = my + h * dx;
+    } else if constexpr (R == 4) {
+        const C s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]), s13 = cadd(v[1], v[3]), d13 = csub(v[1], v[3]);
+        v[0] = cadd(s02, s13);
+        v[2] = csub(s02, s13);
+        v[1] = d02;                                // d02 -/+ i d13
+        v[1].x += d13.y; v[1].y -= d13.x;
+        v[3] = d02;
+        v[3].x -= d13.y; v[3].y += d13.x;
+    } else if constexpr (R == 5) {
+        // w = exp(-2 pi i/5):
         //   y_0 = v0 + s1 + s2,  s1 = v1 + v4,  s2 = v2 + v3,  d1 = v1 - v4,  d2 = v2 - v3,
         //   y_1, y_4 = v0 + c1 s1 + c2 s2 -/+ i (n1 d1 + n2 d2),
         //   y_2, y_3 = v0 + c2 s1 + c1 s2 -/+ i (n2 d1 - n1 d2),
         // c_m = cos(2 pi m/5), n_m = sin(2 pi m/5)
-        const int fifth = M / 5;
-        const int total = nrows * fifth;
         const Rr c1 = Rr(0.30901699437494742410), c2 = Rr(-0.80901699437494742410);
         const Rr n1 = Rr(0.95105651629515357212), n2 = Rr(0.58778525229247312917);
-        for (int t = threadIdx.x; t < total; t += blockDim.x) {
-            const int row = t >> p, j = t & (fifth - 1);
-            const C *src = a + row * P;
-            const C v0 = src[spos(j)], v1 = src[spos(j + fifth)], v2 = src[spos(j + 2 * fifth)], v3 = src[spos(j + 3 * fifth)],
-                    v4 = src[spos(j + 4 * fifth)];
-            const C s1 = cadd(v1, v4), s2 = cadd(v2, v3), d1 = csub(v1, v4), d2 = csub(v2, v3);
-            C a1, a2, b1, b2;
-            a1.x = v0.x + c1 * s1.x + c2 * s2.x; a1.y = v0.y + c1 * s1.y + c2 * s2.y;
-            a2.x = v0.x + c2 * s1.x + c1 * s2.x; a2.y = v0.y + c2 * s1.y + c1 * s2.y;
-            b1.x = n1 * d1.x + n2 * d2.x; b1.y = n1 * d1.y + n2 * d2.y;
-            b2.x = n2 * d1.x - n1 * d2.x; b2.y = n2 * d1.y - n1 * d2.y;
-            // -i b = (b.y, -b.x)
-            C *dst = b + row * P;
-            C y;
-            y.x = v0.x + s1.x + s2.x; y.y = v0.y + s1.y + s2.y; dst[spos(5 * j)] = y;
-            y.x = a1.x + b1.y; y.y = a1.y - b1.x; dst[spos(5 * j + 1)] = y;
-            y.x = a2.x + b2.y; y.y = a2.y - b2.x; dst[spos(5 * j + 2)] = y;
-            y.x = a2.x - b2.y; y.y = a2.y + b2.x; dst[spos(5 * j + 3)] = y;
-            y.x = a1.x - b1.y; y.y = a1.y + b1.x; dst[spos(5 * j + 4)] = y;
-        }
-        __syncthreads();
-        C *t2 = a;
-        a = b;
-        b = t2;
-        Ns = 5;
-    } else if (F == 7) {
-        // 7-point DFT of v_k = x[j + k M/7], by the same pairing:
-        //   s_k = v_k + v_{7-k},  d_k = v_k - v_{7-k}  (k = 1, 2, 3),
+        const C s1 = cadd(v[1], v[4]), s2 = cadd(v[2], v[3]), d1 = csub(v[1], v[4]), d2 = csub(v[2], v[3]);
+        C a1, a2, b1, b2;
+        a1.x = v[0].x + c1 * s1.x + c2 * s2.x; a1.y = v[0].y + c1 * s1.y + c2 * s2.y;
+        a2.x = v[0].x + c2 * s1.x + c1 * s2.x; a2.y = v[0].y + c2 * s1.y + c1 * s2.y;
+        b1.x = n1 * d1.x + n2 * d2.x; b1.y = n1 * d1.y + n2 * d2.y;
+        b2.x = n2 * d1.x - n1 * d2.x; b2.y = n2 * d1.y - n1 * d2.y;
+        // -i b = (b.y, -b.x)
+        v[0].x = v[0].x + s1.x + s2.x; v[0].y = v[0].y + s1.y + s2.y;
+        v[1].x = a1.x + b1.y; v[1].y = a1.y - b1.x;
+        v[2].x = a2.x + b2.y; v[2].y = a2.y - b2.x;
+        v[3].x = a2.x - b2.y; v[3].y = a2.y + b2.x;
+        v[4].x = a1.x - b1.y; v[4].y = a1.y + b1.x;
+    } else if constexpr (R == 7) {
+        // by the same pairing: s_k = v_k + v_{7-k},  d_k = v_k - v_{7-k}  (k = 1, 2, 3),
         //   y_m, y_{7-m} = v0 + sum_k cos(2 pi mk/7) s_k -/+ i sum_k sin(2 pi mk/7) d_k  (m = 1, 2, 3)
-        const int sev = M / 7;
-        const int total = nrows * sev;
         const Rr c1 = Rr(0.62348980185873353053), c2 = Rr(-0.22252093395631440429), c3 = Rr(-0.90096886790241912624);
         const Rr n1 = Rr(0.78183148246802980871), n2 = Rr(0.97492791218182360702), n3 = Rr(0.43388373911755812048);
-        for (int t = threadIdx.x; t < total; t += blockDim.x) {
-            const int row = t >> p, j = t & (sev - 1);
-            const C *src = a + row * P;
-            C v[7];
+        const C s1 = cadd(v[1], v[6]), s2 = cadd(v[2], v[5]), s3 = cadd(v[3], v[4]);
+        const C d1 = csub(v[1], v[6]), d2 = csub(v[2], v[5]), d3 = csub(v[3], v[4]);
+        C am[3], bm[3];
+        am[0].x = v[0].x + c1 * s1.x + c2 * s2.x + c3 * s3.x; am[0].y = v[0].y + c1 * s1.y + c2 * s2.y + c3 * s3.y;
+        am[1].x = v[0].x + c2 * s1.x + c3 * s2.x + c1 * s3.x; am[1].y = v[0].y + c2 * s1.y + c3 * s2.y + c1 * s3.y;
+        am[2].x = v[0].x + c3 * s1.x + c1 * s2.x + c2 * s3.x; am[2].y = v[0].y + c3 * s1.y + c1 * s2.y + c2 * s3.y;
+        bm[0].x = n1 * d1.x + n2 * d2.x + n3 * d3.x; bm[0].y = n1 * d1.y + n2 * d2.y + n3 * d3.y;
+        bm[1].x = n2 * d1.x - n3 * d2.x - n1 * d3.x; bm[1].y = n2 * d1.y - n3 * d2.y - n1 * d3.y;
+        bm[2].x = n3 * d1.x - n1 * d2.x + n2 * d3.x; bm[2].y = n3 * d1.y - n1 * d2.y + n2 * d3.y;
+        v[0].x = v[0].x + s1.x + s2.x + s3.x; v[0].y = v[0].y + s1.y + s2.y + s3.y;
 #pragma unroll
-            for (int k = 0; k < 7; ++k) v[k] = src[spos(j + k * sev)];
-            const C s1 = cadd(v[1], v[6]), s2 = cadd(v[2], v[5]), s3 = cadd(v[3], v[4]);
-            const C d1 = csub(v[1], v[6]), d2 = csub(v[2], v[5]), d3 = csub(v[3], v[4]);
-            C am[3], bm[3];
-            am[0].x = v[0].x + c1 * s1.x + c2 * s2.x + c3 * s3.x; am[0].y = v[0].y + c1 * s1.y + c2 * s2.y + c3 * s3.y;
-            am[1].x = v[0].x + c2 * s1.x + c3 * s2.x + c1 * s3.x; am[1].y = v[0].y + c2 * s1.y + c3 * s2.y + c1 * s3.y;
-            am[2].x = v[0].x + c3 * s1.x + c1 * s2.x + c2 * s3.x; am[2].y = v[0].y + c3 * s1.y + c1 * s2.y + c2 * s3.y;
-            bm[0].x = n1 * d1.x + n2 * d2.x + n3 * d3.x; bm[0].y = n1 * d1.y + n2 * d2.y + n3 * d3.y;
-            bm[1].x = n2 * d1.x - n3 * d2.x - n1 * d3.x; bm[1].y = n2 * d1.y - n3 * d2.y - n1 * d3.y;
-            bm[2].x = n3 * d1.x - n1 * d2.x + n2 * d3.x; bm[2].y = n3 * d1.y - n1 * d2.y + n2 * d3.y;
-            C *dst = b + row * P;
-            C y;
-            y.x = v[0].x + s1.x + s2.x + s3.x; y.y = v[0].y + s1.y + s2.y + s3.y; dst[spos(7 * j)] = y;
-#pragma unroll
-            for (int m = 0; m < 3; ++m) {
-                // -i b = (b.y, -b.x)
-                y.x = am[m].x + bm[m].y; y.y = am[m].y - bm[m].x; dst[spos(7 * j + m + 1)] = y;
-                y.x = am[m].x - bm[m].y; y.y = am[m].y + bm[m].x; dst[spos(7 * j + 6 - m)] = y;
-            }
+        for (int m = 0; m < 3; ++m) {
+            // -i b = (b.y, -b.x)
+            v[m + 1].x = am[m].x + bm[m].y; v[m + 1].y = am[m].y - bm[m].x;
+            v[6 - m].x = am[m].x - bm[m].y; v[6 - m].y = am[m].y + bm[m].x;
         }
-        __syncthreads();
-        C *t2 = a;
-        a = b;
-        b = t2;
-        Ns = 7;
-    }
-    const C *wt = F == 7 ? tw.tw7 : (F == 5 ? tw.tw5 : (F == 3 ? tw.tw3 : tw.tw2));
-    const int lg = F == 7 ? tw.lg7 : (F == 5 ? tw.lg5 : (F == 3 ? tw.lg3 : tw.lg2));
-    int s = 0;                                  // Ns = F 2^s
-    while (Ns < M) {
-        if (M / Ns >= 8) {
-            // radix 8: v_r = x[j + r M/8] w^(rk), w = exp(-2 pi i / (8 Ns)),
-            // out[q 8 Ns + k + m Ns] = sum_r v_r exp(-2 pi i rm / 8), as a
-            // radix-2 step (pairs r, r + 4; the odd half turned by
-            // exp(-2 pi i r / 8)) followed by two 4-point transforms
-            const int eighth = M / 8;
-            const int total = nrows * eighth;
-            const int sh = lg - s - 3;
-            const Rr r2 = Rr(0.70710678118654752440);   // 1/sqrt(2)
-            for (int t = threadIdx.x; t < total; t += blockDim.x) {
-                const int row = divF(t >> (p - 3));
-                const int j = t - row * eighth;
-                const int q = divF(j >> s);
-                const int k = j - q * Ns;
-                const C *src = a + row * P;
-                C v[8];
-                v[0] = src[spos(j)];
+    } else {
+        static_assert(R == 8, "radix");
+        // a radix-2 step (pairs r, r + 4; the odd half turned by
+        // exp(-2 pi i r / 8)) followed by two 4-point transforms
+        const Rr r2 = Rr(0.70710678118654752440);  // 1/sqrt(2)
+        C e[4], o[4];
 #pragma unroll
-                for (int r = 1; r < 8; ++r) v[r] = cmul(src[spos(j + r * eighth)], __ldg(&wt[(r * k) << sh]));
-                C e[4], o[4];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    e[r] = cadd(v[r], v[r + 4]);
-                    o[r] = csub(v[r], v[r + 4]);
-                }
-                // o_1 exp(-i pi/4), o_2 (-i), o_3 exp(-3 i pi/4)
-                {
-                    const C t1 = o[1], t3 = o[3];
-                    o[1].x = (t1.x + t1.y) * r2; o[1].y = (t1.y - t1.x) * r2;
-                    const Rr x2 = o[2].x;
-                    o[2].x = o[2].y; o[2].y = -x2;
-                    o[3].x = (t3.y - t3.x) * r2; o[3].y = -(t3.x + t3.y) * r2;
-                }
-                C *dst = b + row * P;
-                const int d0 = q * 8 * Ns + k;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const C *x = h ? o : e;
-                    const C s02 = cadd(x[0], x[2]), d02 = csub(x[0], x[2]), s13 = cadd(x[1], x[3]),
-                            d13 = csub(x[1], x[3]);
-                    C m1 = d02, m3 = d02;                 // d02 -/+ i d13
-                    m1.x += d13.y; m1.y -= d13.x;
-                    m3.x -= d13.y; m3.y += d13.x;
-                    dst[spos(d0 + (0 + h) * Ns)] = cadd(s02, s13);
-                    dst[spos(d0 + (2 + h) * Ns)] = m1;
-                    dst[spos(d0 + (4 + h) * Ns)] = csub(s02, s13);
-                    dst[spos(d0 + (6 + h) * Ns)] = m3;
-                }
-            }
-            Ns *= 8;
-            s += 3;
-        } else if (M / Ns >= 4) {
-            // radix 4: v_r = x[j + r M/4] w^(rk), w = exp(-2 pi i / (4 Ns)),
-            // out[q 4 Ns + k + m Ns] = sum_r v_r (-i)^(rm)
-            const int quarter = M / 4;
-            const int total = nrows * quarter;
-            const int sh = lg - s - 2;
-            for (int t = threadIdx.x; t < total; t += blockDim.x) {
-                const int row = divF(t >> (p - 2));
-                const int j = t - row * quarter;
-                const int q = divF(j >> s);
-                const int k = j - q * Ns;
-                const C *src = a + row * P;
-                const C v0 = src[spos(j)];
-                const C v1 = cmul(src[spos(j + quarter)], __ldg(&wt[k << sh]));
-                const C v2 = cmul(src[spos(j + 2 * quarter)], __ldg(&wt[(2 * k) << sh]));
-                const C v3 = cmul(src[spos(j + 3 * quarter)], __ldg(&wt[(3 * k) << sh]));
-                const C s02 = cadd(v0, v2), d02 = csub(v0, v2), s13 = cadd(v1, v3), d13 = csub(v1, v3);
-                C *dst = b + row * P;
-                const int d0 = q * 4 * Ns + k;
-                dst[spos(d0)] = cadd(s02, s13);
-                dst[spos(d0 + 2 * Ns)] = csub(s02, s13);
-                // -i d13 = (d13.y, -d13.x)
-                C m1 = d02, m3 = d02;
-                m1.x += d13.y; m1.y -= d13.x;
-                m3.x -= d13.y; m3.y += d13.x;
-                dst[spos(d0 + Ns)] = m1;
-                dst[spos(d0 + 3 * Ns)] = m3;
-            }
-            Ns *= 4;
-            s += 2;
-        } else {
-            const int half = M / 2;
-            const int total = nrows * half;
-            const int sh = lg - s - 1;
-            for (int t = threadIdx.x; t < total; t += blockDim.x) {
-                const int row = divF(t >> (p - 1));
-                const int j = t - row * half;
-                const int q = divF(j >> s);
-                const int k = j - q * Ns;
-                C v0 = a[row * P + spos(j)];
-                C v1 = cmul(a[row * P + spos(j + half)], __ldg(&wt[k << sh]));
-                const int idx = q * 2 * Ns + k;
-                b[row * P + spos(idx)] = cadd(v0, v1);
-                b[row * P + spos(idx + Ns)] = csub(v0, v1);
-            }
-            Ns *= 2;
-            s += 1;
+        for (int r = 0; r < 4; ++r) {
+            e[r] = cadd(v[r], v[r + 4]);
+            o[r] = csub(v[r], v[r + 4]);
         }
-        __syncthreads();
-        C *t2 = a;
-        a = b;
-        b = t2;
+        // o_1 exp(-i pi/4), o_2 (-i), o_3 exp(-3 i pi/4)
+        const C t1 = o[1], t3 = o[3];
+        o[1].x = (t1.x + t1.y) * r2; o[1].y = (t1.y - t1.x) * r2;
+        const Rr x2 = o[2].x;
+        o[2].x = o[2].y; o[2].y = -x2;
+        o[3].x = (t3.y - t3.x) * r2; o[3].y = -(t3.x + t3.y) * r2;
+        dft<4>(e);
+        dft<4>(o);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            v[2 * m] = e[m];
+            v[2 * m + 1] = o[m];
+        }
     }
-    return a;
 }
 
-// Transform of rows of length M = 2^q, 3 x 2^q, 5 x 2^q or 7 x 2^q
-// (block-uniform dispatch)
-template <typename C>
-__device__ __forceinline__ C *fft_smem(C *a, C *b, int M, int P, int nrows, const Twiddles<C> &tw)
+// Rows of a transform block: nr rows of length M = F x 2^p, on the threads
+// either along the row (consecutive threads take consecutive elements) or, ACROSS,
+// across 2^lgw >= nr rows (consecutive threads take the same element of
+// consecutive rows).
+struct FftRows {
+    int M, p, nr, lgw;
+};
+
+// One Stockham stage of radix R on every row: out[q R Ns + k + m Ns] =
+// sum_r w^(rk) x[j + r M/R] exp(-2 pi i rm / R) with j = q Ns + k and
+// w = exp(-2 pi i / (R Ns)) (tw: its table [r - 1][k], null in a first
+// stage); get(row, i) and put(row, i, value) read and write an element.  Every
+// index split is a shift, or a shift and a division by the constant F.
+template <typename C, int F, bool ACROSS, int R, typename G, typename S>
+__device__ __forceinline__ void fft_stage(const FftRows &fr, int Ns, int s, const C *__restrict__ tw, G get, S put)
 {
-    const int odd = M >> (__ffs(M) - 1);
-    if (odd == 7) return fft_smem_f<C, 7>(a, b, M, P, nrows, tw);
-    if (odd == 5) return fft_smem_f<C, 5>(a, b, M, P, nrows, tw);
-    if (odd == 3) return fft_smem_f<C, 3>(a, b, M, P, nrows, tw);
-    return fft_smem_f<C, 1>(a, b, M, P, nrows, tw);
+    constexpr int LR = R == 8 ? 3 : (R == 4 ? 2 : (R == 2 ? 1 : 0));
+    auto divF = [](int x) { return F == 1 ? x : int(unsigned(x) / unsigned(F)); };
+    const int nb = R == F ? 1 << fr.p : F << (fr.p - LR);     // butterflies per row
+    const int total = ACROSS ? nb << fr.lgw : nb * fr.nr;
+    for (int t = threadIdx.x; t < total; t += blockDim.x) {
+        int row, j;
+        if (ACROSS) {
+            row = t & ((1 << fr.lgw) - 1);
+            j = t >> fr.lgw;
+            if (row >= fr.nr) continue;
+        } else {
+            row = R == F ? t >> fr.p : divF(t >> (fr.p - LR));
+            j = t - row * nb;
+        }
+        int q = j, k = 0;
+        if (Ns > 1) {
+            q = divF(j >> s);
+            k = j - q * Ns;
+        }
+        C v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = get(row, j + r * nb);
+        if (tw) {
+#pragma unroll
+            for (int r = 1; r < R; ++r) v[r] = cmul(v[r], __ldg(tw + (r - 1) * Ns + k));
+        }
+        dft<R>(v);
+        const int d0 = q * R * Ns + k;
+#pragma unroll
+        for (int m = 0; m < R; ++m) put(row, d0 + m * Ns, v[m]);
+    }
 }
+
+// Stockham transform X_k = sum_j x_j exp(-2 pi i jk / M) of the block's rows:
+// one radix-F stage first when F > 1, then radix-8 stages and, for what is
+// left of the power of two, one radix-4 or radix-2 stage.  The first stage
+// takes its elements from `load` and the last hands them to `store` (SMEM:
+// leaves them in the returned buffer instead, block synchronised), so that
+// between global memory and the registers a transform of up to 512 points
+// crosses shared memory twice, not four times.  a, b: buffers of nr rows of
+// stride P.  Every thread of the block takes part.
+template <typename C, int F, bool ACROSS, bool SMEM, typename G, typename S>
+__device__ __forceinline__ C *fft_block(const FftRows &fr, int P, C *a, C *b, const C *__restrict__ tw, G load, S store)
+{
+    auto from = [&](C *x) { return [x, P](int row, int i) { return x[row * P + spos(i)]; }; };
+    auto into = [&](C *x) { return [x, P](int row, int i, const C &v) { x[row * P + spos(i)] = v; }; };
+    constexpr int R1 = F > 1 ? F : 8;
+    int Ns = R1, s = F > 1 ? 0 : 3;                 // Ns = F 2^s
+    if (F == 1 && fr.M == 8) {
+        if constexpr (SMEM) {
+            fft_stage<C, F, ACROSS, R1>(fr, 1, 0, nullptr, load, into(a));
+            __syncthreads();
+        } else {
+            fft_stage<C, F, ACROSS, R1>(fr, 1, 0, nullptr, load, store);
+        }
+        return a;
+    }
+    fft_stage<C, F, ACROSS, R1>(fr, 1, 0, nullptr, load, into(a));
+    __syncthreads();
+    const C *w = tw + Twiddles<C>::offset(F);
+    for (;; s += 3) {
+        const int lg = fr.p - s;                    // what is left: 2^lg
+        const C *w8 = w + Twiddles<C>::stage(F, s);
+        if (lg > 3) {
+            fft_stage<C, F, ACROSS, 8>(fr, Ns, s, w8, from(a), into(b));
+            __syncthreads();
+            C *t = a;
+            a = b;
+            b = t;
+            Ns *= 8;
+            continue;
+        }
+        if constexpr (SMEM) {
+            if (lg == 3) fft_stage<C, F, ACROSS, 8>(fr, Ns, s, w8, from(a), into(b));
+            else if (lg == 2) fft_stage<C, F, ACROSS, 4>(fr, Ns, s, w8 + 7 * Ns, from(a), into(b));
+            else fft_stage<C, F, ACROSS, 2>(fr, Ns, s, w8 + 10 * Ns, from(a), into(b));
+            __syncthreads();
+        } else {
+            if (lg == 3) fft_stage<C, F, ACROSS, 8>(fr, Ns, s, w8, from(a), store);
+            else if (lg == 2) fft_stage<C, F, ACROSS, 4>(fr, Ns, s, w8 + 7 * Ns, from(a), store);
+            else fft_stage<C, F, ACROSS, 2>(fr, Ns, s, w8 + 10 * Ns, from(a), store);
+        }
+        return b;
+    }
+}
+
+// fft_block of rows of length M = 2^q, 3 x 2^q, 5 x 2^q or 7 x 2^q
+// (block-uniform dispatch); ODD = false: of 2^q or 3 x 2^q, the lengths of N_g
+template <typename C, bool ACROSS, bool SMEM, bool ODD, typename G, typename S>
+__device__ __forceinline__ C *fft_any(int M, int nr, int lgw, int P, C *a, C *b, const C *__restrict__ tw, G load, S store)
+{
+    const FftRows fr{M, __ffs(M) - 1, nr, lgw};
+    const int odd = M >> fr.p;
+    if constexpr (ODD) {
+        if (odd == 7) return fft_block<C, 7, ACROSS, SMEM>(fr, P, a, b, tw, load, store);
+        if (odd == 5) return fft_block<C, 5, ACROSS, SMEM>(fr, P, a, b, tw, load, store);
+    }
+    if (odd == 3) return fft_block<C, 3, ACROSS, SMEM>(fr, P, a, b, tw, load, store);
+    return fft_block<C, 1, ACROSS, SMEM>(fr, P, a, b, tw, load, store);
+}
+
+// no store: the transform's result stays in shared memory
+struct NoStore {
+    template <typename C> __device__ void operator()(int, int, const C &) const {}
+};
 
 // ---------------------------------------------------------------------------
 template <typename R>
@@ -330,13 +310,9 @@ k_fft_z_real(const R *__restrict__ in, typename Cx<R>::T *__restrict__ out, int 
     C *b = a + rt * P;
     const int64_t row0 = int64_t(blockIdx.x) * rt;
     const int nrow = int(min(int64_t(rt), rows - row0));
-    DivIter ld(threadIdx.x, blockDim.x, M);
-    for (int t = threadIdx.x; t < nrow * M; t += blockDim.x, ld.next()) {
-        const int r = ld.q, j = ld.r;
-        a[r * P + spos(j)] = cmk<C>(double(in[(row0 + r) * M + j]), 0.0);
-    }
-    __syncthreads();
-    const C *res = fft_smem(a, b, M, P, nrow, tw);
+    const R *src = in + row0 * M;
+    const C *res = fft_any<C, false, true, false>(
+        M, nrow, 0, P, a, b, tw.t, [&](int r, int i) { return cmk<C>(double(src[r * M + i]), 0.0); }, NoStore{});
     DivIter st(threadIdx.x, blockDim.x, nrow);
     for (int t = threadIdx.x; t < nkeep * nrow; t += blockDim.x, st.next()) {
         const int k = st.q, r = st.r;
@@ -347,8 +323,7 @@ k_fft_z_real(const R *__restrict__ in, typename Cx<R>::T *__restrict__ out, int 
 template <typename R>
 __global__ void __launch_bounds__(256)
 k_fft_rows_T(const typename Cx<R>::T *__restrict__ in, typename Cx<R>::T *__restrict__ out, int M,
-             int nrow, int ntile, const int64_t *__restrict__ out_off, R scale, int zero_dc, int rt,
-             Twiddles<typename Cx<R>::T> tw, int64_t fs)
+             int nrow, int ntile, R scale, int zero_dc, int rt, Twiddles<typename Cx<R>::T> tw, int64_t fs)
 {
     using C = typename Cx<R>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -361,15 +336,10 @@ k_fft_rows_T(const typename Cx<R>::T *__restrict__ in, typename Cx<R>::T *__rest
     const int tile = int(blockIdx.x - bt * ntile);
     const int row0 = tile * rt;
     const int nr = min(rt, nrow - row0);
-    const C *src = in + bt * int64_t(M) * nrow;
-    DivIter ld(threadIdx.x, blockDim.x, M);
-    for (int t = threadIdx.x; t < nr * M; t += blockDim.x, ld.next()) {
-        const int r = ld.q, j = ld.r;
-        a[r * P + spos(j)] = src[int64_t(row0 + r) * M + j];
-    }
-    __syncthreads();
-    const C *res = fft_smem(a, b, M, P, nr, tw);
-    C *dst = out + (out_off ? out_off[bt] : bt * int64_t(M) * nrow);
+    const C *src = in + bt * int64_t(M) * nrow + int64_t(row0) * M;
+    const C *res = fft_any<C, false, true, false>(M, nr, 0, P, a, b, tw.t, [&](int r, int i) { return src[r * M + i]; },
+                                                  NoStore{});
+    C *dst = out + bt * int64_t(M) * nrow;
     DivIter st(threadIdx.x, blockDim.x, nr);
     for (int t = threadIdx.x; t < M * nr; t += blockDim.x, st.next()) {
         const int k = st.q, r = st.r;
@@ -378,72 +348,6 @@ k_fft_rows_T(const typename Cx<R>::T *__restrict__ in, typename Cx<R>::T *__rest
         v.y *= scale;
         if (zero_dc && bt == 0 && row0 + r == 0 && k == 0) v = cmk<C>(0.0, 0.0);
         dst[int64_t(k) * nrow + row0 + r] = v;
-    }
-}
-
-template <typename R, bool UNIT>
-__global__ void __launch_bounds__(256)
-k_ring_gather(const typename Cx<R>::T *__restrict__ planes, int ng, RingArg rings,
-              const Job *__restrict__ jobs, int M, int ntile, int rt, typename Cx<R>::T *__restrict__ gt,
-              Twiddles<typename Cx<R>::T> tw, const float *__restrict__ scale, int64_t fs)
-{
-    using C = typename Cx<R>::T;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    planes = field_ptr(planes, fs);
-    gt = field_ptr(gt, fs);
-    scale = scale ? field_ptr(scale, fs) : scale;
-    const int P = fft_stride(M);
-    C *a = reinterpret_cast<C *>(smem_raw);
-    C *b = a + rt * P;
-    const int64_t jb = blockIdx.x / ntile;
-    const int tile = int(blockIdx.x - jb * ntile);
-    const Job J = jobs[jb];
-    const C *pl = planes + int64_t(J.n) * ng * ng;
-    const int64_t lo = rings.e3sq[J.r], hi = rings.e3sq[J.r + 1];
-    const int mc = rings.maxc[J.r];
-    const R fac = scale ? R(scale[J.n * kMaxRings + J.r]) : R(1);
-    const int row0 = tile * rt;
-    const int nr = min(rt, M - row0);
-    // rows i hold ring members only where |u_x| <= maxc for u_x = i or i - M;
-    // a block of rows without members is zero after the transform too, and
-    // the column pass reads such rows as zero without loading them
-    if (row0 > mc && row0 + nr - 1 < M - mc) return;
-    DivIter ld(threadIdx.x, blockDim.x, M);
-    for (int t = threadIdx.x; t < nr * M; t += blockDim.x, ld.next()) {
-        const int tr = ld.q, j = ld.r;
-        const int i = row0 + tr;
-        R vr = 0, vi = 0;
-        // members u with u_x = i or i - M and u_y = j or j - M (mod M folding;
-        // |u_x|, |u_y| <= maxc < M, so no other alias exists)
-#pragma unroll
-        for (int ca = 0; ca < 2; ++ca) {
-            const int ux = ca ? i - M : i;
-            if (ux > mc || ux < -mc) continue;
-#pragma unroll
-            for (int cb = 0; cb < 2; ++cb) {
-                const int uy = cb ? j - M : j;
-                if (uy > mc || uy < -mc) continue;
-                const int64_t q9 = 9 * (int64_t(ux) * ux + int64_t(uy) * uy);
-                if (q9 < lo || q9 >= hi) continue;
-                if (UNIT) {
-                    vr += R(1);
-                } else {
-                    const C v = pl[int64_t(ux < 0 ? ux + ng : ux) * ng + (uy < 0 ? uy + ng : uy)];
-                    vr += v.x * fac;
-                    vi += v.y * fac;
-                }
-            }
-        }
-        a[tr * P + spos(j)] = cmk<C>(double(vr), double(vi));
-    }
-    __syncthreads();
-    const C *res = fft_smem(a, b, M, P, nr, tw);
-    // rows of the job's M x M field in place (u_x, k_y), whole rows: coalesced
-    C *dst = gt + jb * int64_t(M) * M + int64_t(row0) * M;
-    DivIter st(threadIdx.x, blockDim.x, M);
-    for (int t = threadIdx.x; t < M * nr; t += blockDim.x, st.next()) {
-        const int r = st.q, k = st.r;
-        dst[t] = res[r * P + spos(k)];
     }
 }
 
@@ -499,41 +403,106 @@ k_ring_scale(const float2 *__restrict__ planes, int ng, RingArg rings, float *__
     scale[n * kMaxRings + r] = ldexpf(1.0f, e);
 }
 
-// Step I second pass: transforms along the first axis of each job's M x M
-// field (rows u_x of the gather's output), a strip of w columns k_y per
-// block, read and written in place order (runs of w consecutive elements
-// of every row), so the D field comes out as [k_x][k_y].
-template <typename R>
+// the grid of a Step-I block (the grids of a launch in order of their blocks)
+__device__ __forceinline__ const StepGrid &grid_of_block(const StepGrids &gs)
+{
+    int i = 0;
+    while (i + 1 < gs.n && blockIdx.x >= gs.g[i + 1].blk0) ++i;
+    return gs.g[i];
+}
+
+template <typename R, bool UNIT>
 __global__ void __launch_bounds__(256)
-k_fft_cols(const typename Cx<R>::T *__restrict__ in, typename Cx<R>::T *__restrict__ out, int M, int ntile, int w,
-           const int64_t *__restrict__ out_off, const Job *__restrict__ jobs, RingArg rings,
-           Twiddles<typename Cx<R>::T> tw, int64_t fs)
+k_ring_gather(const typename Cx<R>::T *__restrict__ planes, int ng, const __grid_constant__ RingArg rings,
+              const __grid_constant__ StepGrids gs, typename Cx<R>::T *__restrict__ out,
+              Twiddles<typename Cx<R>::T> tw, const float *__restrict__ scale, int64_t fs)
 {
     using C = typename Cx<R>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    in = field_ptr(in, fs);
+    planes = field_ptr(planes, fs);
     out = field_ptr(out, fs);
+    scale = scale ? field_ptr(scale, fs) : scale;
+    const StepGrid &gr = grid_of_block(gs);
+    const int M = gr.M, rt = gr.rt;
+    const int P = fft_stride(M);
+    C *a = reinterpret_cast<C *>(smem_raw);
+    C *b = a + rt * P;
+    const int blk = int(blockIdx.x - gr.blk0), jb = blk / gr.ntile;
+    const Job J = gr.jobs[jb];
+    const C *pl = planes + int64_t(J.n) * ng * ng;
+    // members: lo <= |u|^2 < hi (9 |u|^2 is compared with squares of 3 e_r)
+    const int lo = int((rings.e3sq[J.r] + 8) / 9), hi = int((rings.e3sq[J.r + 1] + 8) / 9);
+    const int mc = rings.maxc[J.r];
+    const R fac = scale ? R(scale[J.n * kMaxRings + J.r]) : R(1);
+    const int row0 = (blk - jb * gr.ntile) * rt;
+    const int nr = min(rt, M - row0);
+    // rows i hold ring members only where |u_x| <= maxc for u_x = i or i - M;
+    // a block of rows without members is zero after the transform too, and
+    // the column pass reads such rows as zero without loading them
+    if (row0 > mc && row0 + nr - 1 < M - mc) return;
+    // element (row, j): members u with u_x = i or i - M and u_y = j or j - M
+    // (mod M folding; |u_x|, |u_y| <= maxc < M, so no other alias exists)
+    auto load = [&](int row, int j) {
+        const int i = row0 + row;
+        R vr = 0, vi = 0;
+#pragma unroll
+        for (int ca = 0; ca < 2; ++ca) {
+            const int ux = ca ? i - M : i;
+            if (ux > mc || ux < -mc) continue;
+            const C *prow = pl + int64_t(ux < 0 ? ux + ng : ux) * ng;
+#pragma unroll
+            for (int cb = 0; cb < 2; ++cb) {
+                const int uy = cb ? j - M : j;
+                if (uy > mc || uy < -mc) continue;
+                const int q = ux * ux + uy * uy;
+                if (q < lo || q >= hi) continue;
+                if (UNIT) {
+                    vr += R(1);
+                } else {
+                    const C v = prow[uy < 0 ? uy + ng : uy];
+                    vr += v.x * fac;
+                    vi += v.y * fac;
+                }
+            }
+        }
+        C v;
+        v.x = vr;
+        v.y = vi;
+        return v;
+    };
+    // whole rows (u_x, k_y) of the job's M x M field in place: coalesced
+    C *dst = out + J.out_off + int64_t(row0) * M;
+    fft_any<C, false, false, true>(M, nr, 0, P, a, b, tw.t, load, [&](int row, int k, const C &v) { dst[row * M + k] = v; });
+}
+
+// Step I second pass: transforms along the first axis of each job's M x M
+// field (rows u_x of the gather's output), in place: a strip of w columns
+// k_y per block, read (by the first stage) and written (by the last) in runs
+// of w consecutive elements of every row, so the D field comes out as
+// [k_x][k_y].  The threads run across the strip first: the runs are whole
+// 32-byte sectors for w >= 4, and the lanes of a warp take few different twiddles.
+template <typename R>
+__global__ void __launch_bounds__(256)
+k_fft_cols(typename Cx<R>::T *__restrict__ out, const __grid_constant__ StepGrids gs,
+           const __grid_constant__ RingArg rings, Twiddles<typename Cx<R>::T> tw, int64_t fs)
+{
+    using C = typename Cx<R>::T;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    out = field_ptr(out, fs);
+    const StepGrid &gr = grid_of_block(gs);
+    const int M = gr.M, w = gr.rt;
     const int P = fft_stride(M);
     C *a = reinterpret_cast<C *>(smem_raw);
     C *b = a + w * P;
-    const int64_t jb = blockIdx.x / ntile;
-    const int c0 = int(blockIdx.x - jb * ntile) * w;
+    const int blk = int(blockIdx.x - gr.blk0), jb = blk / gr.ntile;
+    const Job J = gr.jobs[jb];
+    const int c0 = (blk - jb * gr.ntile) * w;
     const int nc = min(w, M - c0);
-    const C *src = in + jb * int64_t(M) * M + c0;
-    const int mc = rings.maxc[jobs[jb].r];      // rows mc < i < M - mc hold no ring member: zero
-    DivIter ld(threadIdx.x, blockDim.x, nc);
-    for (int t = threadIdx.x; t < M * nc; t += blockDim.x, ld.next()) {
-        const int i = ld.q, c = ld.r;
-        a[c * P + spos(i)] = (i <= mc || i >= M - mc) ? src[int64_t(i) * M + c] : cmk<C>(0.0, 0.0);
-    }
-    __syncthreads();
-    const C *res = fft_smem(a, b, M, P, nc, tw);
-    C *dst = out + out_off[jb] + c0;
-    DivIter st(threadIdx.x, blockDim.x, nc);
-    for (int t = threadIdx.x; t < M * nc; t += blockDim.x, st.next()) {
-        const int k = st.q, c = st.r;
-        dst[int64_t(k) * M + c] = res[c * P + spos(k)];
-    }
+    const int mc = rings.maxc[J.r];             // rows mc < i < M - mc hold no ring member: zero
+    C *f = out + J.out_off + c0;
+    auto load = [&](int c, int i) { return (i <= mc || i >= M - mc) ? f[i * M + c] : cmk<C>(0.0, 0.0); };
+    fft_any<C, true, false, true>(M, nc, gr.lgw, P, a, b, tw.t, load,
+                                  [&](int c, int k, const C &v) { f[k * M + c] = v; });
 }
 
 // ---------------------------------------------------------------------------
@@ -966,7 +935,7 @@ cudaError_t launch_fft_z_real(const R *in, typename Cx<R>::T *out, int ng, int64
 
 template <typename R>
 cudaError_t launch_fft_rows_T(const typename Cx<R>::T *in, typename Cx<R>::T *out, int M, int nrow,
-                              int64_t nb, const int64_t *out_off, R scale, bool zero_dc,
+                              int64_t nb, R scale, bool zero_dc,
                               const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s, int rt)
 {
     using C = typename Cx<R>::T;
@@ -976,31 +945,49 @@ cudaError_t launch_fft_rows_T(const typename Cx<R>::T *in, typename Cx<R>::T *ou
     const int ntile = (nrow + rt - 1) / rt;
     const int64_t nblk = nb * ntile;
     if (nblk == 0) return cudaSuccess;
-    k_fft_rows_T<R><<<dim3(unsigned(nblk), fb.nf), 256, smem, s>>>(in, out, M, nrow, ntile, out_off, scale,
-                                                                   zero_dc ? 1 : 0, rt, tw, fb.fs_in);
+    k_fft_rows_T<R><<<dim3(unsigned(nblk), fb.nf), 256, smem, s>>>(in, out, M, nrow, ntile, scale, zero_dc ? 1 : 0, rt,
+                                                                   tw, fb.fs_in);
     return cudaGetLastError();
 }
 
-template <typename R>
-cudaError_t launch_ring_gather(const typename Cx<R>::T *planes, int ng, const RingArg &rings, const Job *jobs,
-                               int64_t njobs, int M, bool unit, typename Cx<R>::T *gt,
-                               const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s, int rt,
-                               const float *scale)
+// The blocks of a Step-I launch over several grids, and its shared memory.
+template <typename C> static cudaError_t step_blocks(StepGrids &gs, bool cols, unsigned *nblk, size_t *smem)
 {
-    using C = typename Cx<R>::T;
-    if (rt <= 0) rt = int(fft_rows_per_block(M, sizeof(C)));
-    rt = std::min(rt, M);
-    const size_t smem = size_t(2) * rt * fft_stride(M) * sizeof(C);
-    const int ntile = (M + rt - 1) / rt;
-    const int64_t nblk = njobs * ntile;
+    int64_t blk = 0;
+    *smem = 0;
+    for (int i = 0; i < gs.n; ++i) {
+        StepGrid &g = gs.g[i];
+        if (g.rt <= 0) g.rt = cols ? 8 : int(fft_rows_per_block(g.M, sizeof(C)));
+        g.rt = std::min(g.rt, g.M);
+        if (cols) {                              // strips of a power of two
+            g.lgw = 0;
+            while ((2 << g.lgw) <= g.rt) ++g.lgw;
+            g.rt = 1 << g.lgw;
+        }
+        g.ntile = (g.M + g.rt - 1) / g.rt;
+        g.blk0 = unsigned(blk);
+        blk += g.njobs * g.ntile;
+        *smem = std::max(*smem, size_t(2) * g.rt * fft_stride(g.M) * sizeof(C));
+    }
+    if (blk > 0x7FFFFFFF || *smem > 227 * 1024) return cudaErrorInvalidValue;
+    *nblk = unsigned(blk);
+    return cudaSuccess;
+}
+
+template <typename R>
+cudaError_t launch_ring_gather(const typename Cx<R>::T *planes, int ng, const RingArg &rings, StepGrids gs, bool unit,
+                               typename Cx<R>::T *out, const Twiddles<typename Cx<R>::T> &tw, const Batch &fb,
+                               cudaStream_t s, const float *scale)
+{
+    unsigned nblk;
+    size_t smem;
+    if (cudaError_t e = step_blocks<typename Cx<R>::T>(gs, false, &nblk, &smem); e != cudaSuccess) return e;
     if (nblk == 0) return cudaSuccess;
-    const dim3 grid(unsigned(nblk), fb.nf);
+    const dim3 grid(nblk, fb.nf);
     if (unit)
-        k_ring_gather<R, true><<<grid, 256, smem, s>>>(planes, ng, rings, jobs, M, ntile, rt, gt, tw, scale,
-                                                        fb.fs_in);
+        k_ring_gather<R, true><<<grid, 256, smem, s>>>(planes, ng, rings, gs, out, tw, scale, fb.fs_in);
     else
-        k_ring_gather<R, false><<<grid, 256, smem, s>>>(planes, ng, rings, jobs, M, ntile, rt, gt, tw, scale,
-                                                         fb.fs_in);
+        k_ring_gather<R, false><<<grid, 256, smem, s>>>(planes, ng, rings, gs, out, tw, scale, fb.fs_in);
     return cudaGetLastError();
 }
 
@@ -1012,20 +999,14 @@ cudaError_t launch_ring_scale(const float2 *planes, int ng, int nz1, const RingA
 }
 
 template <typename R>
-cudaError_t launch_fft_cols(const typename Cx<R>::T *in, typename Cx<R>::T *out, int M, int64_t njobs,
-                            const int64_t *out_off, const Job *jobs, const RingArg &rings,
-                            const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s, int w)
+cudaError_t launch_fft_cols(typename Cx<R>::T *out, StepGrids gs, const RingArg &rings,
+                            const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s)
 {
-    using C = typename Cx<R>::T;
-    if (w <= 0) w = 8;
-    w = std::min(w, M);
-    const size_t smem = size_t(2) * w * fft_stride(M) * sizeof(C);
-    if (smem > 227 * 1024) return cudaErrorInvalidValue;
-    const int ntile = (M + w - 1) / w;
-    const int64_t nblk = njobs * ntile;
+    unsigned nblk;
+    size_t smem;
+    if (cudaError_t e = step_blocks<typename Cx<R>::T>(gs, true, &nblk, &smem); e != cudaSuccess) return e;
     if (nblk == 0) return cudaSuccess;
-    k_fft_cols<R><<<dim3(unsigned(nblk), fb.nf), 256, smem, s>>>(in, out, M, ntile, w, out_off, jobs, rings, tw,
-                                                                 fb.fs_in);
+    k_fft_cols<R><<<dim3(nblk, fb.nf), 256, smem, s>>>(out, gs, rings, tw, fb.fs_in);
     return cudaGetLastError();
 }
 
@@ -1183,16 +1164,12 @@ cudaError_t set_ylm_constants(const double nlm[9][9], const double pref[9], cuda
 // explicit instantiations
 template cudaError_t launch_fft_z_real<float>(const float *, float2 *, int, int64_t, int, const Twiddles<float2> &, const Batch &, cudaStream_t, int);
 template cudaError_t launch_fft_z_real<double>(const double *, double2 *, int, int64_t, int, const Twiddles<double2> &, const Batch &, cudaStream_t, int);
-template cudaError_t launch_fft_rows_T<float>(const float2 *, float2 *, int, int, int64_t, const int64_t *, float, bool, const Twiddles<float2> &, const Batch &, cudaStream_t, int);
-template cudaError_t launch_fft_rows_T<double>(const double2 *, double2 *, int, int, int64_t, const int64_t *, double, bool, const Twiddles<double2> &, const Batch &, cudaStream_t, int);
-template cudaError_t launch_ring_gather<float>(const float2 *, int, const RingArg &, const Job *, int64_t, int, bool, float2 *, const Twiddles<float2> &, const Batch &, cudaStream_t, int, const float *);
-template cudaError_t launch_ring_gather<double>(const double2 *, int, const RingArg &, const Job *, int64_t, int, bool, double2 *, const Twiddles<double2> &, const Batch &, cudaStream_t, int, const float *);
-template cudaError_t launch_fft_cols<float>(const float2 *, float2 *, int, int64_t, const int64_t *, const Job *,
-                                            const RingArg &, const Twiddles<float2> &,
-                                            const Batch &, cudaStream_t, int);
-template cudaError_t launch_fft_cols<double>(const double2 *, double2 *, int, int64_t, const int64_t *, const Job *,
-                                             const RingArg &,
-                                             const Twiddles<double2> &, const Batch &, cudaStream_t, int);
+template cudaError_t launch_fft_rows_T<float>(const float2 *, float2 *, int, int, int64_t, float, bool, const Twiddles<float2> &, const Batch &, cudaStream_t, int);
+template cudaError_t launch_fft_rows_T<double>(const double2 *, double2 *, int, int, int64_t, double, bool, const Twiddles<double2> &, const Batch &, cudaStream_t, int);
+template cudaError_t launch_ring_gather<float>(const float2 *, int, const RingArg &, StepGrids, bool, float2 *, const Twiddles<float2> &, const Batch &, cudaStream_t, const float *);
+template cudaError_t launch_ring_gather<double>(const double2 *, int, const RingArg &, StepGrids, bool, double2 *, const Twiddles<double2> &, const Batch &, cudaStream_t, const float *);
+template cudaError_t launch_fft_cols<float>(float2 *, StepGrids, const RingArg &, const Twiddles<float2> &, const Batch &, cudaStream_t);
+template cudaError_t launch_fft_cols<double>(double2 *, StepGrids, const RingArg &, const Twiddles<double2> &, const Batch &, cudaStream_t);
 template cudaError_t launch_step2<float>(const StepIIArgs &, const float2 *, const int64_t *, const int64_t *, int,
                                          cudaStream_t);
 template cudaError_t launch_step2<double>(const StepIIArgs &, const double2 *, const int64_t *, const int64_t *, int,

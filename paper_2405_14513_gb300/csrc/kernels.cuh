@@ -21,19 +21,22 @@ struct RingArg {
     int maxc[kMaxRings];
 };
 
-// Twiddle tables of the transforms: tw2[k] = exp(-2 pi i k / 2^lg2) for
-// lengths 2^q <= 2^lg2, tw3[k] = exp(-2 pi i k / (3 x 2^lg3)) for lengths
-// 3 x 2^q <= 3 x 2^lg3, and likewise tw5 and tw7 for lengths 5 x 2^q and
-// 7 x 2^q (tw3, tw5, tw7 may be null when no such length is used).
+// Twiddle table of the transforms, computed on the host in double.  A stage of
+// a transform of length F x 2^q (F = 1, 3, 5, 7) that starts from Ns = F x 2^s
+// interleaved results (s = 0, 3, 6, ..; Ns <= 512) takes, with w_R = exp(-2 pi i
+// / (R Ns)), w_8^(rk) in [r - 1][k] (r = 1 .. 7), then w_4^(rk) (r = 1 .. 3), then
+// w_2^k, k < Ns: 11 Ns values, each run contiguous in k.
 template <typename C> struct Twiddles {
-    const C *tw2;
-    const C *tw3;
-    int lg2, lg3;
-    const C *tw5;
-    int lg5;
-    const C *tw7;
-    int lg7;
+    const C *t;
+    // first element of length family F, and of its stage Ns = F x 2^s (relative)
+    static BISP_HD constexpr int offset(int F)
+    {
+        return 11 * (F == 1 ? 0 : (F == 3 ? 585 : (F == 5 ? 804 : 1169)));
+    }
+    static BISP_HD constexpr int stage(int F, int s) { return 11 * F * (((1 << s) - 1) / 7); }
 };
+constexpr int kTwiddles = 11 * 1680;             // F = 1: Ns = 1 .. 512; 3: 3 .. 192; 5: 5 .. 320; 7: 7 .. 448
+void make_twiddles(double2 *t);                  // fills kTwiddles values
 
 // Side lengths of the plan's reduction grids, by level index.
 struct GridArg {
@@ -52,6 +55,21 @@ struct Batch {
 struct Job {
     int32_t n, r;
     int64_t out_off;   // complex elements into the destination store
+};
+
+// The reduction grids of a Step-I launch: grid i's jobs take the blocks from
+// blk0 on, ntile blocks of rt rows (first pass) or columns (second) per job.  The
+// caller fills M, rt (0: the default), jobs and njobs.
+struct StepGrid {
+    int M, rt;
+    const Job *jobs;
+    int64_t njobs;
+    int ntile, lgw;
+    unsigned blk0;
+};
+struct StepGrids {
+    int n = 0;
+    StepGrid g[kMaxLevels];
 };
 
 struct StepIIArgs {
@@ -74,26 +92,24 @@ template <typename R>
 cudaError_t launch_fft_z_real(const R *in, typename Cx<R>::T *out, int ng, int64_t rows, int nkeep,
                               const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s, int rt = 0);
 
-// Batched row transforms written transposed: in[b][nrow][M] -> out[b][M][nrow]
-// (out at out_off[b] when out_off is not null, else b * M * nrow), times
-// scale; zero_dc clears element [0][0] of batch 0.
+// Batched row transforms written transposed: in[b][nrow][M] -> out[b][M][nrow],
+// times scale; zero_dc clears element [0][0] of batch 0.
 template <typename R>
 cudaError_t launch_fft_rows_T(const typename Cx<R>::T *in, typename Cx<R>::T *out, int M, int nrow,
-                              int64_t nb, const int64_t *out_off, R scale, bool zero_dc,
+                              int64_t nb, R scale, bool zero_dc,
                               const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s,
                               int rt = 0);
 
-// Step I, first pass: ring r of plane n of Delta (planes [nz+1][ng][ng]),
-// folded onto the M x M grid, transformed along u_y, written in place order
-// to gt[job][u_x][k_y].  unit = true uses Delta = 1 (the unit fields of
+// Step I, first pass: for every job of the grids, ring r of plane n of Delta
+// (planes [nz+1][ng][ng]), folded onto the M x M grid, transformed along u_y,
+// written in place order [u_x][k_y] at out + out_off; rows that hold no member
+// of the ring are not written.  unit = true uses Delta = 1 (the unit fields of
 // Eq. 2FT).  scale: optional factors [nz1][kMaxRings] of the members' values
 // (one field's; the next field's lie fb.fs_in bytes further).
 template <typename R>
-cudaError_t launch_ring_gather(const typename Cx<R>::T *planes, int ng, const RingArg &rings,
-                               const Job *jobs, int64_t njobs, int M, bool unit,
-                               typename Cx<R>::T *gt, const Twiddles<typename Cx<R>::T> &tw,
-                               const Batch &fb, cudaStream_t s, int rt = 0,
-                               const float *scale = nullptr);
+cudaError_t launch_ring_gather(const typename Cx<R>::T *planes, int ng, const RingArg &rings, StepGrids gs, bool unit,
+                               typename Cx<R>::T *out, const Twiddles<typename Cx<R>::T> &tw, const Batch &fb,
+                               cudaStream_t s, const float *scale = nullptr);
 
 // Power-of-two factor of every (plane, ring) field D(r, n), [nz1][kMaxRings]
 // (see k_ring_scale): with it, every |D| on the grid is at most kFieldBound.
@@ -103,15 +119,12 @@ constexpr float kFieldBound = 250.0f;
 cudaError_t launch_ring_scale(const float2 *planes, int ng, int nz1, const RingArg &rings, float *scale,
                               const Batch &fb, cudaStream_t s);
 
-// Step I second pass: for each of njobs M x M fields in gt ([u_x][k_y],
-// the gather's output), transforms along u_x in strips of w columns and
-// writes the field [k_x][k_y] at out + out_off[job].  Rows that hold no
-// member of the job's ring (jobs[job].r, its largest |u_x| in rings) are
-// taken as zero without being read (the gather does not write them).
+// Step I second pass: the M x M field of every job, as the first pass left it,
+// transformed along u_x in place, in strips of columns: [k_x][k_y].  Rows
+// that hold no member of the job's ring are taken as zero without being read.
 template <typename R>
-cudaError_t launch_fft_cols(const typename Cx<R>::T *in, typename Cx<R>::T *out, int M, int64_t njobs,
-                            const int64_t *out_off, const Job *jobs, const RingArg &rings,
-                            const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s, int w = 0);
+cudaError_t launch_fft_cols(typename Cx<R>::T *out, StepGrids gs, const RingArg &rings,
+                            const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s);
 
 // Step II: partial triple sums of units, one block per unit, one launch per
 // block class (units [lo[c], hi[c]) run in blocks of 2^c warps with

@@ -771,7 +771,6 @@ std::string enumerate(HostPlan &P, int64_t x_chunk)
     P.doff.assign(size_t(kMaxLevels) * (nz + 1) * kMaxRings, -1);
     P.levels.clear();
     int64_t cursor = 0;
-    P.gt_elems = 0;
     for (int lv = 0; lv < R.ngrid; ++lv) {
         Level L;
         L.lev = lv;
@@ -785,10 +784,7 @@ std::string enumerate(HostPlan &P, int64_t x_chunk)
                     cursor += M2;
                     L.njobs++;
                 }
-        if (L.njobs) {
-            P.levels.push_back(L);
-            P.gt_elems = std::max(P.gt_elems, L.njobs * M2);
-        }
+        if (L.njobs) P.levels.push_back(L);
     }
     P.dstore_elems = cursor;
 

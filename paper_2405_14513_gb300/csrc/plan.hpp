@@ -263,7 +263,6 @@ struct HostPlan {
     std::vector<int64_t> doff;
     std::vector<Level> levels;          // levels in use
     int64_t dstore_elems = 0;
-    int64_t gt_elems = 0;               // largest per-level Step-I scratch
 };
 
 // N_g = 2^k or 3 x 2^k in [8, 1024] (the transform lengths the kernels handle).

@@ -179,8 +179,6 @@ struct bisp_shell_plan {
     double *d_den = nullptr;
     int64_t *d_bin_start = nullptr;
     int32_t *d_bin_tri = nullptr;
-    float2 *tw2f = nullptr, *tw3f = nullptr;
-    double2 *tw2d = nullptr, *tw3d = nullptr;
     Twiddles<float2> twf{};
     Twiddles<double2> twd{};
     // workspace layout (bytes)
@@ -221,9 +219,9 @@ cudaError_t fft3(typename Cx<R>::T *a, typename Cx<R>::T *b, int ng, int64_t nb,
                  const Twiddles<typename Cx<R>::T> &tw, cudaStream_t s)
 {
     const int nrow = ng * ng;
-    cudaError_t e = launch_fft_rows_T<R>(a, b, ng, nrow, nb, nullptr, R(1), false, tw, Batch{}, s);
-    if (e == cudaSuccess) e = launch_fft_rows_T<R>(b, a, ng, nrow, nb, nullptr, R(1), false, tw, Batch{}, s);
-    if (e == cudaSuccess) e = launch_fft_rows_T<R>(a, b, ng, nrow, nb, nullptr, R(1), false, tw, Batch{}, s);
+    cudaError_t e = launch_fft_rows_T<R>(a, b, ng, nrow, nb, R(1), false, tw, Batch{}, s);
+    if (e == cudaSuccess) e = launch_fft_rows_T<R>(b, a, ng, nrow, nb, R(1), false, tw, Batch{}, s);
+    if (e == cudaSuccess) e = launch_fft_rows_T<R>(a, b, ng, nrow, nb, R(1), false, tw, Batch{}, s);
     return e;
 }
 
@@ -240,29 +238,20 @@ bool triple_bin(const bisp_shell_plan &P, double kp1, double kp2, double kp3, in
     return true;
 }
 
-int make_twiddles(bisp_shell_plan *p, cudaStream_t s)
+int upload_twiddles(bisp_shell_plan *p, cudaStream_t s)
 {
-    const int ng = p->ng;
-    int lg2 = 0, lg3 = 0;
-    while ((2 << lg2) <= ng) ++lg2;
-    while (3 * (2 << lg3) <= ng) ++lg3;
-    if (lg3 < 1) lg3 = 1;
-    auto table = [&](int base, int count, float2 **f, double2 **d) -> int {
-        std::vector<double2> vd(count);
-        std::vector<float2> vf(count);
-        for (int k = 0; k < count; ++k) {
-            const double a = -kShellTwoPi * double(k) / double(base);
-            vd[k] = make_double2(std::cos(a), std::sin(a));
-            vf[k] = make_float2(float(vd[k].x), float(vd[k].y));
-        }
-        int st = sup(p, d, vd, s);
-        return st ? st : sup(p, f, vf, s);
-    };
-    int st = table(1 << lg2, (7 * (1 << lg2) + 7) / 8, &p->tw2f, &p->tw2d);
-    if (!st) st = table(3 << lg3, (7 * (3 << lg3) + 7) / 8, &p->tw3f, &p->tw3d);
+    std::vector<double2> vd(kTwiddles);
+    std::vector<float2> vf(kTwiddles);
+    make_twiddles(vd.data());
+    for (int k = 0; k < kTwiddles; ++k) vf[k] = make_float2(float(vd[k].x), float(vd[k].y));
+    double2 *d = nullptr;
+    float2 *f = nullptr;
+    int st = sup(p, &d, vd, s);
+    if (!st) st = sup(p, &f, vf, s);
     if (st) return st;
-    p->twf = Twiddles<float2>{p->tw2f, p->tw3f, lg2, lg3};
-    p->twd = Twiddles<double2>{p->tw2d, p->tw3d, lg2, lg3};
+    SCK(cudaStreamSynchronize(s));
+    p->twf = Twiddles<float2>{f};
+    p->twd = Twiddles<double2>{d};
     return BISP_OK;
 }
 
@@ -325,7 +314,7 @@ int build_shell_plan(bisp_shell_plan *p, const bisp_desc *d, cudaStream_t s)
                 cand.insert(cand.end(), {s1, s2, s3});
                 cbin.push_back(bin);
             }
-    int st = make_twiddles(p, s);
+    int st = upload_twiddles(p, s);
     if (!st) st = sup(p, &p->d_e3sq, p->e3sq, s);
     if (st) return st;
     const int64_t n3 = int64_t(ng) * ng * ng;
@@ -516,8 +505,8 @@ int estimator_shell_estimate(bisp_shell_plan *p, const float *delta, void *works
     const double V = p->desc.box_len * p->desc.box_len * p->desc.box_len;
     // forward transform (planes 0..N_g/3 kept, scaled by V/N^3, Delta(0) = 0)
     SCK(launch_fft_z_real<float>(delta, A_, ng, ng2, p->nz + 1, p->twf, Batch{}, s));
-    SCK(launch_fft_rows_T<float>(A_, B_, ng, ng, p->nz + 1, nullptr, 1.0f, false, p->twf, Batch{}, s));
-    SCK(launch_fft_rows_T<float>(B_, A_, ng, ng, p->nz + 1, nullptr, float(V / double(n3)), true, p->twf, Batch{}, s));
+    SCK(launch_fft_rows_T<float>(A_, B_, ng, ng, p->nz + 1, 1.0f, false, p->twf, Batch{}, s));
+    SCK(launch_fft_rows_T<float>(B_, A_, ng, ng, p->nz + 1, float(V / double(n3)), true, p->twf, Batch{}, s));
     if (p->njobs > 0) {
         k_shell_spectrum<float2><<<dim3(blocks_for(n3), unsigned(p->njobs)), 256, 0, s>>>(A_, ng, p->d_e3sq, p->d_jobs, sa);
         SCK(cudaGetLastError());
