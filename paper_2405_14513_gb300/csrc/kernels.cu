@@ -520,10 +520,33 @@ k_fft_cols(typename Cx<R>::T *__restrict__ out, const __grid_constant__ StepGrid
 // chunk, reduced across the warp at the end.  Negative planes enter through
 // D(r, -n) = conj D(r, n) as sign factors.  Blocks of 4, 8 and 16 warps
 // (unit classes) let small units share an SM.
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
+//
+// A tile's 64 entries are a quarter to a half combinations (64^3 23%, 256^3
+// 54%): FP32 computes them all (a test costs as much as the two FMAs), FP64,
+// bound by its pipe of two lanes a clock and SM, tests each entry (the mask is
+// uniform over the warp) and leaves the others out.
+//
+// FP32 is bound by instruction issue (75% of the slots), of which the FMAs of a
+// tile are a third: so the staging and the addresses are kept lean (stages of a
+// constant 64 or 128 points, slot addresses in registers, one piece column per
+// thread, signs on sign bits), and the warps that a unit's tiles leave over take
+// turns at the points (128^3: 61% of the warp slots had a tile).  Without these
+// 128^3 took 6.3 ms and 96^3 x 2 3.6 ms, with them 3.8 and 2.1; FP64 at 64^3 4.3
+// and 2.2 ms, most of it from the entries left out.
+// (The asm statements below clobber memory at the barriers' sides only, so
+// the loads of a stage may move among each other.)
+template <typename C> __device__ __forceinline__ C lds_complex(uint32_t a)
 {
-    const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem));
+    C v;
+    if constexpr (sizeof(C) == 8) asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+    else asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a));
+    return v;
+}
+// x, with the other sign where bit = 0x80000000
+__device__ __forceinline__ float flip_sign(float x, uint32_t bit) { return __uint_as_float(__float_as_uint(x) ^ bit); }
+__device__ __forceinline__ double flip_sign(double x, uint32_t bit)
+{
+    return __hiloint2double(__double2hiint(x) ^ int(bit), __double2loint(x));
 }
 
 template <typename R, int NW>
@@ -534,6 +557,7 @@ k_step2(StepIIArgs args, int64_t unit0, const typename Cx<R>::T *__restrict__ ds
     args.partials = field_ptr(args.partials, args.fs);
     using C = typename Cx<R>::T;
     constexpr int NT = 32 * NW;
+    constexpr bool SKIP = sizeof(R) == 8;     // see above
     constexpr int PER16 = 16 / sizeof(C);     // complex values per 16-byte copy
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const Unit U = args.units[unit0 + blockIdx.x];
@@ -548,10 +572,9 @@ k_step2(StepIIArgs args, int64_t unit0, const typename Cx<R>::T *__restrict__ ds
     int64_t *offs = reinterpret_cast<int64_t *>(smem_raw);
     const size_t off = (size_t(ns) * sizeof(int64_t) + 127) & ~size_t(127);
     C *buf = reinterpret_cast<C *>(smem_raw + off);
-    // grid points per stage: as many as fit, a multiple of 64, at most 256
-    int TX = int((size_t(smem_bytes) - off) / (2 * size_t(ns) * sizeof(C)));
-    TX = min(256, TX & ~63);
-    const size_t stage_elems = size_t(ns) * TX;
+    // grid points per stage: 64 (the plan saw to it that they fit), 128 where
+    // they do; constants, so that the slots' addresses are a base and an immediate
+    const bool wide = off + 2 * size_t(ns) * 128 * sizeof(C) <= size_t(smem_bytes);
 
     for (int s = threadIdx.x; s < ns; s += NT) {
         const int q = s < nq0 ? 0 : (s < nq0 + nq1 ? 1 : 2);
@@ -561,82 +584,105 @@ k_step2(StepIIArgs args, int64_t unit0, const typename Cx<R>::T *__restrict__ ds
     }
     __syncthreads();
 
-    // sign factors of conj(D) for negative planes: with D1 -> (a.x, g1 a.y),
-    // D2 -> (b.x, g2 b.y), D3 -> (c.x, g3 c.y):
-    //   Re(P D3) = Pr c.x - g3 Pi c.y,  Pr = a.x b.x - g1 g2 a.y b.y,
-    //   g3 Pi = g3 g2 a.x b.y + g3 g1 a.y b.x
-    const R g1 = G.n1 < 0 ? R(-1) : R(1), g2 = G.n2 < 0 ? R(-1) : R(1), g3 = G.n3 < 0 ? R(-1) : R(1);
-    const R k12 = -g1 * g2, k32 = g3 * g2, k31 = g3 * g1;
+    // signs of conj(D) for negative planes (n1 >= 0): with D2 -> (b.x, g2 b.y),
+    // D3 -> (c.x, g3 c.y):  Re(P D3) = Pr c.x + Pi (-g3 c.y); applied to the
+    // fields' sign bits
+    const uint32_t flip2 = G.n2 < 0 ? 0x80000000u : 0u, flip3 = G.n3 < 0 ? 0u : 0x80000000u;
 
+    // tile of the warp, and which of the tile's warps it is: a unit with fewer
+    // tiles than warps gives each tile nw2 of them, which take turns at 32 points
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const bool active = warp < U.nt;
+    int ntile2 = 1;
+    while (ntile2 < U.nt) ntile2 *= 2;
+    const int nw2 = NW / ntile2, tile = warp & (ntile2 - 1), turn = warp / ntile2;
+    const bool active = tile < U.nt;
     Tile T;
-    if (active) T = args.tiles[U.t0 + warp];
+    if (active) T = args.tiles[U.t0 + tile];
     R a[kTileRows * kTileCols];
 #pragma unroll
     for (int i = 0; i < kTileRows * kTileCols; ++i) a[i] = R(0);
 
-    const int nstage = int((x1 - x0 + TX - 1) / TX);
-    auto issue = [&](int st) {
-        C *dst = buf + size_t(st & 1) * stage_elems;
-        const int64_t xs = x0 + int64_t(st) * TX;
-        const int nx = int(min(int64_t(TX), x1 - xs));
-        const int per = TX / PER16;                   // 16-byte pieces per slot row
-        for (int k = threadIdx.x; k < ns * per; k += NT) {
-            const int s = k / per, c = (k - s * per) * PER16;
-            C *d = dst + size_t(s) * TX + c;
-            if (offs[s] >= 0 && c < nx) cp_async16(d, dstore + offs[s] + xs + c);
-            else *reinterpret_cast<float4 *>(d) = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        asm volatile("cp.async.commit_group;\n" ::);
-    };
-    issue(0);
-    for (int st = 0; st < nstage; ++st) {
-        if (st + 1 < nstage) {
-            issue(st + 1);
-            asm volatile("cp.async.wait_group 1;\n" ::);
-        } else {
-            asm volatile("cp.async.wait_group 0;\n" ::);
-        }
-        __syncthreads();
-        const C *b = buf + size_t(st & 1) * stage_elems;
-        const int nx = int(min(int64_t(TX), x1 - (x0 + int64_t(st) * TX)));
+    // the stage loop, TX points a stage
+    auto run = [&](auto txc) {
+        constexpr int TX = decltype(txc)::value;
+        constexpr int per = TX / PER16;               // 16-byte pieces per slot row
+        static_assert(NT % per == 0, "a thread copies one piece of its slots");
+        const uint32_t buf0 = uint32_t(__cvta_generic_to_shared(buf)), stage_bytes = uint32_t(ns * TX * sizeof(C));
+        const int nstage = int((x1 - x0 + TX - 1) / TX);
+        auto issue = [&](int st) {
+            const uint32_t dst = buf0 + (st & 1) * stage_bytes;
+            const C *src = dstore + x0 + int64_t(st) * TX;
+            const int nx = int(min(int64_t(TX), x1 - x0 - int64_t(st) * TX));
+            // the thread's piece of every (NT / per)-th slot
+            const int c = int(threadIdx.x % per) * PER16;
+            uint32_t d = dst + 16 * threadIdx.x;
+            for (int s = threadIdx.x / per; s < ns; s += NT / per, d += 16 * NT) {
+                const int64_t o = offs[s];
+                if (o >= 0 && c < nx)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src + c + o));
+                else
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};\n" ::"r"(d), "r"(0) : "memory");
+            }
+            asm volatile("cp.async.commit_group;\n" ::: "memory");
+        };
+        // shared-memory addresses of the tile's slots in stage buffer 0 (this
+        // lane's point), kept: the compiler would rebuild them from their bytes
+        // for every stage
+        uint32_t a1[kTileRows], a2[kTileRows], a3 = 0;
         if (active) {
-            // per-stage slot pointers (lane offset included); the x loop
-            // advances them by 64 points and reads two points per lane
-            const int o3 = T.s3 * TX + lane;
-            int o1[kTileRows], o2[kTileRows];
+            a3 = buf0 + uint32_t((T.s3 * TX + lane) * sizeof(C));
 #pragma unroll
             for (int i = 0; i < kTileRows; ++i) {
-                o1[i] = T.s1[i] * TX + lane;
-                o2[i] = T.s2[i] * TX + lane;
+                a1[i] = buf0 + uint32_t((T.s1[i] * TX + lane) * sizeof(C));
+                a2[i] = buf0 + uint32_t((T.s2[i] * TX + lane) * sizeof(C));
+                asm volatile("" : "+r"(a1[i]), "+r"(a2[i]));
             }
-            for (int xc = 0; xc < nx; xc += 64) {
+        }
+        issue(0);
+        for (int st = 0; st < nstage; ++st) {
+            if (st + 1 < nstage) {
+                issue(st + 1);
+                asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+            }
+            __syncthreads();
+            const int nx = int(min(int64_t(TX), x1 - (x0 + int64_t(st) * TX)));
+            if (active) {
 #pragma unroll 1
-                for (int h = 0; h < 2; ++h) {
-                    const int x = xc + 32 * h;
+                for (int x = 32 * turn; x < nx; x += 32 * nw2) {      // 32 points, one per lane
+                    const uint32_t at = (st & 1) * stage_bytes + uint32_t(x * sizeof(C));
                     C w[kTileCols];
 #pragma unroll
-                    for (int j = 0; j < kTileCols; ++j) w[j] = b[o3 + j * TX + x];
+                    for (int j = 0; j < kTileCols; ++j) {
+                        w[j] = lds_complex<C>(a3 + at + uint32_t(j * TX * sizeof(C)));
+                        w[j].y = flip_sign(w[j].y, flip3);
+                    }
 #pragma unroll
                     for (int i = 0; i < kTileRows; ++i) {
-                        const C u = b[o1[i] + x];
-                        const C v = b[o2[i] + x];
-                        const R pr = fma(u.x, v.x, k12 * (u.y * v.y));
-                        const R npi = -fma(k32 * u.x, v.y, k31 * (u.y * v.x));
+                        // FP64: entries that are no combination are left out
+                        const uint32_t live = SKIP ? (T.mask[i / 4] >> (8 * (i % 4))) & 255u : 255u;
+                        if (SKIP && live == 0) continue;
+                        const C u = lds_complex<C>(a1[i] + at);
+                        const C v = lds_complex<C>(a2[i] + at);
+                        const R vy = flip_sign(v.y, flip2);
+                        const R pr = fma(u.x, v.x, -(u.y * vy));
+                        const R pi = fma(u.x, vy, u.y * v.x);
 #pragma unroll
                         for (int j = 0; j < kTileCols; ++j) {
+                            if (SKIP && !((live >> j) & 1u)) continue;
                             R &acc = a[i * kTileCols + j];
                             acc = fma(pr, w[j].x, acc);
-                            acc = fma(npi, w[j].y, acc);
+                            acc = fma(pi, w[j].y, acc);
                         }
                     }
                 }
             }
+            __syncthreads();
         }
-        __syncthreads();
-    }
-    if (!active) return;
+    };
+    if (wide) run(std::integral_constant<int, 128>{});
+    else run(std::integral_constant<int, 64>{});
     // butterfly reduction across the warp: after the step with offset o the
     // lane keeps the half of its sums selected by (lane & o); at the end lane
     // l holds the sums of tile entries 2 l and 2 l + 1
@@ -651,11 +697,27 @@ k_step2(StepIIArgs args, int64_t unit0, const typename Cx<R>::T *__restrict__ ds
             a[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
         }
     }
+    // the warps of a tile: their sums in order, in FP64 (the stages' buffers
+    // are free after the loop's last barrier)
+    double sum[2] = {double(a[0]), double(a[1])};
+    if (nw2 > 1) {
+        double *sh = reinterpret_cast<double *>(buf);
+        if (turn > 0) {
+            sh[64 * warp + 2 * lane] = sum[0];
+            sh[64 * warp + 2 * lane + 1] = sum[1];
+        }
+        __syncthreads();
+        if (turn > 0) return;
+        for (int g = 1; g < nw2; ++g)
+#pragma unroll
+            for (int k = 0; k < 2; ++k) sum[k] += sh[64 * (warp + g * ntile2) + 2 * lane + k];
+    }
+    if (!active) return;
     double *dst = args.partials + G.part0 + int64_t(U.chunk) * G.ncombo;
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const int idx = 2 * lane + k;
-        if ((T.mask[idx >> 5] >> (idx & 31)) & 1u) dst[T.coff[idx / kTileCols] + (idx % kTileCols)] = double(a[k]);
+        if ((T.mask[idx >> 5] >> (idx & 31)) & 1u) dst[T.coff[idx / kTileCols] + (idx % kTileCols)] = sum[k];
     }
 }
 
