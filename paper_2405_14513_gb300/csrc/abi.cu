@@ -37,7 +37,8 @@ int fail(int code, const std::string &msg)
     } while (0)
 
 constexpr double kTwoPi = 6.283185307179586476925286766559;
-constexpr int64_t kXChunk = 16384;        // grid points of one Step-II unit
+constexpr int64_t kXChunk = 16384;        // grid points of one Step-II unit, at most
+constexpr int64_t kXChunkMin = 512, kUnitsWanted = 1216;   // shorter where there are few (4 per place of a unit)
 constexpr size_t kStepShare = size_t(64) << 20;   // bytes of fields up to which Step-I grids share launches
 
 size_t align256(size_t v) { return (v + 255) & ~size_t(255); }
@@ -592,6 +593,19 @@ int build_plan(bisp_plan *p, const bisp_desc *desc, cudaStream_t s)
     p->x_chunk = kXChunk;
     std::string err = enumerate(P, p->x_chunk);
     if (!err.empty()) return fail(BISP_INTERNAL, err);
+    if (P.tensor) {
+        // a plan of few tiles: shorter x chunks, so that every SM has several
+        // units to take in turn (64^3, 311 tiles on 304 places: the last wave and
+        // the largest grid's units decided the time)
+        auto units = [&](int64_t chunk) {
+            int64_t n = 0;
+            for (const TcTile &T : P.tc_tiles) n += (int64_t(T.M) * T.M + chunk - 1) / chunk;
+            return n;
+        };
+        while (p->x_chunk > kXChunkMin && units(p->x_chunk) < kUnitsWanted) p->x_chunk /= 2;
+        if (p->x_chunk != kXChunk) err = enumerate(P, p->x_chunk);
+        if (!err.empty()) return fail(BISP_INTERNAL, err);
+    }
     unit_costs(P, p->x_chunk);
     build_views(P, mu_l.empty() ? nullptr : mu_l.data(), t_l.empty() ? nullptr : t_l.data());
     sort_records(P);
@@ -658,7 +672,7 @@ int build_plan(bisp_plan *p, const bisp_desc *desc, cudaStream_t s)
     // Step-I jobs per grid, and the launches: consecutive small grids share one
     // while their fields together take at most kStepShare bytes; their kernels
     // last a few us each, so a plan of small grids was bound by the launches
-    // (64^3, 11 grids: 22 launches, 151 us; in two, see DESIGN), while a large grid
+    // (64^3, 11 grids: 22 launches, 157 us; in two, 63 us), while a large grid
     // fills the GPU by itself and keeps the shared memory that suits it
     size_t share = 0;
     for (const Level &L : P.levels) {

@@ -215,18 +215,21 @@ void enumerate_pair(const HostPlan &P, int n1, int n2, PairOut &out)
 // (b, x), (b, y) halve both loads, two rows of one D1 field on lanes 2q, 2q + 1
 // halve the first, two of one D2 field the second.  The condition is on whole
 // warps, so the lanes are filled in the order: quads, D1 pairs, rows alone,
-// D2 pairs, and where the tile has lanes to spare, each kind starts a warp.
-// key1, key2: the rows' fields.  Returns lane -> row (-1: no row) and the
-// row whose fields a lane without a row repeats (so that it breaks no pair).
+// D2 pairs, and where the last warp has lanes to spare, each kind starts a warp.
+// key1, key2: the fields of rows first .. last - 1, which take as few warps as
+// they can, from lane `lane0` on (a multiple of 32).  Sets lane -> row (-1: no
+// row) and the row whose fields a lane without a row repeats (so that it breaks
+// no pair).  Returns the lane after the last warp.
 struct LaneOrder {
     int row[kTcRows], like[kTcRows];
     bool pair1[kTcRows / 32], pair2[kTcRows / 32];    // per warp: the D1 / D2 loads take two passes
 };
-LaneOrder arrange_lanes(const std::vector<int32_t> &key1, const std::vector<int32_t> &key2)
+int arrange_lanes(const std::vector<int32_t> &key1, const std::vector<int32_t> &key2, int first, int last, int lane0,
+                  LaneOrder &L)
 {
-    const int n = int(key1.size());
+    const int n = last - first;
     std::vector<int> by1(n);
-    for (int i = 0; i < n; ++i) by1[i] = i;
+    for (int i = 0; i < n; ++i) by1[i] = first + i;
     std::sort(by1.begin(), by1.end(), [&](int a, int b) {
         return key1[a] != key1[b] ? key1[a] < key1[b] : key2[a] < key2[b];
     });
@@ -273,9 +276,9 @@ LaneOrder arrange_lanes(const std::vector<int32_t> &key1, const std::vector<int3
     std::stable_sort(kind[2].begin(), kind[2].end(), [&](int a, int b) {
         return key1[a] != key1[b] ? key1[a] < key1[b] : key2[a] < key2[b];
     });
-    LaneOrder L;
-    int at = 0, spare = kTcRows - n;
-    for (int i = 0; i < kTcRows; ++i) L.row[i] = -1;
+    const int end = lane0 + (n + 31) / 32 * 32;
+    int at = lane0, spare = end - lane0 - n;
+    for (int i = lane0; i < end; ++i) L.row[i] = -1;
     for (int k = 0; k < 4; ++k) {
         const int pad = (32 - at % 32) % 32;
         if (!kind[k].empty() && pad <= spare) {
@@ -284,16 +287,9 @@ LaneOrder arrange_lanes(const std::vector<int32_t> &key1, const std::vector<int3
         }
         for (int r : kind[k]) L.row[at++] = r;
     }
-    // a lane without a row repeats the lane that its pairing mirrors, else the nearest row before it
-    for (int i = 0; i < kTcRows; ++i) {
-        L.like[i] = L.row[i];
-        if (L.row[i] >= 0) continue;
-        const int q = i & ~3;
-        L.like[i] = i == 0 ? 0 : L.like[i - 1];
-        if (i >= 4 && (i & 3)) L.like[i] = L.like[i - 1];
-        if (i != q && L.row[q] < 0) L.like[i] = L.like[q];
-    }
-    for (int w = 0; w < kTcRows / 32; ++w) {
+    // a lane without a row repeats the lane before it (lane lane0 has a row)
+    for (int i = lane0; i < end; ++i) L.like[i] = L.row[i] >= 0 ? L.row[i] : L.like[i - 1];
+    for (int w = lane0 / 32; w < end / 32; ++w) {
         auto merged = [&](const std::vector<int32_t> &key, int x) {
             for (int l = 0; l < 32; ++l)
                 if (key[L.like[32 * w + l]] != key[L.like[32 * w + (l ^ x)]]) return false;
@@ -302,13 +298,16 @@ LaneOrder arrange_lanes(const std::vector<int32_t> &key1, const std::vector<int3
         L.pair1[w] = merged(key1, 1) || merged(key1, 2);
         L.pair2[w] = merged(key2, 1) || merged(key2, 2);
     }
-    return L;
+    return end;
 }
 
 // tcgen05 tiles (see TcTile): the groups of each (grid, |n3|, signs of n1,
 // n2, n3) in order of n1, their rows by the centre of their r3 run, cut
 // greedily into tiles of at most 128 rows and a window of at most 64 r3
-// whose fields fit kTcMinRing ring buffers of shared memory; then units (tile,
+// whose fields fit kTcMinRing ring buffers of shared memory.  The last, partly
+// filled tiles of the sign patterns of one (grid, |n3|) are put into one tile
+// where they fit, each pattern in warps of its own (at 64^3 such tiles are most of
+// them: they filled 30% of their lanes, merged ones 53%).  Then units (tile,
 // x chunk) by class.
 // Requires the groups' partial-sum layout.  Marks the fields the tiles read.
 template <typename UsedFn>
@@ -333,7 +332,7 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
         std::vector<int32_t> slots;
         int lo = 1 << 30, hi = -1;
     } cur;
-    int cur_lev = 0, cur_n3 = 0, cur_flags = 0;
+    int cur_lev = 0, cur_n3 = 0;
     auto slot_of = [&](std::vector<int32_t> &sl, int32_t key) {
         for (size_t i = 0; i < sl.size(); ++i)
             if (sl[i] == key) return int(i);
@@ -353,8 +352,6 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
         T.ncol = ((cur.hi - cur.lo + 1 + 15) / 16) * 16;
         const int64_t M2 = int64_t(T.M) * T.M;
         T.nchunk = int32_t((M2 + x_chunk - 1) / x_chunk);
-        T.flags = cur_flags;
-        if (cur_flags & 1) return "tcgen05 tiles need n1 >= 0";
         if (T.ncol > kTcMaxCols || T.nslot > kTcMaxSlots || T.nrow > kTcRows || tc_ring(T.ncol, T.nslot) == 0)
             return "tcgen05 tile limits";
         // rows in order of their D1 field, then D2 field, and the staged
@@ -365,8 +362,10 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
             const int a1 = G.n1 < 0 ? -G.n1 : G.n1, a2 = G.n2 < 0 ? -G.n2 : G.n2;
             return std::make_pair((a1 << 8) | rw.r1, (a2 << 8) | rw.r2);
         };
-        std::stable_sort(cur.rows.begin(), cur.rows.end(),
-                         [&](const auto &x, const auto &y) { return keys(x) < keys(y); });
+        auto flags_of = [&](const std::pair<int32_t, int32_t> &gr) { return gflags(P.groups[gr.first]); };
+        std::stable_sort(cur.rows.begin(), cur.rows.end(), [&](const auto &x, const auto &y) {
+            return std::make_pair(flags_of(x), keys(x)) < std::make_pair(flags_of(y), keys(y));
+        });
         cur.slots.clear();
         for (auto &gr : cur.rows) {
             const auto k = keys(gr);
@@ -379,7 +378,18 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
             key1.push_back(keys(gr).first);
             key2.push_back(keys(gr).second);
         }
-        const LaneOrder lanes = arrange_lanes(key1, key2);
+        LaneOrder lanes;
+        int nlane = 0;                               // lanes in use (whole warps)
+        T.flags = flags_of(cur.rows[0]);
+        for (size_t i = 0, j; i < cur.rows.size(); i = j) {
+            const int fl = flags_of(cur.rows[i]);
+            if (fl & 1) return "tcgen05 tiles need n1 >= 0";
+            if (fl != T.flags) T.flags = kTcMixed;
+            for (j = i; j < cur.rows.size() && flags_of(cur.rows[j]) == fl; ++j) {}
+            if (nlane + int(j - i + 31) / 32 * 32 > kTcRows) return "tcgen05 tile lanes";
+            const int end = arrange_lanes(key1, key2, int(i), int(j), nlane, lanes);
+            for (; nlane < end; nlane += 32) T.qflags[nlane / 32] = uint8_t(fl);
+        }
         // Bank groups: a 16-byte load of slot s falls in bank group s % 8
         // (slot stride 272 bytes), and the lanes of a pass (8, or 16 that pair
         // up) that read different slots of one group are served one after
@@ -393,7 +403,7 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
         {
             std::vector<std::vector<int>> adj(ns);
             for (int side = 0; side < 2; ++side)
-                for (int g0 = 0; g0 < kTcRows;) {
+                for (int g0 = 0; g0 < nlane;) {
                     const int np = (side ? lanes.pair2 : lanes.pair1)[g0 / 32] ? 16 : 8;
                     std::vector<int> grp;
                     for (int l = g0; l < g0 + np; ++l) {
@@ -447,63 +457,90 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
             for (int j = 0; j < rw.n; ++j) U_(cur_lev, cur_n3, rw.r3a + j) = 1;
         }
         for (int l = 0; l < kTcRows; ++l)
-            P.tc_lanes.push_back(TcLane{uint8_t(slot_of(cur.slots, key1[lanes.like[l]])),
-                                        uint8_t(slot_of(cur.slots, key2[lanes.like[l]])),
-                                        uint8_t(lanes.row[l] < 0 ? kTcNoRow : lanes.row[l]), 0});
+            P.tc_lanes.push_back(l >= nlane ? TcLane{0, 0, uint8_t(kTcNoRow), 0}
+                                            : TcLane{uint8_t(slot_of(cur.slots, key1[lanes.like[l]])),
+                                                     uint8_t(slot_of(cur.slots, key2[lanes.like[l]])),
+                                                     uint8_t(lanes.row[l] < 0 ? kTcNoRow : lanes.row[l]), 0});
         P.tc_slots.insert(P.tc_slots.end(), cur.slots.begin(), cur.slots.end());
         P.tc_mma_products += double(kTcRows) * T.ncol * double(M2);
         P.tc_tiles.push_back(T);
         cur = Cur{};
         return "";
     };
+    auto add_slot = [&](Cur &c, int32_t key) {
+        if (slot_of(c.slots, key) < 0) c.slots.push_back(key);
+    };
+    // whether a tile with this window and this many slots is within the limits
+    auto fits = [&](int lo, int hi, int nslot) {
+        return hi - lo + 1 <= kTcMaxCols && nslot <= kTcMaxSlots && tc_ring(((hi - lo + 1 + 15) / 16) * 16, nslot) > 0;
+    };
     for (int lv = 0; lv < R.ngrid; ++lv)
-        for (int n3 = 0; n3 <= nz; ++n3)
-            for (int fl = 0; fl < 8; ++fl) {
-            std::vector<int32_t> &gl = pool[(size_t(lv) * (nz + 1) + n3) * 8 + fl];
-            if (gl.empty()) continue;
-            std::stable_sort(gl.begin(), gl.end(), [&](int32_t a, int32_t b) {
-                return P.groups[a].n1 < P.groups[b].n1;
-            });
-            std::string e = close();
-            if (!e.empty()) return e;
+        for (int n3 = 0; n3 <= nz; ++n3) {
             cur_lev = lv;
             cur_n3 = n3;
-            cur_flags = fl;
-            for (int32_t g : gl) {
-                const Group &G = P.groups[g];
-                std::vector<int32_t> order(G.nrow);
-                for (int q = 0; q < G.nrow; ++q) order[q] = G.row0 + q;
-                std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
-                    const Row &X = P.rows[x], &Y = P.rows[y];
-                    const int cx = 2 * X.r3a + X.n, cy = 2 * Y.r3a + Y.n;
-                    return cx != cy ? cx < cy : X.r3a < Y.r3a;
+            std::vector<Cur> rest;                   // the last tile of every sign pattern
+            for (int fl = 0; fl < 8; ++fl) {
+                std::vector<int32_t> &gl = pool[(size_t(lv) * (nz + 1) + n3) * 8 + fl];
+                if (gl.empty()) continue;
+                std::stable_sort(gl.begin(), gl.end(), [&](int32_t a, int32_t b) {
+                    return P.groups[a].n1 < P.groups[b].n1;
                 });
-                const int a1 = G.n1 < 0 ? -G.n1 : G.n1, a2 = G.n2 < 0 ? -G.n2 : G.n2;
-                for (int32_t ri : order) {
-                    const Row &rw = P.rows[ri];
-                    if (rw.n > kTcMaxCols) return "a row's r3 run is longer than a tcgen05 window";
-                    const int k1 = (a1 << 8) | rw.r1, k2 = (a2 << 8) | rw.r2;
-                    if (!cur.rows.empty()) {
-                        const int lo = std::min(cur.lo, int(rw.r3a)), hi = std::max(cur.hi, rw.r3a + rw.n - 1);
-                        const int add = (slot_of(cur.slots, k1) < 0) + (k2 != k1 && slot_of(cur.slots, k2) < 0);
-                        const int ncol = ((hi - lo + 1 + 15) / 16) * 16;
-                        const int ns = int(cur.slots.size()) + add;
-                        if (int(cur.rows.size()) >= kTcRows || hi - lo + 1 > kTcMaxCols || ns > kTcMaxSlots ||
-                            tc_ring(ncol, ns) == 0) {
-                            e = close();
-                            if (!e.empty()) return e;
+                for (int32_t g : gl) {
+                    const Group &G = P.groups[g];
+                    std::vector<int32_t> order(G.nrow);
+                    for (int q = 0; q < G.nrow; ++q) order[q] = G.row0 + q;
+                    std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
+                        const Row &X = P.rows[x], &Y = P.rows[y];
+                        const int cx = 2 * X.r3a + X.n, cy = 2 * Y.r3a + Y.n;
+                        return cx != cy ? cx < cy : X.r3a < Y.r3a;
+                    });
+                    const int a1 = G.n1 < 0 ? -G.n1 : G.n1, a2 = G.n2 < 0 ? -G.n2 : G.n2;
+                    for (int32_t ri : order) {
+                        const Row &rw = P.rows[ri];
+                        if (rw.n > kTcMaxCols) return "a row's r3 run is longer than a tcgen05 window";
+                        const int k1 = (a1 << 8) | rw.r1, k2 = (a2 << 8) | rw.r2;
+                        if (!cur.rows.empty()) {
+                            const int lo = std::min(cur.lo, int(rw.r3a)), hi = std::max(cur.hi, rw.r3a + rw.n - 1);
+                            const int add = (slot_of(cur.slots, k1) < 0) + (k2 != k1 && slot_of(cur.slots, k2) < 0);
+                            if (int(cur.rows.size()) >= kTcRows || !fits(lo, hi, int(cur.slots.size()) + add)) {
+                                const std::string e = close();
+                                if (!e.empty()) return e;
+                            }
                         }
+                        add_slot(cur, k1);
+                        add_slot(cur, k2);
+                        cur.lo = std::min(cur.lo, int(rw.r3a));
+                        cur.hi = std::max(cur.hi, rw.r3a + rw.n - 1);
+                        cur.rows.emplace_back(g, ri);
                     }
-                    if (slot_of(cur.slots, k1) < 0) cur.slots.push_back(k1);
-                    if (slot_of(cur.slots, k2) < 0) cur.slots.push_back(k2);
-                    cur.lo = std::min(cur.lo, int(rw.r3a));
-                    cur.hi = std::max(cur.hi, rw.r3a + rw.n - 1);
-                    cur.rows.emplace_back(g, ri);
                 }
+                rest.push_back(cur);
+                cur = Cur{};
+            }
+            // the rest: as many sign patterns to a tile as fit, fullest first
+            std::stable_sort(rest.begin(), rest.end(), [](const Cur &x, const Cur &y) { return x.rows.size() > y.rows.size(); });
+            std::vector<uint8_t> done(rest.size(), 0);
+            for (size_t i = 0; i < rest.size(); ++i) {
+                if (done[i]) continue;
+                cur = rest[i];
+                int lanes = int(cur.rows.size() + 31) / 32 * 32;
+                for (size_t j = i + 1; j < rest.size(); ++j) {
+                    const int more = int(rest[j].rows.size() + 31) / 32 * 32;
+                    if (done[j] || lanes + more > kTcRows) continue;
+                    Cur both = cur;
+                    for (int32_t k : rest[j].slots) add_slot(both, k);
+                    both.lo = std::min(cur.lo, rest[j].lo);
+                    both.hi = std::max(cur.hi, rest[j].hi);
+                    if (!fits(both.lo, both.hi, int(both.slots.size()))) continue;
+                    both.rows.insert(both.rows.end(), rest[j].rows.begin(), rest[j].rows.end());
+                    cur = both;
+                    lanes += more;
+                    done[j] = 1;
+                }
+                const std::string e = close();
+                if (!e.empty()) return e;
             }
         }
-    std::string e = close();
-    if (!e.empty()) return e;
     // units: class, then biggest grids first, x chunk, tile
     for (int c = 0; c < kTcClasses; ++c) {
         P.tc_class_begin[c] = int64_t(P.tc_units.size());

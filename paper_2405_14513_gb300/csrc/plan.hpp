@@ -124,9 +124,10 @@ struct TcTile {
     int32_t slot0, nslot;      // staged D1 / D2 fields in tc_slots: (plane << 8) | ring
     int32_t n3abs, r3lo;       // B window: rings r3lo .. r3lo + ncol - 1 of plane |n3|
     int32_t ncol, nchunk;      // NC; x chunks of the M^2 grid
-    int32_t flags;             // the rows' flags (all rows of a tile share them)
-    int32_t pad;
+    int32_t flags;             // the rows' flags where all rows share them, else kTcMixed
+    uint8_t qflags[4];         // flags of the rows of lanes 32 q .. 32 q + 31
 };
+constexpr int kTcMixed = 8;
 // What tensor-memory lane `lane` of a tile does: its row of the tile (kTcNoRow:
 // none) and the two staged slots it multiplies (see arrange_lanes).
 constexpr int kTcNoRow = 255;

@@ -283,6 +283,7 @@ struct CompArgs {
     volatile int *abort;
     TcSync *sy;
     int rowb, nslot, S, nstage, ntail, spins, t, half, s1, s2;   // ntail: points of the last stage (16 or 32)
+    int flags;                 // the warp's sign pattern, -1: none of its lanes has a row
 };
 
 // Tensor-memory column of accumulator buffer 0 and the distance to buffer 1
@@ -301,7 +302,9 @@ template <int NC> __device__ constexpr uint32_t acc_step() { return tc_abuf(NC) 
 // 8 (c / 8) ..), row c % 8; this thread's pieces are i = t and t + 256
 // (i = p NC + c), fixed for the tile, so their offsets are computed once.
 // The last stage may hold 16 points (ntail); its second half is left alone.
-template <int NC, bool G1, bool G2, bool G3>
+// PATTERN: the tile's flags, or kTcMixed: each warp takes its own (uniform over
+// the warp).  A warp without rows leaves its lanes of A as they are.
+template <int NC, int PATTERN>
 __device__ __forceinline__ bool compute_loop(const CompArgs &ca, float (&acc)[NC / 2])
 {
     constexpr int NH = NC / 2;
@@ -332,7 +335,20 @@ __device__ __forceinline__ bool compute_loop(const CompArgs &ca, float (&acc)[NC
     auto form = [&](int st) -> bool {
         if (!mbar_wait_abort(&sy->full[q], ph, ca.abort, ca.spins)) return false;
         const bool whole = st + 1 < ca.nstage || ca.ntail == kTX;
-        if (whole || ca.half == 0) form_a<G1, G2, G3>(sq + uoff, sq + voff, ca.tlane + 64 * ia, ca.half);
+        if ((whole || ca.half == 0) && ca.flags >= 0) {
+            const unsigned char *u = sq + uoff, *v = sq + voff;
+            const uint32_t a = ca.tlane + 64 * ia;
+            if constexpr (PATTERN != kTcMixed) {
+                form_a<false, (PATTERN & 2) != 0, (PATTERN & 4) != 0>(u, v, a, ca.half);
+            } else {
+                switch (ca.flags) {
+                case 0: form_a<false, false, false>(u, v, a, ca.half); break;
+                case 2: form_a<false, true, false>(u, v, a, ca.half); break;
+                case 4: form_a<false, false, true>(u, v, a, ca.half); break;
+                default: form_a<false, true, true>(u, v, a, ca.half); break;
+                }
+            }
+        }
 #pragma unroll
         for (int k = 0; k < NP; ++k) {
             if (src[k] < 0) continue;
@@ -575,21 +591,22 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
     } else {
         // compute warps: the thread owns tensor-memory lane 32 (warp % 4) +
         // lane; a lane without a row repeats a neighbour's fields, and its sums
-        // go nowhere.  The loop is instantiated per sign pattern (uniform over
-        // the tile; n1 >= 0)
+        // go nowhere.  The loop is instantiated per sign pattern (n1 >= 0)
         const int quarter = warp & 3, half = warp >> 2;
         const TcLane ln = args.lanes[size_t(U.tile) * kTcRows + quarter * 32 + lane];
         const bool live = ln.row != kTcNoRow;
         TcRow R{};
         if (live) R = args.rows[T.row0 + ln.row];
         CompArgs ca{sS, sHi, sLo, tmem + (uint32_t(quarter * 32) << 16), abort, sy, rowb, nslot, S, nstage, ntail, spins,
-                    t, half, int(ln.s1), int(ln.s2)};
+                    t, half, int(ln.s1), int(ln.s2),
+                    __any_sync(0xFFFFFFFFu, live) ? int(T.qflags[quarter]) : -1};
         float acc[NC / 2];
         switch (T.flags) {
-        case 0: ok = compute_loop<NC, false, false, false>(ca, acc); break;
-        case 2: ok = compute_loop<NC, false, true, false>(ca, acc); break;
-        case 4: ok = compute_loop<NC, false, false, true>(ca, acc); break;
-        default: ok = compute_loop<NC, false, true, true>(ca, acc); break;
+        case 0: ok = compute_loop<NC, 0>(ca, acc); break;
+        case 2: ok = compute_loop<NC, 2>(ca, acc); break;
+        case 4: ok = compute_loop<NC, 4>(ca, acc); break;
+        case 6: ok = compute_loop<NC, 6>(ca, acc); break;
+        default: ok = compute_loop<NC, kTcMixed>(ca, acc); break;
         }
         if (live) {
             double *dst = args.partials + R.p0 + int64_t(U.chunk) * R.stride;
