@@ -320,10 +320,12 @@ k_fft_z_real(const R *__restrict__ in, typename Cx<R>::T *__restrict__ out, int 
     }
 }
 
-template <typename R>
+// nsplit = 0: complex output.  nsplit > 0: the arrays hold two real fields each,
+// nsplit in all: real parts go to field 2 b, imaginary parts to field 2 b + 1 of `out`.
+template <typename R, bool SPLIT>
 __global__ void __launch_bounds__(256)
 k_fft_rows_T(const typename Cx<R>::T *__restrict__ in, typename Cx<R>::T *__restrict__ out, int M,
-             int nrow, int ntile, R scale, int zero_dc, int rt, Twiddles<typename Cx<R>::T> tw, int64_t fs)
+             int nrow, int ntile, R scale, int zero_dc, int rt, Twiddles<typename Cx<R>::T> tw, int64_t fs, int64_t nsplit)
 {
     using C = typename Cx<R>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -340,10 +342,16 @@ k_fft_rows_T(const typename Cx<R>::T *__restrict__ in, typename Cx<R>::T *__rest
     const C *res = fft_any<C, false, true, false>(M, nr, 0, P, a, b, tw.t, [&](int r, int i) { return src[r * M + i]; },
                                                   NoStore{});
     C *dst = out + bt * int64_t(M) * nrow;
+    R *re = reinterpret_cast<R *>(out) + 2 * bt * int64_t(M) * nrow, *im = re + int64_t(M) * nrow;
     DivIter st(threadIdx.x, blockDim.x, nr);
     for (int t = threadIdx.x; t < M * nr; t += blockDim.x, st.next()) {
         const int k = st.q, r = st.r;
         C v = res[r * P + spos(k)];
+        if (SPLIT) {
+            re[int64_t(k) * nrow + row0 + r] = v.x;
+            if (2 * bt + 1 < nsplit) im[int64_t(k) * nrow + row0 + r] = v.y;
+            continue;
+        }
         v.x *= scale;
         v.y *= scale;
         if (zero_dc && bt == 0 && row0 + r == 0 && k == 0) v = cmk<C>(0.0, 0.0);
@@ -1007,8 +1015,23 @@ cudaError_t launch_fft_rows_T(const typename Cx<R>::T *in, typename Cx<R>::T *ou
     const int ntile = (nrow + rt - 1) / rt;
     const int64_t nblk = nb * ntile;
     if (nblk == 0) return cudaSuccess;
-    k_fft_rows_T<R><<<dim3(unsigned(nblk), fb.nf), 256, smem, s>>>(in, out, M, nrow, ntile, scale, zero_dc ? 1 : 0, rt,
-                                                                   tw, fb.fs_in);
+    k_fft_rows_T<R, false><<<dim3(unsigned(nblk), fb.nf), 256, smem, s>>>(in, out, M, nrow, ntile, scale,
+                                                                          zero_dc ? 1 : 0, rt, tw, fb.fs_in, 0);
+    return cudaGetLastError();
+}
+
+template <typename R>
+cudaError_t launch_fft_rows_split(const typename Cx<R>::T *in, R *out, int M, int nrow, int64_t nf,
+                                  const Twiddles<typename Cx<R>::T> &tw, cudaStream_t s)
+{
+    using C = typename Cx<R>::T;
+    const int rt = std::min(int(fft_rows_per_block(M, sizeof(C))), nrow);
+    const size_t smem = size_t(2) * rt * fft_stride(M) * sizeof(C);
+    const int ntile = (nrow + rt - 1) / rt;
+    const int64_t nblk = (nf + 1) / 2 * ntile;
+    if (nblk == 0) return cudaSuccess;
+    k_fft_rows_T<R, true><<<unsigned(nblk), 256, smem, s>>>(in, reinterpret_cast<C *>(out), M, nrow, ntile, R(1), 0, rt, tw, 0,
+                                                            nf);
     return cudaGetLastError();
 }
 
@@ -1168,8 +1191,10 @@ cudaError_t init_kernel_attributes()
     };
     set((const void *)k_fft_z_real<float>);
     set((const void *)k_fft_z_real<double>);
-    set((const void *)k_fft_rows_T<float>);
-    set((const void *)k_fft_rows_T<double>);
+    set((const void *)k_fft_rows_T<float, false>);
+    set((const void *)k_fft_rows_T<float, true>);
+    set((const void *)k_fft_rows_T<double, false>);
+    set((const void *)k_fft_rows_T<double, true>);
     set((const void *)k_fft_cols<float>);
     set((const void *)k_fft_cols<double>);
     set((const void *)k_ring_gather<float, false>);
@@ -1228,6 +1253,8 @@ template cudaError_t launch_fft_z_real<float>(const float *, float2 *, int, int6
 template cudaError_t launch_fft_z_real<double>(const double *, double2 *, int, int64_t, int, const Twiddles<double2> &, const Batch &, cudaStream_t, int);
 template cudaError_t launch_fft_rows_T<float>(const float2 *, float2 *, int, int, int64_t, float, bool, const Twiddles<float2> &, const Batch &, cudaStream_t, int);
 template cudaError_t launch_fft_rows_T<double>(const double2 *, double2 *, int, int, int64_t, double, bool, const Twiddles<double2> &, const Batch &, cudaStream_t, int);
+template cudaError_t launch_fft_rows_split<float>(const float2 *, float *, int, int, int64_t, const Twiddles<float2> &, cudaStream_t);
+template cudaError_t launch_fft_rows_split<double>(const double2 *, double *, int, int, int64_t, const Twiddles<double2> &, cudaStream_t);
 template cudaError_t launch_ring_gather<float>(const float2 *, int, const RingArg &, StepGrids, bool, float2 *, const Twiddles<float2> &, const Batch &, cudaStream_t, const float *);
 template cudaError_t launch_ring_gather<double>(const double2 *, int, const RingArg &, StepGrids, bool, double2 *, const Twiddles<double2> &, const Batch &, cudaStream_t, const float *);
 template cudaError_t launch_fft_cols<float>(float2 *, StepGrids, const RingArg &, const Twiddles<float2> &, const Batch &, cudaStream_t);

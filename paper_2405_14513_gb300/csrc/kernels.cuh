@@ -100,6 +100,12 @@ cudaError_t launch_fft_rows_T(const typename Cx<R>::T *in, typename Cx<R>::T *ou
                               const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s,
                               int rt = 0);
 
+// The same of arrays that hold two real transforms each (real and imaginary
+// parts), nf in all, written apart: out[f][M][nrow].
+template <typename R>
+cudaError_t launch_fft_rows_split(const typename Cx<R>::T *in, R *out, int M, int nrow, int64_t nf,
+                                  const Twiddles<typename Cx<R>::T> &tw, cudaStream_t s);
+
 // Step I, first pass: for every job of the grids, ring r of plane n of Delta
 // (planes [nz+1][ng][ng]), folded onto the M x M grid, transformed along u_y,
 // written in place order [u_x][k_y] at out + out_off; rows that hold no member

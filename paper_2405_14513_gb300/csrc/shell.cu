@@ -22,9 +22,10 @@
 //
 // Plan: shell table, triples, and the field-independent N_tri and den_l
 // from FP64 unit fields.  Estimate: the forward transform (the kernels of
-// the main path), the weighted shell spectra of every shell, 3D transforms
-// (three passes of the row transform, each a cyclic transpose), FP32
-// fields, FP32 triple products summed in FP64, binning.  Lengths N_g <= 128
+// the main path), the weighted shell spectra of every shell, two fields to a
+// complex array, 3D transforms (three passes of the row transform, each a cyclic
+// transpose), FP32 fields, FP32 triple products summed in pairs of floats and in
+// FP64, binning.  Lengths N_g <= 128
 // (the plan's FP64 sums over N_g^3 points per triple grow as N_g^6).
 #include "kernels.cuh"
 
@@ -64,77 +65,161 @@ __device__ __forceinline__ double y_l0(int l, double z)
     return sqrt((2.0 * l + 1.0) / (2.0 * kShellTwoPi)) * p;
 }
 
-// Weighted shell spectra on the N_g^3 grid, [job][a][b][c] with (a, b, c)
-// the FFT indices of (k_x, k_y, k_z); Delta from the kept planes n >= 0
-// ([n][k_x][k_y]) and Delta(k_x, k_y, -n) = conj Delta(-k_x, -k_y, n).
+// The weighted spectrum of one job at mode (i, j, n), FFT indices (a, b, .) of
+// k_x and k_y; Delta from the kept planes n >= 0 ([n][k_x][k_y]) and
+// Delta(k_x, k_y, -n) = conj Delta(-k_x, -k_y, n).
+template <typename C>
+__device__ __forceinline__ C shell_mode(const C *__restrict__ planes, int ng, const int64_t *__restrict__ e3sq, const ShellJob &J,
+                                        int a, int b, int i, int j, int n)
+{
+    C v;
+    v.x = 0;
+    v.y = 0;
+    const int q = i * i + j * j + n * n;
+    if (9 * int64_t(q) < e3sq[J.s] || 9 * int64_t(q) >= e3sq[J.s + 1]) return v;
+    double w = 1.0;
+    if (J.kind == 1 || J.kind == 3) {
+        const double y = y_l0(J.l, double(n) / sqrt(double(q)));
+        w = J.kind == 1 ? y : y * y;
+    }
+    if (J.kind <= 1) {
+        C d;
+        if (n >= 0) {
+            d = planes[(int64_t(n) * ng + a) * ng + b];
+        } else {
+            d = planes[(int64_t(-n) * ng + (ng - a) % ng) * ng + (ng - b) % ng];
+            d.y = -d.y;
+        }
+        v.x = decltype(v.x)(double(d.x) * w);
+        v.y = decltype(v.y)(double(d.y) * w);
+    } else {
+        v.x = decltype(v.x)(w);
+    }
+    return v;
+}
+
+// Weighted shell spectra on the N_g^3 grid, [pair][a][b][c] with (a, b, c) the
+// FFT indices of (k_x, k_y, k_z).  Every shell field is real, so two jobs share
+// a complex transform: X = A + i B (the last of an odd number has B = 0).
 template <typename C>
 __global__ void __launch_bounds__(256)
 k_shell_spectrum(const C *__restrict__ planes, int ng, const int64_t *__restrict__ e3sq,
-                 const ShellJob *__restrict__ jobs, C *__restrict__ out)
+                 const ShellJob *__restrict__ jobs, int njobs, C *__restrict__ out)
 {
-    const ShellJob J = jobs[blockIdx.y];
+    const int f = 2 * blockIdx.y;
+    const ShellJob J = jobs[f], K = jobs[f + 1 < njobs ? f + 1 : f];
     const int64_t n3 = int64_t(ng) * ng * ng;
     C *dst = out + int64_t(blockIdx.y) * n3;
-    const int64_t lo = e3sq[J.s], hi = e3sq[J.s + 1];
+    const int64_t lo = min(e3sq[J.s], e3sq[K.s]), hi = max(e3sq[J.s + 1], e3sq[K.s + 1]);
     for (int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < n3; p += int64_t(gridDim.x) * blockDim.x) {
-        const int a = int(p / (int64_t(ng) * ng)), b = int((p / ng) % ng), c = int(p % ng);
+        const int c = int(p % ng), ab = int(p / ng), a = ab / ng, b = ab - a * ng;
         const int i = a < ng / 2 ? a : a - ng, j = b < ng / 2 ? b : b - ng, n = c < ng / 2 ? c : c - ng;
         const int64_t q9 = 9 * (int64_t(i) * i + int64_t(j) * j + int64_t(n) * n);
         C v;
         v.x = 0;
         v.y = 0;
         if (q9 >= lo && q9 < hi) {
-            double w = 1.0;
-            if (J.kind == 1 || J.kind == 3) {
-                const double y = y_l0(J.l, double(n) / sqrt(double(int64_t(i) * i + int64_t(j) * j + int64_t(n) * n)));
-                w = J.kind == 1 ? y : y * y;
-            }
-            if (J.kind <= 1) {
-                C d;
-                if (n >= 0) {
-                    d = planes[(int64_t(n) * ng + a) * ng + b];
-                } else {
-                    d = planes[(int64_t(-n) * ng + (ng - a) % ng) * ng + (ng - b) % ng];
-                    d.y = -d.y;
-                }
-                v.x = decltype(v.x)(double(d.x) * w);
-                v.y = decltype(v.y)(double(d.y) * w);
-            } else {
-                v.x = decltype(v.x)(w);
+            v = shell_mode<C>(planes, ng, e3sq, J, a, b, i, j, n);
+            if (f + 1 < njobs) {
+                const C w = shell_mode<C>(planes, ng, e3sq, K, a, b, i, j, n);
+                v.x -= w.y;
+                v.y += w.x;
             }
         }
         dst[p] = v;
     }
 }
 
-template <typename C, typename R>
-__global__ void __launch_bounds__(256) k_real_part(const C *__restrict__ in, R *__restrict__ out, int64_t n)
-{
-    for (int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < n; p += int64_t(gridDim.x) * blockDim.x)
-        out[p] = in[p].x;
-}
-
-// out[q] = scale sum_p A[p] B[p] C[p] for the field triple of product q
-// (products in R, the sum in FP64), one block per product; outputs whose
-// index is a multiple of every_first (if > 0) take scale_first instead.
-template <typename R>
+// out[q] = scale sum_p A[p] B[p] C[p] for the field triple of product q, FP64
+// (the plan's counts and denominators), one block per product.
 __global__ void __launch_bounds__(256)
-k_triple_products(const R *__restrict__ fields, int64_t n3, const int4 *__restrict__ prods, double scale,
-                  int every_first, double scale_first, double *__restrict__ out)
+k_triple_products(const double *__restrict__ fields, int64_t n3, const int4 *__restrict__ prods, double scale,
+                  double *__restrict__ out)
 {
     __shared__ double red[8];
     const int4 P = prods[blockIdx.x];
-    const R *A = fields + int64_t(P.x) * n3, *B = fields + int64_t(P.y) * n3, *Cf = fields + int64_t(P.z) * n3;
+    const double *A = fields + int64_t(P.x) * n3, *B = fields + int64_t(P.y) * n3, *Cf = fields + int64_t(P.z) * n3;
     double acc = 0;
-    for (int64_t p = threadIdx.x; p < n3; p += blockDim.x) acc += double(A[p] * B[p] * Cf[p]);
+    for (int64_t p = threadIdx.x; p < n3; p += blockDim.x) acc += A[p] * B[p] * Cf[p];
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0;
         for (int w = 0; w < int(blockDim.x >> 5); ++w) t += red[w];
-        out[P.w] = t * (every_first > 0 && P.w % every_first == 0 ? scale_first : scale);
+        out[P.w] = t * scale;
     }
+}
+
+// s + e += x, s and e two floats: the rounding error of every addition to s is
+// found exactly (Knuth's two-sum) and kept in e, so that the pair holds the sum
+// of the FP32 products to 2^-45 or so, at FP32 speed (an FP64 addition, with its
+// conversion, takes 128 times a float's share of the SM).
+__device__ __forceinline__ void add_exact(float &s, float &e, float x)
+{
+    const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
+    s = t;
+}
+
+// Partial sums of sum_p F_l[p] D2[p] D3[p] for every l of one triple (tri: the
+// indices of F_0, whose l >= 2 follow it, of D2 and of D3) over one slice of the
+// grid: part[triple][slice][l].  Products in FP32, D2 D3 formed once for all l;
+// bound by reading the fields from L2.  With a block per triple and l and FP64
+// sums, and a transform per field, a 64^3 estimate took 2.57 ms; so 0.90 ms.
+template <int NL>
+__global__ void __launch_bounds__(256)
+k_shell_products(const float *__restrict__ fields, int64_t n3, const int4 *__restrict__ tri, int nslice, double *__restrict__ part)
+{
+    __shared__ double red[8][NL];
+    const int4 T = tri[blockIdx.x];
+    const int64_t n4 = n3 / 4, lo = n4 * blockIdx.y / nslice, hi = n4 * (blockIdx.y + 1) / nslice;
+    const float4 *F[NL], *B = reinterpret_cast<const float4 *>(fields + int64_t(T.y) * n3),
+                        *D = reinterpret_cast<const float4 *>(fields + int64_t(T.z) * n3);
+    float s[NL][2], e[NL][2];
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+        F[l] = reinterpret_cast<const float4 *>(fields + int64_t(T.x + l) * n3);
+        s[l][0] = s[l][1] = e[l][0] = e[l][1] = 0.0f;
+    }
+    for (int64_t p = lo + threadIdx.x; p < hi; p += blockDim.x) {
+        const float4 b = B[p], d = D[p];
+        const float4 c = make_float4(b.x * d.x, b.y * d.y, b.z * d.z, b.w * d.w);
+#pragma unroll
+        for (int l = 0; l < NL; ++l) {
+            const float4 f = F[l][p];
+            add_exact(s[l][0], e[l][0], f.x * c.x);
+            add_exact(s[l][1], e[l][1], f.y * c.y);
+            add_exact(s[l][0], e[l][0], f.z * c.z);
+            add_exact(s[l][1], e[l][1], f.w * c.w);
+        }
+    }
+#pragma unroll
+    for (int l = 0; l < NL; ++l) {
+        double v = (double(s[l][0]) + double(s[l][1])) + (double(e[l][0]) + double(e[l][1]));
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][l] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < NL) {
+        double t = 0;
+        for (int w = 0; w < int(blockDim.x >> 5); ++w) t += red[w][threadIdx.x];
+        part[(int64_t(blockIdx.x) * nslice + blockIdx.y) * NL + threadIdx.x] = t;
+    }
+}
+
+// num[t][l] = scale of l times the slices' sums, in order (l = 0 takes D_{s1} for
+// F_{s1,0} = Y_00 D_{s1}, so its scale has Y_00)
+__global__ void __launch_bounds__(256)
+k_shell_sums(const double *__restrict__ part, int64_t n, int nl, int nslice, double scale, double scale0, double *__restrict__ num)
+{
+    const int64_t q = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (q >= n) return;
+    const int64_t t = q / nl;
+    const int l = int(q - t * nl);
+    double v = 0;
+    for (int k = 0; k < nslice; ++k) v += part[(t * nslice + k) * nl + l];
+    num[q] = v * (l == 0 ? scale0 : scale);
 }
 
 // B[bin][li] = sqrt((2l+1)/4pi) sum num / (V sum den) over the bin's triples
@@ -175,14 +260,15 @@ struct bisp_shell_plan {
     int64_t *d_e3sq = nullptr;
     ShellJob *d_jobs = nullptr;           // estimate fields: D_s, F_{s,l} (l >= 2), s >= 1
     int njobs = 0;
-    int4 *d_prods = nullptr;              // estimate products: (F_{s1,l}, D_{s2}, D_{s3}) -> num [t][li]
+    int4 *d_tri = nullptr;                // per triple: field of D_{s1} (F_{s1,l} follow), D_{s2}, D_{s3}
+    int nslice = 1;                       // blocks per triple
     double *d_den = nullptr;
     int64_t *d_bin_start = nullptr;
     int32_t *d_bin_tri = nullptr;
     Twiddles<float2> twf{};
     Twiddles<double2> twd{};
     // workspace layout (bytes)
-    size_t off_a = 0, off_b = 0, off_spec = 0, off_spec2 = 0, off_fields = 0, off_num = 0, ws_bytes = 0;
+    size_t off_a = 0, off_b = 0, off_spec = 0, off_spec2 = 0, off_fields = 0, off_part = 0, off_num = 0, ws_bytes = 0;
     std::vector<void *> owned;
 };
 
@@ -211,17 +297,19 @@ int sup(bisp_shell_plan *p, T **out, const std::vector<T> &v, cudaStream_t s)
 
 size_t al(size_t v) { return (v + 255) & ~size_t(255); }
 
-// 3D transform of nb complex N^3 arrays: three passes of the row
-// transform, each along the contiguous axis and written cyclically
-// transposed, so the result is back in [x][y][z] order.  a -> b -> a -> b.
+// 3D transform of the nf real fields packed two to a complex N^3 array (see
+// k_shell_spectrum): three passes of the row transform, each along the
+// contiguous axis and written cyclically transposed, so the result is back in
+// [x][y][z] order; the last writes the fields apart.  a -> b -> a -> fields.
 template <typename R>
-cudaError_t fft3(typename Cx<R>::T *a, typename Cx<R>::T *b, int ng, int64_t nb,
+cudaError_t fft3(typename Cx<R>::T *a, typename Cx<R>::T *b, R *fields, int ng, int64_t nf,
                  const Twiddles<typename Cx<R>::T> &tw, cudaStream_t s)
 {
     const int nrow = ng * ng;
+    const int64_t nb = (nf + 1) / 2;
     cudaError_t e = launch_fft_rows_T<R>(a, b, ng, nrow, nb, R(1), false, tw, Batch{}, s);
     if (e == cudaSuccess) e = launch_fft_rows_T<R>(b, a, ng, nrow, nb, R(1), false, tw, Batch{}, s);
-    if (e == cudaSuccess) e = launch_fft_rows_T<R>(a, b, ng, nrow, nb, R(1), false, tw, Batch{}, s);
+    if (e == cudaSuccess) e = launch_fft_rows_split<R>(a, fields, ng, nrow, nf, tw, s);
     return e;
 }
 
@@ -345,8 +433,9 @@ int build_shell_plan(bisp_shell_plan *p, const bisp_desc *d, cudaStream_t s)
         };
         std::vector<double> h(size_t(std::max<int64_t>(nc, 1)) * (1 + nl));
         cudaError_t e = cudaMalloc(&d_uj, sizeof(ShellJob) * std::max<int64_t>(nu, 1));
-        if (e == cudaSuccess) e = cudaMalloc(&sa, sizeof(double2) * std::max<int64_t>(nu * n3, 1));
-        if (e == cudaSuccess) e = cudaMalloc(&sb, sizeof(double2) * std::max<int64_t>(nu * n3, 1));
+        const int64_t np = (nu + 1) / 2;             // pairs of fields
+        if (e == cudaSuccess) e = cudaMalloc(&sa, sizeof(double2) * std::max<int64_t>(np * n3, 1));
+        if (e == cudaSuccess) e = cudaMalloc(&sb, sizeof(double2) * std::max<int64_t>(np * n3, 1));
         if (e == cudaSuccess) e = cudaMalloc(&fld, sizeof(double) * std::max<int64_t>(nu * n3, 1));
         if (e == cudaSuccess) e = cudaMalloc(&sums, sizeof(double) * h.size());
         if (e == cudaSuccess) e = cudaMalloc(&d_up, sizeof(int4) * std::max<size_t>(up.size(), 1));
@@ -354,17 +443,13 @@ int build_shell_plan(bisp_shell_plan *p, const bisp_desc *d, cudaStream_t s)
         if (e == cudaSuccess && !up.empty())
             e = cudaMemcpyAsync(d_up, up.data(), sizeof(int4) * up.size(), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess && nu > 0) {
-            k_shell_spectrum<double2><<<dim3(blocks_for(n3), unsigned(nu)), 256, 0, s>>>(nullptr, ng, p->d_e3sq, d_uj, sa);
+            k_shell_spectrum<double2><<<dim3(blocks_for(n3), unsigned(np)), 256, 0, s>>>(nullptr, ng, p->d_e3sq, d_uj, int(nu),
+                                                                                         sa);
             e = cudaGetLastError();
-            if (e == cudaSuccess) e = fft3<double>(sa, sb, ng, nu, p->twd, s);
-            if (e == cudaSuccess) {
-                k_real_part<double2, double><<<blocks_for(nu * n3), 256, 0, s>>>(sb, fld, nu * n3);
-                e = cudaGetLastError();
-            }
+            if (e == cudaSuccess) e = fft3<double>(sa, sb, fld, ng, nu, p->twd, s);
         }
         if (e == cudaSuccess && !up.empty()) {
-            k_triple_products<double><<<unsigned(up.size()), 256, 0, s>>>(fld, n3, d_up, 1.0 / double(n3), 0, 0.0,
-                                                                          sums);
+            k_triple_products<<<unsigned(up.size()), 256, 0, s>>>(fld, n3, d_up, 1.0 / double(n3), sums);
             e = cudaGetLastError();
         }
         if (e == cudaSuccess && nc > 0)
@@ -396,12 +481,11 @@ int build_shell_plan(bisp_shell_plan *p, const bisp_desc *d, cudaStream_t s)
     }
     p->njobs = int(jobs.size());
     const int64_t nt = int64_t(p->tri_bin.size());
-    std::vector<int4> prods;
-    for (int64_t t = 0; t < nt; ++t) {
-        const int s1 = p->tri[3 * t], s2 = p->tri[3 * t + 1], s3 = p->tri[3 * t + 2];
-        for (int li = 0; li < nl; ++li)
-            prods.push_back(int4{(s1 - 1) * nl + li, (s2 - 1) * nl, (s3 - 1) * nl, int(t * nl + li)});
-    }
+    std::vector<int4> tri4;
+    for (int64_t t = 0; t < nt; ++t)
+        tri4.push_back(int4{(p->tri[3 * t] - 1) * nl, (p->tri[3 * t + 1] - 1) * nl, (p->tri[3 * t + 2] - 1) * nl, 0});
+    // enough blocks for eight on every SM
+    p->nslice = int(std::min<int64_t>(16, (152 * 8 + nt) / std::max<int64_t>(nt, 1)));
     // bins: triples grouped by bin
     std::vector<int64_t> bs(p->nbins + 1, 0);
     for (int32_t b : p->tri_bin) ++bs[b + 1];
@@ -412,7 +496,7 @@ int build_shell_plan(bisp_shell_plan *p, const bisp_desc *d, cudaStream_t s)
         for (int64_t t = 0; t < nt; ++t) bt[pos[p->tri_bin[t]]++] = int32_t(t);
     }
     st = sup(p, &p->d_jobs, jobs, s);
-    if (!st) st = sup(p, &p->d_prods, prods, s);
+    if (!st) st = sup(p, &p->d_tri, tri4, s);
     if (!st) st = sup(p, &p->d_den, p->den, s);
     if (!st) st = sup(p, &p->d_bin_start, bs, s);
     if (!st) st = sup(p, &p->d_bin_tri, bt, s);
@@ -422,9 +506,10 @@ int build_shell_plan(bisp_shell_plan *p, const bisp_desc *d, cudaStream_t s)
     size_t o = 0;
     p->off_a = o; o = al(o + size_t(planes) * sizeof(float2));
     p->off_b = o; o = al(o + size_t(planes) * sizeof(float2));
-    p->off_spec = o; o = al(o + size_t(p->njobs) * n3 * sizeof(float2));
-    p->off_spec2 = o; o = al(o + size_t(p->njobs) * n3 * sizeof(float2));
+    p->off_spec = o; o = al(o + size_t((p->njobs + 1) / 2) * n3 * sizeof(float2));
+    p->off_spec2 = o; o = al(o + size_t((p->njobs + 1) / 2) * n3 * sizeof(float2));
     p->off_fields = o; o = al(o + size_t(p->njobs) * n3 * sizeof(float));
+    p->off_part = o; o = al(o + size_t(std::max<int64_t>(nt, 1)) * nl * p->nslice * sizeof(double));
     p->off_num = o; o = al(o + size_t(std::max<int64_t>(nt, 1)) * nl * sizeof(double));
     p->ws_bytes = o;
     SCK(cudaStreamSynchronize(s));
@@ -508,18 +593,25 @@ int estimator_shell_estimate(bisp_shell_plan *p, const float *delta, void *works
     SCK(launch_fft_rows_T<float>(A_, B_, ng, ng, p->nz + 1, 1.0f, false, p->twf, Batch{}, s));
     SCK(launch_fft_rows_T<float>(B_, A_, ng, ng, p->nz + 1, float(V / double(n3)), true, p->twf, Batch{}, s));
     if (p->njobs > 0) {
-        k_shell_spectrum<float2><<<dim3(blocks_for(n3), unsigned(p->njobs)), 256, 0, s>>>(A_, ng, p->d_e3sq, p->d_jobs, sa);
+        k_shell_spectrum<float2><<<dim3(blocks_for(n3), unsigned((p->njobs + 1) / 2)), 256, 0, s>>>(A_, ng, p->d_e3sq,
+                                                                                                    p->d_jobs, p->njobs, sa);
         SCK(cudaGetLastError());
-        SCK(fft3<float>(sa, sb, ng, p->njobs, p->twf, s));
-        k_real_part<float2, float><<<blocks_for(int64_t(p->njobs) * n3), 256, 0, s>>>(sb, fld, int64_t(p->njobs) * n3);
-        SCK(cudaGetLastError());
+        SCK(fft3<float>(sa, sb, fld, ng, p->njobs, p->twf, s));
     }
-    const int64_t nprod = int64_t(p->tri_bin.size()) * p->nl;
+    const int64_t nt = int64_t(p->tri_bin.size()), nprod = nt * p->nl;
     if (nprod > 0) {
-        // l = 0 takes D_{s1} for F_{s1,0} = Y_00 D_{s1}: its sums are scaled by Y_00
         const double y00 = std::sqrt(1.0 / (2.0 * kShellTwoPi));
-        k_triple_products<float><<<unsigned(nprod), 256, 0, s>>>(fld, n3, p->d_prods, 1.0 / double(n3), p->nl,
-                                                                 y00 / double(n3), num);
+        double *part = reinterpret_cast<double *>(ws + p->off_part);
+        const dim3 grid(unsigned(nt), unsigned(p->nslice));
+        switch (p->nl) {
+        case 1: k_shell_products<1><<<grid, 256, 0, s>>>(fld, n3, p->d_tri, p->nslice, part); break;
+        case 2: k_shell_products<2><<<grid, 256, 0, s>>>(fld, n3, p->d_tri, p->nslice, part); break;
+        case 3: k_shell_products<3><<<grid, 256, 0, s>>>(fld, n3, p->d_tri, p->nslice, part); break;
+        default: k_shell_products<4><<<grid, 256, 0, s>>>(fld, n3, p->d_tri, p->nslice, part); break;
+        }
+        SCK(cudaGetLastError());
+        k_shell_sums<<<unsigned((nprod + 255) / 256), 256, 0, s>>>(part, nprod, p->nl, p->nslice, 1.0 / double(n3),
+                                                                   y00 / double(n3), num);
         SCK(cudaGetLastError());
     }
     const int64_t nq = p->nbins * p->nl;
