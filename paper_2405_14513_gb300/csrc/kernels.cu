@@ -484,11 +484,13 @@ k_ring_gather(const typename Cx<R>::T *__restrict__ planes, int ng, const __grid
 }
 
 // Step I second pass: transforms along the first axis of each job's M x M
-// field (rows u_x of the gather's output), in place: a strip of w columns
-// k_y per block, read (by the first stage) and written (by the last) in runs
-// of w consecutive elements of every row, so the D field comes out as
-// [k_x][k_y].  The threads run across the strip first: the runs are whole
-// 32-byte sectors for w >= 4, and the lanes of a warp take few different twiddles.
+// field (rows u_x of the gather's output), in place: a strip of w columns k_y
+// per block, of all the columns of the grid's jobs one after another (a block of a
+// small grid takes several jobs' columns), read (by the first stage) and written
+// (by the last) in runs of consecutive elements of every row, so the D field
+// comes out as [k_x][k_y].  The threads run across the strip first: the runs are
+// whole 32-byte sectors for w >= 4, the lanes of a warp take few different
+// twiddles, and a thread's column is the same throughout.
 template <typename R>
 __global__ void __launch_bounds__(256)
 k_fft_cols(typename Cx<R>::T *__restrict__ out, const __grid_constant__ StepGrids gs,
@@ -502,15 +504,16 @@ k_fft_cols(typename Cx<R>::T *__restrict__ out, const __grid_constant__ StepGrid
     const int P = fft_stride(M);
     C *a = reinterpret_cast<C *>(smem_raw);
     C *b = a + w * P;
-    const int blk = int(blockIdx.x - gr.blk0), jb = blk / gr.ntile;
+    const int64_t c0 = int64_t(blockIdx.x - gr.blk0) * w, cols = gr.njobs * M;
+    const int nc = int(min(int64_t(w), cols - c0));
+    // this thread's column (of the grid's jobs' M each)
+    const int64_t c = min(c0 + (threadIdx.x & (w - 1)), cols - 1);
+    const int64_t jb = c / M;
     const Job J = gr.jobs[jb];
-    const int c0 = (blk - jb * gr.ntile) * w;
-    const int nc = min(w, M - c0);
     const int mc = rings.maxc[J.r];             // rows mc < i < M - mc hold no ring member: zero
-    C *f = out + J.out_off + c0;
-    auto load = [&](int c, int i) { return (i <= mc || i >= M - mc) ? f[i * M + c] : cmk<C>(0.0, 0.0); };
-    fft_any<C, true, false, true>(M, nc, gr.lgw, P, a, b, tw.t, load,
-                                  [&](int c, int k, const C &v) { f[k * M + c] = v; });
+    C *f = out + J.out_off + (c - jb * M);
+    auto load = [&](int, int i) { return (i <= mc || i >= M - mc) ? f[i * M] : cmk<C>(0.0, 0.0); };
+    fft_any<C, true, false, true>(M, nc, gr.lgw, P, a, b, tw.t, load, [&](int, int k, const C &v) { f[k * M] = v; });
 }
 
 // ---------------------------------------------------------------------------
@@ -731,17 +734,22 @@ k_step2(StepIIArgs args, int64_t unit0, const typename Cx<R>::T *__restrict__ ds
 
 template <typename A>
 __global__ void __launch_bounds__(256)
-k_reduce(const Group *__restrict__ groups, const double *__restrict__ partials, int ng, double *__restrict__ S,
-         int64_t fs)
+k_reduce(const Group *__restrict__ groups, int64_t ngroups, const double *__restrict__ partials, int ng,
+         double *__restrict__ S, int64_t fs)
 {
     partials = field_ptr(partials, fs);
     S = field_ptr(S, fs);
-    const Group G = groups[blockIdx.x];
+    // one warp per group: groups hold 14 (64^3) to 140 (512^3) combinations
+    const int64_t g = int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5);
+    if (g >= ngroups) return;
+    const Group G = groups[g];
     const double f = double(ng) / double(G.M);
     const A scale = A(f * f);
-    for (int j = threadIdx.x; j < G.ncombo; j += blockDim.x) {
+    for (int j = threadIdx.x & 31; j < G.ncombo; j += 32) {
+        const double *p = partials + G.part0 + j;
         A s = A(0);
-        for (int k = 0; k < G.nchunk; ++k) s += A(partials[G.part0 + int64_t(k) * G.ncombo + j]);
+#pragma unroll 4
+        for (int k = 0; k < G.nchunk; ++k) s += A(p[int64_t(k) * G.ncombo]);
         S[G.c0 + j] = double(s * scale);
     }
 }
@@ -901,29 +909,38 @@ k_epi_part(int mode, const Record *__restrict__ rec, const RecordF *__restrict__
     if ((lane & (32 / P2 - 1)) == 0 && idx < NLM) partial[ch * NLM + idx] = double(red[0]) * (WIDEN ? 0x1p448 : 1.0);
 }
 
-// One thread per bin and moment: the bin's chunks' partial sums in chunk
-// order, then (mode 0) the ratio of Eq. bs_lm2_1 or (mode 1) the sum itself.
+// One block per bin: 128 / P2 threads per moment (P2 = NLM rounded up to a power
+// of two) take the bin's chunks in turn, and their partial sums are added in
+// order; then (mode 0) the ratio of Eq. bs_lm2_1 or (mode 1) the sum itself.
+// A thread per bin and moment walked up to 80 chunks alone (64^3: 14 us).
 template <int LMAX>
-__global__ void __launch_bounds__(256)
-k_epi_fin(int mode, const int64_t *__restrict__ bin_chunk, int64_t nbins, const double *__restrict__ partial,
+__global__ void __launch_bounds__(128)
+k_epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *__restrict__ partial,
           const double *__restrict__ den, double norm, double *__restrict__ out, int64_t fs_part, int64_t fs_out,
           int lm_lo, int nlm_out)
 {
     partial = field_ptr(partial, fs_part);
     out = field_ptr(out, fs_out);
     constexpr int NLM = (LMAX / 2 + 1) * (LMAX / 2 + 1);
-    const int64_t o = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (o >= nbins * nlm_out) return;
-    const int64_t b = o / nlm_out;
-    const int i = int(o - b * nlm_out) + lm_lo;
+    constexpr int P2 = NLM <= 1 ? 1 : (NLM <= 4 ? 4 : (NLM <= 16 ? 16 : 32));
+    constexpr int NS = 128 / P2;
+    __shared__ double red[128];
+    const int64_t b = blockIdx.x;
+    const int i = threadIdx.x % P2, sub = threadIdx.x / P2;
     const int64_t c0 = bin_chunk[b], c1 = bin_chunk[b + 1];
     double v = 0.0;
-#pragma unroll 8
-    for (int64_t ch = c0; ch < c1; ++ch) v += partial[ch * NLM + i];
+    if (i < NLM)
+#pragma unroll 4
+        for (int64_t ch = c0 + sub; ch < c1; ch += NS) v += partial[ch * NLM + i];
+    red[threadIdx.x] = v;
+    __syncthreads();
+    if (sub > 0 || i < lm_lo || i >= NLM) return;
+    const int64_t o = b * nlm_out + (i - lm_lo);
+    const double d = mode == 0 ? den[o] : 0.0;
+    for (int k = 1; k < NS; ++k) v += red[k * P2 + i];
     if (mode == 0) {
         int l = 0;
         while ((l / 2 + 1) * (l / 2 + 1) <= i) l += 2;
-        const double d = den[o];
         out[o] = d > 0.0 ? c_pref[l] * v * norm / d : __longlong_as_double(0x7ff8000000000000LL);
     } else {
         out[o] = v;
@@ -1035,6 +1052,15 @@ cudaError_t launch_fft_rows_split(const typename Cx<R>::T *in, R *out, int M, in
     return cudaGetLastError();
 }
 
+// Shared-memory buffers of a Step-I transform of length M: its stages hand the
+// data on between the first, from global memory, and the last, to it.
+static int fft_buffers(int M)
+{
+    const int lg = __builtin_ctz(unsigned(M)), odd = M >> lg;
+    const int stages = odd > 1 ? 1 + (lg + 2) / 3 : (lg + 2) / 3;
+    return stages > 2 ? 2 : 1;
+}
+
 // The blocks of a Step-I launch over several grids, and its shared memory.
 template <typename C> static cudaError_t step_blocks(StepGrids &gs, bool cols, unsigned *nblk, size_t *smem)
 {
@@ -1051,12 +1077,23 @@ template <typename C> static cudaError_t step_blocks(StepGrids &gs, bool cols, u
         }
         g.ntile = (g.M + g.rt - 1) / g.rt;
         g.blk0 = unsigned(blk);
-        blk += g.njobs * g.ntile;
-        *smem = std::max(*smem, size_t(2) * g.rt * fft_stride(g.M) * sizeof(C));
+        blk += cols ? (g.njobs * g.M + g.rt - 1) / g.rt : g.njobs * g.ntile;
+        *smem = std::max(*smem, size_t(fft_buffers(g.M)) * g.rt * fft_stride(g.M) * sizeof(C));
     }
     if (blk > 0x7FFFFFFF || *smem > 227 * 1024) return cudaErrorInvalidValue;
     *nblk = unsigned(blk);
     return cudaSuccess;
+}
+
+// Threads of a Step-I block: 128 up to M = 256, whose tiles give more threads
+// little to do in a stage and whose blocks are then finer to place (all grids of
+// 64^3 63 -> 49 us with the columns of several jobs per block, of 128^3 x 16 5.0 ->
+// 4.0 ms); 256 above (at 512^3, 128 for all took 29.9 ms, 256 27.0).
+static unsigned step_threads(const StepGrids &gs)
+{
+    int m = 0;
+    for (int i = 0; i < gs.n; ++i) m = std::max(m, gs.g[i].M);
+    return m <= 256 ? 128 : 256;
 }
 
 template <typename R>
@@ -1069,10 +1106,11 @@ cudaError_t launch_ring_gather(const typename Cx<R>::T *planes, int ng, const Ri
     if (cudaError_t e = step_blocks<typename Cx<R>::T>(gs, false, &nblk, &smem); e != cudaSuccess) return e;
     if (nblk == 0) return cudaSuccess;
     const dim3 grid(nblk, fb.nf);
+    const unsigned threads = step_threads(gs);
     if (unit)
-        k_ring_gather<R, true><<<grid, 256, smem, s>>>(planes, ng, rings, gs, out, tw, scale, fb.fs_in);
+        k_ring_gather<R, true><<<grid, threads, smem, s>>>(planes, ng, rings, gs, out, tw, scale, fb.fs_in);
     else
-        k_ring_gather<R, false><<<grid, 256, smem, s>>>(planes, ng, rings, gs, out, tw, scale, fb.fs_in);
+        k_ring_gather<R, false><<<grid, threads, smem, s>>>(planes, ng, rings, gs, out, tw, scale, fb.fs_in);
     return cudaGetLastError();
 }
 
@@ -1091,7 +1129,7 @@ cudaError_t launch_fft_cols(typename Cx<R>::T *out, StepGrids gs, const RingArg 
     size_t smem;
     if (cudaError_t e = step_blocks<typename Cx<R>::T>(gs, true, &nblk, &smem); e != cudaSuccess) return e;
     if (nblk == 0) return cudaSuccess;
-    k_fft_cols<R><<<dim3(nblk, fb.nf), 256, smem, s>>>(out, gs, rings, tw, fb.fs_in);
+    k_fft_cols<R><<<dim3(nblk, fb.nf), step_threads(gs), smem, s>>>(out, gs, rings, tw, fb.fs_in);
     return cudaGetLastError();
 }
 
@@ -1129,7 +1167,7 @@ cudaError_t launch_reduce_partials(const Group *groups, int64_t ngroups, const d
                                    double *S, const Batch &fb, cudaStream_t s)
 {
     if (ngroups == 0) return cudaSuccess;
-    k_reduce<A><<<dim3(unsigned(ngroups), fb.nf), 256, 0, s>>>(groups, partials, ng, S, fb.fs_in);
+    k_reduce<A><<<dim3(unsigned((ngroups + 7) / 8), fb.nf), 256, 0, s>>>(groups, ngroups, partials, ng, S, fb.fs_in);
     return cudaGetLastError();
 }
 
@@ -1137,12 +1175,11 @@ template <typename W, typename Y, int LMAX>
 cudaError_t epilogue_l(int mode, const EpiArgs &e, const double *value, const double *den, double norm, double *out,
                        const Batch &fb, int lo, int n, cudaStream_t s)
 {
-    const dim3 g1(unsigned((e.nchunks * 32 + 255) / 256), fb.nf), g2(unsigned((e.nbins * n + 255) / 256), fb.nf);
+    const dim3 g1(unsigned((e.nchunks * 32 + 255) / 256), fb.nf), g2(unsigned(e.nbins), fb.nf);
     if (e.nchunks > 0)
         k_epi_part<W, Y, LMAX><<<g1, 256, 0, s>>>(mode, e.rec, e.recf, e.chunk_lo, e.chunk_hi, e.nchunks, value, e.partial,
                                                   fb.fs_in, e.fs_part);
-    k_epi_fin<LMAX><<<g2, 256, 0, s>>>(mode, e.bin_chunk, e.nbins, e.partial, den, norm, out, e.fs_part, fb.fs_out,
-                                       lo, n);
+    k_epi_fin<LMAX><<<g2, 128, 0, s>>>(mode, e.bin_chunk, e.partial, den, norm, out, e.fs_part, fb.fs_out, lo, n);
     return cudaGetLastError();
 }
 
