@@ -909,12 +909,19 @@ k_epi_part(int mode, const Record *__restrict__ rec, const RecordF *__restrict__
     if ((lane & (32 / P2 - 1)) == 0 && idx < NLM) partial[ch * NLM + idx] = double(red[0]) * (WIDEN ? 0x1p448 : 1.0);
 }
 
-// One block per bin: 128 / P2 threads per moment (P2 = NLM rounded up to a power
-// of two) take the bin's chunks in turn, and their partial sums are added in
-// order; then (mode 0) the ratio of Eq. bs_lm2_1 or (mode 1) the sum itself.
-// A thread per bin and moment walked up to 80 chunks alone (64^3: 14 us).
+// One block per bin: kFinSplit threads per moment take the bin's chunks in turn,
+// and their partial sums are added in order (the same for every LMAX, so that a
+// moment does not depend on the others binned with it); then (mode 0) the ratio
+// of Eq. bs_lm2_1 or (mode 1) the sum itself.  A thread per bin and moment walked
+// up to 80 chunks alone (64^3: 14 us).
+constexpr int kFinSplit = 8;
+template <int LMAX> constexpr int fin_threads()
+{
+    const int n = (LMAX / 2 + 1) * (LMAX / 2 + 1);
+    return n <= 4 ? 32 : (n <= 16 ? 128 : 256);
+}
 template <int LMAX>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(fin_threads<LMAX>())
 k_epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *__restrict__ partial,
           const double *__restrict__ den, double norm, double *__restrict__ out, int64_t fs_part, int64_t fs_out,
           int lm_lo, int nlm_out)
@@ -922,22 +929,21 @@ k_epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *__restr
     partial = field_ptr(partial, fs_part);
     out = field_ptr(out, fs_out);
     constexpr int NLM = (LMAX / 2 + 1) * (LMAX / 2 + 1);
-    constexpr int P2 = NLM <= 1 ? 1 : (NLM <= 4 ? 4 : (NLM <= 16 ? 16 : 32));
-    constexpr int NS = 128 / P2;
-    __shared__ double red[128];
+    constexpr int P2 = fin_threads<LMAX>() / kFinSplit;     // at least NLM
+    __shared__ double red[fin_threads<LMAX>()];
     const int64_t b = blockIdx.x;
     const int i = threadIdx.x % P2, sub = threadIdx.x / P2;
     const int64_t c0 = bin_chunk[b], c1 = bin_chunk[b + 1];
     double v = 0.0;
     if (i < NLM)
 #pragma unroll 4
-        for (int64_t ch = c0 + sub; ch < c1; ch += NS) v += partial[ch * NLM + i];
+        for (int64_t ch = c0 + sub; ch < c1; ch += kFinSplit) v += partial[ch * NLM + i];
     red[threadIdx.x] = v;
     __syncthreads();
     if (sub > 0 || i < lm_lo || i >= NLM) return;
     const int64_t o = b * nlm_out + (i - lm_lo);
     const double d = mode == 0 ? den[o] : 0.0;
-    for (int k = 1; k < NS; ++k) v += red[k * P2 + i];
+    for (int k = 1; k < kFinSplit; ++k) v += red[k * P2 + i];
     if (mode == 0) {
         int l = 0;
         while ((l / 2 + 1) * (l / 2 + 1) <= i) l += 2;
@@ -1179,7 +1185,7 @@ cudaError_t epilogue_l(int mode, const EpiArgs &e, const double *value, const do
     if (e.nchunks > 0)
         k_epi_part<W, Y, LMAX><<<g1, 256, 0, s>>>(mode, e.rec, e.recf, e.chunk_lo, e.chunk_hi, e.nchunks, value, e.partial,
                                                   fb.fs_in, e.fs_part);
-    k_epi_fin<LMAX><<<g2, 128, 0, s>>>(mode, e.bin_chunk, e.partial, den, norm, out, e.fs_part, fb.fs_out, lo, n);
+    k_epi_fin<LMAX><<<g2, fin_threads<LMAX>(), 0, s>>>(mode, e.bin_chunk, e.partial, den, norm, out, e.fs_part, fb.fs_out, lo, n);
     return cudaGetLastError();
 }
 
