@@ -349,7 +349,8 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
         T.nslot = int32_t(cur.slots.size());
         T.n3abs = cur_n3;
         T.r3lo = cur.lo;
-        T.ncol = ((cur.hi - cur.lo + 1 + 15) / 16) * 16;
+        T.nwin = cur.hi - cur.lo + 1;
+        T.ncol = ((T.nwin + 15) / 16) * 16;
         const int64_t M2 = int64_t(T.M) * T.M;
         T.nchunk = int32_t((M2 + x_chunk - 1) / x_chunk);
         if (T.ncol > kTcMaxCols || T.nslot > kTcMaxSlots || T.nrow > kTcRows || tc_ring(T.ncol, T.nslot) == 0)
@@ -395,13 +396,15 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
         // up) that read different slots of one group are served one after
         // another.  Colour the fields greedily (first appearance order) so
         // that the distinct D1 fields of each pass, and its distinct D2
-        // fields, take distinct colours where they can, and number them
-        // colour + 8 k; numbers left free are padding slots that hold a field
-        // nothing stores (they read as zero).  Kept only if the tile still fits.
+        // fields, take distinct colours where they can, then move single
+        // fields to a colour that saves accesses while there are any (512^3:
+        // 6.1 -> 5.8 accesses for the two loads), and number them colour + 8 k;
+        // numbers left free are padding slots that hold a field nothing stores
+        // (they read as zero).  Kept only if the tile still fits.
         const int ns = T.nslot;
         std::vector<int> num(ns);
         {
-            std::vector<std::vector<int>> adj(ns);
+            std::vector<std::vector<int>> adj(ns), pass, in(ns);   // passes, and those of each field
             for (int side = 0; side < 2; ++side)
                 for (int g0 = 0; g0 < nlane;) {
                     const int np = (side ? lanes.pair2 : lanes.pair1)[g0 / 32] ? 16 : 8;
@@ -410,9 +413,12 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
                         const int f = slot_of(cur.slots, (side ? key2 : key1)[lanes.like[l]]);
                         if (std::find(grp.begin(), grp.end(), f) == grp.end()) grp.push_back(f);
                     }
-                    for (int a : grp)
+                    for (int a : grp) {
+                        in[a].push_back(int(pass.size()));
                         for (int b : grp)
                             if (a != b) adj[a].push_back(b);
+                    }
+                    pass.push_back(grp);
                     g0 += np;
                 }
             std::vector<int> col(ns, -1), cnt(8, 0), next(8, 0);
@@ -426,7 +432,41 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
                     if (use[c] < use[best] || (use[c] == use[best] && cnt[c] < cnt[best])) best = c;
                 col[f] = best;
                 ++cnt[best];
-                num[f] = best + 8 * next[best]++;
+            }
+            // accesses of a field's passes (the most fields of one colour in each)
+            auto accesses = [&](int f) {
+                int n = 0;
+                for (int k : in[f]) {
+                    int c[8] = {0}, most = 0;
+                    for (int g : pass[size_t(k)]) most = std::max(most, ++c[col[g]]);
+                    n += most;
+                }
+                return n;
+            };
+            for (int round = 0, moved = 1; round < 3 && moved; ++round) {
+                moved = 0;
+                for (int f = 0; f < ns; ++f) {
+                    const int was = col[f], now = accesses(f);
+                    if (now == int(in[f].size())) continue;      // no conflict
+                    int best = was, fewest = now;
+                    for (int c = 0; c < 8; ++c) {
+                        if (c == was || cnt[c] > ns / 8 + 1) continue;
+                        col[f] = c;
+                        const int n = accesses(f);
+                        if (n < fewest) {
+                            fewest = n;
+                            best = c;
+                        }
+                    }
+                    col[f] = best;
+                    if (best == was) continue;
+                    --cnt[was];
+                    ++cnt[best];
+                    moved = 1;
+                }
+            }
+            for (int f = 0; f < ns; ++f) {
+                num[f] = col[f] + 8 * next[col[f]]++;
                 top = std::max(top, num[f] + 1);
             }
             if (top <= kTcMaxSlots && tc_ring(T.ncol, top) > 0) {

@@ -100,15 +100,17 @@ BISP_HD inline size_t tc_fixed_smem(int ncol, int nslot)
     return size_t(2 * tc_abuf(ncol)) * ncol * kTcTX * 4 + ((8 * size_t(nslot + ncol) + 256 + 127) & ~size_t(127));
 }
 // Buffers of the stage ring for a tile (0 if fewer than kTcMinRing fit):
-// each holds a stage of the tile's nslot + ncol fields.
-BISP_HD inline int tc_ring(int ncol, int nslot)
+// each holds a stage of the tile's nslot + nwin fields (nwin columns of the
+// window of ncol; the two-argument form counts all of them).
+BISP_HD inline int tc_ring(int ncol, int nslot, int nwin)
 {
     const size_t fixed = tc_fixed_smem(ncol, nslot);
     if (fixed >= kTcSmem) return 0;
-    const size_t per = size_t(nslot + ncol) * kTcSlotBytes;
+    const size_t per = size_t(nslot + nwin) * kTcSlotBytes;
     const int n = int((kTcSmem - fixed) / per);
     return n < kTcMinRing ? 0 : (n > kTcMaxRing ? kTcMaxRing : n);
 }
+BISP_HD inline int tc_ring(int ncol, int nslot) { return tc_ring(ncol, nslot, ncol); }
 struct TcRow {
     int64_t p0;                // partial sum of (x chunk 0, first combination of the run)
     int32_t stride;            // partial sums of one x chunk of the row's group (its ncombo)
@@ -126,6 +128,7 @@ struct TcTile {
     int32_t ncol, nchunk;      // NC; x chunks of the M^2 grid
     int32_t flags;             // the rows' flags where all rows share them, else kTcMixed
     uint8_t qflags[4];         // flags of the rows of lanes 32 q .. 32 q + 31
+    int32_t nwin;              // columns of the window that a row uses: r3lo .. r3lo + nwin - 1
 };
 constexpr int kTcMixed = 8;
 // What tensor-memory lane `lane` of a tile does: its row of the tile (kTcNoRow:

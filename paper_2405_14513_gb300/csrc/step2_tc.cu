@@ -206,7 +206,9 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *m)
 }
 
 // Bounded wait for phase `parity` of m; gives up (false) when the block is
-// aborting or after `spins` polls, and then raises the abort flag.  A poll
+// aborting or after `spins` more polls, and then raises the abort flag.  The
+// first poll is a test_wait: most waits are over when they are reached.  A later
+// one
 // is a try_wait, which may suspend the thread for a while before it reports;
 // under kTestPolls polls (a limit set to exercise the give-up path) it is a
 // test_wait, which reports at once, so that such a limit really cuts the
@@ -215,9 +217,12 @@ constexpr int kTestPolls = 64;
 __device__ __forceinline__ bool mbar_wait_abort(uint64_t *m, uint32_t parity, volatile int *abort, int spins)
 {
     const uint32_t a = su32(m);
+    uint32_t ok;
+    asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(ok) : "r"(a), "r"(parity) : "memory");
+    if (ok) return true;
     const bool test = spins < kTestPolls;
     for (int i = 0; i < spins; ++i) {
-        uint32_t ok;
         if (test)
             asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
                          : "=r"(ok) : "r"(a), "r"(parity) : "memory");
@@ -282,7 +287,7 @@ struct CompArgs {
     uint32_t tlane;            // tensor-memory address of lane 0 of this warp's quarter
     volatile int *abort;
     TcSync *sy;
-    int rowb, nslot, S, nstage, ntail, spins, t, half, s1, s2;   // ntail: points of the last stage (16 or 32)
+    int rowb, nslot, nwin, S, nstage, ntail, spins, t, half, s1, s2;   // ntail: points of the last stage (16 or 32)
     int flags;                 // the warp's sign pattern, -1: none of its lanes has a row
 };
 
@@ -298,9 +303,10 @@ template <int NC> __device__ constexpr uint32_t acc_step() { return tc_abuf(NC) 
 // overwrite that accumulator buffer, and wait only for A(st), signalled
 // after the read) can start as soon as A(st) is written, and have the whole
 // next stage to finish.  Returns false if a wait gave up.  B piece p
-// (grid points 4p .. 4p + 3) of column c goes to core matrix (K block p, rows
-// 8 (c / 8) ..), row c % 8; this thread's pieces are i = t and t + 256
-// (i = p NC + c), fixed for the tile, so their offsets are computed once.
+// (grid points 4p .. 4p + 3) of column c < nwin goes to core matrix (K block p,
+// rows 8 (c / 8) ..), row c % 8 (columns that no row uses hold what they hold);
+// this thread's pieces are i = t and t + 256 (i = p nwin + c), fixed for the
+// tile, so their offsets are computed once.
 // The last stage may hold 16 points (ntail); its second half is left alone.
 // PATTERN: the tile's flags, or kTcMixed: each warp takes its own (uniform over
 // the warp).  A warp without rows leaves its lanes of A as they are.
@@ -318,8 +324,8 @@ __device__ __forceinline__ bool compute_loop(const CompArgs &ca, float (&acc)[NC
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
         const int i = ca.t + k * kCompute;
-        const int c = i % NC, p = i / NC;
-        src[k] = i < NC * 8 ? (ca.nslot + c) * kSlotBytes + p * 32 : -1;
+        const int p = i / ca.nwin, c = i - p * ca.nwin;
+        src[k] = p < 8 ? (ca.nslot + c) * kSlotBytes + p * 32 : -1;
         dst[k] = (p * NB + c / 8) * 128 + (c % 8) * 16;
     }
     const int uoff = ca.s1 * kSlotBytes, voff = ca.s2 * kSlotBytes;
@@ -352,7 +358,7 @@ __device__ __forceinline__ bool compute_loop(const CompArgs &ca, float (&acc)[NC
 #pragma unroll
         for (int k = 0; k < NP; ++k) {
             if (src[k] < 0) continue;
-            if (!whole && ca.t + k * kCompute >= NC * 4) continue;        // pieces of points 16 ..
+            if (!whole && ca.t + k * kCompute >= ca.nwin * 4) continue;   // pieces of points 16 ..
             const float4 v = *reinterpret_cast<const float4 *>(sq + src[k]);
             const float4 w = *reinterpret_cast<const float4 *>(sq + src[k] + 16);
             const int o = ia * BB + dst[k];
@@ -372,7 +378,6 @@ __device__ __forceinline__ bool compute_loop(const CompArgs &ca, float (&acc)[NC
             sq += ca.rowb;
         }
         asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
         mbar_arrive(&sy->aready[ia]);
         if (++ia == NA) ia = 0;
@@ -474,8 +479,8 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
     args.scale = reinterpret_cast<const float *>(reinterpret_cast<const char *>(args.scale) + int64_t(blockIdx.y) * args.fs);
     args.status = reinterpret_cast<int *>(reinterpret_cast<char *>(args.status) + int64_t(blockIdx.y) * args.fs);
     const int spins = args.wait_spins;
-    const int nslot = T.nslot, nf = nslot + NC;
-    const int S = tc_ring(NC, nslot);            // ring buffers (>= 2; the plan checked)
+    const int nslot = T.nslot, nf = nslot + T.nwin;
+    const int S = tc_ring(NC, nslot, T.nwin);    // ring buffers (>= 2; the plan checked)
     const int rowb = nf * kSlotBytes;            // one ring buffer: nf fields
     // shared memory: B high and low parts [NA][BB] each (canonical layout),
     // field offsets [nf], barriers, ring [S][nf][kSlotBytes] (a stage of D1 / D2
@@ -483,7 +488,7 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
     unsigned char *sHi = smem;
     unsigned char *sLo = smem + NA * BB;
     int64_t *offs = reinterpret_cast<int64_t *>(smem + 2 * NA * BB);
-    TcSync *sy = reinterpret_cast<TcSync *>(smem + 2 * NA * BB + 8 * size_t(nf));
+    TcSync *sy = reinterpret_cast<TcSync *>(smem + 2 * NA * BB + 8 * size_t(nslot + NC));
     unsigned char *sS = smem + tc_fixed_smem(NC, nslot);
 
     for (int f = t; f < nf; f += kThreads) {
@@ -564,6 +569,11 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
                 // stage's ring buffer are done (the MMAs do not read the ring)
                 if (lane == 0) mbar_arrive(&sy->empty[qr]);
                 if (++qr == S) qr = 0;
+                // the compute threads' generic writes of B, which the barrier has
+                // ordered before this point, before the tensor core's reads: one
+                // fence here, on the way from the writes to the reads, in place of one by
+                // each of the writers
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t a = tmem + 64 * ia;
                 const uint32_t d = tmem + acc_col0<NC>() + acc_step<NC>() * b;
@@ -597,8 +607,8 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
         const bool live = ln.row != kTcNoRow;
         TcRow R{};
         if (live) R = args.rows[T.row0 + ln.row];
-        CompArgs ca{sS, sHi, sLo, tmem + (uint32_t(quarter * 32) << 16), abort, sy, rowb, nslot, S, nstage, ntail, spins,
-                    t, half, int(ln.s1), int(ln.s2),
+        CompArgs ca{sS, sHi, sLo, tmem + (uint32_t(quarter * 32) << 16), abort, sy, rowb, nslot, T.nwin, S, nstage, ntail,
+                    spins, t, half, int(ln.s1), int(ln.s2),
                     __any_sync(0xFFFFFFFFu, live) ? int(T.qflags[quarter]) : -1};
         float acc[NC / 2];
         switch (T.flags) {
