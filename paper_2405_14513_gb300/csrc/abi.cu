@@ -470,7 +470,7 @@ int autotune_transforms(bisp_plan *p, cudaStream_t s)
         int best = 0;
         float best_ms = 1e30f;
         for (int w : {2, 4, 8, 16, 32}) {
-            if (w > M || size_t(2) * w * fft_stride(M) * sizeof(C) > 227 * 1024) continue;
+            if (w > M || size_t(2) * w * fft_stride<C>(M, w) * sizeof(C) > 227 * 1024) continue;
             if (w > 4 && size_t(w) * M * sizeof(C) > most) continue;
             if (launch(w) != cudaSuccess) return -1;
             cudaEventRecord(e0, s);

@@ -76,11 +76,13 @@ struct DivIter {
     }
 };
 
-// Shared-memory position of element i of a transform row: a padding slot
-// after every 8 elements, so that the strided stores of the first radix-8
-// stages (elements 8 and 64 apart) fall in different banks.  A row takes
-// fft_stride(M) elements (kernels.cuh).
-__device__ __forceinline__ int spos(int i) { return i + (i >> 3); }
+// Shared-memory position of element i of a transform row: the low four bits
+// exchanged with those of i / 8, so that runs of 16 elements and elements 8 or 64
+// apart (the strided stores of the first radix-8 stages) each fall in different
+// banks.  (A padding slot after every 8 elements, which this replaces, made runs
+// take two accesses where one will do: the kernels were bound by them, up to 93% of
+// the L1's wavefronts.)
+__device__ __forceinline__ int spos(int i) { return i ^ ((i >> 3) & 15); }
 
 // DFT of R values in registers, X_m = sum_r v_r exp(-2 pi i r m / R), in place.
 template <int R, typename C> __device__ __forceinline__ void dft(C (&v)[R])
@@ -305,7 +307,7 @@ k_fft_z_real(const R *__restrict__ in, typename Cx<R>::T *__restrict__ out, int 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     in = field_ptr(in, fs_in);
     out = field_ptr(out, fs_out);
-    const int P = fft_stride(M);
+    const int P = fft_stride<C>(M, rt);
     C *a = reinterpret_cast<C *>(smem_raw);
     C *b = a + rt * P;
     const int64_t row0 = int64_t(blockIdx.x) * rt;
@@ -331,7 +333,7 @@ k_fft_rows_T(const typename Cx<R>::T *__restrict__ in, typename Cx<R>::T *__rest
     extern __shared__ __align__(16) unsigned char smem_raw[];
     in = field_ptr(in, fs);
     out = field_ptr(out, fs);
-    const int P = fft_stride(M);
+    const int P = fft_stride<C>(M, rt);
     C *a = reinterpret_cast<C *>(smem_raw);
     C *b = a + rt * P;
     const int64_t bt = blockIdx.x / ntile;
@@ -411,6 +413,9 @@ k_ring_scale(const float2 *__restrict__ planes, int ng, RingArg rings, float *__
     scale[n * kMaxRings + r] = ldexpf(1.0f, e);
 }
 
+// rows that the lanes of a first-pass warp run across: several where a row is short
+__host__ __device__ __forceinline__ constexpr int gather_across(int M) { return M >= 128 ? 16 : 2; }
+
 // the grid of a Step-I block (the grids of a launch in order of their blocks)
 __device__ __forceinline__ const StepGrid &grid_of_block(const StepGrids &gs)
 {
@@ -432,7 +437,7 @@ k_ring_gather(const typename Cx<R>::T *__restrict__ planes, int ng, const __grid
     scale = scale ? field_ptr(scale, fs) : scale;
     const StepGrid &gr = grid_of_block(gs);
     const int M = gr.M, rt = gr.rt;
-    const int P = fft_stride(M);
+    const int P = fft_stride<C>(M, gather_across(M));
     C *a = reinterpret_cast<C *>(smem_raw);
     C *b = a + rt * P;
     const int blk = int(blockIdx.x - gr.blk0), jb = blk / gr.ntile;
@@ -501,7 +506,7 @@ k_fft_cols(typename Cx<R>::T *__restrict__ out, const __grid_constant__ StepGrid
     out = field_ptr(out, fs);
     const StepGrid &gr = grid_of_block(gs);
     const int M = gr.M, w = gr.rt;
-    const int P = fft_stride(M);
+    const int P = fft_stride<C>(M, w);
     C *a = reinterpret_cast<C *>(smem_raw);
     C *b = a + w * P;
     const int64_t c0 = int64_t(blockIdx.x - gr.blk0) * w, cols = gr.njobs * M;
@@ -1019,7 +1024,7 @@ cudaError_t launch_fft_z_real(const R *in, typename Cx<R>::T *out, int ng, int64
 {
     using C = typename Cx<R>::T;
     if (rt <= 0) rt = int(fft_rows_per_block(ng, sizeof(C)));
-    const size_t smem = size_t(2) * rt * fft_stride(ng) * sizeof(C);
+    const size_t smem = size_t(2) * rt * fft_stride<C>(ng, rt) * sizeof(C);
     const int64_t nblk = (rows + rt - 1) / rt;
     k_fft_z_real<R><<<dim3(unsigned(nblk), fb.nf), 256, smem, s>>>(in, out, ng, rows, nkeep, rt, tw, fb.fs_in,
                                                                    fb.fs_out);
@@ -1034,7 +1039,7 @@ cudaError_t launch_fft_rows_T(const typename Cx<R>::T *in, typename Cx<R>::T *ou
     using C = typename Cx<R>::T;
     if (rt <= 0) rt = int(fft_rows_per_block(M, sizeof(C)));
     rt = std::min(rt, nrow);
-    const size_t smem = size_t(2) * rt * fft_stride(M) * sizeof(C);
+    const size_t smem = size_t(2) * rt * fft_stride<C>(M, rt) * sizeof(C);
     const int ntile = (nrow + rt - 1) / rt;
     const int64_t nblk = nb * ntile;
     if (nblk == 0) return cudaSuccess;
@@ -1049,7 +1054,7 @@ cudaError_t launch_fft_rows_split(const typename Cx<R>::T *in, R *out, int M, in
 {
     using C = typename Cx<R>::T;
     const int rt = std::min(int(fft_rows_per_block(M, sizeof(C))), nrow);
-    const size_t smem = size_t(2) * rt * fft_stride(M) * sizeof(C);
+    const size_t smem = size_t(2) * rt * fft_stride<C>(M, rt) * sizeof(C);
     const int ntile = (nrow + rt - 1) / rt;
     const int64_t nblk = (nf + 1) / 2 * ntile;
     if (nblk == 0) return cudaSuccess;
@@ -1084,7 +1089,7 @@ template <typename C> static cudaError_t step_blocks(StepGrids &gs, bool cols, u
         g.ntile = (g.M + g.rt - 1) / g.rt;
         g.blk0 = unsigned(blk);
         blk += cols ? (g.njobs * g.M + g.rt - 1) / g.rt : g.njobs * g.ntile;
-        *smem = std::max(*smem, size_t(fft_buffers(g.M)) * g.rt * fft_stride(g.M) * sizeof(C));
+        *smem = std::max(*smem, size_t(fft_buffers(g.M)) * g.rt * fft_stride<C>(g.M, cols ? g.rt : gather_across(g.M)) * sizeof(C));
     }
     if (blk > 0x7FFFFFFF || *smem > 227 * 1024) return cudaErrorInvalidValue;
     *nblk = unsigned(blk);

@@ -224,9 +224,15 @@ cudaError_t launch_ntri(const double2 *ifields, const int64_t *ioff, const int32
 // launchers above selects this with the default 16 KB; the plan's autotuner
 // passes its own choice.
 size_t fft_rows_per_block(int M, size_t elem, size_t bytes = 16384);
-// Elements of one row of a transform's shared-memory buffers: M values with
-// a padding slot after every 8, and one more so that consecutive rows start
-// in different banks.
-inline __host__ __device__ constexpr int fft_stride(int M) { return M + (M >> 3) + 1; }
+// Elements from one row of a transform's shared-memory buffer to the next.  An
+// element's place in its row is its index with the low four bits exchanged
+// (spos in kernels.cu), so a row takes a multiple of 16; what is added to it
+// spreads the rows over the banks (16 of 8 bytes, or 8 of 16) where a warp's
+// lanes run across `across` rows first and along them second.
+template <typename C> inline __host__ __device__ constexpr int fft_stride(int M, int across)
+{
+    const int banks = 128 / int(sizeof(C));
+    return ((M + 15) & ~15) + (across >= banks ? 1 : (2 * across >= banks ? 2 : (4 * across >= banks ? 4 : banks / 2)));
+}
 
 }  // namespace bisp
