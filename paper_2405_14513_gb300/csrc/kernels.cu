@@ -310,15 +310,32 @@ k_fft_z_real(const R *__restrict__ in, typename Cx<R>::T *__restrict__ out, int 
     const int P = fft_stride<C>(M, rt);
     C *a = reinterpret_cast<C *>(smem_raw);
     C *b = a + rt * P;
-    const int64_t row0 = int64_t(blockIdx.x) * rt;
-    const int nrow = int(min(int64_t(rt), rows - row0));
+    // two real rows a, b share a transform of a + i b (the number of rows is
+    // even): half the transforms of a kernel that is bound by its shared-memory
+    // accesses (forward transform, 384^3 x 10: 4.5 -> 3.4 ms)
+    const int64_t row0 = int64_t(blockIdx.x) * 2 * rt;
+    const int npair = int(min(int64_t(rt), (rows - row0) / 2));
     const R *src = in + row0 * M;
     const C *res = fft_any<C, false, true, false>(
-        M, nrow, 0, P, a, b, tw.t, [&](int r, int i) { return cmk<C>(double(src[r * M + i]), 0.0); }, NoStore{});
-    DivIter st(threadIdx.x, blockDim.x, nrow);
-    for (int t = threadIdx.x; t < nkeep * nrow; t += blockDim.x, st.next()) {
+        M, npair, 0, P, a, b, tw.t,
+        [&](int r, int i) {
+            C v;
+            v.x = src[2 * r * M + i];
+            v.y = src[(2 * r + 1) * M + i];
+            return v;
+        },
+        NoStore{});
+    // A_k = (X_k + conj X_{M-k}) / 2,  B_k = (X_k - conj X_{M-k}) / (2 i)
+    DivIter st(threadIdx.x, blockDim.x, npair);
+    for (int t = threadIdx.x; t < nkeep * npair; t += blockDim.x, st.next()) {
         const int k = st.q, r = st.r;
-        out[int64_t(k) * rows + row0 + r] = res[r * P + spos(k)];
+        const C x = res[r * P + spos(k)], y = res[r * P + spos(k == 0 ? 0 : M - k)];
+        C *o = out + int64_t(k) * rows + row0 + 2 * r;
+        C u, v;
+        u.x = R(0.5) * (x.x + y.x); u.y = R(0.5) * (x.y - y.y);
+        v.x = R(0.5) * (x.y + y.y); v.y = R(0.5) * (y.x - x.x);
+        o[0] = u;
+        o[1] = v;
     }
 }
 
@@ -1024,8 +1041,9 @@ cudaError_t launch_fft_z_real(const R *in, typename Cx<R>::T *out, int ng, int64
 {
     using C = typename Cx<R>::T;
     if (rt <= 0) rt = int(fft_rows_per_block(ng, sizeof(C)));
+    rt = std::max(1, int(std::min<int64_t>(rt, rows / 2)));        // pairs of rows
     const size_t smem = size_t(2) * rt * fft_stride<C>(ng, rt) * sizeof(C);
-    const int64_t nblk = (rows + rt - 1) / rt;
+    const int64_t nblk = (rows / 2 + rt - 1) / rt;
     k_fft_z_real<R><<<dim3(unsigned(nblk), fb.nf), 256, smem, s>>>(in, out, ng, rows, nkeep, rt, tw, fb.fs_in,
                                                                    fb.fs_out);
     return cudaGetLastError();
