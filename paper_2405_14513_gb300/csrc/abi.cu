@@ -672,7 +672,7 @@ int build_plan(bisp_plan *p, const bisp_desc *desc, cudaStream_t s)
     // Step-I jobs per grid, and the launches: consecutive small grids share one
     // while their fields together take at most kStepShare bytes; their kernels
     // last a few us each, so a plan of small grids was bound by the launches
-    // (64^3, 11 grids: 22 launches, 157 us; in two, 63 us), while a large grid
+    // (64^3, 11 grids: 22 launches, 157 us; in two, 48 us), while a large grid
     // fills the GPU by itself and keeps the shared memory that suits it
     size_t share = 0;
     for (const Level &L : P.levels) {
@@ -704,7 +704,12 @@ int build_plan(bisp_plan *p, const bisp_desc *desc, cudaStream_t s)
     p->off_part = o; o = align256(o + size_t(P.n_partials) * sizeof(double));
     p->off_S = o; o = align256(o + size_t(P.n_combos) * sizeof(double));
     p->off_status = o; o = align256(o + sizeof(int));
-    p->off_epi = o; o = align256(o + size_t(P.max_chunks * epi_nlm) * sizeof(double));
+    p->off_epi = o;
+    {
+        int64_t n = 0;                       // every view's chunks x moments of l <= its l_hi
+        for (const View &v : P.views) n += v.n_chunks * (v.l_hi / 2 + 1) * (v.l_hi / 2 + 1);
+        o = align256(o + size_t(n) * sizeof(double));
+    }
     p->off_scale = o;
     if (P.tensor) o = align256(o + size_t(R.nz + 1) * kMaxRings * sizeof(float));
     p->region_bytes = o;
@@ -747,11 +752,11 @@ int run_estimate(bisp_plan *p, const R *delta, int batch, unsigned char *ws, dou
     const Batch in_field{nf, int64_t(ng2) * ng * int64_t(sizeof(R)), fs};   // input field -> region
     const Batch region{nf, fs, fs};
     const Batch to_out{nf, fs, P.n_out * int64_t(sizeof(double))};
-    // the wait status of each field starts clear
-    CK(cudaMemset2DAsync(ws + p->off_status, size_t(fs), 0, sizeof(int), nf, s));
     {   // forward transform: z (real, planes 0..N_g/3 kept) -> y -> x, scaled by V/N_g^3, Delta(0) = 0
+        // (its first kernel also clears each field's wait status)
         StageMark m(p, BISP_STAGE_FORWARD, 3, s);
-        CK(launch_fft_z_real<R>(delta, A_, ng, ng2, Rg.nz + 1, tw, in_field, s, p->rt_z));
+        CK(launch_fft_z_real<R>(delta, A_, ng, ng2, Rg.nz + 1, tw, in_field, s, p->rt_z,
+                                 reinterpret_cast<int *>(ws + p->off_status)));
         CK(launch_fft_rows_T<R>(A_, B_, ng, ng, Rg.nz + 1, R(1), false, tw, region, s, p->rt_xy));
         CK(launch_fft_rows_T<R>(B_, A_, ng, ng, Rg.nz + 1, scale, true, tw, region, s, p->rt_xy));
     }
@@ -799,12 +804,26 @@ int run_estimate(bisp_plan *p, const R *delta, int batch, unsigned char *ws, dou
         CK(launch_reduce_partials<RA>(p->d_groups, int64_t(P.groups.size()), part, ng, Ssum, region, s));
     }
     {   // binning and the ratio of Eq. bs_lm2_1
-        StageMark m(p, BISP_STAGE_BIN, int(2 * P.views.size()), s);
-        for (const View &v : P.views) {
+        StageMark m(p, BISP_STAGE_BIN, 2, s);
+        const double norm = 1.0 / (P.volume * double(ng2));
+        double *epi = reinterpret_cast<double *>(ws + p->off_epi);
+        if (P.views.size() == 1) {
+            const View &v = P.views[0];
             const EpiArgs ea{p->d_rec, p->d_recf, p->d_chunk_lo + v.chunk_off, p->d_chunk_hi + v.chunk_off, v.n_chunks,
-                             p->d_bin_chunk + v.bc_off, v.n_bins, reinterpret_cast<double *>(ws + p->off_epi), fs};
-            CK(launch_epilogue<W>(0, ea, Ssum, v.l_lo, v.l_hi, p->d_den + v.out_off, 1.0 / (P.volume * double(ng2)),
-                                  B + v.out_off, to_out, s, p->precision != BISP_PREC_FP64));
+                             p->d_bin_chunk + v.bc_off, v.n_bins, epi, fs};
+            CK(launch_epilogue<W>(0, ea, Ssum, v.l_lo, v.l_hi, p->d_den + v.out_off, norm, B + v.out_off, to_out, s,
+                                  p->precision != BISP_PREC_FP64));
+        } else {
+            EpiViews ev{};
+            ev.rec = p->d_rec;
+            ev.recf = p->d_recf;
+            for (const View &v : P.views) {
+                ev.v[ev.n++] = EpiView{p->d_chunk_lo + v.chunk_off, p->d_chunk_hi + v.chunk_off, p->d_bin_chunk + v.bc_off,
+                                       v.n_chunks, v.n_bins, epi, p->d_den + v.out_off, B + v.out_off, v.l_hi, v.lm_lo,
+                                       v.n_lm, 0, 0};
+                epi += v.n_chunks * (v.l_hi / 2 + 1) * (v.l_hi / 2 + 1);
+            }
+            CK(launch_epilogue_views<W>(ev, Ssum, norm, to_out, s, p->precision != BISP_PREC_FP64));
         }
     }
     p->last_field = batch - 1;

@@ -301,12 +301,13 @@ struct NoStore {
 template <typename R>
 __global__ void __launch_bounds__(256)
 k_fft_z_real(const R *__restrict__ in, typename Cx<R>::T *__restrict__ out, int M, int64_t rows,
-             int nkeep, int rt, Twiddles<typename Cx<R>::T> tw, int64_t fs_in, int64_t fs_out)
+             int nkeep, int rt, Twiddles<typename Cx<R>::T> tw, int64_t fs_in, int64_t fs_out, int *clear)
 {
     using C = typename Cx<R>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     in = field_ptr(in, fs_in);
     out = field_ptr(out, fs_out);
+    if (clear && blockIdx.x == 0 && threadIdx.x == 0) *field_ptr(clear, fs_out) = 0;
     const int P = fft_stride<C>(M, rt);
     C *a = reinterpret_cast<C *>(smem_raw);
     C *b = a + rt * P;
@@ -828,10 +829,10 @@ __device__ __forceinline__ double widen_scaled(float w)
 // records) 7.5 -> 3.2 ms, 256^3 1.21 -> 0.52 ms; 64^3, mostly for its shorter chunks
 // (bin_chunk_len), 184 -> 26 us.
 template <typename W, typename Y, int LMAX>
-__global__ void __launch_bounds__(256)
-k_epi_part(int mode, const Record *__restrict__ rec, const RecordF *__restrict__ recf,
-           const int64_t *__restrict__ chunk_lo, const int64_t *__restrict__ chunk_hi, int64_t nchunks,
-           const double *__restrict__ value, double *__restrict__ partial, int64_t fs_in, int64_t fs_part)
+__device__ __forceinline__ void
+epi_part(int mode, const Record *__restrict__ rec, const RecordF *__restrict__ recf,
+         const int64_t *__restrict__ chunk_lo, const int64_t *__restrict__ chunk_hi, int64_t nchunks, int64_t ch,
+         const double *__restrict__ value, double *__restrict__ partial, int64_t fs_in, int64_t fs_part)
 {
     constexpr bool F32 = sizeof(Y) == 4;                  // FP32 weights (mode 0 only)
     constexpr bool WIDEN = F32 && sizeof(W) == 8;
@@ -841,7 +842,6 @@ k_epi_part(int mode, const Record *__restrict__ rec, const RecordF *__restrict__
     value = field_ptr(value, fs_in);
     partial = field_ptr(partial, fs_part);
     constexpr int NLM = (LMAX / 2 + 1) * (LMAX / 2 + 1);
-    const int64_t ch = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (ch >= nchunks) return;   // whole warps leave together
     W acc[NLM];
@@ -931,6 +931,44 @@ k_epi_part(int mode, const Record *__restrict__ rec, const RecordF *__restrict__
     if ((lane & (32 / P2 - 1)) == 0 && idx < NLM) partial[ch * NLM + idx] = double(red[0]) * (WIDEN ? 0x1p448 : 1.0);
 }
 
+template <typename W, typename Y, int LMAX>
+__global__ void __launch_bounds__(256)
+k_epi_part(int mode, const Record *__restrict__ rec, const RecordF *__restrict__ recf,
+           const int64_t *__restrict__ chunk_lo, const int64_t *__restrict__ chunk_hi, int64_t nchunks,
+           const double *__restrict__ value, double *__restrict__ partial, int64_t fs_in, int64_t fs_part)
+{
+    epi_part<W, Y, LMAX>(mode, rec, recf, chunk_lo, chunk_hi, nchunks, (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5,
+                         value, partial, fs_in, fs_part);
+}
+
+// The view that block blockIdx.x of a launch over all views works on
+template <bool FIN> __device__ __forceinline__ const EpiView &view_of_block(const EpiViews &ev)
+{
+    int i = 0;
+    while (i + 1 < ev.n && blockIdx.x >= (FIN ? ev.v[i + 1].bin0 : ev.v[i + 1].blk0)) ++i;
+    return ev.v[i];
+}
+
+// k_epi_part (mode 0) for several views in one launch
+template <typename W, typename Y>
+__global__ void __launch_bounds__(256)
+k_epi_part_views(const __grid_constant__ EpiViews ev, const double *__restrict__ value, int64_t fs_in)
+{
+    const EpiView &v = view_of_block<false>(ev);
+    const int64_t ch = int64_t(blockIdx.x - v.blk0) * 8 + (threadIdx.x >> 5);
+    auto run = [&](auto lmax) {
+        epi_part<W, Y, decltype(lmax)::value>(0, ev.rec, ev.recf, v.chunk_lo, v.chunk_hi, v.nchunks, ch, value, v.partial,
+                                              fs_in, fs_in);
+    };
+    switch (v.l_hi) {
+    case 0: run(std::integral_constant<int, 0>{}); break;
+    case 2: run(std::integral_constant<int, 2>{}); break;
+    case 4: run(std::integral_constant<int, 4>{}); break;
+    case 6: run(std::integral_constant<int, 6>{}); break;
+    default: run(std::integral_constant<int, 8>{}); break;
+    }
+}
+
 // One block per bin: kFinSplit threads per moment take the bin's chunks in turn,
 // and their partial sums are added in order (the same for every LMAX, so that a
 // moment does not depend on the others binned with it); then (mode 0) the ratio
@@ -943,21 +981,19 @@ template <int LMAX> constexpr int fin_threads()
     return n <= 4 ? 32 : (n <= 16 ? 128 : 256);
 }
 template <int LMAX>
-__global__ void __launch_bounds__(fin_threads<LMAX>())
-k_epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *__restrict__ partial,
-          const double *__restrict__ den, double norm, double *__restrict__ out, int64_t fs_part, int64_t fs_out,
-          int lm_lo, int nlm_out)
+__device__ __forceinline__ void
+epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *__restrict__ partial,
+        const double *__restrict__ den, double norm, double *__restrict__ out, int64_t fs_part, int64_t fs_out,
+        int lm_lo, int nlm_out, int64_t b, double *red)
 {
     partial = field_ptr(partial, fs_part);
     out = field_ptr(out, fs_out);
     constexpr int NLM = (LMAX / 2 + 1) * (LMAX / 2 + 1);
     constexpr int P2 = fin_threads<LMAX>() / kFinSplit;     // at least NLM
-    __shared__ double red[fin_threads<LMAX>()];
-    const int64_t b = blockIdx.x;
     const int i = threadIdx.x % P2, sub = threadIdx.x / P2;
     const int64_t c0 = bin_chunk[b], c1 = bin_chunk[b + 1];
     double v = 0.0;
-    if (i < NLM)
+    if (i < NLM && sub < kFinSplit)               // (a launch over several views may have threads to spare)
 #pragma unroll 4
         for (int64_t ch = c0 + sub; ch < c1; ch += kFinSplit) v += partial[ch * NLM + i];
     red[threadIdx.x] = v;
@@ -972,6 +1008,35 @@ k_epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *__restr
         out[o] = d > 0.0 ? c_pref[l] * v * norm / d : __longlong_as_double(0x7ff8000000000000LL);
     } else {
         out[o] = v;
+    }
+}
+
+template <int LMAX>
+__global__ void __launch_bounds__(fin_threads<LMAX>())
+k_epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *__restrict__ partial,
+          const double *__restrict__ den, double norm, double *__restrict__ out, int64_t fs_part, int64_t fs_out,
+          int lm_lo, int nlm_out)
+{
+    __shared__ double red[fin_threads<LMAX>()];
+    epi_fin<LMAX>(mode, bin_chunk, partial, den, norm, out, fs_part, fs_out, lm_lo, nlm_out, blockIdx.x, red);
+}
+
+// k_epi_fin (mode 0) for several views in one launch
+__global__ void __launch_bounds__(256)
+k_epi_fin_views(const __grid_constant__ EpiViews ev, double norm, int64_t fs_part, int64_t fs_out)
+{
+    __shared__ double red[256];
+    const EpiView &v = view_of_block<true>(ev);
+    const int64_t b = blockIdx.x - v.bin0;
+    auto run = [&](auto lmax) {
+        epi_fin<decltype(lmax)::value>(0, v.bin_chunk, v.partial, v.den, norm, v.out, fs_part, fs_out, v.lm_lo, v.nlm, b, red);
+    };
+    switch (v.l_hi) {
+    case 0: run(std::integral_constant<int, 0>{}); break;
+    case 2: run(std::integral_constant<int, 2>{}); break;
+    case 4: run(std::integral_constant<int, 4>{}); break;
+    case 6: run(std::integral_constant<int, 6>{}); break;
+    default: run(std::integral_constant<int, 8>{}); break;
     }
 }
 
@@ -1037,7 +1102,7 @@ size_t fft_rows_per_block(int M, size_t elem, size_t bytes)
 
 template <typename R>
 cudaError_t launch_fft_z_real(const R *in, typename Cx<R>::T *out, int ng, int64_t rows, int nkeep,
-                              const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s, int rt)
+                              const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s, int rt, int *clear)
 {
     using C = typename Cx<R>::T;
     if (rt <= 0) rt = int(fft_rows_per_block(ng, sizeof(C)));
@@ -1045,7 +1110,7 @@ cudaError_t launch_fft_z_real(const R *in, typename Cx<R>::T *out, int ng, int64
     const size_t smem = size_t(2) * rt * fft_stride<C>(ng, rt) * sizeof(C);
     const int64_t nblk = (rows / 2 + rt - 1) / rt;
     k_fft_z_real<R><<<dim3(unsigned(nblk), fb.nf), 256, smem, s>>>(in, out, ng, rows, nkeep, rt, tw, fb.fs_in,
-                                                                   fb.fs_out);
+                                                                   fb.fs_out, clear);
     return cudaGetLastError();
 }
 
@@ -1238,6 +1303,30 @@ cudaError_t launch_epilogue(int mode, const EpiArgs &e, const double *value, int
     return epilogue_lmax<W, W>(mode, e, value, l_lo, l_hi, den, norm, out, fb, s);
 }
 
+template <typename W>
+cudaError_t launch_epilogue_views(EpiViews ev, const double *value, double norm, const Batch &fb, cudaStream_t s,
+                                  bool fp32_weights)
+{
+    unsigned blk = 0, bin = 0;
+    int threads = 32;
+    for (int i = 0; i < ev.n; ++i) {
+        EpiView &v = ev.v[i];
+        if (v.l_hi < 0 || v.l_hi > 8 || (v.l_hi & 1)) return cudaErrorInvalidValue;
+        v.blk0 = blk;
+        v.bin0 = bin;
+        blk += unsigned((v.nchunks + 7) / 8);
+        bin += unsigned(v.nbins);
+        threads = std::max(threads, v.l_hi < 4 ? fin_threads<2>() : (v.l_hi < 8 ? fin_threads<6>() : fin_threads<8>()));
+    }
+    if (bin == 0) return cudaSuccess;
+    if (blk > 0) {
+        if (fp32_weights) k_epi_part_views<W, float><<<dim3(blk, fb.nf), 256, 0, s>>>(ev, value, fb.fs_in);
+        else k_epi_part_views<W, W><<<dim3(blk, fb.nf), 256, 0, s>>>(ev, value, fb.fs_in);
+    }
+    k_epi_fin_views<<<dim3(bin, fb.nf), threads, 0, s>>>(ev, norm, fb.fs_in, fb.fs_out);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_records_f(const Record *rec, RecordF *recf, int64_t n, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
@@ -1315,8 +1404,8 @@ cudaError_t set_ylm_constants(const double nlm[9][9], const double pref[9], cuda
 }
 
 // explicit instantiations
-template cudaError_t launch_fft_z_real<float>(const float *, float2 *, int, int64_t, int, const Twiddles<float2> &, const Batch &, cudaStream_t, int);
-template cudaError_t launch_fft_z_real<double>(const double *, double2 *, int, int64_t, int, const Twiddles<double2> &, const Batch &, cudaStream_t, int);
+template cudaError_t launch_fft_z_real<float>(const float *, float2 *, int, int64_t, int, const Twiddles<float2> &, const Batch &, cudaStream_t, int, int *);
+template cudaError_t launch_fft_z_real<double>(const double *, double2 *, int, int64_t, int, const Twiddles<double2> &, const Batch &, cudaStream_t, int, int *);
 template cudaError_t launch_fft_rows_T<float>(const float2 *, float2 *, int, int, int64_t, float, bool, const Twiddles<float2> &, const Batch &, cudaStream_t, int);
 template cudaError_t launch_fft_rows_T<double>(const double2 *, double2 *, int, int, int64_t, double, bool, const Twiddles<double2> &, const Batch &, cudaStream_t, int);
 template cudaError_t launch_fft_rows_split<float>(const float2 *, float *, int, int, int64_t, const Twiddles<float2> &, cudaStream_t);
@@ -1335,5 +1424,7 @@ template cudaError_t launch_epilogue<float>(int, const EpiArgs &, const double *
                                             double *, const Batch &, cudaStream_t, bool);
 template cudaError_t launch_epilogue<double>(int, const EpiArgs &, const double *, int, int, const double *, double,
                                              double *, const Batch &, cudaStream_t, bool);
+template cudaError_t launch_epilogue_views<float>(EpiViews, const double *, double, const Batch &, cudaStream_t, bool);
+template cudaError_t launch_epilogue_views<double>(EpiViews, const double *, double, const Batch &, cudaStream_t, bool);
 
 }  // namespace bisp

@@ -87,10 +87,12 @@ struct StepIIArgs {
 // --- launch helpers (kernels.cu); all return cudaGetLastError() --------------
 
 // z pass of the forward 3D transform: real rows of length ng -> kept
-// frequencies [0, nkeep) written transposed as out[k][row].
+// frequencies [0, nkeep) written transposed as out[k][row].  clear: an int of each
+// output region set to zero (a memset of its own cost as much as a small kernel).
 template <typename R>
 cudaError_t launch_fft_z_real(const R *in, typename Cx<R>::T *out, int ng, int64_t rows, int nkeep,
-                              const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s, int rt = 0);
+                              const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s, int rt = 0,
+                              int *clear = nullptr);
 
 // Batched row transforms written transposed: in[b][nrow][M] -> out[b][M][nrow],
 // times scale; zero_dc clears element [0][0] of batch 0.
@@ -187,7 +189,7 @@ cudaError_t launch_reduce_partials(const Group *groups, int64_t ngroups, const d
 // fp32_weights: the Y_lm of each record in FP32 (sums stay in W).
 // The records are walked in chunks of one bin each (one warp per chunk, FP64
 // partial sums per moment in `partial` [nchunks][moments of l <= l_hi]),
-// then each bin adds its chunks in order (one thread per bin).
+// then each bin adds its chunks in a fixed order (one block per bin).
 struct EpiArgs {
     const Record *rec;                    // fp32_weights: not read (recf is)
     const RecordF *recf;
@@ -201,6 +203,28 @@ struct EpiArgs {
 template <typename W>
 cudaError_t launch_epilogue(int mode, const EpiArgs &e, const double *value, int l_lo, int l_hi, const double *den,
                             double norm, double *out, const Batch &fb, cudaStream_t s, bool fp32_weights = false);
+
+// The same (mode 0) for all views of a plan in one launch per pass: the views do
+// not depend on one another, and at a few thousand chunks each a launch is short
+// and leaves most of the GPU idle.  blk0 and bin0 are the launcher's.
+struct EpiView {
+    const int64_t *chunk_lo, *chunk_hi, *bin_chunk;
+    int64_t nchunks, nbins;
+    double *partial;                      // this view's own [nchunks][moments of l <= l_hi]
+    const double *den;
+    double *out;
+    int l_hi, lm_lo, nlm;                 // first moment and moments written
+    unsigned blk0, bin0;                  // first block of the chunks' and of the bins' launch
+};
+struct EpiViews {
+    int n;
+    const Record *rec;
+    const RecordF *recf;
+    EpiView v[5];                         // even l <= 8
+};
+template <typename W>
+cudaError_t launch_epilogue_views(EpiViews ev, const double *value, double norm, const Batch &fb, cudaStream_t s,
+                                  bool fp32_weights);
 
 // The records' FP32 form.
 cudaError_t launch_records_f(const Record *rec, RecordF *recf, int64_t n, cudaStream_t s);

@@ -307,7 +307,7 @@ int arrange_lanes(const std::vector<int32_t> &key1, const std::vector<int32_t> &
 // whose fields fit kTcMinRing ring buffers of shared memory.  The last, partly
 // filled tiles of the sign patterns of one (grid, |n3|) are put into one tile
 // where they fit, each pattern in warps of its own (at 64^3 such tiles are most of
-// them: they filled 30% of their lanes, merged ones 53%).  Then units (tile,
+// them: they filled 30% of their lanes, merged ones 52%).  Then units (tile,
 // x chunk) by class.
 // Requires the groups' partial-sum layout.  Marks the fields the tiles read.
 template <typename UsedFn>
@@ -397,8 +397,8 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
         // another.  Colour the fields greedily (first appearance order) so
         // that the distinct D1 fields of each pass, and its distinct D2
         // fields, take distinct colours where they can, then move single
-        // fields to a colour that saves accesses while there are any (512^3:
-        // 6.1 -> 5.8 accesses for the two loads), and number them colour + 8 k;
+        // fields to a colour that saves accesses while there are any (256^3:
+        // 6.2 -> 6.0 accesses for the two loads), and number them colour + 8 k;
         // numbers left free are padding slots that hold a field nothing stores
         // (they read as zero).  Kept only if the tile still fits.
         const int ns = T.nslot;

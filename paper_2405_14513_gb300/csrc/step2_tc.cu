@@ -34,7 +34,14 @@
 // buffers holds 16 points, so the barriers, fences and accumulator reads, a
 // third of the time, came twice as often.  512^3, all of Step II: 587 ms with
 // TF32 pairs and 16-point stages, 462 ms so; the error against 64 bits fell
-// from 1.1e-6 to 0.7e-6 (2-norm over the bins, 128^3).
+// from 1.1e-6 to 0.7e-6 (2-norm over the bins, 128^3).  With lanes paired by
+// field (plan.cpp), tiles shared by sign patterns, one proxy fence per stage and
+// waits tested before they are polled it now takes 404 ms (256^3: 27.8 -> 17.0).
+//
+// What bounds it: the shared-memory reads of the two fields per row and point
+// and the issue around them.  At 256^3 (17.0 ms), leaving out one part at a time:
+// those reads 12.9 ms, the producers' copies 14.5, the B conversion 15.6, the
+// accumulator reads 16.7, the split of A into pairs 16.9.
 #include "kernels.cuh"
 
 #include <algorithm>
@@ -208,11 +215,10 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *m)
 // Bounded wait for phase `parity` of m; gives up (false) when the block is
 // aborting or after `spins` more polls, and then raises the abort flag.  The
 // first poll is a test_wait: most waits are over when they are reached.  A later
-// one
-// is a try_wait, which may suspend the thread for a while before it reports;
-// under kTestPolls polls (a limit set to exercise the give-up path) it is a
-// test_wait, which reports at once, so that such a limit really cuts the
-// wait short.
+// one is a try_wait, which may suspend the thread for a while before it reports
+// (256^3: 17.3 -> 17.0 ms against try_wait alone); under kTestPolls polls (a limit
+// set to exercise the give-up path) it is a test_wait, which reports at once, so
+// that such a limit really cuts the wait short.
 constexpr int kTestPolls = 64;
 __device__ __forceinline__ bool mbar_wait_abort(uint64_t *m, uint32_t parity, volatile int *abort, int spins)
 {
@@ -552,9 +558,9 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
     } else if (warp == 8) {
         // MMA issue: low A x high B, high A x low B and high A x high B over
         // the four k-steps of the stage: the small products first, so that the
-        // accumulator truncates at its full size only four times.  The whole warp runs the loop (all
-        // lanes wait, one elected lane issues), so that its operands are
-        // warp-uniform; a lane's wait that gives up stops the warp.
+        // accumulator truncates at its full size only four times.  The whole warp
+        // runs the loop (all lanes wait, one elected lane issues), so that its
+        // operands are warp-uniform; a lane's wait that gives up stops the warp.
         {
             const uint64_t dh = smem_desc(su32(sHi), LBO, SBO), dl = smem_desc(su32(sLo), LBO, SBO);
             int ia = 0;                                         // A / B buffer of stage st
@@ -571,8 +577,8 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
                 if (++qr == S) qr = 0;
                 // the compute threads' generic writes of B, which the barrier has
                 // ordered before this point, before the tensor core's reads: one
-                // fence here, on the way from the writes to the reads, in place of one by
-                // each of the writers
+                // fence here, on the way from the writes to the reads, in place of
+                // one by each of the writers (256^3: 18.1 -> 17.3 ms)
                 asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t a = tmem + 64 * ia;

@@ -1,6 +1,6 @@
 """Edges of the kernels' own forms: the FP16 pairs of scaled fields (tensor-core
-Step II), the moment counts of the binning's warp sums, and the shell fields
-packed two to a transform."""
+Step II), the moment counts of the binning's warp sums, views binned together, and
+the shell fields packed two to a transform."""
 import numpy as np
 import pytest
 
@@ -81,3 +81,26 @@ def test_shell_fields_in_pairs(ng, l_max):
     plan = api.ShellPlan(ng, L, edges, 3, 3, l_max)
     B = plan.estimate(torch.from_numpy(field).cuda(), plan.workspace()).cpu().numpy()
     assert _floored(B, ref) < 1e-4
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "mixed_tc"])
+@pytest.mark.parametrize("ng,bins", [(12, [3, 1]), (24, [2, 2, 1]), (32, [9, 5, 3, 2, 1]), (32, [2, 3, 3, 4, 4])])
+def test_views_binned_together(precision, ng, bins):
+    """Views of every l_hi, of few and of many bins, binned in one launch, two fields
+    at once: each equals, bit for bit, the same moments of a plan with that one view."""
+    L, l_max = 10.0 * ng, 2 * len(bins) - 2
+    edges = synth.default_k1_edges(ng, L, 3)
+    dt = np.float64 if precision == "fp64" else np.float32
+    d = torch.from_numpy(np.stack([synth.make_field(ng, L, s).astype(dt) for s in (7, 8)])).cuda()
+    plan = api.Plan(ng, L, edges, 1, 1, l_max, precision=precision, mu_t_bins_l=bins, max_batch=2)
+    assert len(plan.views) == len(set(bins))
+    ws = plan.workspace(2)
+    blocks = plan.split(plan.estimate(d, ws).cpu().numpy())
+    assert plan.workspace_status(ws, 2) == 0
+    for v, blk in zip(plan.views, blocks):
+        one = api.Plan(ng, L, edges, v["n_mu"], v["n_t"], l_max, precision=precision, max_batch=2)
+        want = one.estimate(d, one.workspace(2)).cpu().numpy()
+        lo = (v["l_lo"] // 2) ** 2
+        assert np.array_equal(blk, want[..., lo:lo + v["n_lm"]], equal_nan=True), v
+        one.close()
+    plan.close()
