@@ -305,6 +305,7 @@ k_fft_z_real(const R *__restrict__ in, typename Cx<R>::T *__restrict__ out, int 
 {
     using C = typename Cx<R>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    grid_begin();
     in = field_ptr(in, fs_in);
     out = field_ptr(out, fs_out);
     if (clear && blockIdx.x == 0 && threadIdx.x == 0) *field_ptr(clear, fs_out) = 0;
@@ -344,11 +345,12 @@ k_fft_z_real(const R *__restrict__ in, typename Cx<R>::T *__restrict__ out, int 
 // nsplit in all: real parts go to field 2 b, imaginary parts to field 2 b + 1 of `out`.
 template <typename R, bool SPLIT>
 __global__ void __launch_bounds__(256)
-k_fft_rows_T(const typename Cx<R>::T *__restrict__ in, typename Cx<R>::T *__restrict__ out, int M,
+k_fft_rows_T(const typename Cx<R>::T *in, typename Cx<R>::T *__restrict__ out, int M,
              int nrow, int ntile, R scale, int zero_dc, int rt, Twiddles<typename Cx<R>::T> tw, int64_t fs, int64_t nsplit)
 {
     using C = typename Cx<R>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    grid_begin();
     in = field_ptr(in, fs);
     out = field_ptr(out, fs);
     const int P = fft_stride<C>(M, rt);
@@ -391,8 +393,9 @@ k_fft_rows_T(const typename Cx<R>::T *__restrict__ in, typename Cx<R>::T *__rest
 // 384^3, this one a tenth of it).  Every sum is in a fixed order.  Empty or
 // non-finite rings get 1.
 __global__ void __launch_bounds__(256)
-k_ring_scale(const float2 *__restrict__ planes, int ng, RingArg rings, float *__restrict__ scale, int64_t fs)
+k_ring_scale(const float2 *planes, int ng, RingArg rings, float *__restrict__ scale, int64_t fs)
 {
+    grid_begin();
     planes = field_ptr(planes, fs);
     scale = field_ptr(scale, fs);
     const int r = blockIdx.x % rings.nr, n = blockIdx.x / rings.nr;
@@ -444,12 +447,13 @@ __device__ __forceinline__ const StepGrid &grid_of_block(const StepGrids &gs)
 
 template <typename R, bool UNIT>
 __global__ void __launch_bounds__(256)
-k_ring_gather(const typename Cx<R>::T *__restrict__ planes, int ng, const __grid_constant__ RingArg rings,
+k_ring_gather(const typename Cx<R>::T *planes, int ng, const __grid_constant__ RingArg rings,
               const __grid_constant__ StepGrids gs, typename Cx<R>::T *__restrict__ out,
-              Twiddles<typename Cx<R>::T> tw, const float *__restrict__ scale, int64_t fs)
+              Twiddles<typename Cx<R>::T> tw, const float *scale, int64_t fs)
 {
     using C = typename Cx<R>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    grid_begin();
     planes = field_ptr(planes, fs);
     out = field_ptr(out, fs);
     scale = scale ? field_ptr(scale, fs) : scale;
@@ -516,11 +520,12 @@ k_ring_gather(const typename Cx<R>::T *__restrict__ planes, int ng, const __grid
 // twiddles, and a thread's column is the same throughout.
 template <typename R>
 __global__ void __launch_bounds__(256)
-k_fft_cols(typename Cx<R>::T *__restrict__ out, const __grid_constant__ StepGrids gs,
+k_fft_cols(typename Cx<R>::T *out, const __grid_constant__ StepGrids gs,
            const __grid_constant__ RingArg rings, Twiddles<typename Cx<R>::T> tw, int64_t fs)
 {
     using C = typename Cx<R>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    grid_begin();
     out = field_ptr(out, fs);
     const StepGrid &gr = grid_of_block(gs);
     const int M = gr.M, w = gr.rt;
@@ -587,6 +592,7 @@ template <typename R, int NW>
 __global__ void __launch_bounds__(32 * NW, (sizeof(R) == 8 ? 8 : 16) / NW)
 k_step2(StepIIArgs args, int64_t unit0, const typename Cx<R>::T *__restrict__ dstore, int smem_bytes)
 {
+    grid_begin();
     dstore = field_ptr(dstore, args.fs);
     args.partials = field_ptr(args.partials, args.fs);
     using C = typename Cx<R>::T;
@@ -757,9 +763,10 @@ k_step2(StepIIArgs args, int64_t unit0, const typename Cx<R>::T *__restrict__ ds
 
 template <typename A>
 __global__ void __launch_bounds__(256)
-k_reduce(const Group *__restrict__ groups, int64_t ngroups, const double *__restrict__ partials, int ng,
+k_reduce(const Group *__restrict__ groups, int64_t ngroups, const double *partials, int ng,
          double *__restrict__ S, int64_t fs)
 {
+    grid_begin();
     partials = field_ptr(partials, fs);
     S = field_ptr(S, fs);
     // one warp per group: groups hold 14 (64^3) to 140 (512^3) combinations
@@ -832,7 +839,7 @@ template <typename W, typename Y, int LMAX>
 __device__ __forceinline__ void
 epi_part(int mode, const Record *__restrict__ rec, const RecordF *__restrict__ recf,
          const int64_t *__restrict__ chunk_lo, const int64_t *__restrict__ chunk_hi, int64_t nchunks, int64_t ch,
-         const double *__restrict__ value, double *__restrict__ partial, int64_t fs_in, int64_t fs_part)
+         const double *value, double *__restrict__ partial, int64_t fs_in, int64_t fs_part)
 {
     constexpr bool F32 = sizeof(Y) == 4;                  // FP32 weights (mode 0 only)
     constexpr bool WIDEN = F32 && sizeof(W) == 8;
@@ -935,8 +942,9 @@ template <typename W, typename Y, int LMAX>
 __global__ void __launch_bounds__(256)
 k_epi_part(int mode, const Record *__restrict__ rec, const RecordF *__restrict__ recf,
            const int64_t *__restrict__ chunk_lo, const int64_t *__restrict__ chunk_hi, int64_t nchunks,
-           const double *__restrict__ value, double *__restrict__ partial, int64_t fs_in, int64_t fs_part)
+           const double *value, double *__restrict__ partial, int64_t fs_in, int64_t fs_part)
 {
+    grid_begin();
     epi_part<W, Y, LMAX>(mode, rec, recf, chunk_lo, chunk_hi, nchunks, (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5,
                          value, partial, fs_in, fs_part);
 }
@@ -952,8 +960,9 @@ template <bool FIN> __device__ __forceinline__ const EpiView &view_of_block(cons
 // k_epi_part (mode 0) for several views in one launch
 template <typename W, typename Y>
 __global__ void __launch_bounds__(256)
-k_epi_part_views(const __grid_constant__ EpiViews ev, const double *__restrict__ value, int64_t fs_in)
+k_epi_part_views(const __grid_constant__ EpiViews ev, const double *value, int64_t fs_in)
 {
+    grid_begin();
     const EpiView &v = view_of_block<false>(ev);
     const int64_t ch = int64_t(blockIdx.x - v.blk0) * 8 + (threadIdx.x >> 5);
     auto run = [&](auto lmax) {
@@ -982,7 +991,7 @@ template <int LMAX> constexpr int fin_threads()
 }
 template <int LMAX>
 __device__ __forceinline__ void
-epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *__restrict__ partial,
+epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *partial,
         const double *__restrict__ den, double norm, double *__restrict__ out, int64_t fs_part, int64_t fs_out,
         int lm_lo, int nlm_out, int64_t b, double *red)
 {
@@ -1013,11 +1022,12 @@ epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *__restric
 
 template <int LMAX>
 __global__ void __launch_bounds__(fin_threads<LMAX>())
-k_epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *__restrict__ partial,
+k_epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *partial,
           const double *__restrict__ den, double norm, double *__restrict__ out, int64_t fs_part, int64_t fs_out,
           int lm_lo, int nlm_out)
 {
     __shared__ double red[fin_threads<LMAX>()];
+    grid_begin();
     epi_fin<LMAX>(mode, bin_chunk, partial, den, norm, out, fs_part, fs_out, lm_lo, nlm_out, blockIdx.x, red);
 }
 
@@ -1026,6 +1036,7 @@ __global__ void __launch_bounds__(256)
 k_epi_fin_views(const __grid_constant__ EpiViews ev, double norm, int64_t fs_part, int64_t fs_out)
 {
     __shared__ double red[256];
+    grid_begin();
     const EpiView &v = view_of_block<true>(ev);
     const int64_t b = blockIdx.x - v.bin0;
     auto run = [&](auto lmax) {
@@ -1126,9 +1137,8 @@ cudaError_t launch_fft_rows_T(const typename Cx<R>::T *in, typename Cx<R>::T *ou
     const int ntile = (nrow + rt - 1) / rt;
     const int64_t nblk = nb * ntile;
     if (nblk == 0) return cudaSuccess;
-    k_fft_rows_T<R, false><<<dim3(unsigned(nblk), fb.nf), 256, smem, s>>>(in, out, M, nrow, ntile, scale,
-                                                                          zero_dc ? 1 : 0, rt, tw, fb.fs_in, 0);
-    return cudaGetLastError();
+    return launch_next(k_fft_rows_T<R, false>, dim3(unsigned(nblk), fb.nf), 256, smem, s, in, out, M, nrow, ntile, scale,
+                       zero_dc ? 1 : 0, rt, tw, fb.fs_in, 0);
 }
 
 template <typename R>
@@ -1141,9 +1151,8 @@ cudaError_t launch_fft_rows_split(const typename Cx<R>::T *in, R *out, int M, in
     const int ntile = (nrow + rt - 1) / rt;
     const int64_t nblk = (nf + 1) / 2 * ntile;
     if (nblk == 0) return cudaSuccess;
-    k_fft_rows_T<R, true><<<unsigned(nblk), 256, smem, s>>>(in, reinterpret_cast<C *>(out), M, nrow, ntile, R(1), 0, rt, tw, 0,
-                                                            nf);
-    return cudaGetLastError();
+    return launch_next(k_fft_rows_T<R, true>, unsigned(nblk), 256, smem, s, in, reinterpret_cast<C *>(out), M, nrow, ntile, R(1),
+                       0, rt, tw, 0, nf);
 }
 
 // Shared-memory buffers of a Step-I transform of length M: its stages hand the
@@ -1201,18 +1210,14 @@ cudaError_t launch_ring_gather(const typename Cx<R>::T *planes, int ng, const Ri
     if (nblk == 0) return cudaSuccess;
     const dim3 grid(nblk, fb.nf);
     const unsigned threads = step_threads(gs);
-    if (unit)
-        k_ring_gather<R, true><<<grid, threads, smem, s>>>(planes, ng, rings, gs, out, tw, scale, fb.fs_in);
-    else
-        k_ring_gather<R, false><<<grid, threads, smem, s>>>(planes, ng, rings, gs, out, tw, scale, fb.fs_in);
-    return cudaGetLastError();
+    return launch_next(unit ? k_ring_gather<R, true> : k_ring_gather<R, false>, grid, threads, smem, s, planes, ng, rings, gs,
+                       out, tw, scale, fb.fs_in);
 }
 
 cudaError_t launch_ring_scale(const float2 *planes, int ng, int nz1, const RingArg &rings, float *scale,
                               const Batch &fb, cudaStream_t s)
 {
-    k_ring_scale<<<dim3(unsigned(nz1 * rings.nr), fb.nf), 256, 0, s>>>(planes, ng, rings, scale, fb.fs_in);
-    return cudaGetLastError();
+    return launch_next(k_ring_scale, dim3(unsigned(nz1 * rings.nr), fb.nf), 256, 0, s, planes, ng, rings, scale, fb.fs_in);
 }
 
 template <typename R>
@@ -1223,8 +1228,7 @@ cudaError_t launch_fft_cols(typename Cx<R>::T *out, StepGrids gs, const RingArg 
     size_t smem;
     if (cudaError_t e = step_blocks<typename Cx<R>::T>(gs, true, &nblk, &smem); e != cudaSuccess) return e;
     if (nblk == 0) return cudaSuccess;
-    k_fft_cols<R><<<dim3(nblk, fb.nf), step_threads(gs), smem, s>>>(out, gs, rings, tw, fb.fs_in);
-    return cudaGetLastError();
+    return launch_next(k_fft_cols<R>, dim3(nblk, fb.nf), step_threads(gs), smem, s, out, gs, rings, tw, fb.fs_in);
 }
 
 template <typename R, int NW>
@@ -1232,8 +1236,7 @@ cudaError_t launch_step2_class(const StepIIArgs &a, const typename Cx<R>::T *dst
                                size_t smem, int nf, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    k_step2<R, NW><<<dim3(unsigned(n), nf), 32 * NW, smem, s>>>(a, u0, dstore, int(smem));
-    return cudaGetLastError();
+    return launch_next(k_step2<R, NW>, dim3(unsigned(n), nf), 32 * NW, smem, s, a, u0, dstore, int(smem));
 }
 
 template <typename R>
@@ -1261,8 +1264,7 @@ cudaError_t launch_reduce_partials(const Group *groups, int64_t ngroups, const d
                                    double *S, const Batch &fb, cudaStream_t s)
 {
     if (ngroups == 0) return cudaSuccess;
-    k_reduce<A><<<dim3(unsigned((ngroups + 7) / 8), fb.nf), 256, 0, s>>>(groups, ngroups, partials, ng, S, fb.fs_in);
-    return cudaGetLastError();
+    return launch_next(k_reduce<A>, dim3(unsigned((ngroups + 7) / 8), fb.nf), 256, 0, s, groups, ngroups, partials, ng, S, fb.fs_in);
 }
 
 template <typename W, typename Y, int LMAX>
@@ -1270,11 +1272,14 @@ cudaError_t epilogue_l(int mode, const EpiArgs &e, const double *value, const do
                        const Batch &fb, int lo, int n, cudaStream_t s)
 {
     const dim3 g1(unsigned((e.nchunks * 32 + 255) / 256), fb.nf), g2(unsigned(e.nbins), fb.nf);
+    cudaError_t st = cudaSuccess;
     if (e.nchunks > 0)
-        k_epi_part<W, Y, LMAX><<<g1, 256, 0, s>>>(mode, e.rec, e.recf, e.chunk_lo, e.chunk_hi, e.nchunks, value, e.partial,
-                                                  fb.fs_in, e.fs_part);
-    k_epi_fin<LMAX><<<g2, fin_threads<LMAX>(), 0, s>>>(mode, e.bin_chunk, e.partial, den, norm, out, e.fs_part, fb.fs_out, lo, n);
-    return cudaGetLastError();
+        st = launch_next(k_epi_part<W, Y, LMAX>, g1, 256, 0, s, mode, e.rec, e.recf, e.chunk_lo, e.chunk_hi, e.nchunks, value,
+                         e.partial, fb.fs_in, e.fs_part);
+    if (st == cudaSuccess)
+        st = launch_next(k_epi_fin<LMAX>, g2, fin_threads<LMAX>(), 0, s, mode, e.bin_chunk, e.partial, den, norm, out,
+                         e.fs_part, fb.fs_out, lo, n);
+    return st;
 }
 
 template <typename W, typename Y>
@@ -1320,11 +1325,11 @@ cudaError_t launch_epilogue_views(EpiViews ev, const double *value, double norm,
     }
     if (bin == 0) return cudaSuccess;
     if (blk > 0) {
-        if (fp32_weights) k_epi_part_views<W, float><<<dim3(blk, fb.nf), 256, 0, s>>>(ev, value, fb.fs_in);
-        else k_epi_part_views<W, W><<<dim3(blk, fb.nf), 256, 0, s>>>(ev, value, fb.fs_in);
+        const cudaError_t e = launch_next(fp32_weights ? k_epi_part_views<W, float> : k_epi_part_views<W, W>, dim3(blk, fb.nf),
+                                          256, 0, s, ev, value, fb.fs_in);
+        if (e != cudaSuccess) return e;
     }
-    k_epi_fin_views<<<dim3(bin, fb.nf), threads, 0, s>>>(ev, norm, fb.fs_in, fb.fs_out);
-    return cudaGetLastError();
+    return launch_next(k_epi_fin_views, dim3(bin, fb.nf), threads, 0, s, ev, norm, fb.fs_in, fb.fs_out);
 }
 
 cudaError_t launch_records_f(const Record *rec, RecordF *recf, int64_t n, cudaStream_t s)

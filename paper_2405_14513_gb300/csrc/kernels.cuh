@@ -84,6 +84,38 @@ struct StepIIArgs {
     int64_t fs;              // bytes between the workspace regions of the fields of a batch
 };
 
+// The kernels of an estimate follow one another on a stream, each reading what the
+// one before wrote, and at small N_g each lasts a few us: they are launched with
+// programmatic stream serialisation, so that a kernel's blocks are placed while the
+// last blocks of the one before still run.  Every kernel so launched, and the first of
+// an estimate, calls grid_begin before it reads or writes global memory that another
+// kernel writes or reads: the next kernel may be placed from here on; this one
+// goes on when every kernel before it has completed (each waits so, also blocks
+// without work) and its writes are visible.  Pointers to such memory are not
+// __restrict__: the compiler may then neither take the read-only path, which is for
+// data that nobody writes while the kernel lasts, nor move their loads before the wait.
+// 32^3 (11 kernels) 79 -> 59 us, 48^3 x 3 202 -> 177, 64^3 173 -> 161; from 128^3 on, 2% of Step I.
+__device__ __forceinline__ void grid_begin()
+{
+    asm volatile("griddepcontrol.launch_dependents;\ngriddepcontrol.wait;\n" ::: "memory");
+}
+template <typename... P, typename... A>
+cudaError_t launch_next(void (*k)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A &&...args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&c, k, P(args)...);
+    return e == cudaSuccess ? e : cudaGetLastError();
+}
+
 // --- launch helpers (kernels.cu); all return cudaGetLastError() --------------
 
 // z pass of the forward 3D transform: real rows of length ng -> kept

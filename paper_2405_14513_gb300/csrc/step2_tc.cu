@@ -534,6 +534,7 @@ k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    grid_begin();                                // the plan's tables apart, nothing was read before
     const uint32_t tmem = sy->tmem;
     volatile int *abort = &sy->abort;
 
@@ -653,8 +654,7 @@ template <int NC>
 cudaError_t launch_class(const TcArgs &a, const float2 *dstore, int64_t u0, int64_t n, int nf, cudaStream_t s)
 {
     if (n == 0) return cudaSuccess;
-    k_step2_tc<NC><<<dim3(unsigned(n), unsigned(nf)), kThreads, kTcSmem, s>>>(a, u0, dstore);
-    return cudaGetLastError();
+    return launch_next(k_step2_tc<NC>, dim3(unsigned(n), unsigned(nf)), kThreads, kTcSmem, s, a, u0, dstore);
 }
 
 }  // namespace

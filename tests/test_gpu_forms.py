@@ -104,3 +104,29 @@ def test_views_binned_together(precision, ng, bins):
         assert np.array_equal(blk, want[..., lo:lo + v["n_lm"]], equal_nan=True), v
         one.close()
     plan.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed", "mixed_tc"])
+@pytest.mark.parametrize("ng", [8, 32, 64])
+def test_back_to_back_estimates_wait_for_each_other(precision, ng):
+    """The kernels of an estimate are placed before the ones ahead of them end: forty
+    estimates of alternating fields in one workspace, the input written by the kernel
+    ahead and the output read by the one behind, none synchronised, give the bits of
+    single ones."""
+    L = 10.0 * ng
+    dt = torch.float64 if precision == "fp64" else torch.float32
+    plan = api.Plan(ng, L, synth.default_k1_edges(ng, L, 2), 4, 4, 4, precision=precision)
+    ws = plan.workspace()
+    fields = [torch.from_numpy(synth.make_field(ng, L, s)).to("cuda", dt) for s in (1, 2)]
+    want = []
+    for f in fields:
+        want.append(plan.estimate(f, ws).cpu().numpy())
+    buf = torch.empty_like(fields[0])
+    got = []
+    for i in range(40):
+        buf.copy_(fields[i % 2])
+        got.append(plan.estimate(buf, ws).clone())
+        buf.zero_()
+    for i, g in enumerate(got):
+        assert np.array_equal(g.cpu().numpy(), want[i % 2], equal_nan=True), i
+    plan.close()
