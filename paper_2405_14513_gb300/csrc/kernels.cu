@@ -594,6 +594,9 @@ k_step2(StepIIArgs args, int64_t unit0, const typename Cx<R>::T *__restrict__ ds
 {
     grid_begin();
     dstore = field_ptr(dstore, args.fs);
+    // an address of its own to the compiler, which otherwise works out that of every
+    // copy from the kernel's arguments anew (128^3: 3.79 -> 3.49 ms)
+    asm volatile("" : "+l"(dstore));
     args.partials = field_ptr(args.partials, args.fs);
     using C = typename Cx<R>::T;
     constexpr int NT = 32 * NW;
