@@ -910,8 +910,8 @@ int estimator_plan_info(const bisp_plan *p, bisp_plan_info *info)
             const double m2 = double(T.M) * T.M;
             info->tc_row_points += double(T.nrow) * m2;
             info->tc_lane_points += double(kTcRows) * m2;
-            // every stage stages each slot and window field (16 points, 8 bytes each)
-            info->tc_staged_bytes += double(T.nslot + T.ncol) * m2 * 8.0;
+            // every grid point of each slot and window field, 8 bytes
+            info->tc_staged_bytes += double(T.nslot + T.nwin) * m2 * 8.0;
         }
     return BISP_OK;
 }

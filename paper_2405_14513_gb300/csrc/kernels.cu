@@ -570,8 +570,9 @@ k_fft_cols(typename Cx<R>::T *out, const __grid_constant__ StepGrids gs,
 // constant 64 or 128 points, slot addresses in registers, one piece column per
 // thread, signs on sign bits), and the warps that a unit's tiles leave over take
 // turns at the points (128^3: 61% of the warp slots had a tile).  Without these
-// 128^3 took 6.3 ms and 96^3 x 2 3.6 ms, with them 3.8 and 2.1; FP64 at 64^3 4.3
-// and 2.2 ms, most of it from the entries left out.
+// 128^3 took 6.3 ms and 96^3 x 2 3.6 ms, with them 3.8 and 2.1 (128^3 with the
+// store's base address in registers 3.5); FP64 at 64^3 4.3 and 2.2 ms, most of it
+// from the entries left out.
 // (The asm statements below clobber memory at the barriers' sides only, so
 // the loads of a stage may move among each other.)
 template <typename C> __device__ __forceinline__ C lds_complex(uint32_t a)
