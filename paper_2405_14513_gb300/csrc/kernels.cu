@@ -11,7 +11,7 @@
 //   k_ring_scale    power-of-two factors of the D fields (tensor-core Step II)
 //   k_step2         Step II: partial triple sums sum_x D1 D2 D3 (Eq. fftbs)
 //   k_reduce        partial sums -> S per combination, grid normalisation
-//   k_epilogue      Y_lm weights, (k1, mu, t) binning and the ratio of
+//   k_epi_part, k_epi_fin  Y_lm weights, (k1, mu, t) binning and the ratio of
 //                   Eq. bs_lm2_1; or the plan-time denominators
 //   k_ntri          N_tri = M^-2 sum_y I1 I2 I3 on the unit fields (Eq. Ntri2)
 //
