@@ -5,6 +5,8 @@
 //                   keeping planes 0..N_g/3, written plane-major
 //   k_fft_rows_T    batched row transforms written transposed (the y and x
 //                   passes of the forward transform)
+//   k_fft_z_back    real fields from their half spectra, along the line of sight
+//                   (the shell estimator's fields)
 //   k_ring_gather   Step I first pass: ring mask (and fold onto the M x M
 //                   reduction grid) fused into the load, transform along u_y
 //   k_fft_cols      Step I second pass: transform along u_x, in place
@@ -341,12 +343,10 @@ k_fft_z_real(const R *__restrict__ in, typename Cx<R>::T *__restrict__ out, int 
     }
 }
 
-// nsplit = 0: complex output.  nsplit > 0: the arrays hold two real fields each,
-// nsplit in all: real parts go to field 2 b, imaginary parts to field 2 b + 1 of `out`.
-template <typename R, bool SPLIT>
+template <typename R>
 __global__ void __launch_bounds__(256)
 k_fft_rows_T(const typename Cx<R>::T *in, typename Cx<R>::T *__restrict__ out, int M,
-             int nrow, int ntile, R scale, int zero_dc, int rt, Twiddles<typename Cx<R>::T> tw, int64_t fs, int64_t nsplit)
+             int nrow, int ntile, R scale, int zero_dc, int rt, Twiddles<typename Cx<R>::T> tw, int64_t fs)
 {
     using C = typename Cx<R>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -364,20 +364,62 @@ k_fft_rows_T(const typename Cx<R>::T *in, typename Cx<R>::T *__restrict__ out, i
     const C *res = fft_any<C, false, true, false>(M, nr, 0, P, a, b, tw.t, [&](int r, int i) { return src[r * M + i]; },
                                                   NoStore{});
     C *dst = out + bt * int64_t(M) * nrow;
-    R *re = reinterpret_cast<R *>(out) + 2 * bt * int64_t(M) * nrow, *im = re + int64_t(M) * nrow;
     DivIter st(threadIdx.x, blockDim.x, nr);
     for (int t = threadIdx.x; t < M * nr; t += blockDim.x, st.next()) {
         const int k = st.q, r = st.r;
         C v = res[r * P + spos(k)];
-        if (SPLIT) {
-            re[int64_t(k) * nrow + row0 + r] = v.x;
-            if (2 * bt + 1 < nsplit) im[int64_t(k) * nrow + row0 + r] = v.y;
-            continue;
-        }
         v.x *= scale;
         v.y *= scale;
         if (zero_dc && bt == 0 && row0 + r == 0 && k == 0) v = cmk<C>(0.0, 0.0);
         dst[int64_t(k) * nrow + row0 + r] = v;
+    }
+}
+
+// Real fields of half spectra in[f][k][p], k < nkeep along the line of sight, p the
+// M^2 points of a plane: out[f][p][z] = Re A_0 + sum over 0 < k < nkeep of
+// 2 Re(A_k exp(-2 pi i kz / M)) (A_{-k} = conj A_k).  Two rows A, B share a transform
+// of A + i B, neighbours of one field, so that a field's rounding errors are those
+// of its own size whatever the other fields hold.  A block takes w = 2^lgw pairs: the
+// threads run across them, so that the loads are runs of 2 w elements of a plane, and
+// the rows leave shared memory whole.  Bound by its loads and stores.
+template <typename R>
+__global__ void __launch_bounds__(256)
+k_fft_z_back(const typename Cx<R>::T *in, R *__restrict__ out, int M, int nkeep, int ntile, int lgw,
+             Twiddles<typename Cx<R>::T> tw)
+{
+    using C = typename Cx<R>::T;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    grid_begin();
+    const int w = 1 << lgw, npos = M * M;
+    const int P = fft_stride<C>(M, w);
+    C *a = reinterpret_cast<C *>(smem_raw);
+    C *b = a + w * P;
+    const int64_t f = blockIdx.x / ntile;
+    const int p0 = int(blockIdx.x - f * ntile) * 2 * w;
+    const int nr = min(w, (npos - p0) / 2);        // pairs of rows (npos is even)
+    const C *src = in + f * nkeep * npos + p0;
+    auto load = [&](int r, int i) {
+        const bool neg = 2 * i > M;                // A_{i - M} = conj A_{M - i}
+        const int k = neg ? M - i : i;
+        if (k >= nkeep) return cmk<C>(0.0, 0.0);
+        const C *q = src + int64_t(k) * npos + 2 * r;
+        const C u = q[0], v = q[1];
+        C x;
+        if (k == 0) {                              // real
+            x.x = u.x;
+            x.y = v.x;
+        } else {
+            x.x = neg ? u.x + v.y : u.x - v.y;
+            x.y = neg ? v.x - u.y : v.x + u.y;
+        }
+        return x;
+    };
+    const C *res = fft_any<C, true, true, false>(M, nr, lgw, P, a, b, tw.t, load, NoStore{});
+    R *dst = out + (f * npos + p0) * M;
+    DivIter st(threadIdx.x, blockDim.x, M);
+    for (int t = threadIdx.x; t < 2 * nr * M; t += blockDim.x, st.next()) {
+        const C v = res[(st.q >> 1) * P + spos(st.r)];
+        dst[t] = (st.q & 1) ? v.y : v.x;
     }
 }
 
@@ -1141,22 +1183,23 @@ cudaError_t launch_fft_rows_T(const typename Cx<R>::T *in, typename Cx<R>::T *ou
     const int ntile = (nrow + rt - 1) / rt;
     const int64_t nblk = nb * ntile;
     if (nblk == 0) return cudaSuccess;
-    return launch_next(k_fft_rows_T<R, false>, dim3(unsigned(nblk), fb.nf), 256, smem, s, in, out, M, nrow, ntile, scale,
-                       zero_dc ? 1 : 0, rt, tw, fb.fs_in, 0);
+    return launch_next(k_fft_rows_T<R>, dim3(unsigned(nblk), fb.nf), 256, smem, s, in, out, M, nrow, ntile, scale,
+                       zero_dc ? 1 : 0, rt, tw, fb.fs_in);
 }
 
 template <typename R>
-cudaError_t launch_fft_rows_split(const typename Cx<R>::T *in, R *out, int M, int nrow, int64_t nf,
-                                  const Twiddles<typename Cx<R>::T> &tw, cudaStream_t s)
+cudaError_t launch_fft_z_back(const typename Cx<R>::T *in, R *out, int M, int nkeep, int64_t nf,
+                              const Twiddles<typename Cx<R>::T> &tw, cudaStream_t s)
 {
     using C = typename Cx<R>::T;
-    const int rt = std::min(int(fft_rows_per_block(M, sizeof(C))), nrow);
-    const size_t smem = size_t(2) * rt * fft_stride<C>(M, rt) * sizeof(C);
-    const int ntile = (nrow + rt - 1) / rt;
-    const int64_t nblk = (nf + 1) / 2 * ntile;
+    const int lgw = sizeof(R) == 4 ? 4 : 3, w = 1 << lgw;      // 256 bytes of a plane per load
+    const size_t smem = size_t(2) * w * fft_stride<C>(M, w) * sizeof(C);
+    if (M % 2 || 2 * nkeep > M + 1 || smem > 48 * 1024) return cudaErrorInvalidValue;
+    const int ntile = (M * M / 2 + w - 1) / w;
+    const int64_t nblk = nf * ntile;
+    if (nblk > 0x7FFFFFFF) return cudaErrorInvalidValue;
     if (nblk == 0) return cudaSuccess;
-    return launch_next(k_fft_rows_T<R, true>, unsigned(nblk), 256, smem, s, in, reinterpret_cast<C *>(out), M, nrow, ntile, R(1),
-                       0, rt, tw, 0, nf);
+    return launch_next(k_fft_z_back<R>, unsigned(nblk), 256, smem, s, in, out, M, nkeep, ntile, lgw, tw);
 }
 
 // Shared-memory buffers of a Step-I transform of length M: its stages hand the
@@ -1355,10 +1398,8 @@ cudaError_t init_kernel_attributes()
     };
     set((const void *)k_fft_z_real<float>);
     set((const void *)k_fft_z_real<double>);
-    set((const void *)k_fft_rows_T<float, false>);
-    set((const void *)k_fft_rows_T<float, true>);
-    set((const void *)k_fft_rows_T<double, false>);
-    set((const void *)k_fft_rows_T<double, true>);
+    set((const void *)k_fft_rows_T<float>);
+    set((const void *)k_fft_rows_T<double>);
     set((const void *)k_fft_cols<float>);
     set((const void *)k_fft_cols<double>);
     set((const void *)k_ring_gather<float, false>);
@@ -1417,8 +1458,8 @@ template cudaError_t launch_fft_z_real<float>(const float *, float2 *, int, int6
 template cudaError_t launch_fft_z_real<double>(const double *, double2 *, int, int64_t, int, const Twiddles<double2> &, const Batch &, cudaStream_t, int, int *);
 template cudaError_t launch_fft_rows_T<float>(const float2 *, float2 *, int, int, int64_t, float, bool, const Twiddles<float2> &, const Batch &, cudaStream_t, int);
 template cudaError_t launch_fft_rows_T<double>(const double2 *, double2 *, int, int, int64_t, double, bool, const Twiddles<double2> &, const Batch &, cudaStream_t, int);
-template cudaError_t launch_fft_rows_split<float>(const float2 *, float *, int, int, int64_t, const Twiddles<float2> &, cudaStream_t);
-template cudaError_t launch_fft_rows_split<double>(const double2 *, double *, int, int, int64_t, const Twiddles<double2> &, cudaStream_t);
+template cudaError_t launch_fft_z_back<float>(const float2 *, float *, int, int, int64_t, const Twiddles<float2> &, cudaStream_t);
+template cudaError_t launch_fft_z_back<double>(const double2 *, double *, int, int, int64_t, const Twiddles<double2> &, cudaStream_t);
 template cudaError_t launch_ring_gather<float>(const float2 *, int, const RingArg &, StepGrids, bool, float2 *, const Twiddles<float2> &, const Batch &, cudaStream_t, const float *);
 template cudaError_t launch_ring_gather<double>(const double2 *, int, const RingArg &, StepGrids, bool, double2 *, const Twiddles<double2> &, const Batch &, cudaStream_t, const float *);
 template cudaError_t launch_fft_cols<float>(float2 *, StepGrids, const RingArg &, const Twiddles<float2> &, const Batch &, cudaStream_t);

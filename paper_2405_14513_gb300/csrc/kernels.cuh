@@ -134,11 +134,11 @@ cudaError_t launch_fft_rows_T(const typename Cx<R>::T *in, typename Cx<R>::T *ou
                               const Twiddles<typename Cx<R>::T> &tw, const Batch &fb, cudaStream_t s,
                               int rt = 0);
 
-// The same of arrays that hold two real transforms each (real and imaginary
-// parts), nf in all, written apart: out[f][M][nrow].
+// Real fields out[f][p][z], f < nf, p < M^2, from half spectra in[f][k][p], k < nkeep
+// <= M/2 along the line of sight (of k = 0 the real part counts).  M even, at most 128.
 template <typename R>
-cudaError_t launch_fft_rows_split(const typename Cx<R>::T *in, R *out, int M, int nrow, int64_t nf,
-                                  const Twiddles<typename Cx<R>::T> &tw, cudaStream_t s);
+cudaError_t launch_fft_z_back(const typename Cx<R>::T *in, R *out, int M, int nkeep, int64_t nf,
+                              const Twiddles<typename Cx<R>::T> &tw, cudaStream_t s);
 
 // Step I, first pass: for every job of the grids, ring r of plane n of Delta
 // (planes [nz+1][ng][ng]), folded onto the M x M grid, transformed along u_y,

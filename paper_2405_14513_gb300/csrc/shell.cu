@@ -22,9 +22,9 @@
 //
 // Plan: shell table, triples, and the field-independent N_tri and den_l
 // from FP64 unit fields.  Estimate: the forward transform (the kernels of
-// the main path), the weighted shell spectra of every shell, two fields to a
-// complex array, 3D transforms (three passes of the row transform, each a cyclic
-// transpose), FP32 fields, FP32 triple products summed in pairs of floats and in
+// the main path), the weighted shell spectra of every shell (their planes n >= 0),
+// 3D transforms to real fields (two passes of the row transform, then the line of
+// sight), FP32 fields, FP32 triple products summed in pairs of floats and in
 // FP64, binning.  Lengths N_g <= 128
 // (the plan's FP64 sums over N_g^3 points per triple grow as N_g^6).
 #include "kernels.cuh"
@@ -65,65 +65,40 @@ __device__ __forceinline__ double y_l0(int l, double z)
     return sqrt((2.0 * l + 1.0) / (2.0 * kShellTwoPi)) * p;
 }
 
-// The weighted spectrum of one job at mode (i, j, n), FFT indices (a, b, .) of
-// k_x and k_y; Delta from the kept planes n >= 0 ([n][k_x][k_y]) and
-// Delta(k_x, k_y, -n) = conj Delta(-k_x, -k_y, n).
-template <typename C>
-__device__ __forceinline__ C shell_mode(const C *__restrict__ planes, int ng, const int64_t *__restrict__ e3sq, const ShellJob &J,
-                                        int a, int b, int i, int j, int n)
-{
-    C v;
-    v.x = 0;
-    v.y = 0;
-    const int q = i * i + j * j + n * n;
-    if (9 * int64_t(q) < e3sq[J.s] || 9 * int64_t(q) >= e3sq[J.s + 1]) return v;
-    double w = 1.0;
-    if (J.kind == 1 || J.kind == 3) {
-        const double y = y_l0(J.l, double(n) / sqrt(double(q)));
-        w = J.kind == 1 ? y : y * y;
-    }
-    if (J.kind <= 1) {
-        C d;
-        if (n >= 0) {
-            d = planes[(int64_t(n) * ng + a) * ng + b];
-        } else {
-            d = planes[(int64_t(-n) * ng + (ng - a) % ng) * ng + (ng - b) % ng];
-            d.y = -d.y;
-        }
-        v.x = decltype(v.x)(double(d.x) * w);
-        v.y = decltype(v.y)(double(d.y) * w);
-    } else {
-        v.x = decltype(v.x)(w);
-    }
-    return v;
-}
-
-// Weighted shell spectra on the N_g^3 grid, [pair][a][b][c] with (a, b, c) the
-// FFT indices of (k_x, k_y, k_z).  Every shell field is real, so two jobs share
-// a complex transform: X = A + i B (the last of an odd number has B = 0).
+// Weighted shell spectra, the planes n >= 0 of each: out[job][n][a][b], (a, b) the FFT
+// indices of (k_x, k_y), n < nz1, from the kept planes of Delta ([n][k_x][k_y]).  The
+// other half is the conjugate of (-k_x, -k_y, n): the fields are real.  (Full spectra
+// of two fields in one complex transform gave a field the error of the larger of the
+// two: with every third shell 1000 times its neighbours, 1e-5 to 2e-4 of the 2-norm of
+// a triple's products, where a field by itself has less than 2e-6.)
 template <typename C>
 __global__ void __launch_bounds__(256)
-k_shell_spectrum(const C *__restrict__ planes, int ng, const int64_t *__restrict__ e3sq,
-                 const ShellJob *__restrict__ jobs, int njobs, C *__restrict__ out)
+k_shell_spectrum(const C *__restrict__ planes, int ng, int nz1, const int64_t *__restrict__ e3sq,
+                 const ShellJob *__restrict__ jobs, C *__restrict__ out)
 {
-    const int f = 2 * blockIdx.y;
-    const ShellJob J = jobs[f], K = jobs[f + 1 < njobs ? f + 1 : f];
-    const int64_t n3 = int64_t(ng) * ng * ng;
-    C *dst = out + int64_t(blockIdx.y) * n3;
-    const int64_t lo = min(e3sq[J.s], e3sq[K.s]), hi = max(e3sq[J.s + 1], e3sq[K.s + 1]);
-    for (int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < n3; p += int64_t(gridDim.x) * blockDim.x) {
-        const int c = int(p % ng), ab = int(p / ng), a = ab / ng, b = ab - a * ng;
-        const int i = a < ng / 2 ? a : a - ng, j = b < ng / 2 ? b : b - ng, n = c < ng / 2 ? c : c - ng;
-        const int64_t q9 = 9 * (int64_t(i) * i + int64_t(j) * j + int64_t(n) * n);
+    const ShellJob J = jobs[blockIdx.y];
+    const int64_t np = int64_t(nz1) * ng * ng;
+    C *dst = out + int64_t(blockIdx.y) * np;
+    const int64_t lo = e3sq[J.s], hi = e3sq[J.s + 1];
+    for (int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < np; p += int64_t(gridDim.x) * blockDim.x) {
+        const int b = int(p % ng), na = int(p / ng), n = na / ng, a = na - n * ng;
+        const int i = a < ng / 2 ? a : a - ng, j = b < ng / 2 ? b : b - ng;
+        const int q = i * i + j * j + n * n;
         C v;
         v.x = 0;
         v.y = 0;
-        if (q9 >= lo && q9 < hi) {
-            v = shell_mode<C>(planes, ng, e3sq, J, a, b, i, j, n);
-            if (f + 1 < njobs) {
-                const C w = shell_mode<C>(planes, ng, e3sq, K, a, b, i, j, n);
-                v.x -= w.y;
-                v.y += w.x;
+        if (9 * int64_t(q) >= lo && 9 * int64_t(q) < hi) {
+            double w = 1.0;
+            if (J.kind == 1 || J.kind == 3) {
+                const double y = y_l0(J.l, double(n) / sqrt(double(q)));
+                w = J.kind == 1 ? y : y * y;
+            }
+            if (J.kind <= 1) {
+                const C d = planes[p];
+                v.x = decltype(v.x)(double(d.x) * w);
+                v.y = decltype(v.y)(double(d.y) * w);
+            } else {
+                v.x = decltype(v.x)(w);
             }
         }
         dst[p] = v;
@@ -297,19 +272,17 @@ int sup(bisp_shell_plan *p, T **out, const std::vector<T> &v, cudaStream_t s)
 
 size_t al(size_t v) { return (v + 255) & ~size_t(255); }
 
-// 3D transform of the nf real fields packed two to a complex N^3 array (see
-// k_shell_spectrum): three passes of the row transform, each along the
-// contiguous axis and written cyclically transposed, so the result is back in
-// [x][y][z] order; the last writes the fields apart.  a -> b -> a -> fields.
+// The nf real fields [f][x][y][z] of half spectra [f][n][a][b], n < nz1 (see
+// k_shell_spectrum): two passes of the row transform, each along the contiguous axis
+// and written transposed ([f][n][y][a], then [f][n][x][y]), then the line of sight.
+// a -> b -> a -> fields.
 template <typename R>
-cudaError_t fft3(typename Cx<R>::T *a, typename Cx<R>::T *b, R *fields, int ng, int64_t nf,
+cudaError_t fft3(typename Cx<R>::T *a, typename Cx<R>::T *b, R *fields, int ng, int nz1, int64_t nf,
                  const Twiddles<typename Cx<R>::T> &tw, cudaStream_t s)
 {
-    const int nrow = ng * ng;
-    const int64_t nb = (nf + 1) / 2;
-    cudaError_t e = launch_fft_rows_T<R>(a, b, ng, nrow, nb, R(1), false, tw, Batch{}, s);
-    if (e == cudaSuccess) e = launch_fft_rows_T<R>(b, a, ng, nrow, nb, R(1), false, tw, Batch{}, s);
-    if (e == cudaSuccess) e = launch_fft_rows_split<R>(a, fields, ng, nrow, nf, tw, s);
+    cudaError_t e = launch_fft_rows_T<R>(a, b, ng, ng, nf * nz1, R(1), false, tw, Batch{}, s);
+    if (e == cudaSuccess) e = launch_fft_rows_T<R>(b, a, ng, ng, nf * nz1, R(1), false, tw, Batch{}, s);
+    if (e == cudaSuccess) e = launch_fft_z_back<R>(a, fields, ng, nz1, nf, tw, s);
     return e;
 }
 
@@ -405,7 +378,7 @@ int build_shell_plan(bisp_shell_plan *p, const bisp_desc *d, cudaStream_t s)
     int st = upload_twiddles(p, s);
     if (!st) st = sup(p, &p->d_e3sq, p->e3sq, s);
     if (st) return st;
-    const int64_t n3 = int64_t(ng) * ng * ng;
+    const int64_t n3 = int64_t(ng) * ng * ng, planes = int64_t(p->nz + 1) * ng * ng;
     const int64_t nc = int64_t(cbin.size());
     // plan-time FP64 unit fields: I_s (kind 2) and Y_l0^2-weighted (kind 3), s >= 1
     {
@@ -433,9 +406,8 @@ int build_shell_plan(bisp_shell_plan *p, const bisp_desc *d, cudaStream_t s)
         };
         std::vector<double> h(size_t(std::max<int64_t>(nc, 1)) * (1 + nl));
         cudaError_t e = cudaMalloc(&d_uj, sizeof(ShellJob) * std::max<int64_t>(nu, 1));
-        const int64_t np = (nu + 1) / 2;             // pairs of fields
-        if (e == cudaSuccess) e = cudaMalloc(&sa, sizeof(double2) * std::max<int64_t>(np * n3, 1));
-        if (e == cudaSuccess) e = cudaMalloc(&sb, sizeof(double2) * std::max<int64_t>(np * n3, 1));
+        if (e == cudaSuccess) e = cudaMalloc(&sa, sizeof(double2) * std::max<int64_t>(nu * planes, 1));
+        if (e == cudaSuccess) e = cudaMalloc(&sb, sizeof(double2) * std::max<int64_t>(nu * planes, 1));
         if (e == cudaSuccess) e = cudaMalloc(&fld, sizeof(double) * std::max<int64_t>(nu * n3, 1));
         if (e == cudaSuccess) e = cudaMalloc(&sums, sizeof(double) * h.size());
         if (e == cudaSuccess) e = cudaMalloc(&d_up, sizeof(int4) * std::max<size_t>(up.size(), 1));
@@ -443,10 +415,10 @@ int build_shell_plan(bisp_shell_plan *p, const bisp_desc *d, cudaStream_t s)
         if (e == cudaSuccess && !up.empty())
             e = cudaMemcpyAsync(d_up, up.data(), sizeof(int4) * up.size(), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess && nu > 0) {
-            k_shell_spectrum<double2><<<dim3(blocks_for(n3), unsigned(np)), 256, 0, s>>>(nullptr, ng, p->d_e3sq, d_uj, int(nu),
-                                                                                         sa);
+            k_shell_spectrum<double2><<<dim3(blocks_for(planes), unsigned(nu)), 256, 0, s>>>(nullptr, ng, p->nz + 1, p->d_e3sq,
+                                                                                             d_uj, sa);
             e = cudaGetLastError();
-            if (e == cudaSuccess) e = fft3<double>(sa, sb, fld, ng, nu, p->twd, s);
+            if (e == cudaSuccess) e = fft3<double>(sa, sb, fld, ng, p->nz + 1, nu, p->twd, s);
         }
         if (e == cudaSuccess && !up.empty()) {
             k_triple_products<<<unsigned(up.size()), 256, 0, s>>>(fld, n3, d_up, 1.0 / double(n3), sums);
@@ -502,12 +474,11 @@ int build_shell_plan(bisp_shell_plan *p, const bisp_desc *d, cudaStream_t s)
     if (!st) st = sup(p, &p->d_bin_tri, bt, s);
     if (st) return st;
     // workspace
-    const int64_t planes = int64_t(p->nz + 1) * ng * ng;
     size_t o = 0;
     p->off_a = o; o = al(o + size_t(planes) * sizeof(float2));
     p->off_b = o; o = al(o + size_t(planes) * sizeof(float2));
-    p->off_spec = o; o = al(o + size_t((p->njobs + 1) / 2) * n3 * sizeof(float2));
-    p->off_spec2 = o; o = al(o + size_t((p->njobs + 1) / 2) * n3 * sizeof(float2));
+    p->off_spec = o; o = al(o + size_t(p->njobs) * planes * sizeof(float2));
+    p->off_spec2 = o; o = al(o + size_t(p->njobs) * planes * sizeof(float2));
     p->off_fields = o; o = al(o + size_t(p->njobs) * n3 * sizeof(float));
     p->off_part = o; o = al(o + size_t(std::max<int64_t>(nt, 1)) * nl * p->nslice * sizeof(double));
     p->off_num = o; o = al(o + size_t(std::max<int64_t>(nt, 1)) * nl * sizeof(double));
@@ -593,10 +564,10 @@ int estimator_shell_estimate(bisp_shell_plan *p, const float *delta, void *works
     SCK(launch_fft_rows_T<float>(A_, B_, ng, ng, p->nz + 1, 1.0f, false, p->twf, Batch{}, s));
     SCK(launch_fft_rows_T<float>(B_, A_, ng, ng, p->nz + 1, float(V / double(n3)), true, p->twf, Batch{}, s));
     if (p->njobs > 0) {
-        k_shell_spectrum<float2><<<dim3(blocks_for(n3), unsigned((p->njobs + 1) / 2)), 256, 0, s>>>(A_, ng, p->d_e3sq,
-                                                                                                    p->d_jobs, p->njobs, sa);
+        k_shell_spectrum<float2><<<dim3(blocks_for(ng2 * (p->nz + 1)), unsigned(p->njobs)), 256, 0, s>>>(
+            A_, ng, p->nz + 1, p->d_e3sq, p->d_jobs, sa);
         SCK(cudaGetLastError());
-        SCK(fft3<float>(sa, sb, fld, ng, p->njobs, p->twf, s));
+        SCK(fft3<float>(sa, sb, fld, ng, p->nz + 1, p->njobs, p->twf, s));
     }
     const int64_t nt = int64_t(p->tri_bin.size()), nprod = nt * p->nl;
     if (nprod > 0) {
