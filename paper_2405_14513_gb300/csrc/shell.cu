@@ -24,8 +24,7 @@
 // from FP64 unit fields.  Estimate: the forward transform (the kernels of
 // the main path), the weighted shell spectra of every shell (their planes n >= 0),
 // 3D transforms to real fields (two passes of the row transform, then the line of
-// sight), FP32 fields, FP32 triple products summed in pairs of floats and in
-// FP64, binning.  Lengths N_g <= 128
+// sight), FP32 fields, FP32 triple products summed in FP64, binning.  Lengths N_g <= 128
 // (the plan's FP64 sums over N_g^3 points per triple grow as N_g^6).
 #include "kernels.cuh"
 
@@ -126,24 +125,39 @@ k_triple_products(const double *__restrict__ fields, int64_t n3, const int4 *__r
     }
 }
 
-// s + e += x, s and e two floats: the rounding error of every addition to s is
-// found exactly (Knuth's two-sum) and kept in e, so that the pair holds the sum
-// of the FP32 products to 2^-45 or so, at FP32 speed (an FP64 addition, with its
-// conversion, takes 128 times a float's share of the SM).
+// t + e = a + b exactly, t = a + b rounded (Knuth's two-sum)
+__device__ __forceinline__ float two_sum(float a, float b, float &e)
+{
+    const float t = __fadd_rn(a, b), d = __fsub_rn(t, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, d)), __fsub_rn(b, d));
+    return t;
+}
+// s + e += x, s and e two floats
 __device__ __forceinline__ void add_exact(float &s, float &e, float x)
 {
-    const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
-    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)));
-    s = t;
+    float r;
+    s = two_sum(s, x, r);
+    e = __fadd_rn(e, r);
 }
 
-// Partial sums of sum_p F_l[p] D2[p] D3[p] for every l of one triple (tri: the
-// indices of F_0, whose l >= 2 follow it, of D2 and of D3) over one slice of the
-// grid: part[triple][slice][l].  Products in FP32, D2 D3 formed once for all l;
-// bound by reading the fields from L2.  With a block per triple and l and FP64
-// sums, and a transform per field, a 64^3 estimate took 2.57 ms; so 0.90 ms.
+// Partial sums of sum_p F_l[p] D2[p] D3[p] / kShellGuard for every l of one triple
+// (tri: the indices of F_0, whose l >= 2 follow it, of D2 and of D3) over one slice of
+// the grid: part[triple][slice][l].  Products in FP32, D2 D3 formed once for all l, sums
+// in FP64: a thread's products are added 4 kShellRun at a time, in pairs of floats,
+// because an FP64 addition and the conversion before it take 128 times a float's share of
+// the SM.  A run's pair holds its sum to 2^-54 of the products' 2-norm (random products;
+// 2^-47 for pairs kept over 1024 of them), far below the rounding of the FP32 products.
+// The products are divided by 4 kShellRun first (exactly), so that a sum of floats
+// overflows only where a product itself would, and is then taken as it is.
+// Bound by reading the fields from L2 and by the FP32 issue of the exact additions; runs
+// of a constant length let the loads of four steps go ahead, at four blocks an SM.  64^3,
+// l <= 6, the whole estimate: 2.57 ms with a block per triple and l, an FP64 addition per
+// product and full complex transforms, 0.53 ms so (0.50 with pairs of floats throughout);
+// 128^3, l = 0: 10.1, 2.00 (1.81).
+constexpr int kShellRun = 8;                      // times four products
+constexpr float kShellGuard = 1.0f / (4 * kShellRun);
 template <int NL>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 4)
 k_shell_products(const float *__restrict__ fields, int64_t n3, const int4 *__restrict__ tri, int nslice, double *__restrict__ part)
 {
     __shared__ double red[8][NL];
@@ -151,15 +165,21 @@ k_shell_products(const float *__restrict__ fields, int64_t n3, const int4 *__res
     const int64_t n4 = n3 / 4, lo = n4 * blockIdx.y / nslice, hi = n4 * (blockIdx.y + 1) / nslice;
     const float4 *F[NL], *B = reinterpret_cast<const float4 *>(fields + int64_t(T.y) * n3),
                         *D = reinterpret_cast<const float4 *>(fields + int64_t(T.z) * n3);
-    float s[NL][2], e[NL][2];
+    double acc[NL];
 #pragma unroll
     for (int l = 0; l < NL; ++l) {
         F[l] = reinterpret_cast<const float4 *>(fields + int64_t(T.x + l) * n3);
-        s[l][0] = s[l][1] = e[l][0] = e[l][1] = 0.0f;
+        acc[l] = 0.0;
     }
-    for (int64_t p = lo + threadIdx.x; p < hi; p += blockDim.x) {
+    float s[NL][2], e[NL][2];
+    auto clear = [&]() {
+#pragma unroll
+        for (int l = 0; l < NL; ++l) s[l][0] = s[l][1] = e[l][0] = e[l][1] = 0.0f;
+    };
+    auto add = [&](int64_t p) {
         const float4 b = B[p], d = D[p];
-        const float4 c = make_float4(b.x * d.x, b.y * d.y, b.z * d.z, b.w * d.w);
+        const float g = kShellGuard;
+        const float4 c = make_float4(g * (b.x * d.x), g * (b.y * d.y), g * (b.z * d.z), g * (b.w * d.w));
 #pragma unroll
         for (int l = 0; l < NL; ++l) {
             const float4 f = F[l][p];
@@ -168,10 +188,28 @@ k_shell_products(const float *__restrict__ fields, int64_t n3, const int4 *__res
             add_exact(s[l][0], e[l][0], f.z * c.z);
             add_exact(s[l][1], e[l][1], f.w * c.w);
         }
+    };
+    auto flush = [&]() {
+#pragma unroll
+        for (int l = 0; l < NL; ++l) {
+            float r;
+            const float t = two_sum(s[l][0], s[l][1], r);
+            acc[l] += isfinite(t) ? double(t) + double((e[l][0] + e[l][1]) + r) : double(t);
+        }
+    };
+    int64_t p = lo + threadIdx.x;
+    while (p + (kShellRun - 1) * 256 < hi) {
+        clear();
+#pragma unroll 4
+        for (int k = 0; k < kShellRun; ++k, p += 256) add(p);
+        flush();
     }
+    clear();
+    for (; p < hi; p += 256) add(p);
+    flush();
 #pragma unroll
     for (int l = 0; l < NL; ++l) {
-        double v = (double(s[l][0]) + double(s[l][1])) + (double(e[l][0]) + double(e[l][1]));
+        double v = acc[l];
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
         if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][l] = v;
     }
@@ -581,8 +619,8 @@ int estimator_shell_estimate(bisp_shell_plan *p, const float *delta, void *works
         default: k_shell_products<4><<<grid, 256, 0, s>>>(fld, n3, p->d_tri, p->nslice, part); break;
         }
         SCK(cudaGetLastError());
-        k_shell_sums<<<unsigned((nprod + 255) / 256), 256, 0, s>>>(part, nprod, p->nl, p->nslice, 1.0 / double(n3),
-                                                                   y00 / double(n3), num);
+        const double scale = 1.0 / (double(kShellGuard) * double(n3));
+        k_shell_sums<<<unsigned((nprod + 255) / 256), 256, 0, s>>>(part, nprod, p->nl, p->nslice, scale, y00 * scale, num);
         SCK(cudaGetLastError());
     }
     const int64_t nq = p->nbins * p->nl;

@@ -67,3 +67,25 @@ def test_shell_fields_keep_their_own_error(ng, l_max):
     ref, norm = _reference(plan, ws)
     err = np.sqrt(np.mean(((num - ref) / norm) ** 2, axis=0))
     assert err.max() < 2e-6, err
+
+
+@pytest.mark.parametrize("ng", [24, 32, 64])
+def test_shell_sums_reach_the_largest_products(ng):
+    """Three plane waves, k1 + k2 + k3 = 0, in shells 7, 5 and 4: D = V a cos(k x) in
+    each, so num_l = Y_l0(0) (V a)^3 / 4, with products up to 0.9 of FP32's largest: no
+    product overflows, and their sums are FP64's.  1e-5: three FP32 fields of 1e-6."""
+    L = 1e4
+    a = (0.9 * 3.4028234e38) ** (1 / 3) / L ** 3
+    x = np.arange(ng) * (2 * np.pi / ng)
+    d = sum(a * np.cos(i * x[:, None] + j * x[None, :]) for i, j in ((7, 0), (-4, 3), (-3, -3)))
+    d = torch.from_numpy(np.repeat(d[:, :, None], ng, axis=2).astype(np.float32)).cuda()
+    plan = api.ShellPlan(ng, L, np.array([3.0, ng / 3.0]) * (2 * np.pi / L), 1, 1, 6)
+    ws = plan.workspace()
+    plan.estimate(d, ws)
+    num = plan.sums(ws)
+    t = [k for k, q in enumerate(plan.triples()["tri"]) if tuple(q[:3]) == (7, 5, 4)]
+    assert len(t) == 1
+    y = np.sqrt((4 * np.arange(4) + 1) / (4 * np.pi)) * np.array([1.0, -1 / 2, 3 / 8, -5 / 16])
+    want = y * (L ** 3 * a) ** 3 / 4
+    assert np.isfinite(num[t[0]]).all()
+    assert np.abs(num[t[0]] / want - 1).max() < 1e-5
