@@ -999,7 +999,7 @@ k_epi_part(int mode, const Record *__restrict__ rec, const RecordF *__restrict__
 template <bool FIN> __device__ __forceinline__ const EpiView &view_of_block(const EpiViews &ev)
 {
     int i = 0;
-    while (i + 1 < ev.n && blockIdx.x >= (FIN ? ev.v[i + 1].bin0 : ev.v[i + 1].blk0)) ++i;
+    while (i + 1 < ev.n && blockIdx.x >= (FIN ? ev.v[i + 1].fin0 : ev.v[i + 1].blk0)) ++i;
     return ev.v[i];
 }
 
@@ -1024,11 +1024,15 @@ k_epi_part_views(const __grid_constant__ EpiViews ev, const double *value, int64
     }
 }
 
-// One block per bin: kFinSplit threads per moment take the bin's chunks in turn,
-// and their partial sums are added in order (the same for every LMAX, so that a
-// moment does not depend on the others binned with it); then (mode 0) the ratio
-// of Eq. bs_lm2_1 or (mode 1) the sum itself.  A thread per bin and moment walked
-// up to 80 chunks alone (64^3: 14 us).
+// The bins b0 .. b1 - 1 of a block (see fin_bins_per_block): their chunks' partial sums
+// added up, then (mode 0) the ratio of Eq. bs_lm2_1 or (mode 1) the sum itself.  The sum
+// of a moment: kFinSplit running sums take the bin's chunks in turn, and are added in
+// order (the same for every LMAX, so that a moment does not depend on the others binned
+// with it).  A bin of at most kFinSplit chunks takes one thread per moment, which comes to
+// the same; one of more takes kFinSplit threads per moment, so that none walks many
+// chunks alone (64^3, up to 80 of them: 14 us).  A block per bin throughout was bound by
+// the launch of empty blocks where bins are many, one thread per bin by its strided
+// stores (64^3, 3e6 bins of 4 moments, the binning: 3.1 ms and 0.52; so 0.24 ms).
 constexpr int kFinSplit = 8;
 template <int LMAX> constexpr int fin_threads()
 {
@@ -1039,42 +1043,67 @@ template <int LMAX>
 __device__ __forceinline__ void
 epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *partial,
         const double *__restrict__ den, double norm, double *__restrict__ out, int64_t fs_part, int64_t fs_out,
-        int lm_lo, int nlm_out, int64_t b, double *red)
+        int lm_lo, int nlm_out, int64_t b0, int64_t b1, double *red)
 {
     partial = field_ptr(partial, fs_part);
     out = field_ptr(out, fs_out);
     constexpr int NLM = (LMAX / 2 + 1) * (LMAX / 2 + 1);
     constexpr int P2 = fin_threads<LMAX>() / kFinSplit;     // at least NLM
+    auto store = [&](int64_t b, int i, double v) {
+        const int64_t o = b * nlm_out + (i - lm_lo);
+        if (mode == 0) {
+            const double d = den[o];
+            int l = 0;
+            while ((l / 2 + 1) * (l / 2 + 1) <= i) l += 2;
+            out[o] = d > 0.0 ? c_pref[l] * v * norm / d : __longlong_as_double(0x7ff8000000000000LL);
+        } else {
+            out[o] = v;
+        }
+    };
+    const int64_t total = (b1 - b0) * nlm_out;
+    bool more = false;                                      // a bin of more chunks seen
+    for (int64_t t = threadIdx.x; t < total; t += blockDim.x) {
+        const int64_t q = t / nlm_out, b = b0 + q, c0 = bin_chunk[b], c1 = bin_chunk[b + 1];
+        if (c1 - c0 > kFinSplit) {
+            more = true;
+            continue;
+        }
+        const int i = lm_lo + int(t - q * nlm_out);
+        double v = 0.0;
+        for (int64_t ch = c0; ch < c1; ++ch) v += partial[ch * NLM + i];
+        store(b, i, v);
+    }
+    if (!__syncthreads_or(more)) return;
     const int i = threadIdx.x % P2, sub = threadIdx.x / P2;
-    const int64_t c0 = bin_chunk[b], c1 = bin_chunk[b + 1];
-    double v = 0.0;
-    if (i < NLM && sub < kFinSplit)               // (a launch over several views may have threads to spare)
+    for (int64_t b = b0; b < b1; ++b) {                     // (the same bins for every thread)
+        const int64_t c0 = bin_chunk[b], c1 = bin_chunk[b + 1];
+        if (c1 - c0 <= kFinSplit) continue;
+        double v = 0.0;
+        if (sub < kFinSplit) {                              // (a launch may have threads to spare)
+            if (i < NLM)
 #pragma unroll 4
-        for (int64_t ch = c0 + sub; ch < c1; ch += kFinSplit) v += partial[ch * NLM + i];
-    red[threadIdx.x] = v;
-    __syncthreads();
-    if (sub > 0 || i < lm_lo || i >= NLM) return;
-    const int64_t o = b * nlm_out + (i - lm_lo);
-    const double d = mode == 0 ? den[o] : 0.0;
-    for (int k = 1; k < kFinSplit; ++k) v += red[k * P2 + i];
-    if (mode == 0) {
-        int l = 0;
-        while ((l / 2 + 1) * (l / 2 + 1) <= i) l += 2;
-        out[o] = d > 0.0 ? c_pref[l] * v * norm / d : __longlong_as_double(0x7ff8000000000000LL);
-    } else {
-        out[o] = v;
+                for (int64_t ch = c0 + sub; ch < c1; ch += kFinSplit) v += partial[ch * NLM + i];
+            red[threadIdx.x] = v;
+        }
+        __syncthreads();
+        if (sub == 0 && i >= lm_lo && i < NLM) {
+            for (int k = 1; k < kFinSplit; ++k) v += red[k * P2 + i];
+            store(b, i, v);
+        }
+        __syncthreads();
     }
 }
 
 template <int LMAX>
-__global__ void __launch_bounds__(fin_threads<LMAX>())
-k_epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *partial,
+__global__ void __launch_bounds__(256)
+k_epi_fin(int mode, const int64_t *__restrict__ bin_chunk, int64_t nbins, int64_t per, const double *partial,
           const double *__restrict__ den, double norm, double *__restrict__ out, int64_t fs_part, int64_t fs_out,
           int lm_lo, int nlm_out)
 {
     __shared__ double red[fin_threads<LMAX>()];
     grid_begin();
-    epi_fin<LMAX>(mode, bin_chunk, partial, den, norm, out, fs_part, fs_out, lm_lo, nlm_out, blockIdx.x, red);
+    const int64_t b0 = int64_t(blockIdx.x) * per;
+    epi_fin<LMAX>(mode, bin_chunk, partial, den, norm, out, fs_part, fs_out, lm_lo, nlm_out, b0, min(nbins, b0 + per), red);
 }
 
 // k_epi_fin (mode 0) for several views in one launch
@@ -1084,9 +1113,9 @@ k_epi_fin_views(const __grid_constant__ EpiViews ev, double norm, int64_t fs_par
     __shared__ double red[256];
     grid_begin();
     const EpiView &v = view_of_block<true>(ev);
-    const int64_t b = blockIdx.x - v.bin0;
+    const int64_t b0 = int64_t(blockIdx.x - v.fin0) * ev.per, b1 = min(v.nbins, b0 + ev.per);
     auto run = [&](auto lmax) {
-        epi_fin<decltype(lmax)::value>(0, v.bin_chunk, v.partial, v.den, norm, v.out, fs_part, fs_out, v.lm_lo, v.nlm, b, red);
+        epi_fin<decltype(lmax)::value>(0, v.bin_chunk, v.partial, v.den, norm, v.out, fs_part, fs_out, v.lm_lo, v.nlm, b0, b1, red);
     };
     switch (v.l_hi) {
     case 0: run(std::integral_constant<int, 0>{}); break;
@@ -1318,14 +1347,15 @@ template <typename W, typename Y, int LMAX>
 cudaError_t epilogue_l(int mode, const EpiArgs &e, const double *value, const double *den, double norm, double *out,
                        const Batch &fb, int lo, int n, cudaStream_t s)
 {
-    const dim3 g1(unsigned((e.nchunks * 32 + 255) / 256), fb.nf), g2(unsigned(e.nbins), fb.nf);
+    const int64_t per = fin_bins_per_block(e.nbins);
+    const dim3 g1(unsigned((e.nchunks * 32 + 255) / 256), fb.nf), g2(unsigned((e.nbins + per - 1) / per), fb.nf);
     cudaError_t st = cudaSuccess;
     if (e.nchunks > 0)
         st = launch_next(k_epi_part<W, Y, LMAX>, g1, 256, 0, s, mode, e.rec, e.recf, e.chunk_lo, e.chunk_hi, e.nchunks, value,
                          e.partial, fb.fs_in, e.fs_part);
     if (st == cudaSuccess)
-        st = launch_next(k_epi_fin<LMAX>, g2, fin_threads<LMAX>(), 0, s, mode, e.bin_chunk, e.partial, den, norm, out,
-                         e.fs_part, fb.fs_out, lo, n);
+        st = launch_next(k_epi_fin<LMAX>, g2, per > 1 ? 256 : fin_threads<LMAX>(), 0, s, mode, e.bin_chunk, e.nbins, per, e.partial,
+                         den, norm, out, e.fs_part, fb.fs_out, lo, n);
     return st;
 }
 
@@ -1359,24 +1389,27 @@ template <typename W>
 cudaError_t launch_epilogue_views(EpiViews ev, const double *value, double norm, const Batch &fb, cudaStream_t s,
                                   bool fp32_weights)
 {
-    unsigned blk = 0, bin = 0;
-    int threads = 32;
+    int64_t bins = 0;
+    for (int i = 0; i < ev.n; ++i) bins += ev.v[i].nbins;
+    ev.per = fin_bins_per_block(bins);
+    unsigned blk = 0, fin = 0;
+    int threads = ev.per > 1 ? 256 : 32;
     for (int i = 0; i < ev.n; ++i) {
         EpiView &v = ev.v[i];
         if (v.l_hi < 0 || v.l_hi > 8 || (v.l_hi & 1)) return cudaErrorInvalidValue;
         v.blk0 = blk;
-        v.bin0 = bin;
+        v.fin0 = fin;
         blk += unsigned((v.nchunks + 7) / 8);
-        bin += unsigned(v.nbins);
+        fin += unsigned((v.nbins + ev.per - 1) / ev.per);
         threads = std::max(threads, v.l_hi < 4 ? fin_threads<2>() : (v.l_hi < 8 ? fin_threads<6>() : fin_threads<8>()));
     }
-    if (bin == 0) return cudaSuccess;
+    if (fin == 0) return cudaSuccess;
     if (blk > 0) {
         const cudaError_t e = launch_next(fp32_weights ? k_epi_part_views<W, float> : k_epi_part_views<W, W>, dim3(blk, fb.nf),
                                           256, 0, s, ev, value, fb.fs_in);
         if (e != cudaSuccess) return e;
     }
-    return launch_next(k_epi_fin_views, dim3(bin, fb.nf), threads, 0, s, ev, norm, fb.fs_in, fb.fs_out);
+    return launch_next(k_epi_fin_views, dim3(fin, fb.nf), threads, 0, s, ev, norm, fb.fs_in, fb.fs_out);
 }
 
 cudaError_t launch_records_f(const Record *rec, RecordF *recf, int64_t n, cudaStream_t s)

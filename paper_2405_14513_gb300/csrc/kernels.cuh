@@ -221,7 +221,8 @@ cudaError_t launch_reduce_partials(const Group *groups, int64_t ngroups, const d
 // fp32_weights: the Y_lm of each record in FP32 (sums stay in W).
 // The records are walked in chunks of one bin each (one warp per chunk, FP64
 // partial sums per moment in `partial` [nchunks][moments of l <= l_hi]),
-// then each bin adds its chunks in a fixed order (one block per bin).
+// then each bin adds its chunks in a fixed order (a block per bin, or per
+// fin_bins_per_block of them).
 struct EpiArgs {
     const Record *rec;                    // fp32_weights: not read (recf is)
     const RecordF *recf;
@@ -238,7 +239,7 @@ cudaError_t launch_epilogue(int mode, const EpiArgs &e, const double *value, int
 
 // The same (mode 0) for all views of a plan in one launch per pass: the views do
 // not depend on one another, and at a few thousand chunks each a launch is short
-// and leaves most of the GPU idle.  blk0 and bin0 are the launcher's.
+// and leaves most of the GPU idle.  blk0, fin0 and per are the launcher's.
 struct EpiView {
     const int64_t *chunk_lo, *chunk_hi, *bin_chunk;
     int64_t nchunks, nbins;
@@ -246,12 +247,13 @@ struct EpiView {
     const double *den;
     double *out;
     int l_hi, lm_lo, nlm;                 // first moment and moments written
-    unsigned blk0, bin0;                  // first block of the chunks' and of the bins' launch
+    unsigned blk0, fin0;                  // first block of the chunks' and of the bins' launch
 };
 struct EpiViews {
     int n;
     const Record *rec;
     const RecordF *recf;
+    int64_t per;                          // bins of a block of the bins' launch
     EpiView v[5];                         // even l <= 8
 };
 template <typename W>

@@ -206,6 +206,12 @@ inline int64_t bin_chunk_len(int64_t nrec)
     return len < 64 ? 64 : (len > 2048 ? 2048 : len);
 }
 
+// Bins that a block of the binning's last pass takes: one where there are at most
+// kFinBlocks (a block then adds the many chunks of a bin), several where there are more,
+// nearly all of them empty or of a chunk or two.
+constexpr int64_t kFinBlocks = 16384;
+inline int64_t fin_bins_per_block(int64_t nbins) { return nbins <= kFinBlocks ? 1 : (nbins + kFinBlocks - 1) / kFinBlocks; }
+
 struct Level {
     int lev = 0;               // index into Rings::grid
     int M = 0;                 // grid side
