@@ -603,8 +603,7 @@ int build_plan(bisp_plan *p, const bisp_desc *desc, cudaStream_t s)
             return n;
         };
         while (p->x_chunk > kXChunkMin && units(p->x_chunk) < kUnitsWanted) p->x_chunk /= 2;
-        if (p->x_chunk != kXChunk) err = enumerate(P, p->x_chunk);
-        if (!err.empty()) return fail(BISP_INTERNAL, err);
+        if (p->x_chunk != kXChunk) set_x_chunk(P, p->x_chunk);
     }
     unit_costs(P, p->x_chunk);
     build_views(P, mu_l.empty() ? nullptr : mu_l.data(), t_l.empty() ? nullptr : t_l.data());

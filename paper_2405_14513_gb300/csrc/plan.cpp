@@ -307,19 +307,18 @@ int arrange_lanes(const std::vector<int32_t> &key1, const std::vector<int32_t> &
 // whose fields fit kTcMinRing ring buffers of shared memory.  The last, partly
 // filled tiles of the sign patterns of one (grid, |n3|) are put into one tile
 // where they fit, each pattern in warps of its own (at 64^3 such tiles are most of
-// them: they filled 30% of their lanes, merged ones 52%).  Then units (tile,
-// x chunk) by class.
-// Requires the groups' partial-sum layout.  Marks the fields the tiles read.
+// them: they filled 30% of their lanes, merged ones 52%).  set_x_chunk gives them
+// their partial sums and units.  Marks the fields the tiles read.
 template <typename UsedFn>
-std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
+std::string build_tc(HostPlan &P, UsedFn &&U_)
 {
     const Rings &R = P.rings;
     const int nz = R.nz;
     P.tc_tiles.clear();
     P.tc_rows.clear();
+    P.tc_row_of.clear();
     P.tc_slots.clear();
     P.tc_lanes.clear();
-    P.tc_units.clear();
     P.tc_mma_products = 0;
     auto gflags = [](const Group &G) { return (G.n1 < 0 ? 1 : 0) | (G.n2 < 0 ? 2 : 0) | (G.n3 < 0 ? 4 : 0); };
     std::vector<std::vector<int32_t>> pool(size_t(R.ngrid) * (nz + 1) * 8);
@@ -352,7 +351,6 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
         T.nwin = cur.hi - cur.lo + 1;
         T.ncol = ((T.nwin + 15) / 16) * 16;
         const int64_t M2 = int64_t(T.M) * T.M;
-        T.nchunk = int32_t((M2 + x_chunk - 1) / x_chunk);
         if (T.ncol > kTcMaxCols || T.nslot > kTcMaxSlots || T.nrow > kTcRows || tc_ring(T.ncol, T.nslot) == 0)
             return "tcgen05 tile limits";
         // rows in order of their D1 field, then D2 field, and the staged
@@ -482,7 +480,6 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
             const Group &G = P.groups[gr.first];
             const Row &rw = P.rows[gr.second];
             TcRow t{};
-            t.p0 = G.part0 + rw.coff;
             t.stride = G.ncombo;
             const int a1 = G.n1 < 0 ? -G.n1 : G.n1, a2 = G.n2 < 0 ? -G.n2 : G.n2;
             const auto k = keys(gr);
@@ -492,6 +489,7 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
             t.n = rw.n;
             t.flags = uint8_t((G.n1 < 0 ? 1 : 0) | (G.n2 < 0 ? 2 : 0) | (G.n3 < 0 ? 4 : 0));
             P.tc_rows.push_back(t);
+            P.tc_row_of.push_back(TcRowOf{gr.first, rw.coff});
             U_(cur_lev, a1, rw.r1) = 1;
             U_(cur_lev, a2, rw.r2) = 1;
             for (int j = 0; j < rw.n; ++j) U_(cur_lev, cur_n3, rw.r3a + j) = 1;
@@ -581,6 +579,30 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
                 if (!e.empty()) return e;
             }
         }
+    return "";
+}
+
+// Partial sums [group][x chunk][combination]
+void layout_partials(HostPlan &P, int64_t x_chunk)
+{
+    int64_t part = 0;
+    for (auto &G : P.groups) {
+        G.nchunk = int32_t((int64_t(G.M) * G.M + x_chunk - 1) / x_chunk);
+        G.part0 = part;
+        part += int64_t(G.nchunk) * G.ncombo;
+    }
+    P.n_partials = part;
+}
+
+}  // namespace
+
+void set_x_chunk(HostPlan &P, int64_t x_chunk)
+{
+    const Rings &R = P.rings;
+    layout_partials(P, x_chunk);
+    for (size_t r = 0; r < P.tc_rows.size(); ++r) P.tc_rows[r].p0 = P.groups[P.tc_row_of[r].group].part0 + P.tc_row_of[r].coff;
+    for (TcTile &T : P.tc_tiles) T.nchunk = int32_t((int64_t(T.M) * T.M + x_chunk - 1) / x_chunk);
+    P.tc_units.clear();
     // units: class, then biggest grids first, x chunk, tile
     for (int c = 0; c < kTcClasses; ++c) {
         P.tc_class_begin[c] = int64_t(P.tc_units.size());
@@ -597,10 +619,7 @@ std::string build_tc(HostPlan &P, int64_t x_chunk, UsedFn &&U_)
         }
     }
     P.tc_class_begin[kTcClasses] = int64_t(P.tc_units.size());
-    return "";
 }
-
-}  // namespace
 
 std::string enumerate(HostPlan &P, int64_t x_chunk)
 {
@@ -730,8 +749,6 @@ std::string enumerate(HostPlan &P, int64_t x_chunk)
             if (ncombo == 0) continue;
             G.nrow = int32_t(P.rows.size()) - G.row0;
             G.ncombo = ncombo;
-            const int64_t M2 = int64_t(G.M) * G.M;
-            G.nchunk = int32_t((M2 + x_chunk - 1) / x_chunk);
             cidx += ncombo;
 
             if (P.tensor) {             // tcgen05 tiles span groups: built after the loop
@@ -832,16 +849,12 @@ std::string enumerate(HostPlan &P, int64_t x_chunk)
     P.n_combos = cidx;
     if (P.n_combos >= (int64_t(1) << 31) - 1) return "too many combinations for 32-bit indices";
 
-    // partial sums [group][x chunk][combination]
-    int64_t part = 0;
-    for (auto &G : P.groups) {
-        G.part0 = part;
-        part += int64_t(G.nchunk) * G.ncombo;
-    }
-    P.n_partials = part;
     if (P.tensor) {
-        std::string e = build_tc(P, x_chunk, U_);
+        std::string e = build_tc(P, U_);
         if (!e.empty()) return e;
+        set_x_chunk(P, x_chunk);
+    } else {
+        layout_partials(P, x_chunk);
     }
 
     // D-store layout, grid by grid, plane by plane, ring by ring

@@ -140,6 +140,10 @@ struct TcLane {
 struct TcUnit {
     int32_t tile, chunk;
 };
+// Where the partial sums of a TcRow are: its group, and its first combination there.
+struct TcRowOf {
+    int32_t group, coff;
+};
 
 // One Step-II block: an x chunk of a group with up to 16 of its tiles (one
 // per warp), and the ring ranges it stages per plane (plane 3 may reach
@@ -238,6 +242,7 @@ struct HostPlan {
     bool tensor = false;                // build tcgen05 tiles (set before enumerate)
     std::vector<TcTile> tc_tiles;
     std::vector<TcRow> tc_rows;
+    std::vector<TcRowOf> tc_row_of;     // of every row
     std::vector<int32_t> tc_slots;
     std::vector<TcLane> tc_lanes;       // kTcRows per tile
     std::vector<TcUnit> tc_units;       // by class (NC), then grid, x chunk, tile
@@ -291,6 +296,10 @@ int triple_level(const Rings &R, int r1, int r2, int r3);
 // fill groups, rows, tiles, units, records and the D-store layout.
 // Requires rings and ntri.  Returns "" or an error message.
 std::string enumerate(HostPlan &P, int64_t x_chunk);
+
+// The x chunk length of a tensor-core plan that has been enumerated: the layout of its
+// partial sums and its units (its tiles, and what they read, do not depend on it).
+void set_x_chunk(HostPlan &P, int64_t x_chunk);
 
 // Views of the plan (from desc n_mu, n_t, or the per-l grids n_mu_l, n_t_l
 // for l = 0, 2, .., l_max), their output offsets and n_out.
