@@ -329,28 +329,32 @@ std::string build_tc(HostPlan &P, UsedFn &&U_)
     struct Cur {
         std::vector<std::pair<int32_t, int32_t>> rows;   // (group, row index in P.rows)
         std::vector<int32_t> slots;
-        int lo = 1 << 30, hi = -1;
+        int lo = 1 << 30, hi = -1, lev = 0, n3 = 0;
     } cur;
+    struct Built {
+        std::string err;
+        TcTile T{};
+        std::vector<TcRow> rows;
+        std::vector<int32_t> slots;
+        TcLane lanes[kTcRows];
+    };
     int cur_lev = 0, cur_n3 = 0;
-    auto slot_of = [&](std::vector<int32_t> &sl, int32_t key) {
+    auto slot_of = [](const std::vector<int32_t> &sl, int32_t key) {
         for (size_t i = 0; i < sl.size(); ++i)
             if (sl[i] == key) return int(i);
         return -1;
     };
-    auto close = [&]() -> std::string {
-        if (cur.rows.empty()) return "";
+    // a tile's rows in order, slots and lanes
+    auto finish = [&](Cur &cur, Built &out) -> std::string {
         TcTile T{};
-        T.lev = cur_lev;
-        T.M = R.grid[cur_lev];
-        T.row0 = int32_t(P.tc_rows.size());
+        T.lev = cur.lev;
+        T.M = R.grid[cur.lev];
         T.nrow = int32_t(cur.rows.size());
-        T.slot0 = int32_t(P.tc_slots.size());
         T.nslot = int32_t(cur.slots.size());
-        T.n3abs = cur_n3;
+        T.n3abs = cur.n3;
         T.r3lo = cur.lo;
         T.nwin = cur.hi - cur.lo + 1;
         T.ncol = ((T.nwin + 15) / 16) * 16;
-        const int64_t M2 = int64_t(T.M) * T.M;
         if (T.ncol > kTcMaxCols || T.nslot > kTcMaxSlots || T.nrow > kTcRows || tc_ring(T.ncol, T.nslot) == 0)
             return "tcgen05 tile limits";
         // rows in order of their D1 field, then D2 field, and the staged
@@ -403,12 +407,14 @@ std::string build_tc(HostPlan &P, UsedFn &&U_)
         std::vector<int> num(ns);
         {
             std::vector<std::vector<int>> adj(ns), pass, in(ns);   // passes, and those of each field
-            for (int side = 0; side < 2; ++side)
+            for (int side = 0; side < 2; ++side) {
+                const bool *pair = side ? lanes.pair2 : lanes.pair1;
+                const std::vector<int32_t> &key = side ? key2 : key1;
                 for (int g0 = 0; g0 < nlane;) {
-                    const int np = (side ? lanes.pair2 : lanes.pair1)[g0 / 32] ? 16 : 8;
+                    const int np = pair[g0 / 32] ? 16 : 8;
                     std::vector<int> grp;
                     for (int l = g0; l < g0 + np; ++l) {
-                        const int f = slot_of(cur.slots, (side ? key2 : key1)[lanes.like[l]]);
+                        const int f = slot_of(cur.slots, key[lanes.like[l]]);
                         if (std::find(grp.begin(), grp.end(), f) == grp.end()) grp.push_back(f);
                     }
                     for (int a : grp) {
@@ -419,6 +425,7 @@ std::string build_tc(HostPlan &P, UsedFn &&U_)
                     pass.push_back(grp);
                     g0 += np;
                 }
+            }
             std::vector<int> col(ns, -1), cnt(8, 0), next(8, 0);
             int top = 0;
             for (int f = 0; f < ns; ++f) {
@@ -481,29 +488,75 @@ std::string build_tc(HostPlan &P, UsedFn &&U_)
             const Row &rw = P.rows[gr.second];
             TcRow t{};
             t.stride = G.ncombo;
-            const int a1 = G.n1 < 0 ? -G.n1 : G.n1, a2 = G.n2 < 0 ? -G.n2 : G.n2;
             const auto k = keys(gr);
             t.s1 = uint8_t(slot_of(cur.slots, k.first));     // the field's number (its slot)
             t.s2 = uint8_t(slot_of(cur.slots, k.second));
             t.col0 = uint8_t(rw.r3a - cur.lo);
             t.n = rw.n;
-            t.flags = uint8_t((G.n1 < 0 ? 1 : 0) | (G.n2 < 0 ? 2 : 0) | (G.n3 < 0 ? 4 : 0));
-            P.tc_rows.push_back(t);
-            P.tc_row_of.push_back(TcRowOf{gr.first, rw.coff});
-            U_(cur_lev, a1, rw.r1) = 1;
-            U_(cur_lev, a2, rw.r2) = 1;
-            for (int j = 0; j < rw.n; ++j) U_(cur_lev, cur_n3, rw.r3a + j) = 1;
+            t.flags = uint8_t(gflags(G));
+            out.rows.push_back(t);
         }
         for (int l = 0; l < kTcRows; ++l)
-            P.tc_lanes.push_back(l >= nlane ? TcLane{0, 0, uint8_t(kTcNoRow), 0}
-                                            : TcLane{uint8_t(slot_of(cur.slots, key1[lanes.like[l]])),
-                                                     uint8_t(slot_of(cur.slots, key2[lanes.like[l]])),
-                                                     uint8_t(lanes.row[l] < 0 ? kTcNoRow : lanes.row[l]), 0});
-        P.tc_slots.insert(P.tc_slots.end(), cur.slots.begin(), cur.slots.end());
-        P.tc_mma_products += double(kTcRows) * T.ncol * double(M2);
-        P.tc_tiles.push_back(T);
-        cur = Cur{};
+            out.lanes[l] = l >= nlane ? TcLane{0, 0, uint8_t(kTcNoRow), 0}
+                                      : TcLane{uint8_t(slot_of(cur.slots, key1[lanes.like[l]])),
+                                               uint8_t(slot_of(cur.slots, key2[lanes.like[l]])),
+                                               uint8_t(lanes.row[l] < 0 ? kTcNoRow : lanes.row[l]), 0};
+        out.slots = cur.slots;
+        out.T = T;
         return "";
+    };
+    // The tiles cut so far, finished by several threads (a tile's lanes and slots take
+    // longer than cutting it) and appended in the order they were cut.
+    std::vector<Cur> cut;
+    auto flush = [&]() -> std::string {
+        std::vector<Built> built(cut.size());
+        std::atomic<size_t> next{0};
+        auto work = [&]() {
+            for (size_t k; (k = next.fetch_add(1)) < cut.size();) {
+                try {
+                    built[k].err = finish(cut[k], built[k]);
+                } catch (const std::exception &) {
+                    built[k].err = "out of memory";
+                }
+            }
+        };
+        const size_t nt = std::min<size_t>(std::min(32u, std::thread::hardware_concurrency()), cut.size() / 32);
+        std::vector<std::thread> th;
+        try {
+            for (size_t t = 1; t < nt; ++t) th.emplace_back(work);
+        } catch (const std::exception &) {              // fewer threads, then
+        }
+        work();
+        for (auto &t : th) t.join();
+        for (size_t k = 0; k < cut.size(); ++k) {
+            Built &b = built[k];
+            if (!b.err.empty()) return b.err;
+            b.T.row0 = int32_t(P.tc_rows.size());
+            b.T.slot0 = int32_t(P.tc_slots.size());
+            P.tc_rows.insert(P.tc_rows.end(), b.rows.begin(), b.rows.end());
+            P.tc_slots.insert(P.tc_slots.end(), b.slots.begin(), b.slots.end());
+            P.tc_lanes.insert(P.tc_lanes.end(), b.lanes, b.lanes + kTcRows);
+            for (auto &gr : cut[k].rows) {
+                const Group &G = P.groups[gr.first];
+                const Row &rw = P.rows[gr.second];
+                P.tc_row_of.push_back(TcRowOf{gr.first, rw.coff});
+                U_(b.T.lev, G.n1 < 0 ? -G.n1 : G.n1, rw.r1) = 1;
+                U_(b.T.lev, G.n2 < 0 ? -G.n2 : G.n2, rw.r2) = 1;
+                for (int j = 0; j < rw.n; ++j) U_(b.T.lev, b.T.n3abs, rw.r3a + j) = 1;
+            }
+            P.tc_mma_products += double(kTcRows) * b.T.ncol * double(b.T.M) * b.T.M;
+            P.tc_tiles.push_back(b.T);
+        }
+        cut.clear();
+        return "";
+    };
+    auto close = [&]() -> std::string {
+        if (cur.rows.empty()) return "";
+        cur.lev = cur_lev;
+        cur.n3 = cur_n3;
+        cut.push_back(std::move(cur));
+        cur = Cur{};
+        return cut.size() < 4096 ? "" : flush();
     };
     auto add_slot = [&](Cur &c, int32_t key) {
         if (slot_of(c.slots, key) < 0) c.slots.push_back(key);
@@ -579,7 +632,7 @@ std::string build_tc(HostPlan &P, UsedFn &&U_)
                 if (!e.empty()) return e;
             }
         }
-    return "";
+    return flush();
 }
 
 // Partial sums [group][x chunk][combination]
