@@ -633,7 +633,7 @@ __device__ __forceinline__ double flip_sign(double x, uint32_t bit)
 
 template <typename R, int NW>
 __global__ void __launch_bounds__(32 * NW, (sizeof(R) == 8 ? 8 : 16) / NW)
-k_step2(StepIIArgs args, int64_t unit0, const typename Cx<R>::T *__restrict__ dstore, int smem_bytes)
+k_step2(StepIIArgs args, int64_t unit0, const typename Cx<R>::T *dstore, int smem_bytes)
 {
     grid_begin();
     dstore = field_ptr(dstore, args.fs);

@@ -91,9 +91,11 @@ struct StepIIArgs {
 // an estimate, calls grid_begin before it reads or writes global memory that another
 // kernel writes or reads: the next kernel may be placed from here on; this one
 // goes on when every kernel before it has completed (each waits so, also blocks
-// without work) and its writes are visible.  Pointers to such memory are not
-// __restrict__: the compiler may then neither take the read-only path, which is for
-// data that nobody writes while the kernel lasts, nor move their loads before the wait.
+// without work) and its writes are visible.  Pointers that such memory is read through
+// are not __restrict__: the compiler may then neither take the read-only path, which is
+// for data that nobody writes while the kernel lasts, nor move loads before the wait.
+// (The plan's tables are, and the input of an estimate's first kernel, which is launched
+// the ordinary way.)
 // 32^3 (11 kernels) 79 -> 59 us, 48^3 x 3 202 -> 177, 64^3 173 -> 161; from 128^3 on, 2% of Step I.
 __device__ __forceinline__ void grid_begin()
 {

@@ -466,7 +466,7 @@ __device__ __forceinline__ bool produce(const ProdArgs &pa)
 // thread (an 88-register build ran one block per SM and was 45% slower).
 template <int NC>
 __global__ void __launch_bounds__(kThreads, 2)
-k_step2_tc(TcArgs args, int64_t unit0, const float2 *__restrict__ dstore)
+k_step2_tc(TcArgs args, int64_t unit0, const float2 *dstore)
 {
     constexpr int NB = NC / 8;                   // 8-row groups of B
     constexpr uint32_t LBO = NB * 128;           // next core matrix along K
