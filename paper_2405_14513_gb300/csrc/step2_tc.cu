@@ -20,10 +20,12 @@
 //
 // Precision.  Every FP32 operand is split x = hi + lo into two FP16 numbers,
 // hi rounded to nearest and lo the remainder (exact in FP32) rounded to
-// nearest, so that hi + lo holds x to 2^-24; the product is taken as
-// hi hi' + lo hi' + hi lo' (lo lo' is below FP32 rounding).  The stored
+// nearest.  hi + lo holds x to 2^-23 of itself, and no closer than 2^-25 (FP16 has
+// no spacing below 2^-24): relative to x that is less where |x| < 1/4.  The product
+// is taken as hi hi' + lo hi' + hi lo'; lo lo', left out, is at most 2^-22 of it.  The stored
 // fields are D times a power of two per field that puts them, their products
-// and the low parts inside FP16's range (k_ring_scale); it is undone, exactly,
+// and the low parts inside FP16's range and their root mean square at 1/3 or more
+// (k_ring_scale), so that the 2^-25 is small against a sum; it is undone, exactly,
 // on the FP64 partial sums.  The tensor-memory accumulator truncates when it
 // accumulates, so it holds one stage of 32 grid points (12 MMAs); every stage
 // is added into FP32 registers, and each unit's sums go out as FP64 partials,
@@ -34,7 +36,9 @@
 // buffers holds 16 points, so the barriers, fences and accumulator reads, a
 // third of the time, came twice as often.  512^3, all of Step II: 587 ms with
 // TF32 pairs and 16-point stages, 462 ms so; the error against 64 bits fell
-// from 1.1e-6 to 0.7e-6 (2-norm over the bins, 128^3).  With lanes paired by
+// from 1.1e-6 to 0.7e-6 (2-norm over the bins, 128^3), also on fields whose values
+// differ by orders of magnitude (a point on a field 10^-6 of it, log-normal, a bright
+// slab: 0.3 to 0.5 of what the TF32 pairs gave).  With lanes paired by
 // field (plan.cpp), tiles shared by sign patterns, one proxy fence per stage and
 // waits tested before they are polled it now takes 404 ms (256^3: 27.8 -> 17.0).
 //
