@@ -91,7 +91,6 @@ struct bisp_plan {
     int64_t *d_doff = nullptr;
     Record *d_rec = nullptr;             // binning records: FP64 plans keep these,
     RecordF *d_recf = nullptr;           // the others their FP32 form
-    int64_t *d_bin_start = nullptr;
     int64_t *d_chunk_lo = nullptr, *d_chunk_hi = nullptr, *d_bin_chunk = nullptr;   // binning chunks
     double *d_den = nullptr;
     std::vector<double> h_den;
@@ -621,7 +620,6 @@ int build_plan(bisp_plan *p, const bisp_desc *desc, cudaStream_t s)
     const bool fp64 = desc->precision == BISP_PREC_FP64;
     if (!st && fp64) st = upload(p, &p->d_rec, P.records, s);
     if (!st && !fp64) st = dev_alloc(p, &p->d_recf, P.records.size());
-    if (!st) st = upload(p, &p->d_bin_start, P.bin_start, s);
     if (!st) st = upload(p, &p->d_chunk_lo, P.chunk_lo, s);
     if (!st) st = upload(p, &p->d_chunk_hi, P.chunk_hi, s);
     if (!st) st = upload(p, &p->d_bin_chunk, P.bin_chunk, s);

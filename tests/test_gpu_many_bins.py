@@ -58,3 +58,13 @@ def test_bins_of_few_combinations(l_max):
     # FP64 sums of at most a few hundred terms, relative to the terms' sizes
     size = np.bincount(tab["bin"], weights=mult * np.abs(S), minlength=plan.n_bins)[f] / (L ** 3 * ng ** 2 * nt[f])
     assert (np.abs(B[f, 0] - want[f]) <= 1e-12 * size).all()
+
+
+def test_resident_bytes_of_a_bin():
+    """On the device a bin is its first chunk (8 bytes) and its moments' denominators."""
+    ng, L, lmax, n = 16, 160.0, 2, 50000
+    kf = 2 * np.pi / L
+    edges = np.append(np.linspace(0.0, 0.5 * kf, n), ng / 3 * kf)
+    many, one = (api.Plan(ng, L, e, 1, 1, lmax, precision="mixed") for e in (edges, edges[-2:]))
+    assert many.n_bins == n and many.n_combos == one.n_combos
+    assert many.info["resident_bytes"] - one.info["resident_bytes"] <= (n - 1) * (8 + 8 * many.n_lm) + 64
