@@ -68,7 +68,7 @@ METRIC = "B_l^m(k1,mu,t) configs/s at N_g={ng}"
 
 
 PRECISION_TEXT = {
-    "mixed_tc": "FP32 transforms; Step-II products on tcgen05 tensor cores (FP16 high/low split of scaled values, 3 passes, FP32 accuracy); FP32 sums per 16384-point chunk, FP64 across chunks and in the binning",
+    "mixed_tc": "FP32 transforms; Step-II products on tcgen05 tensor cores (FP16 high/low split of scaled values, 3 passes, FP32 accuracy); FP32 sums per chunk of at most 16384 points, FP64 across chunks and in the binning",
     "mixed": "FP32 transforms and products on CUDA cores, FP64 sums",
     "fp32": "FP32 throughout",
     "fp64": "FP64 throughout",

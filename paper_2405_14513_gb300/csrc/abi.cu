@@ -366,7 +366,7 @@ int init_attributes()
 
 // Transform tile autotuner.  Each transform kernel holds rt rows (or, in
 // Step I's second pass, w columns) of its length M in two shared-memory
-// buffers; the best tile depends on M, the kernel and the GPU (large tiles
+// buffers (Step I in one where two stages do); the best tile depends on M, the kernel and the GPU (large tiles
 // leave one block per SM).  For the forward z pass, the forward row passes
 // and each reduction grid's gather, candidate tiles of 4-64 KB per buffer,
 // and for each grid's second pass strips of 2-32 columns, are timed on

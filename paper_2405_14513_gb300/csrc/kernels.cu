@@ -231,9 +231,9 @@ __device__ __forceinline__ void fft_stage(const FftRows &fr, int Ns, int s, cons
 // left of the power of two, one radix-4 or radix-2 stage.  The first stage
 // takes its elements from `load` and the last hands them to `store` (SMEM:
 // leaves them in the returned buffer instead, block synchronised), so that
-// between global memory and the registers a transform of up to 512 points
-// crosses shared memory twice, not four times.  a, b: buffers of nr rows of
-// stride P.  Every thread of the block takes part.
+// between global memory and the registers a transform of three stages (2^q up to
+// 512, F x 2^q with q up to 6) crosses shared memory twice, not four times.  a, b:
+// buffers of nr rows of stride P.  Every thread of the block takes part.
 template <typename C, int F, bool ACROSS, bool SMEM, typename G, typename S>
 __device__ __forceinline__ C *fft_block(const FftRows &fr, int P, C *a, C *b, const C *__restrict__ tw, G load, S store)
 {
@@ -1392,6 +1392,7 @@ cudaError_t launch_epilogue_views(EpiViews ev, const double *value, double norm,
     int64_t bins = 0;
     for (int i = 0; i < ev.n; ++i) bins += ev.v[i].nbins;
     ev.per = fin_bins_per_block(bins);
+    // (a view has fewer than 2^31 chunks, as a plan has fewer combinations: 5 x 2^28 blocks)
     unsigned blk = 0, fin = 0;
     int threads = ev.per > 1 ? 256 : 32;
     for (int i = 0; i < ev.n; ++i) {
