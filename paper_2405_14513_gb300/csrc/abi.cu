@@ -366,12 +366,12 @@ int init_attributes()
 
 // Transform tile autotuner.  Each transform kernel holds rt rows (or, in
 // Step I's second pass, w columns) of its length M in two shared-memory
-// buffers (Step I in one where two stages do); the best tile depends on M, the kernel and the GPU (large tiles
-// leave one block per SM).  For the forward z pass, the forward row passes
-// and each reduction grid's gather, candidate tiles of 4-64 KB per buffer,
-// and for each grid's second pass strips of 2-32 columns, are timed on
-// scratch buffers holding a sample of the plan's rows (16 planes, 64K z
-// rows, and at most kTuneJobs fields of a grid, evenly spaced over its
+// buffers (Step I in one where two stages do); the best tile depends on M, the
+// kernel and the GPU (large tiles leave one block per SM).  For the forward z
+// pass, the forward row passes and each reduction grid's gather, candidate tiles
+// of 4-64 KB per buffer, and for each grid's second pass strips of 2-32 columns,
+// are timed on scratch buffers holding a sample of the plan's rows (16 planes, 64K
+// z rows, and at most kTuneJobs fields of a grid, evenly spaced over its
 // fields so that their rings, and the launch's size, are those of the
 // estimate), and the fastest is kept.  Rows and columns are transformed
 // independently, so the choice changes the speed, not the results.
