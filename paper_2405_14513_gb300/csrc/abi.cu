@@ -975,11 +975,10 @@ int estimator_estimate_host(bisp_plan *p, const void *delta_host, int batch, dou
     const size_t field = size_t(P.desc.n_g) * P.desc.n_g * P.desc.n_g *
                          (p->precision == BISP_PREC_FP64 ? sizeof(double) : sizeof(float));
     const size_t outb = size_t(P.n_out) * sizeof(double);
-    if (!p->own_ws) {
-        CK(cudaMalloc(&p->own_ws, std::max<size_t>(size_t(P.desc.max_batch) * p->region_bytes, 256)));
-        CK(cudaMalloc(&p->own_in, field * P.desc.max_batch));
-        CK(cudaMalloc((void **)&p->own_out, outb * P.desc.max_batch));
-    }
+    // (the workspace may be there already, from estimator_host_submit)
+    if (!p->own_ws) CK(cudaMalloc(&p->own_ws, std::max<size_t>(size_t(P.desc.max_batch) * p->region_bytes, 256)));
+    if (!p->own_in) CK(cudaMalloc(&p->own_in, field * P.desc.max_batch));
+    if (!p->own_out) CK(cudaMalloc((void **)&p->own_out, outb * P.desc.max_batch));
     CK(cudaMemcpyAsync(p->own_in, delta_host, field * batch, cudaMemcpyHostToDevice, s));
     int st = dispatch_estimate(p, p->own_in, batch, p->own_ws, p->own_out, s);
     if (st) return st;
