@@ -1028,11 +1028,12 @@ k_epi_part_views(const __grid_constant__ EpiViews ev, const double *value, int64
 // added up, then (mode 0) the ratio of Eq. bs_lm2_1 or (mode 1) the sum itself.  The sum
 // of a moment: kFinSplit running sums take the bin's chunks in turn, and are added in
 // order (the same for every LMAX, so that a moment does not depend on the others binned
-// with it).  A bin of at most kFinSplit chunks takes one thread per moment, which comes to
-// the same; one of more takes kFinSplit threads per moment, so that none walks many
-// chunks alone (64^3, up to 80 of them: 14 us).  A block per bin throughout was bound by
-// the launch of empty blocks where bins are many, one thread per bin by its strided
-// stores (64^3, 3e6 bins of 4 moments, the binning: 3.1 ms and 0.52; so 0.24 ms).
+// with it).  They take kFinSplit threads per moment, so that none walks many chunks
+// alone (64^3, up to 80 of them: 14 us); of several bins, those of at most kFinSplit
+// chunks take one thread per moment, which comes to the same.  A block per bin
+// throughout was bound by the launch of empty blocks where bins are many, one thread per
+// bin by its strided stores (64^3, 3e6 bins of 4 moments, the binning: 3.1 ms and 0.52;
+// so 0.24 ms).
 constexpr int kFinSplit = 8;
 template <int LMAX> constexpr int fin_threads()
 {
@@ -1060,8 +1061,9 @@ epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *partial,
             out[o] = v;
         }
     };
-    const int64_t total = (b1 - b0) * nlm_out;
-    bool more = false;                                      // a bin of more chunks seen
+    const bool several = b1 - b0 > 1;
+    const int64_t total = several ? (b1 - b0) * nlm_out : 0;
+    bool more = !several;                                   // a bin of more chunks seen
     for (int64_t t = threadIdx.x; t < total; t += blockDim.x) {
         const int64_t q = t / nlm_out, b = b0 + q, c0 = bin_chunk[b], c1 = bin_chunk[b + 1];
         if (c1 - c0 > kFinSplit) {
@@ -1073,11 +1075,11 @@ epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *partial,
         for (int64_t ch = c0; ch < c1; ++ch) v += partial[ch * NLM + i];
         store(b, i, v);
     }
-    if (!__syncthreads_or(more)) return;
+    if (several && !__syncthreads_or(more)) return;
     const int i = threadIdx.x % P2, sub = threadIdx.x / P2;
     for (int64_t b = b0; b < b1; ++b) {                     // (the same bins for every thread)
         const int64_t c0 = bin_chunk[b], c1 = bin_chunk[b + 1];
-        if (c1 - c0 <= kFinSplit) continue;
+        if (several && c1 - c0 <= kFinSplit) continue;
         double v = 0.0;
         if (sub < kFinSplit) {                              // (a launch may have threads to spare)
             if (i < NLM)
@@ -1090,7 +1092,7 @@ epi_fin(int mode, const int64_t *__restrict__ bin_chunk, const double *partial,
             for (int k = 1; k < kFinSplit; ++k) v += red[k * P2 + i];
             store(b, i, v);
         }
-        __syncthreads();
+        if (several) __syncthreads();
     }
 }
 
