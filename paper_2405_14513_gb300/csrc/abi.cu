@@ -28,12 +28,16 @@ int fail(int code, const std::string &msg)
     return code;
 }
 
+// A failed call returns its status; the error is taken off the runtime's record, where
+// the launches of the next call would find it as theirs.
 #define CK(x)                                                                                     \
     do {                                                                                          \
         cudaError_t e_ = (x);                                                                     \
-        if (e_ != cudaSuccess)                                                                    \
+        if (e_ != cudaSuccess) {                                                                  \
+            cudaGetLastError();                                                                   \
             return fail(e_ == cudaErrorMemoryAllocation ? BISP_OUT_OF_MEMORY : BISP_CUDA_ERROR,   \
                         std::string(#x) + ": " + cudaGetErrorString(e_));                         \
+        }                                                                                         \
     } while (0)
 
 constexpr double kTwoPi = 6.283185307179586476925286766559;

@@ -292,9 +292,11 @@ int sfail(int code, const std::string &msg) { return record_error(code, msg.c_st
 #define SCK(x)                                                                                     \
     do {                                                                                           \
         cudaError_t e_ = (x);                                                                      \
-        if (e_ != cudaSuccess)                                                                     \
+        if (e_ != cudaSuccess) {                                                                   \
+            cudaGetLastError();                                                                    \
             return sfail(e_ == cudaErrorMemoryAllocation ? BISP_OUT_OF_MEMORY : BISP_CUDA_ERROR,   \
                          std::string(#x) + ": " + cudaGetErrorString(e_));                         \
+        }                                                                                          \
     } while (0)
 
 template <typename T>

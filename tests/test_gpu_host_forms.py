@@ -33,3 +33,17 @@ def test_host_forms_in_either_order(first):
     for f in forms if first == "submit" else forms[::-1]:
         assert np.array_equal(f(), want, equal_nan=True)
     plan.close()
+
+
+def test_a_failed_allocation_is_not_the_next_calls_error():
+    """A workspace of terabytes is refused; the estimate after it is not."""
+    ng, L = 64, 640.0
+    plan = api.Plan(ng, L, synth.default_k1_edges(ng, L, 2), 2, 2, 0, precision="mixed", max_batch=65535)
+    assert plan.workspace_bytes(65535) > 1 << 40
+    d = synth.make_field(ng, L, 2).astype(np.float32)[None]
+    with pytest.raises(api.BispError) as e:
+        plan.estimate_host(d)
+    assert e.value.status == 3                       # BISP_OUT_OF_MEMORY
+    B = plan.estimate(torch.from_numpy(d).cuda(), plan.workspace(1)).cpu().numpy()
+    assert np.isfinite(B).any()
+    plan.close()
