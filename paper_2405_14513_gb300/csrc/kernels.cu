@@ -607,7 +607,7 @@ k_fft_cols(typename Cx<R>::T *out, const __grid_constant__ StepGrids gs,
 // bound by its pipe of two lanes a clock and SM, tests each entry (the mask is
 // uniform over the warp) and leaves the others out.
 //
-// FP32 is bound by instruction issue (75% of the slots), of which the FMAs of a
+// FP32 is bound by instruction issue (66-71% of the slots), of which the FMAs of a
 // tile are a third: so the staging and the addresses are kept lean (stages of a
 // constant 64 or 128 points, slot addresses in registers, one piece column per
 // thread, signs on sign bits), and the warps that a unit's tiles leave over take
