@@ -86,8 +86,34 @@ struct DivIter {
 // the L1's wavefronts.)
 __device__ __forceinline__ int spos(int i) { return i ^ ((i >> 3) & 15); }
 
+// a + c x and c x for a constant c of a butterfly.  FINE: FP32 takes it in two parts, c
+// rounded and what that leaves.  A rounded constant is off the same way in every
+// butterfly (1/sqrt(2) by 1.7e-8 of itself, and most points of a transform meet it two
+// or three times), which makes all amplitudes smaller alike, and a triple product takes
+// that three times: with rounded constants the planes of Delta were 4e-8 (24^3) to 7e-8
+// (96^3) too small, so 2e-8 to 5e-8 (what is left comes from the twiddles), and B's
+// errors against 64 bits fell by 6 to 15% (the shell estimator's by 20 to 40%).  Step I
+// keeps to one part: with two there as well the estimate of 384^3 x 10 took 63.5 ms
+// instead of 63.1.
+struct Const {
+    double c;
+    __host__ __device__ constexpr Const operator-() const { return Const{-c}; }
+};
+template <bool FINE> __device__ __forceinline__ float muladd(Const k, float x, float a)
+{
+    const float h = float(k.c), l = float(k.c - double(h));
+    return fmaf(h, x, FINE ? fmaf(l, x, a) : a);
+}
+template <bool FINE> __device__ __forceinline__ double muladd(Const k, double x, double a) { return fma(k.c, x, a); }
+template <bool FINE> __device__ __forceinline__ float mul(Const k, float x)
+{
+    const float h = float(k.c), l = float(k.c - double(h));
+    return FINE ? fmaf(h, x, l * x) : h * x;
+}
+template <bool FINE> __device__ __forceinline__ double mul(Const k, double x) { return k.c * x; }
+
 // DFT of R values in registers, X_m = sum_r v_r exp(-2 pi i r m / R), in place.
-template <int R, typename C> __device__ __forceinline__ void dft(C (&v)[R])
+template <int R, bool FINE, typename C> __device__ __forceinline__ void dft(C (&v)[R])
 {
     using Rr = decltype(v[0].x);
     if constexpr (R == 2) {
@@ -95,12 +121,12 @@ template <int R, typename C> __device__ __forceinline__ void dft(C (&v)[R])
         v[0] = cadd(v[0], v[1]);
         v[1] = t;
     } else if constexpr (R == 3) {
-        const Rr h = Rr(0.86602540378443864676);   // sqrt(3)/2
+        constexpr Const h{0.86602540378443864676};   // sqrt(3)/2
         const Rr sx = v[1].x + v[2].x, sy = v[1].y + v[2].y, dx = v[1].x - v[2].x, dy = v[1].y - v[2].y;
         const Rr mx = v[0].x - Rr(0.5) * sx, my = v[0].y - Rr(0.5) * sy;
         v[0].x += sx; v[0].y += sy;
-        v[1].x = mx + h * dy; v[1].y = my - h * dx;
-        v[2].x = mx - h * dy; v[2].y = my + h * dx;
+        v[1].x = muladd<FINE>(h, dy, mx); v[1].y = muladd<FINE>(-h, dx, my);
+        v[2].x = muladd<FINE>(-h, dy, mx); v[2].y = muladd<FINE>(h, dx, my);
     } else if constexpr (R == 4) {
         const C s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]), s13 = cadd(v[1], v[3]), d13 = csub(v[1], v[3]);
         v[0] = cadd(s02, s13);
@@ -154,7 +180,7 @@ template <int R, typename C> __device__ __forceinline__ void dft(C (&v)[R])
         static_assert(R == 8, "radix");
         // a radix-2 step (pairs r, r + 4; the odd half turned by
         // exp(-2 pi i r / 8)) followed by two 4-point transforms
-        const Rr r2 = Rr(0.70710678118654752440);  // 1/sqrt(2)
+        constexpr Const r2{0.70710678118654752440};  // 1/sqrt(2)
         C e[4], o[4];
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
@@ -163,12 +189,12 @@ template <int R, typename C> __device__ __forceinline__ void dft(C (&v)[R])
         }
         // o_1 exp(-i pi/4), o_2 (-i), o_3 exp(-3 i pi/4)
         const C t1 = o[1], t3 = o[3];
-        o[1].x = (t1.x + t1.y) * r2; o[1].y = (t1.y - t1.x) * r2;
+        o[1].x = mul<FINE>(r2, t1.x + t1.y); o[1].y = mul<FINE>(r2, t1.y - t1.x);
         const Rr x2 = o[2].x;
         o[2].x = o[2].y; o[2].y = -x2;
-        o[3].x = (t3.y - t3.x) * r2; o[3].y = -(t3.x + t3.y) * r2;
-        dft<4>(e);
-        dft<4>(o);
+        o[3].x = mul<FINE>(r2, t3.y - t3.x); o[3].y = -mul<FINE>(r2, t3.x + t3.y);
+        dft<4, FINE>(e);
+        dft<4, FINE>(o);
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
             v[2 * m] = e[m];
@@ -190,7 +216,7 @@ struct FftRows {
 // w = exp(-2 pi i / (R Ns)) (tw: its table [r - 1][k], null in a first
 // stage); get(row, i) and put(row, i, value) read and write an element.  Every
 // index split is a shift, or a shift and a division by the constant F.
-template <typename C, int F, bool ACROSS, int R, typename G, typename S>
+template <typename C, int F, bool ACROSS, bool FINE, int R, typename G, typename S>
 __device__ __forceinline__ void fft_stage(const FftRows &fr, int Ns, int s, const C *__restrict__ tw, G get, S put)
 {
     constexpr int LR = R == 8 ? 3 : (R == 4 ? 2 : (R == 2 ? 1 : 0));
@@ -219,7 +245,7 @@ __device__ __forceinline__ void fft_stage(const FftRows &fr, int Ns, int s, cons
 #pragma unroll
             for (int r = 1; r < R; ++r) v[r] = cmul(v[r], __ldg(tw + (r - 1) * Ns + k));
         }
-        dft<R>(v);
+        dft<R, FINE>(v);
         const int d0 = q * R * Ns + k;
 #pragma unroll
         for (int m = 0; m < R; ++m) put(row, d0 + m * Ns, v[m]);
@@ -234,7 +260,7 @@ __device__ __forceinline__ void fft_stage(const FftRows &fr, int Ns, int s, cons
 // between global memory and the registers a transform of three stages (2^q up to
 // 512, F x 2^q with q up to 6) crosses shared memory twice, not four times.  a, b:
 // buffers of nr rows of stride P.  Every thread of the block takes part.
-template <typename C, int F, bool ACROSS, bool SMEM, typename G, typename S>
+template <typename C, int F, bool ACROSS, bool SMEM, bool FINE, typename G, typename S>
 __device__ __forceinline__ C *fft_block(const FftRows &fr, int P, C *a, C *b, const C *__restrict__ tw, G load, S store)
 {
     auto from = [&](C *x) { return [x, P](int row, int i) { return x[row * P + spos(i)]; }; };
@@ -243,21 +269,21 @@ __device__ __forceinline__ C *fft_block(const FftRows &fr, int P, C *a, C *b, co
     int Ns = R1, s = F > 1 ? 0 : 3;                 // Ns = F 2^s
     if (F == 1 && fr.M == 8) {
         if constexpr (SMEM) {
-            fft_stage<C, F, ACROSS, R1>(fr, 1, 0, nullptr, load, into(a));
+            fft_stage<C, F, ACROSS, FINE, R1>(fr, 1, 0, nullptr, load, into(a));
             __syncthreads();
         } else {
-            fft_stage<C, F, ACROSS, R1>(fr, 1, 0, nullptr, load, store);
+            fft_stage<C, F, ACROSS, FINE, R1>(fr, 1, 0, nullptr, load, store);
         }
         return a;
     }
-    fft_stage<C, F, ACROSS, R1>(fr, 1, 0, nullptr, load, into(a));
+    fft_stage<C, F, ACROSS, FINE, R1>(fr, 1, 0, nullptr, load, into(a));
     __syncthreads();
     const C *w = tw + Twiddles<C>::offset(F);
     for (;; s += 3) {
         const int lg = fr.p - s;                    // what is left: 2^lg
         const C *w8 = w + Twiddles<C>::stage(F, s);
         if (lg > 3) {
-            fft_stage<C, F, ACROSS, 8>(fr, Ns, s, w8, from(a), into(b));
+            fft_stage<C, F, ACROSS, FINE, 8>(fr, Ns, s, w8, from(a), into(b));
             __syncthreads();
             C *t = a;
             a = b;
@@ -266,32 +292,33 @@ __device__ __forceinline__ C *fft_block(const FftRows &fr, int P, C *a, C *b, co
             continue;
         }
         if constexpr (SMEM) {
-            if (lg == 3) fft_stage<C, F, ACROSS, 8>(fr, Ns, s, w8, from(a), into(b));
-            else if (lg == 2) fft_stage<C, F, ACROSS, 4>(fr, Ns, s, w8 + 7 * Ns, from(a), into(b));
-            else fft_stage<C, F, ACROSS, 2>(fr, Ns, s, w8 + 10 * Ns, from(a), into(b));
+            if (lg == 3) fft_stage<C, F, ACROSS, FINE, 8>(fr, Ns, s, w8, from(a), into(b));
+            else if (lg == 2) fft_stage<C, F, ACROSS, FINE, 4>(fr, Ns, s, w8 + 7 * Ns, from(a), into(b));
+            else fft_stage<C, F, ACROSS, FINE, 2>(fr, Ns, s, w8 + 10 * Ns, from(a), into(b));
             __syncthreads();
         } else {
-            if (lg == 3) fft_stage<C, F, ACROSS, 8>(fr, Ns, s, w8, from(a), store);
-            else if (lg == 2) fft_stage<C, F, ACROSS, 4>(fr, Ns, s, w8 + 7 * Ns, from(a), store);
-            else fft_stage<C, F, ACROSS, 2>(fr, Ns, s, w8 + 10 * Ns, from(a), store);
+            if (lg == 3) fft_stage<C, F, ACROSS, FINE, 8>(fr, Ns, s, w8, from(a), store);
+            else if (lg == 2) fft_stage<C, F, ACROSS, FINE, 4>(fr, Ns, s, w8 + 7 * Ns, from(a), store);
+            else fft_stage<C, F, ACROSS, FINE, 2>(fr, Ns, s, w8 + 10 * Ns, from(a), store);
         }
         return b;
     }
 }
 
 // fft_block of rows of length M = 2^q, 3 x 2^q, 5 x 2^q or 7 x 2^q
-// (block-uniform dispatch); ODD = false: of 2^q or 3 x 2^q, the lengths of N_g
-template <typename C, bool ACROSS, bool SMEM, bool ODD, typename G, typename S>
+// (block-uniform dispatch).  STEP1 = false: of 2^q or 3 x 2^q, the lengths of N_g, with
+// the butterflies' constants in two parts (see muladd)
+template <typename C, bool ACROSS, bool SMEM, bool STEP1, typename G, typename S>
 __device__ __forceinline__ C *fft_any(int M, int nr, int lgw, int P, C *a, C *b, const C *__restrict__ tw, G load, S store)
 {
     const FftRows fr{M, __ffs(M) - 1, nr, lgw};
     const int odd = M >> fr.p;
-    if constexpr (ODD) {
-        if (odd == 7) return fft_block<C, 7, ACROSS, SMEM>(fr, P, a, b, tw, load, store);
-        if (odd == 5) return fft_block<C, 5, ACROSS, SMEM>(fr, P, a, b, tw, load, store);
+    if constexpr (STEP1) {
+        if (odd == 7) return fft_block<C, 7, ACROSS, SMEM, false>(fr, P, a, b, tw, load, store);
+        if (odd == 5) return fft_block<C, 5, ACROSS, SMEM, false>(fr, P, a, b, tw, load, store);
     }
-    if (odd == 3) return fft_block<C, 3, ACROSS, SMEM>(fr, P, a, b, tw, load, store);
-    return fft_block<C, 1, ACROSS, SMEM>(fr, P, a, b, tw, load, store);
+    if (odd == 3) return fft_block<C, 3, ACROSS, SMEM, !STEP1>(fr, P, a, b, tw, load, store);
+    return fft_block<C, 1, ACROSS, SMEM, !STEP1>(fr, P, a, b, tw, load, store);
 }
 
 // no store: the transform's result stays in shared memory
