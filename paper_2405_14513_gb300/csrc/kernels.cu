@@ -408,7 +408,8 @@ k_fft_rows_T(const typename Cx<R>::T *in, typename Cx<R>::T *__restrict__ out, i
 // of A + i B, neighbours of one field, so that a field's rounding errors are those
 // of its own size whatever the other fields hold.  A block takes w = 2^lgw pairs: the
 // threads run across them, so that the loads are runs of 2 w elements of a plane, and
-// the rows leave shared memory whole.  Bound by its loads and stores.
+// the rows leave shared memory whole.  Bound by instruction issue (23 fields of 128^3,
+// 0.14 ms: 72% of the slots, shared memory 54%, DRAM 24%; 64^3: 60%, and barriers).
 template <typename R>
 __global__ void __launch_bounds__(256)
 k_fft_z_back(const typename Cx<R>::T *in, R *__restrict__ out, int M, int nkeep, int ntile, int lgw,
